@@ -1219,6 +1219,8 @@ int pxsne_test_stack_limit(pxsne_ctx *c, int32_t entries) {
     const int lim = entries;  // 0: the full stack
     CK(c, cudaMemcpyAsync(&c->sc->stack_limit, &lim, sizeof(int), cudaMemcpyHostToDevice,
                           c->stream));
+    c->stack_limit = lim;
+    drop_graph(c);  // the choice of the traversal kernel depends on it
     CK(c, cudaStreamSynchronize(c->stream));
     return PXSNE_OK;
 }

@@ -19,13 +19,27 @@ constexpr int kMaxL = 14;           // screen up to 2^14 x 2^14 (Morton keys < 2
 constexpr int64_t kMaxN = 1 << 24;  // cell counts are exact floats below 2^24
 constexpr int kTravWarps = 8;       // warps per CTA in the traversal
 constexpr int kTravStack = 48;      // entries per warp; depth <= 3L - 2 <= 40
-// Persistent grids of the forces: CTAs per SM of the traversal and of the
-// attraction that runs beside it on the side stream.  The traversal alone is
-// fastest at four CTAs (all of the SM's registers); at two it leaves room
-// for three of the attraction's CTAs from the start, and the whole
-// 1000-iteration schedule at n = 1M runs 6.6 % faster than with four.
-constexpr int kTravCtasPerSm = 2;
-constexpr int kAttCtasPerSm = 4;
+constexpr int kExactLevel = 8;      // cells of 2^24 ulps and fewer
+// The traversal's kernel by the number of points (late states of 10- and
+// 100-component mixtures, us per iteration).  Below kTravPointTo one warp per
+// point: 46 against 102 at n = 2000 and 108 against 150 at 20,000, but 187
+// against 171 at 40,000, where the points fill the chip by themselves.  From
+// there one point per lane; with geometric centres, which need no records and
+// so leave the registers, two points per lane from kTravPairFrom on (208
+// against 227 at 150,000, 574 against 642 at 400,000; the records of centres
+// of mass cost the gain back: 28.8 against 27.7 ms for 20 iterations at 1M).
+constexpr int64_t kTravPointTo = 32768;
+constexpr int64_t kTravPairFrom = 150000;
+// Persistent grids of the forces: CTAs per SM of the traversal (one and two
+// points per lane) and of the attraction that runs beside it on the side
+// stream.  The traversal leaves registers for the attraction's CTAs from the
+// start: 20 iterations at n = 1M take 29.6, 27.7 and 30.0 ms with 2, 3 and 4
+// traversal CTAs (two points per lane, geometric centres at 300,000, ten
+// iterations: 4.79 ms with two, 4.74 with three, but 5.74 against 6.12 at
+// 400,000), 27.9 with four of the attraction's CTAs instead of five.
+constexpr int kTravCtasPerSm = 3;
+constexpr int kTravPairCtasPerSm = 2;
+constexpr int kAttCtasPerSm = 5;
 constexpr int kPyrK = 5;            // pyramid levels reduced per CTA pass
 
 // Scalars of the iteration that live on the device so that a captured graph
@@ -66,17 +80,20 @@ struct DevScalars {
     i64 mm3[2][6];       // [t & 1] = {min_x, min_y, min_z, max_x, max_y, max_z} of zhat
 };
 
-// The pyramid of cell records.  Cell (l, m) (level l, Morton index m) is at
-// rec_offset(l) + m of two arrays:
-//   rec  float4 {c_hi_x, c_lo_x, c_hi_y, c_lo_y}: the centre of mass S_c / N_c in
-//        ulps, split at bit 16 (c_hi = floor(com) with the low 16 bits cleared,
-//        exact in float; c_lo = the rest, in [0, 65536]; the centre's offset in
-//        its cell is one FP32 quotient, good to about 2^-23 of the cell width),
-//        so that a point's offset z - com is (z_hi - c_hi) + (z_lo - c_lo)
-//        with one rounding;
-//   recn float N_c (exact below 2^24).
-// The record of an empty cell (N_c = 0) is not written each iteration; it
-// keeps an earlier value and is never read.
+// The pyramid of cell records.  Cell (l, m) (level l, Morton index m):
+//   rec   the centre of mass S_c / N_c in ulps, split at bit 16 and negated:
+//         {-c_hi_x, -c_lo_x, -c_hi_y, -c_lo_y} (c_hi = floor(com) with the low
+//         16 bits cleared, exact in float; c_lo = the rest, in [0, 65536]; the
+//         centre's offset in its cell is one FP32 quotient, good to about
+//         2^-23 of the cell width), so that a point's offset z - com is
+//         (z_hi + -c_hi) + (z_lo + -c_lo) with one rounding.  The four siblings
+//         of a node share 64 bytes as a structure of arrays: the float4s at
+//         rec_offset(l) + 4 (m / 4) + {0, 1, 2, 3} hold the siblings' -c_hi_x,
+//         -c_lo_x, -c_hi_y and -c_lo_y, so that two siblings' words are
+//         adjacent and enter the traversal's packed operations as loaded;
+//   recn  float N_c (exact below 2^24) at rec_offset(l) + m.
+// The record of an empty cell (N_c = 0) is not kept up to date; whatever finite
+// centre it holds weighs nothing.
 // rec_offset pads level 0 to four slots so that every group of four siblings
 // starts on a 16-byte boundary.
 __host__ __device__ inline int64_t rec_offset(int l) {
@@ -207,6 +224,7 @@ struct pxsne_ctx {
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     cudaStream_t side = nullptr;          // stream of the attraction (overlaps the traversal)
+    int stack_limit = 0;                  // host copy of DevScalars::stack_limit
     int sms = 0;                          // streaming multiprocessors of the device
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     int device = 0;

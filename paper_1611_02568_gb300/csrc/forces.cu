@@ -1,10 +1,12 @@
 // Forces of the PixelSNE gradient (Eq. grad) on the pixel-aligned tree.
 //
 //   k_bh_traverse  repulsion by Barnes-Hut (Sec. 3.3, Eq. bh_criteria) on the
-//                  dense pyramid, one warp per 64 points of the Morton order
-//                  (two per lane, as packed FP32 pairs); each point keeps its
-//                  own accept/open decisions (lane masks per stack entry), so
-//                  it sees exactly the cells its own depth-first search would
+//                  dense pyramid, one warp per 32 points of the Morton order
+//                  (64 with geometric centres), the siblings as packed FP32
+//                  pairs; each point keeps its own accept/open decisions (lane
+//                  masks per stack entry), so it sees exactly the cells its
+//                  own depth-first search would
+//   k_bh_traverse_pt  the same for small sets, one warp per point
 //   k_attract      attraction over the CSR of P, one warp per row
 //   k_zsum         Z = sum_i Z_i in FP64, fixed summation order
 //   k_kl           Eq. cost_func in FP64 accumulation
@@ -15,20 +17,32 @@
 
 namespace pxsne {
 
-// One warp = 64 points consecutive in Morton order, two per lane (lane l holds
-// points l and l + 32); the two are held and computed as packed FP32 pairs
-// (each component rounded to nearest exactly as the scalar operation).  Each
-// stack entry is a node whose four children are to be tested, with one mask per
-// half of the warp's points marking the points that opened it, so every point
-// sees exactly the cells its own depth-first search would.  A child's record is
-// loaded once for all the warp's points.  The per-child step is branch-free
-// within a level: every lane computes its points' offsets, distances and kernel
-// values, and the accept/open decisions only gate the accumulation and the
-// push.  Children at the leaf level are always accepted (bounded depth, Sec.
-// 4.1) except for a point's own pixel, which is used without the point itself;
-// children above it follow Eq. bh_criteria, and the cell holding a point's own
-// pixel is opened.  A point accumulates its cells in the fixed depth-first order
-// of the tree, so its result does not depend on the warp it shares.
+// One warp = 32 PPL points consecutive in Morton order, PPL (1 or 2) per lane.
+// Each stack
+// entry is a node whose four children are to be tested, with the mask of the
+// lanes whose point opened it, so every point sees exactly the cells its own
+// depth-first search would.  The four children are taken as two packed FP32
+// pairs of siblings: the records keep each sibling group as a structure of
+// arrays (common.cuh), so that a pair's coordinates are two adjacent words of
+// a 16-byte load and enter the packed operations as they are, while a point's
+// own coordinates are broadcast into packed registers once per 32 points.
+// (Each component is rounded to nearest exactly as the scalar operation.)  The
+// per-node step is branch-free within a level: every lane computes its point's
+// offsets, distances and kernel values, and the accept/open decisions only
+// gate the accumulation and the push.  Empty children add zero.  Children at
+// the leaf level are always accepted (bounded depth, Sec. 4.1) except for a
+// point's own pixel, which is used without the point itself; children above
+// it follow Eq. bh_criteria, and the cell holding a point's own pixel is
+// opened.  A point accumulates its cells in the fixed depth-first order of the
+// tree (even and odd siblings in two sums, added at the end), so its result
+// does not depend on the warp it shares.
+// The kernel is bound by its issue slots: about 110 instructions per node of 32
+// points, of which the packed arithmetic and reciprocals are about 35.  The
+// siblings' pairs replaced pairs of a lane's two points, whose cell data had to
+// be broadcast into packed registers for every child (59 instructions per child
+// of 64 points): together with accepting single points early, 20 iterations at
+// n = 1M went from 31.1 to 27.7 ms and five at 70,000 from 1.37 to 0.88 ms (beside
+// the attraction; 64 points per warp and pairs of siblings: 28.8 and 1.18 ms).
 // CENTRE = 0: centre of mass; 1: geometric cell centre.  COUNT = 1 also
 // counts tested and accepted (point, cell) pairs.
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
@@ -45,34 +59,15 @@ __device__ __forceinline__ float rcp1(float x) {
     return r;
 }
 
-// Offset z - c of a lane's two points from the cell's centre: of mass (the
-// split record r), or (CENTRE = 1) the geometric centre, passed in r.x / r.z
-// as exact floats (multiples of 2^16 below level 16), so that z - c =
-// (z_hi - c) + z_lo with one rounding, as for a centre of mass.
-template <int CENTRE>
-__device__ __forceinline__ void cell_offset2(float4 r, float2 zhx, float2 zlx, float2 zhy,
-                                             float2 zly, float2 &dx, float2 &dy) {
-    if (CENTRE == 0) {
-        dx = add2(add2(zhx, bc2(-r.x)), add2(zlx, bc2(-r.y)));
-        dy = add2(add2(zhy, bc2(-r.z)), add2(zly, bc2(-r.w)));
-    } else {
-        dx = add2(add2(zhx, bc2(-r.x)), zlx);
-        dy = add2(add2(zhy, bc2(-r.z)), zly);
-    }
-}
-
-// COUNT: one warp step's (tested, accepted) pairs and the step itself, added
+// COUNT: one (node, non-empty child) step's tested and accepted points, added
 // to the CTA's counters of the child's level by lane 0.
-__device__ __forceinline__ void count_level(u64 *lv, bool me0, bool me1, bool acc0, bool acc1,
-                                            int lane) {
-    const unsigned t = __popc(__ballot_sync(0xffffffffu, me0)) +
-                       __popc(__ballot_sync(0xffffffffu, me1));
-    const unsigned a = __popc(__ballot_sync(0xffffffffu, acc0)) +
-                       __popc(__ballot_sync(0xffffffffu, acc1));
+__device__ __forceinline__ void count_level(u64 *lv, bool me, bool acc, bool step, int lane) {
+    const unsigned t = __popc(__ballot_sync(0xffffffffu, me));
+    const unsigned a = __popc(__ballot_sync(0xffffffffu, acc));
     if (lane == 0) {
         atomicAdd(&lv[0], (u64)t);
         atomicAdd(&lv[1], (u64)a);
-        atomicAdd(&lv[2], 1ull);
+        if (step) atomicAdd(&lv[2], 1ull);
     }
 }
 
@@ -167,203 +162,301 @@ __device__ __forceinline__ void attract_row(int row, int lane, const AttractArgs
     if (lane == 0) a.Fattr[a.aperm[row]] = make_float2(fx, fy);
 }
 
-struct __align__(16) TravEntry {
-    uint32_t node, m0, m1, pad;
+// A point as the traversal holds it: each coordinate's two 16-bit halves
+// (both exact in float, see rec in common.cuh) broadcast into packed pairs.
+struct TravPoint {
+    float2 hx, lx, hy, ly;
+};
+__device__ __forceinline__ TravPoint trav_point(uint2 z) {
+    return TravPoint{bc2((float)(z.x & 0xffff0000u)), bc2((float)(z.x & 0xffffu)),
+                     bc2((float)(z.y & 0xffff0000u)), bc2((float)(z.y & 0xffffu))};
+}
+
+// The four children of one node as two packed pairs (children 0, 1 and 2, 3).
+// CENTRE = 0: the group's records (negated centres of mass), loaded.
+// CENTRE = 1: the geometric centres from the node's corner (exact floats) and
+// width 2^(33 - lc): child ch's centre is a quarter or three quarters across
+// on each axis, so the two pairs share their x offsets.
+template <int CENTRE>
+struct Siblings {
+    float4 hx, lx, hy, ly;  // CENTRE = 1: hx.xy the pair's x, hy.xy the two rows' y
+    __device__ __forceinline__ void load(const float4 *__restrict__ rec, int at, int lc,
+                                         uint32_t m) {
+        if (CENTRE == 0) {
+            hx = __ldg(rec + at);
+            lx = __ldg(rec + at + 1);
+            hy = __ldg(rec + at + 2);
+            ly = __ldg(rec + at + 3);
+        } else {
+            const float wp = __int_as_float((127 + 33 - lc) << 23);
+            const float px = (float)gather_bits16(m) * wp, py = (float)gather_bits16(m >> 1) * wp;
+            hx = make_float4(-fmaf(wp, 0.25f, px), -fmaf(wp, 0.75f, px), 0.f, 0.f);
+            hy = make_float4(-fmaf(wp, 0.25f, py), -fmaf(wp, 0.75f, py), 0.f, 0.f);
+        }
+    }
+    // Offsets z - c (one rounding) of the point from pair p's two centres.
+    __device__ __forceinline__ void offset(int p, const TravPoint &z, float2 &dx, float2 &dy) const {
+        if (CENTRE == 0) {
+            const float2 cx = p ? make_float2(hx.z, hx.w) : make_float2(hx.x, hx.y);
+            const float2 ex = p ? make_float2(lx.z, lx.w) : make_float2(lx.x, lx.y);
+            const float2 cy = p ? make_float2(hy.z, hy.w) : make_float2(hy.x, hy.y);
+            const float2 ey = p ? make_float2(ly.z, ly.w) : make_float2(ly.x, ly.y);
+            dx = add2(add2(z.hx, cx), add2(z.lx, ex));
+            dy = add2(add2(z.hy, cy), add2(z.ly, ey));
+        } else {
+            dx = add2(add2(z.hx, make_float2(hx.x, hx.y)), z.lx);
+            dy = add2(add2(z.hy, bc2(p ? hy.y : hy.x)), z.ly);
+        }
+    }
 };
 
-template <int CENTRE, int COUNT, bool OWN>
-__global__ void __launch_bounds__(kTravWarps * 32, 4)
+// A stack entry: the record offset of a node's sibling group of children
+// (rec_offset(lc) + 4 m, lc their level, m the node's Morton index; a multiple
+// of 4) in the low 28 bits as a count of groups, lc above, and for each of a
+// lane's PPL points the mask of the lanes whose point opens the node.
+template <int PPL>
+struct TravEntry;
+template <>
+struct __align__(8) TravEntry<1> {
+    uint32_t node, m[1];
+};
+template <>
+struct __align__(16) TravEntry<2> {
+    uint32_t node, m[2], pad;
+};
+
+template <int CENTRE, int COUNT, bool OWN, int PPL>
+__global__ void __launch_bounds__(kTravWarps * 32, PPL == 1 ? 4 : 3)
     k_bh_traverse(int n, int L, const uint2 *__restrict__ z, const uint32_t *__restrict__ perm,
                   const float4 *__restrict__ rec, const float *__restrict__ recn,
                   DevScalars *sc, float2 *__restrict__ Frep, float *__restrict__ Zi) {
-    // stack entry: (level << 28) | Morton index of a node, and for each half of
-    // the warp's points the mask of the lanes whose point opens it
-    __shared__ TravEntry s_stk[kTravWarps][kTravStack];
+    __shared__ TravEntry<PPL> s_stk[kTravWarps][kTravStack];
     __shared__ float s_T[kMaxL + 2];
-    __shared__ int s_off[kMaxL + 2];
     const int stk_lim = sc->stack_limit > 0 ? min(max(sc->stack_limit, 4), kTravStack) : kTravStack;
     // COUNT: (tested, accepted, warp steps) by level of the child
     __shared__ u64 s_lv[COUNT ? kMaxL + 2 : 1][3];
     if (threadIdx.x < kMaxL + 2) {
         s_T[threadIdx.x] = sc->T[threadIdx.x];
-        s_off[threadIdx.x] = threadIdx.x <= L ? (int)rec_offset(threadIdx.x) : 0;
         if (COUNT) s_lv[threadIdx.x][0] = s_lv[threadIdx.x][1] = s_lv[threadIdx.x][2] = 0ull;
     }
     __syncthreads();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int F = 32 - L;
     const float2 sf0 = bc2(sc->sf[0]), sf1 = bc2(sc->sf[1]);
+    const unsigned before = (1u << lane) - 1u;
     uint32_t n_acc = 0u, n_tst = 0u, n_stp = 0u, n_nod = 0u;
-    TravEntry *stk = s_stk[w];
-    // Each warp takes the next 64 points of the Morton order until none are
+    TravEntry<PPL> *stk = s_stk[w];
+    // Each warp takes the next 32 PPL points of the Morton order until none are
     // left: a warp whose points are cheap moves on instead of idling until
     // the slowest warp of its CTA is done.
     for (;;) {
         unsigned chunk = 0u;
         if (lane == 0) chunk = atomicAdd(&sc->trav_next, 1u);
         chunk = __shfl_sync(0xffffffffu, chunk, 0);
-        if ((int64_t)chunk * 64 >= n) break;
-        const int base = (int)chunk * 64;
-        const int idx0 = base + lane, idx1 = base + 32 + lane;
-        const bool valid0 = idx0 < n, valid1 = idx1 < n;
-        const unsigned act0 = __ballot_sync(0xffffffffu, valid0);
-        const unsigned act1 = __ballot_sync(0xffffffffu, valid1);
-        const uint32_t i0 = valid0 ? perm[idx0] : 0u, i1 = valid1 ? perm[idx1] : 0u;
-        const uint2 z0 = z[i0], z1 = z[i1];
-        const uint32_t mi0 = morton2(z0.x >> F, z0.y >> F), mi1 = morton2(z1.x >> F, z1.y >> F);
-        // z split at bit 16, both halves exact in float (see rec in common.cuh)
-        const float2 zhx = make_float2((float)(z0.x & 0xffff0000u), (float)(z1.x & 0xffff0000u));
-        const float2 zlx = make_float2((float)(z0.x & 0xffffu), (float)(z1.x & 0xffffu));
-        const float2 zhy = make_float2((float)(z0.y & 0xffff0000u), (float)(z1.y & 0xffff0000u));
-        const float2 zly = make_float2((float)(z0.y & 0xffffu), (float)(z1.y & 0xffffu));
-        float2 fx = bc2(0.f), fy = bc2(0.f), zs = bc2(0.f);
+        if ((int64_t)chunk * (32 * PPL) >= n) break;
+        unsigned act[PPL];
+        uint32_t i[PPL], mi[PPL];
+        TravPoint pt[PPL];
+        float2 fx[PPL], fy[PPL], zs[PPL];
+#pragma unroll
+        for (int a = 0; a < PPL; a++) {
+            const int idx = (int)chunk * (32 * PPL) + 32 * a + lane;
+            act[a] = __ballot_sync(0xffffffffu, idx < n);
+            i[a] = idx < n ? perm[idx] : 0u;
+            const uint2 zi = z[i[a]];
+            mi[a] = morton2(zi.x >> F, zi.y >> F);
+            pt[a] = trav_point(zi);
+            fx[a] = fy[a] = zs[a] = bc2(0.f);
+        }
 
-        // The root contains every point: start with its four children.
-        if (lane == 0) stk[0] = TravEntry{0u, act0, act1, 0u};  // (level 0 << 28) | morton 0
+        // The root contains every point: start with its four children (level
+        // 1, group 1 of the records).
+        if (lane == 0) {
+            TravEntry<PPL> e;
+            e.node = (1u << 28) | 1u;
+#pragma unroll
+            for (int a = 0; a < PPL; a++) e.m[a] = act[a];
+            stk[0] = e;
+        }
         int sp = 1;
         __syncwarp();
         bool overflow = false;
         while (sp > 0) {
             sp--;
-            TravEntry top = stk[sp];
+            TravEntry<PPL> top = stk[sp];
             __syncwarp();
             // the entry is the same for every lane: taken from lane 0, so that
             // the node, its level and addresses are known to be warp-uniform
             top.node = __shfl_sync(0xffffffffu, top.node, 0);
-            top.m0 = __shfl_sync(0xffffffffu, top.m0, 0);
-            top.m1 = __shfl_sync(0xffffffffu, top.m1, 0);
-            const uint32_t node = top.node;
-            const int lc = (int)(node >> 28) + 1;  // level of the children
-            const uint32_t m0 = (node & 0x0fffffffu) << 2;
-            const int at = s_off[lc] + (int)m0;
-            const float4 nv = __ldg(reinterpret_cast<const float4 *>(recn + at));
-            // the four children's records are requested together with their
-            // counts (one latency per node instead of two)
-            float4 rr[4];
-            if (CENTRE == 0) {
+            bool me[PPL];
 #pragma unroll
-                for (int ch = 0; ch < 4; ch++) rr[ch] = __ldg(rec + at + ch);
-            } else {
-                // geometric centres: the node's corner (exact floats) and width
-                // 2^(33 - lc); child ch's centre is a quarter or three quarters
-                // across on each axis
-                const uint32_t pm = node & 0x0fffffffu;
-                const float wp = __int_as_float((127 + 33 - lc) << 23);
-                const float px = (float)gather_bits16(pm) * wp, py = (float)gather_bits16(pm >> 1) * wp;
-#pragma unroll
-                for (int ch = 0; ch < 4; ch++)
-                    rr[ch] = make_float4(fmaf(wp, (ch & 1) ? 0.75f : 0.25f, px), 0.f,
-                                         fmaf(wp, (ch & 2) ? 0.75f : 0.25f, py), 0.f);
+            for (int a = 0; a < PPL; a++) {
+                top.m[a] = __shfl_sync(0xffffffffu, top.m[a], 0);
+                me[a] = (top.m[a] >> lane) & 1u;
             }
-            const bool me0 = (top.m0 >> lane) & 1u, me1 = (top.m1 >> lane) & 1u;
-            const float Nc[4] = {nv.x, nv.y, nv.z, nv.w};
+            const uint32_t grp = top.node & 0x0fffffffu;
+            const int lc = (int)(top.node >> 28);  // level of the children
+            // the counts and the four children's records are requested
+            // together (one latency per node)
+            const float4 nv = __ldg(reinterpret_cast<const float4 *>(recn) + grp);
+            Siblings<CENTRE> sib;
+            // the node's Morton index, from rec_offset(lc) = (4^lc + 8) / 3
+            const uint32_t m = (CENTRE == 1 || OWN || COUNT) ? grp - (uint32_t)(rec_offset(lc) >> 2) : 0u;
+            sib.load(rec, (int)(4u * grp), lc, m);
             if (COUNT) {
                 n_nod++;
                 n_stp += (nv.x != 0.f) + (nv.y != 0.f) + (nv.z != 0.f) + (nv.w != 0.f);
             }
             if (lc == L) {
-                const uint32_t mine0 = mi0, mine1 = mi1;  // own pixels
+                const uint32_t g0 = (uint32_t)(rec_offset(L) >> 2);
+                bool own[PPL], any = false;
 #pragma unroll
-                for (int ch = 0; ch < 4; ch++) {
-                    const float N = Nc[ch];
-                    if (N == 0.f) continue;
-                    const uint32_t mc = m0 + ch;
-                    const float4 r = rr[ch];
-                    float2 dx, dy;
-                    cell_offset2<CENTRE>(r, zhx, zlx, zhy, zly, dx, dy);
-                    const bool own0 = me0 && (mine0 == mc), own1 = me1 && (mine1 == mc);
-                    float2 Nf = bc2(N);
-                    if (__any_sync(0xffffffffu, own0 || own1)) {  // own pixel: take the point out
-                        if (own0) {
-                            Nf.x = N - 1.0f;
-                            if (CENTRE == 0 && N > 1.0f) {
-                                const float k = N / Nf.x;
-                                dx.x *= k;
-                                dy.x *= k;
+                for (int a = 0; a < PPL; a++) {
+                    own[a] = me[a] && (mi[a] >> 2) + g0 == grp;
+                    any |= own[a];
+                }
+                const bool any_own = __any_sync(0xffffffffu, any);
+#pragma unroll
+                for (int p = 0; p < 2; p++) {
+                    const float2 N0 = p ? make_float2(nv.z, nv.w) : make_float2(nv.x, nv.y);
+                    if (N0.x + N0.y == 0.f) continue;
+#pragma unroll
+                    for (int a = 0; a < PPL; a++) {
+                        float2 N = N0, dx, dy;
+                        sib.offset(p, pt[a], dx, dy);
+                        if (any_own) {  // a point's own pixel: take the point out
+                            const bool o0 = own[a] && (mi[a] & 3u) == 2u * p;
+                            const bool o1 = own[a] && (mi[a] & 3u) == 2u * p + 1u;
+                            if (o0) {
+                                const float r = N.x - 1.0f;
+                                if (CENTRE == 0 && r > 0.0f) {
+                                    const float k = N.x / r;
+                                    dx.x *= k;
+                                    dy.x *= k;
+                                }
+                                N.x = r;
+                            }
+                            if (o1) {
+                                const float r = N.y - 1.0f;
+                                if (CENTRE == 0 && r > 0.0f) {
+                                    const float k = N.y / r;
+                                    dx.y *= k;
+                                    dy.y *= k;
+                                }
+                                N.y = r;
                             }
                         }
-                        if (own1) {
-                            Nf.y = N - 1.0f;
-                            if (CENTRE == 0 && N > 1.0f) {
-                                const float k = N / Nf.y;
-                                dx.y *= k;
-                                dy.y *= k;
+                        dx = mul2(dx, sf0);
+                        dy = mul2(dy, sf1);
+                        const float2 d2 = fma2(dx, dx, mul2(dy, dy));
+                        if (COUNT) {
+                            const bool a0 = me[a] && N.x > 0.f, a1 = me[a] && N.y > 0.f;
+                            if (N0.x != 0.f) {
+                                n_tst += me[a];
+                                n_acc += a0;
+                                count_level(s_lv[lc], me[a], a0, a == 0, lane);
+                            }
+                            if (N0.y != 0.f) {
+                                n_tst += me[a];
+                                n_acc += a1;
+                                count_level(s_lv[lc], me[a], a1, a == 0, lane);
                             }
                         }
+                        const float2 w1 = add2(bc2(1.0f), d2);
+                        const float2 q = make_float2(rcp1(w1.x), rcp1(w1.y));
+                        const float2 Nq =
+                            mul2(make_float2(me[a] ? N.x : 0.0f, me[a] ? N.y : 0.0f), q);
+                        zs[a] = add2(zs[a], Nq);
+                        const float2 Nq2 = mul2(Nq, q);
+                        fx[a] = fma2(Nq2, dx, fx[a]);
+                        fy[a] = fma2(Nq2, dy, fy[a]);
                     }
-                    dx = mul2(dx, sf0);
-                    dy = mul2(dy, sf1);
-                    const float2 d2 = fma2(dx, dx, mul2(dy, dy));
-                    const bool acc0 = me0 && (Nf.x > 0.f), acc1 = me1 && (Nf.y > 0.f);
-                    if (COUNT) {
-                        n_tst += (me0 ? 1u : 0u) + (me1 ? 1u : 0u);
-                        n_acc += (acc0 ? 1u : 0u) + (acc1 ? 1u : 0u);
-                        count_level(s_lv[lc], me0, me1, acc0, acc1, lane);
-                    }
-                    const float2 w1 = add2(bc2(1.0f), d2);
-                    const float2 q = make_float2(rcp1(w1.x), rcp1(w1.y));
-                    const float2 Nq = mul2(make_float2(acc0 ? Nf.x : 0.0f, acc1 ? Nf.y : 0.0f), q);
-                    zs = add2(zs, Nq);
-                    const float2 Nq2 = mul2(Nq, q);
-                    fx = fma2(Nq2, dx, fx);
-                    fy = fma2(Nq2, dy, fy);
                 }
             } else {
+                // Eq. bh_criteria's threshold on d^2.  A cell that holds one
+                // point stands for it exactly from level kExactLevel on (its
+                // offset in the cell is below 2^24 and so exact), so opening it
+                // down to its pixel would end in the same term: it is accepted
+                // at once by every point but the one in it, whose d^2 is 0
+                // (threshold 0).  Empty cells add nothing.
                 const float Tl = s_T[lc];
-                // a point's own cell: opened by the criterion itself when theta < 1
-                // (the point and the centre of mass lie in the cell, so d <= r_c <
-                // r_c / theta); tested explicitly otherwise
-                const int sh = 2 * (L - lc);
-                const uint32_t mine0 = OWN ? mi0 >> sh : 0xffffffffu, mine1 = OWN ? mi1 >> sh : 0xffffffffu;
+                const float few = (CENTRE == 0 && lc >= kExactLevel) ? 1.0f : 0.0f;
                 // room for the (at most four) entries this node may push
                 if (sp + 4 > stk_lim) {
                     overflow = true;
                     break;
                 }
+                unsigned acc[PPL][4];
 #pragma unroll
-                for (int ch = 0; ch < 4; ch++) {
-                    const float N = Nc[ch];
-                    if (N == 0.f) continue;
-                    const uint32_t mc = m0 + ch;
-                    const float4 r = rr[ch];
-                    float2 dx, dy;
-                    cell_offset2<CENTRE>(r, zhx, zlx, zhy, zly, dx, dy);
-                    dx = mul2(dx, sf0);
-                    dy = mul2(dy, sf1);
-                    const float2 d2 = fma2(dx, dx, mul2(dy, dy));
-                    const bool far0 = (d2.x > Tl) && (!OWN || mine0 != mc);
-                    const bool far1 = (d2.y > Tl) && (!OWN || mine1 != mc);
-                    const bool acc0 = me0 && far0, acc1 = me1 && far1;
-                    if (COUNT) {
-                        n_tst += (me0 ? 1u : 0u) + (me1 ? 1u : 0u);
-                        n_acc += (acc0 ? 1u : 0u) + (acc1 ? 1u : 0u);
-                        count_level(s_lv[lc], me0, me1, acc0, acc1, lane);
+                for (int p = 0; p < 2; p++) {
+                    const float2 N = p ? make_float2(nv.z, nv.w) : make_float2(nv.x, nv.y);
+                    const float2 tb = fma2(N, bc2(1e30f), bc2(-1e30f * few));
+                    const float T0 = fminf(tb.x, Tl), T1 = fminf(tb.y, Tl);
+#pragma unroll
+                    for (int a = 0; a < PPL; a++) {
+                        // a point's own cell: opened by the criterion itself when
+                        // theta < 1 (the point and the centre of mass lie in the
+                        // cell, so d <= r_c < r_c / theta); tested explicitly
+                        // otherwise
+                        const uint32_t mine = OWN ? mi[a] >> (2 * (L - lc)) : 0u;
+                        float2 dx, dy;
+                        sib.offset(p, pt[a], dx, dy);
+                        dx = mul2(dx, sf0);
+                        dy = mul2(dy, sf1);
+                        const float2 d2 = fma2(dx, dx, mul2(dy, dy));
+                        const bool a0 = me[a] && d2.x > T0 && (!OWN || mine != 4u * m + 2u * p);
+                        const bool a1 = me[a] && d2.y > T1 && (!OWN || mine != 4u * m + 2u * p + 1u);
+                        if (COUNT) {
+                            if (N.x != 0.f) {
+                                n_tst += me[a];
+                                n_acc += a0;
+                                count_level(s_lv[lc], me[a], a0, a == 0, lane);
+                            }
+                            if (N.y != 0.f) {
+                                n_tst += me[a];
+                                n_acc += a1;
+                                count_level(s_lv[lc], me[a], a1, a == 0, lane);
+                            }
+                        }
+                        const float2 w1 = add2(bc2(1.0f), d2);
+                        const float2 q = make_float2(rcp1(w1.x), rcp1(w1.y));
+                        const float2 Nq = mul2(make_float2(a0 ? N.x : 0.0f, a1 ? N.y : 0.0f), q);
+                        zs[a] = add2(zs[a], Nq);
+                        const float2 Nq2 = mul2(Nq, q);
+                        fx[a] = fma2(Nq2, dx, fx[a]);
+                        fy[a] = fma2(Nq2, dy, fy[a]);
+                        acc[a][2 * p] = __ballot_sync(0xffffffffu, a0);
+                        acc[a][2 * p + 1] = __ballot_sync(0xffffffffu, a1);
                     }
-                    const float2 w1 = add2(bc2(1.0f), d2);
-                    const float2 q = make_float2(rcp1(w1.x), rcp1(w1.y));
-                    const float2 Nq = mul2(make_float2(acc0 ? N : 0.0f, acc1 ? N : 0.0f), q);
-                    zs = add2(zs, Nq);
-                    const float2 Nq2 = mul2(Nq, q);
-                    fx = fma2(Nq2, dx, fx);
-                    fy = fma2(Nq2, dy, fy);
-                    const unsigned ob0 = __ballot_sync(0xffffffffu, me0 && !far0);
-                    const unsigned ob1 = __ballot_sync(0xffffffffu, me1 && !far1);
-                    // written in any case above the top; kept if some point opens it
-                    if (lane == 0) stk[sp] = TravEntry{((uint32_t)lc << 28) | mc, ob0, ob1, 0u};
-                    sp += (ob0 | ob1) != 0u;
                 }
+                // lanes 0..3 push the children that some point opens
+                const float na = (lane & 1) ? nv.y : nv.x, nc = (lane & 1) ? nv.w : nv.z;
+                const float nn = (lane & 2) ? nc : na;
+                TravEntry<PPL> e;
+                unsigned some = 0u;
+#pragma unroll
+                for (int a = 0; a < PPL; a++) {
+                    const unsigned oa = (lane & 1) ? acc[a][1] : acc[a][0];
+                    const unsigned oc = (lane & 1) ? acc[a][3] : acc[a][2];
+                    e.m[a] = top.m[a] & ~((lane & 2) ? oc : oa);
+                    some |= e.m[a];
+                }
+                // the group of child c's children (rec_offset(l + 1) = 4
+                // rec_offset(l) - 8): 4 grp - 2 + c, one level down
+                e.node = ((uint32_t)(lc + 1) << 28) | (4u * grp - 2u + (uint32_t)lane);
+                const bool push = lane < 4 && some != 0u && nn > few;
+                const unsigned pm = __ballot_sync(0xffffffffu, push);
+                if (push) stk[sp + __popc(pm & before)] = e;
+                sp += __popc(pm);
             }
             __syncwarp();
-            if (overflow) break;
         }
-        if (valid0) {
-            Frep[i0] = make_float2(fx.x, fy.x);
-            Zi[i0] = zs.x;
-        }
-        if (valid1) {
-            Frep[i1] = make_float2(fx.y, fy.y);
-            Zi[i1] = zs.y;
-        }
+#pragma unroll
+        for (int a = 0; a < PPL; a++)
+            if ((act[a] >> lane) & 1u) {
+                Frep[i[a]] = make_float2(fx[a].x + fx[a].y, fy[a].x + fy[a].y);
+                Zi[i[a]] = zs[a].x + zs[a].y;
+            }
         if (overflow && lane == 0) atomicOr(&sc->err, (unsigned)PXSNE_DEVERR_STACK);
         __syncwarp();
     }
@@ -383,6 +476,162 @@ __global__ void __launch_bounds__(kTravWarps * 32, 4)
         for (int o = 16; o > 0; o >>= 1) {
             n_acc += __shfl_xor_sync(0xffffffffu, n_acc, o);
             n_tst += __shfl_xor_sync(0xffffffffu, n_tst, o);
+        }
+        if (lane == 0) {
+            atomicAdd(&sc->n_accept, (u64)n_acc);
+            atomicAdd(&sc->n_test, (u64)n_tst);
+            atomicAdd(&sc->n_steps, (u64)n_stp);
+            atomicAdd(&sc->n_nodes, (u64)n_nod);
+        }
+    }
+}
+
+// The traversal of small sets, one warp per point: with a few thousand points
+// the kernel above has a few dozen warps on the whole chip, each walking its
+// tree one node after another, and the time is that chain's latency.  Here the
+// lanes take up to 32 of the point's open nodes at a time (all four children
+// of a node as two packed pairs), so that the chain is about one step per
+// level: 5 us instead of 55 at n = 2000 (20 iterations 0.93 ms, 2.05 with the
+// kernel above).  The open nodes wait in a ring in shared memory, taken oldest first
+// (breadth first); above kPtDeep waiting nodes the newest are taken first,
+// which bounds the ring: such a step takes the 32 newest, of level l or deeper,
+// and puts at most 128 of level l + 1 or deeper in their place, so that a
+// node of level l waits at most 128 l places above kPtDeep + 96.  What a lane
+// sums, and in which order, depends on the point's own walk only.
+constexpr int kPtWarps = 4;
+constexpr int kPtRing = 2048;
+constexpr int kPtDeep = kPtRing - 128 * kMaxL - 128;
+static_assert(kPtDeep >= 128, "ring of the point traversal");
+template <int CENTRE, int COUNT, bool OWN>
+__global__ void __launch_bounds__(kPtWarps * 32)
+    k_bh_traverse_pt(int n, int L, const uint2 *__restrict__ z, const uint32_t *__restrict__ perm,
+                     const float4 *__restrict__ rec, const float *__restrict__ recn,
+                     DevScalars *sc, float2 *__restrict__ Frep, float *__restrict__ Zi) {
+    __shared__ uint32_t s_ring[kPtWarps][kPtRing];
+    __shared__ float s_T[kMaxL + 2];
+    if (threadIdx.x < kMaxL + 2) s_T[threadIdx.x] = sc->T[threadIdx.x];
+    __syncthreads();
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int idx = blockIdx.x * kPtWarps + w;
+    if (idx >= n) return;  // whole warps; no block barrier follows
+    uint32_t *ring = s_ring[w];
+    const int F = 32 - L;
+    const float2 sf0 = bc2(sc->sf[0]), sf1 = bc2(sc->sf[1]);
+    const unsigned before = (1u << lane) - 1u;
+    const uint32_t g0 = (uint32_t)(rec_offset(L) >> 2);
+    const uint32_t i = perm[idx];
+    const uint2 zi = z[i];
+    const uint32_t mi = morton2(zi.x >> F, zi.y >> F);
+    const TravPoint pt = trav_point(zi);
+    float2 fx = bc2(0.f), fy = bc2(0.f), zs = bc2(0.f);
+    uint32_t n_acc = 0u, n_tst = 0u, n_stp = 0u, n_nod = 0u;
+    if (lane == 0) ring[0] = (1u << 28) | 1u;
+    uint32_t head = 0u, size = 1u;
+    __syncwarp();
+    while (size > 0u) {
+        const uint32_t k = min(size, 32u);
+        const uint32_t at = size <= (uint32_t)kPtDeep ? head : head + size - k;
+        if (size <= (uint32_t)kPtDeep) head += k;
+        size -= k;
+        const bool act = (uint32_t)lane < k;
+        const uint32_t node = act ? ring[(at + lane) & (kPtRing - 1)] : (1u << 28) | 1u;
+        __syncwarp();
+        const uint32_t grp = node & 0x0fffffffu;
+        const int lc = (int)(node >> 28);
+        const bool leaf = lc == L;
+        float4 nv = __ldg(reinterpret_cast<const float4 *>(recn) + grp);
+        if (!act) nv = make_float4(0.f, 0.f, 0.f, 0.f);
+        Siblings<CENTRE> sib;
+        const uint32_t m = (CENTRE == 1 || OWN || COUNT) ? grp - (uint32_t)(rec_offset(lc) >> 2) : 0u;
+        sib.load(rec, (int)(4u * grp), lc, m);
+        const float Tl = s_T[lc];
+        const float few = (CENTRE == 0 && lc >= kExactLevel) ? 1.0f : 0.0f;
+        const bool own = leaf && act && (mi >> 2) + g0 == grp;
+        const uint32_t mine = OWN ? mi >> (2 * (L - lc)) : 0u;
+        bool open[4];
+        if (COUNT && act) n_nod++;
+#pragma unroll
+        for (int p = 0; p < 2; p++) {
+            const float2 N0 = p ? make_float2(nv.z, nv.w) : make_float2(nv.x, nv.y);
+            float2 N = N0, dx, dy;
+            sib.offset(p, pt, dx, dy);
+            if (own) {  // the point's own pixel: take the point out
+                const bool second = mi & 1u;
+                if (((mi >> 1) & 1u) == (uint32_t)p) {
+                    const float Nc = second ? N.y : N.x, r = Nc - 1.0f;
+                    const float kk = (CENTRE == 0 && r > 0.0f) ? Nc / r : 1.0f;
+                    if (second) {
+                        N.y = r;
+                        dx.y *= kk;
+                        dy.y *= kk;
+                    } else {
+                        N.x = r;
+                        dx.x *= kk;
+                        dy.x *= kk;
+                    }
+                }
+            }
+            dx = mul2(dx, sf0);
+            dy = mul2(dy, sf1);
+            const float2 d2 = fma2(dx, dx, mul2(dy, dy));
+            // thresholds as above; a pixel is always accepted
+            const float2 tb = fma2(N0, bc2(1e30f), bc2(-1e30f * few));
+            const float T0 = leaf ? -1.0f : fminf(tb.x, Tl), T1 = leaf ? -1.0f : fminf(tb.y, Tl);
+            const bool a0 = d2.x > T0 && (!OWN || leaf || mine != 4u * m + 2u * p);
+            const bool a1 = d2.y > T1 && (!OWN || leaf || mine != 4u * m + 2u * p + 1u);
+            if (COUNT) {
+                const bool f0 = N0.x != 0.f, f1 = N0.y != 0.f;
+                const uint32_t ts = (f0 ? 1u : 0u) + (f1 ? 1u : 0u);
+                const uint32_t ac = (f0 && a0 && N.x > 0.f ? 1u : 0u) + (f1 && a1 && N.y > 0.f ? 1u : 0u);
+                n_tst += ts;
+                n_acc += ac;
+                n_stp += ts;
+                if (ts) {
+                    atomicAdd(&sc->lvl[lc][0], (u64)ts);
+                    atomicAdd(&sc->lvl[lc][2], (u64)ts);
+                }
+                if (ac) atomicAdd(&sc->lvl[lc][1], (u64)ac);
+            }
+            const float2 w1 = add2(bc2(1.0f), d2);
+            const float2 q = make_float2(rcp1(w1.x), rcp1(w1.y));
+            const float2 Nq = mul2(make_float2(a0 ? N.x : 0.0f, a1 ? N.y : 0.0f), q);
+            zs = add2(zs, Nq);
+            const float2 Nq2 = mul2(Nq, q);
+            fx = fma2(Nq2, dx, fx);
+            fy = fma2(Nq2, dy, fy);
+            // (a pixel is never opened, whatever a non-finite distance says)
+            open[2 * p] = !a0 && !leaf && N0.x > few;
+            open[2 * p + 1] = !a1 && !leaf && N0.y > few;
+        }
+        const uint32_t child = ((uint32_t)(lc + 1) << 28) | (4u * grp - 2u);
+        uint32_t end = head + size;
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+            const unsigned b = __ballot_sync(0xffffffffu, open[c]);
+            if (open[c]) ring[(end + __popc(b & before)) & (kPtRing - 1)] = child + (uint32_t)c;
+            end += __popc(b);
+        }
+        size = end - head;
+        __syncwarp();
+    }
+    float vx = fx.x + fx.y, vy = fy.x + fy.y, vz = zs.x + zs.y;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        vx += __shfl_xor_sync(0xffffffffu, vx, o);
+        vy += __shfl_xor_sync(0xffffffffu, vy, o);
+        vz += __shfl_xor_sync(0xffffffffu, vz, o);
+    }
+    if (lane == 0) {
+        Frep[i] = make_float2(vx, vy);
+        Zi[i] = vz;
+    }
+    if (COUNT) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            n_acc += __shfl_xor_sync(0xffffffffu, n_acc, o);
+            n_tst += __shfl_xor_sync(0xffffffffu, n_tst, o);
+            n_stp += __shfl_xor_sync(0xffffffffu, n_stp, o);
+            n_nod += __shfl_xor_sync(0xffffffffu, n_nod, o);
         }
         if (lane == 0) {
             atomicAdd(&sc->n_accept, (u64)n_acc);
@@ -502,15 +751,30 @@ static AttractArgs attract_args(const pxsne_ctx *c) {
     return AttractArgs{c->rp2, c->col2, c->val2, c->zp, c->aperm, c->Fattr};
 }
 
-// One wave of kTravCtasPerSm CTAs per SM (at most the four the launch bounds
-// allow), fewer when the points fill fewer.
-template <int CENTRE, int COUNT, bool OWN>
+// One wave of a few CTAs per SM (kTravCtasPerSm), fewer when the points fill
+// fewer.
+template <int CENTRE, int COUNT, bool OWN, int PPL>
 static void traverse_as(pxsne_ctx *c, cudaStream_t st) {
     const int n = (int)c->n;
-    const int per_block = kTravWarps * 64;
-    const int blocks = std::min((n + per_block - 1) / per_block, kTravCtasPerSm * std::max(c->sms, 1));
-    k_bh_traverse<CENTRE, COUNT, OWN><<<blocks, kTravWarps * 32, 0, st>>>(
+    const int per_block = kTravWarps * 32 * PPL;
+    const int ctas = PPL == 1 ? kTravCtasPerSm : kTravPairCtasPerSm;
+    const int blocks = std::min((n + per_block - 1) / per_block, ctas * std::max(c->sms, 1));
+    k_bh_traverse<CENTRE, COUNT, OWN, PPL><<<blocks, kTravWarps * 32, 0, st>>>(
         n, c->L, c->z, c->perm, c->rec, c->recn, c->sc, c->Frep, c->Zi);
+}
+
+template <int CENTRE, int COUNT, bool OWN>
+static void traverse_n(pxsne_ctx *c, cudaStream_t st) {
+    // (the stack test hook is the other kernels')
+    if (c->n < kTravPointTo && c->stack_limit == 0) {
+        const int n = (int)c->n;
+        k_bh_traverse_pt<CENTRE, COUNT, OWN><<<(n + kPtWarps - 1) / kPtWarps, kPtWarps * 32, 0, st>>>(
+            n, c->L, c->z, c->perm, c->rec, c->recn, c->sc, c->Frep, c->Zi);
+    } else if (CENTRE == 0 || c->n < kTravPairFrom) {
+        traverse_as<CENTRE, COUNT, OWN, 1>(c, st);
+    } else {
+        traverse_as<CENTRE, COUNT, OWN, CENTRE == 0 ? 1 : 2>(c, st);
+    }
 }
 
 static cudaError_t traverse(pxsne_ctx *c, cudaStream_t st, bool count) {
@@ -518,11 +782,11 @@ static cudaError_t traverse(pxsne_ctx *c, cudaStream_t st, bool count) {
     // rounding of d^2)
     const bool own = c->p.theta >= 0.999f;
     if (c->p.centre_mode == 0) {
-        if (count) own ? traverse_as<0, 1, true>(c, st) : traverse_as<0, 1, false>(c, st);
-        else own ? traverse_as<0, 0, true>(c, st) : traverse_as<0, 0, false>(c, st);
+        if (count) own ? traverse_n<0, 1, true>(c, st) : traverse_n<0, 1, false>(c, st);
+        else own ? traverse_n<0, 0, true>(c, st) : traverse_n<0, 0, false>(c, st);
     } else {
-        if (count) own ? traverse_as<1, 1, true>(c, st) : traverse_as<1, 1, false>(c, st);
-        else own ? traverse_as<1, 0, true>(c, st) : traverse_as<1, 0, false>(c, st);
+        if (count) own ? traverse_n<1, 1, true>(c, st) : traverse_n<1, 1, false>(c, st);
+        else own ? traverse_n<1, 0, true>(c, st) : traverse_n<1, 0, false>(c, st);
     }
     return cudaGetLastError();
 }

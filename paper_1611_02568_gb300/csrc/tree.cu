@@ -118,7 +118,8 @@ __global__ void k_snap_hist(int n, int L, int rescale, float theta, u64 Rx, u64 
     if (valid) rank[i] = base + (uint32_t)(lane - start);
 }
 
-// Centre-of-mass record of cell m of level l (layout in common.cuh).
+// Centre-of-mass record of cell m of level l: the four words {-c_hi_x, -c_lo_x,
+// -c_hi_y, -c_lo_y} of the layout in common.cuh (zeros for an empty cell).
 __device__ __forceinline__ float4 make_record(uint32_t N, u64 Sx, u64 Sy, int l, uint32_t m) {
     if (N == 0) return make_float4(0.f, 0.f, 0.f, 0.f);
     const int sh = 32 - l;
@@ -127,7 +128,26 @@ __device__ __forceinline__ float4 make_record(uint32_t N, u64 Sx, u64 Sy, int l,
     float4 r;
     record_axis(N, Sx, bx, sh, r.x, r.y);
     record_axis(N, Sy, by, sh, r.z, r.w);
-    return r;
+    return make_float4(-r.x, -r.y, -r.z, -r.w);
+}
+
+// One cell's record into its sibling group (four words, 16 bytes apart).
+__device__ __forceinline__ void store_record(float4 *rec, int l, uint32_t m, float4 r) {
+    float *g = reinterpret_cast<float *>(rec + rec_offset(l) + (m & ~3u)) + (m & 3u);
+    g[0] = r.x;
+    g[4] = r.y;
+    g[8] = r.z;
+    g[12] = r.w;
+}
+
+// The records of a whole sibling group (cells m .. m + 3, m a multiple of 4).
+__device__ __forceinline__ void store_group(float4 *rec, int l, uint32_t m, float4 a, float4 b,
+                                            float4 c, float4 d) {
+    float4 *g = rec + rec_offset(l) + m;
+    g[0] = make_float4(a.x, b.x, c.x, d.x);
+    g[1] = make_float4(a.y, b.y, c.y, d.y);
+    g[2] = make_float4(a.z, b.z, c.z, d.z);
+    g[3] = make_float4(a.w, b.w, c.w, d.w);
 }
 
 // Block-wide exclusive scan of one value per thread (nt threads, nt <= 1024).
@@ -203,11 +223,10 @@ __global__ void __launch_bounds__(1 << (2 * (K - 1)))
         x23 = reinterpret_cast<const ulonglong2 *>(in_sx)[(cell0 >> 1) + 1];
         y01 = reinterpret_cast<const ulonglong2 *>(in_sy)[cell0 >> 1];
         y23 = reinterpret_cast<const ulonglong2 *>(in_sy)[(cell0 >> 1) + 1];
-        float4 *rl = rec + rec_offset(h) + cell0;
-        rl[0] = make_record(c4.x, x01.x, y01.x, h, (uint32_t)cell0);
-        rl[1] = make_record(c4.y, x01.y, y01.y, h, (uint32_t)cell0 + 1u);
-        rl[2] = make_record(c4.z, x23.x, y23.x, h, (uint32_t)cell0 + 2u);
-        rl[3] = make_record(c4.w, x23.y, y23.y, h, (uint32_t)cell0 + 3u);
+        store_group(rec, h, (uint32_t)cell0, make_record(c4.x, x01.x, y01.x, h, (uint32_t)cell0),
+                    make_record(c4.y, x01.y, y01.y, h, (uint32_t)cell0 + 1u),
+                    make_record(c4.z, x23.x, y23.x, h, (uint32_t)cell0 + 2u),
+                    make_record(c4.w, x23.y, y23.y, h, (uint32_t)cell0 + 3u));
     }
     reinterpret_cast<float4 *>(recn + rec_offset(h))[cell0 >> 2] =
         make_float4((float)c4.x, (float)c4.y, (float)c4.z, (float)c4.w);
@@ -232,7 +251,8 @@ __global__ void __launch_bounds__(1 << (2 * (K - 1)))
         const int cells = 1 << (2 * j);
         if (tid < cells) {
             if (j > 0 || top) {
-                if (sums) rec[rec_offset(lvl) + idx] = make_record(N, X, Y, lvl, (uint32_t)idx);
+                if (sums)
+                    store_record(rec, lvl, (uint32_t)idx, make_record(N, X, Y, lvl, (uint32_t)idx));
                 recn[rec_offset(lvl) + idx] = (float)N;
             }
             if (j == 0) {
@@ -276,8 +296,8 @@ __device__ __forceinline__ u64 shfl_xor_u64(u64 v, int o) {
 
 __device__ __forceinline__ void put_record(float4 *rec, float *recn, int l, uint32_t m,
                                            uint32_t N, u64 X, u64 Y) {
-    // NULL: counts only; an empty cell's record is never read, so not written
-    if (rec != nullptr && N != 0u) rec[rec_offset(l) + m] = make_record(N, X, Y, l, m);
+    // NULL: counts only; an empty cell's record weighs nothing, so not written
+    if (rec != nullptr && N != 0u) store_record(rec, l, m, make_record(N, X, Y, l, m));
     recn[rec_offset(l) + m] = (float)N;
 }
 
@@ -379,12 +399,12 @@ __global__ void __launch_bounds__(256)
         x23 = reinterpret_cast<const ulonglong2 *>(in_sx)[(cell0 >> 1) + 1];
         y01 = reinterpret_cast<const ulonglong2 *>(in_sy)[cell0 >> 1];
         y23 = reinterpret_cast<const ulonglong2 *>(in_sy)[(cell0 >> 1) + 1];
-        float4 *rl = rec + rec_offset(h) + cell0;
-        // (an empty cell's record is never read: not written)
-        if (c4.x) rl[0] = make_record(c4.x, x01.x, y01.x, h, cell0);
-        if (c4.y) rl[1] = make_record(c4.y, x01.y, y01.y, h, cell0 + 1u);
-        if (c4.z) rl[2] = make_record(c4.z, x23.x, y23.x, h, cell0 + 2u);
-        if (c4.w) rl[3] = make_record(c4.w, x23.y, y23.y, h, cell0 + 3u);
+        // (the records of four empty cells are not read: not written)
+        if ((c4.x | c4.y | c4.z | c4.w) != 0u)
+            store_group(rec, h, cell0, make_record(c4.x, x01.x, y01.x, h, cell0),
+                        make_record(c4.y, x01.y, y01.y, h, cell0 + 1u),
+                        make_record(c4.z, x23.x, y23.x, h, cell0 + 2u),
+                        make_record(c4.w, x23.y, y23.y, h, cell0 + 3u));
     }
     reinterpret_cast<float4 *>(recn + rec_offset(h))[cell0 >> 2] =
         make_float4((float)c4.x, (float)c4.y, (float)c4.z, (float)c4.w);

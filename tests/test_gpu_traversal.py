@@ -1,0 +1,82 @@
+"""The traversal's kernels at the sizes where one hands over to the next and at
+the remainders of their warps, against the oracle's forces (1e-4 relative L2,
+the bar of every force comparison), with states whose cells hold one point as
+well as crowded ones."""
+import numpy as np
+import pytest
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+FORCE_TOL = 1e-4
+L = 10
+
+
+def rel(a, b):
+    return float(np.linalg.norm(np.asarray(a, np.float64) - b) / np.linalg.norm(b))
+
+
+def state(n, seed):
+    """Half of the points spread over the screen, half in a small patch, a few
+    on one position; the corners taken, as a rescaled state has them."""
+    rng = np.random.default_rng([seed, n])
+    z = rng.integers(0, 1 << 32, (n, 2), dtype=np.uint64)
+    m = n // 2
+    z[:m] = (1 << 30) + rng.integers(0, 1 << 26, (m, 2), dtype=np.uint64)
+    z[m:m + 5] = z[0]
+    z[-2], z[-1] = 0, (1 << 32) - 1
+    return rng.permutation(z).astype(np.uint32), np.array([50.0, 43.0]) / 2.0 ** 32
+
+
+def ring_P(n):
+    """Each point coupled to its two neighbours by index."""
+    i = np.arange(n)
+    col = np.sort(np.stack([(i + 1) % n, (i - 1) % n], 1), 1)
+    return np.arange(n + 1) * 2, col.reshape(-1), np.full(2 * n, 0.5 / n)
+
+
+@pytest.mark.parametrize("n,centre,theta", [
+    (3, 0, 0.5), (33, 0, 0.5), (33, 1, 1.2), (32767, 0, 0.5), (32768, 0, 0.5), (32801, 0, 1.2),
+    (32801, 0, 0.3), (40000, 1, 0.5), (149_999, 1, 0.5), (150_000, 1, 0.5), (150_033, 1, 1.2)])
+def test_forces_across_the_kernels(n, centre, theta):
+    import paper_1611_02568_gb300 as px
+    from paper_1611_02568_gb300 import build
+    build.build()
+    z, s = state(n, 5)
+    with px.Context(px.Params(log2_r=L, theta=theta, centre_mode=centre)) as ctx:
+        ctx.set_P(*ring_P(n))
+        ctx.set_state(z, s)
+        Frep, Zi, _, Z = ctx.get_forces()
+        acc = ctx.counters()[0]
+        ctx.step(1)
+        ctx.sync()
+    rows = np.unique(np.concatenate([np.arange(min(n, 70)), np.arange(max(0, n - 70), n),
+                                     np.random.default_rng(1).integers(0, n, 1500)]))
+    oF, oZi, _ = oracle.bh_repulsion(z, s, L, theta, rows=rows, centre_mode=centre)
+    assert rel(Frep[rows], oF) <= FORCE_TOL
+    assert rel(Zi[rows], oZi) <= FORCE_TOL
+    assert abs(Z - Zi.astype(np.float64).sum()) <= 1e-6 * Z
+    if n <= 40000:
+        _, oZ, oacc = oracle.bh_repulsion(z, s, L, theta, centre_mode=centre)
+        assert acc == pytest.approx(int(oacc.sum()), rel=1e-4)
+        assert rel(Zi, oZ) <= FORCE_TOL
+
+
+def test_every_cell_opened():
+    """theta = 0 opens every occupied cell: the point traversal's ring at its
+    fullest, and the same sums from the warp's stack."""
+    import paper_1611_02568_gb300 as px
+    from paper_1611_02568_gb300 import build
+    build.build()
+    z, s = state(6000, 7)
+    with px.Context(px.Params(log2_r=L, theta=0.0)) as ctx:
+        ctx.set_P(*ring_P(6000))
+        ctx.set_state(z, s)
+        a = ctx.get_forces()
+        ctx.test_stack_limit(48)
+        ctx.set_state(z, s)
+        b = ctx.get_forces()
+    oF, oZi, _ = oracle.bh_repulsion(z, s, L, 0.0)
+    for Frep, Zi in ((a[0], a[1]), (b[0], b[1])):
+        assert rel(Frep, oF) <= FORCE_TOL and rel(Zi, oZi) <= FORCE_TOL
