@@ -338,8 +338,9 @@ int pxsne_get_counters(pxsne_ctx *ctx, uint64_t *n_accept, uint64_t *n_test,
 int pxsne_get_level_counters(pxsne_ctx *ctx, uint64_t *counts, int32_t levels);
 
 /* Work counters of the last neighbour search: exact FP32 distances computed
- * and list insertions over all rows (tensor-core search only; 0 otherwise),
- * and the search used (1 tensor cores, 0 FP32 CUDA cores, -1 none).
+ * and list insertions over all rows (for the two-pass search the candidates
+ * within the rows' thresholds, which are sorted instead; tensor-core search
+ * only; 0 otherwise), and the search used (1 tensor cores, 0 FP32 CUDA cores, -1 none).
  * Synchronises. */
 int pxsne_get_knn_counters(pxsne_ctx *ctx, uint64_t *exact, uint64_t *inserted, int32_t *path);
 

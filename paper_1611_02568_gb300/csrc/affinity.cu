@@ -24,6 +24,7 @@
 #include <cuda_fp16.h>
 
 #include "common.cuh"
+#include "knn.cuh"
 #include "tc.cuh"
 
 namespace pxsne {
@@ -279,8 +280,6 @@ __global__ void __launch_bounds__(kKnnThreads)
 // distances, one survivor per lane, and, holding the lock its row quarter
 // shares with the other warp on those rows, every lane walks its own row's
 // chain inserting them, all lanes at once, against the lists' current roots.
-constexpr int kTcRows = 128;     // query rows per CTA (MMA M)
-constexpr int kTcCols = 128;     // candidates per tile (MMA N)
 constexpr int kTcStages = 2;     // candidate-tile stages in shared memory
 constexpr int kTcQueue = 384;    // survivor queue per filter warp (entries)
 constexpr uint32_t kTcFlushAt = 48u;   // queued survivors that trigger a flush
@@ -288,11 +287,6 @@ constexpr int kTcAcc = 4;        // TMEM accumulators (4 x 128 columns)
 constexpr int kTcFilterWarps = 8;  // two per TMEM lane quarter, 64 columns each
 constexpr int kTcThreads = 32 * (kTcFilterWarps + 2);  // then the loader, then the MMA issuer
 constexpr int kTcLoadWarp = kTcFilterWarps, kTcMmaWarp = kTcFilterWarps + 1;
-constexpr int kTcPolls = 1 << 22;
-constexpr uint32_t kTcSleepNs = 2000u;  // suspend hint of the pipeline waits
-// per candidate tile: h_j (128), g_j (128), then per 32-column chunk min h and
-// max g (4 + 4): 264 floats, 1056 bytes (a multiple of 16 for the bulk copy)
-constexpr int kHG = 2 * kTcCols + 12;
 
 __global__ void k_absmax(int64_t m, const float *__restrict__ X, unsigned *out) {
     unsigned v = 0u;
@@ -584,17 +578,24 @@ __global__ void __launch_bounds__(kCsRows)
     order[off[(int64_t)c * nb + b] + before + (uint32_t)rw] = (uint32_t)i;
 }
 
-// Xs[r] = X[order[r]], ns[r] = nrm[order[r]]
-__global__ void k_gather_rows(int64_t n, int D, const uint32_t *__restrict__ order,
-                              const float *__restrict__ X, const float *__restrict__ nrm,
-                              float *__restrict__ Xs, float *__restrict__ ns) {
+// Xs[r] = X[order[r]], rows ld >= D floats apart with zeros past D (a zero
+// column changes no sum of squares, so the distances are those of the D
+// columns while every row can be read in 16-byte words)
+__global__ void k_gather_rows(int64_t n, int D, int ld, const uint32_t *__restrict__ order,
+                              const float *__restrict__ X, float *__restrict__ Xs) {
     const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (q >= n * D) return;
-    const int64_t r = q / D;
-    const int d = (int)(q % D);
-    const uint32_t i = order[r];
-    Xs[q] = X[(int64_t)i * D + d];
-    if (d == 0) ns[r] = nrm[i];
+    if (q >= n * ld) return;
+    const int64_t r = q / ld;
+    const int d = (int)(q % ld);
+    Xs[q] = d < D ? X[(int64_t)order[r] * D + d] : 0.f;
+}
+
+// The sample of the two-pass search: every kScanStride-th ordered row.
+__global__ void k_sample_rows(int64_t m, int ld, const float *__restrict__ Xs,
+                              float *__restrict__ out) {
+    const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (q >= m * ld) return;
+    out[q] = Xs[(kScanPhase + (q / ld) * kScanStride) * ld + q % ld];
 }
 
 // ---- random-projection refinement of the locality order, and the
@@ -802,6 +803,7 @@ struct KnnTcArgs {
     const float *rad;     // per tile: an upper bound of |x - centroid| over its rows
     const int32_t *cand;  // approximate search: per query tile its W candidate tiles
     int W;                //   (own tile first); NULL: every tile (the exact search)
+    const uint32_t *qlist;  // the query tiles to search; NULL: all of them
 };
 
 // The i-th candidate tile a CTA visits: its own, then alternately the next
@@ -846,7 +848,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_knn_tc(const KnnTcArgs a) {
     uint16_t *qp_all = reinterpret_cast<uint16_t *>(qd_all + kTcFilterWarps * kTcQueue);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int64_t qt = blockIdx.x;  // query tile
+    const int64_t qt = a.qlist ? a.qlist[blockIdx.x] : blockIdx.x;  // query tile
     const int64_t q0 = qt * kTcRows;
 
     for (int e = tid; e < kTcRows * ks; e += kTcThreads) lst[e] = KnnEntry{INFINITY, 0x7fffffff};
@@ -1450,6 +1452,41 @@ __global__ void k_rank_of(int64_t n, const uint32_t *__restrict__ order, uint32_
     if (p < n) rank[order[p]] = (uint32_t)p;
 }
 
+// What a search reads of ordered rows X (ld floats apart), in one allocation.
+struct KnnSide {
+    KnnRows r{};
+    uint8_t *block = nullptr;
+};
+
+static cudaError_t make_side(int64_t n, int ld, int Dp, float scale, float eps_abs,
+                             const float *X, KnnSide &s, cudaStream_t st) {
+    const int64_t T = (n + kTcCols - 1) / kTcCols;
+    auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
+    const size_t b_img = up((size_t)T * kTcRows * Dp * 2), b_hg = up((size_t)T * kHG * 4),
+                 b_n = up((size_t)n * 4), b_c = up((size_t)T * Dp * 4), b_r = up((size_t)T * 4);
+    cudaError_t e;
+    if ((e = cudaMallocAsync(&s.block, b_img + b_hg + 2 * b_n + b_c + b_r, st))) return e;
+    uint8_t *img = s.block;
+    float *HG = reinterpret_cast<float *>(img + b_img);
+    float *n16 = reinterpret_cast<float *>(img + b_img + b_hg);
+    float *rerr = reinterpret_cast<float *>(img + b_img + b_hg + b_n);
+    float *cent = reinterpret_cast<float *>(img + b_img + b_hg + 2 * b_n);
+    float *rad = reinterpret_cast<float *>(img + b_img + b_hg + 2 * b_n + b_c);
+    const int64_t chunks = T * kTcRows * (Dp / 8);
+    k_to_half_img<<<(unsigned)((chunks + 255) / 256), 256, 0, st>>>(n, ld, Dp, T, scale, X, img);
+    k_round_err<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, ld, scale, X, n16, rerr);
+    k_tile_norms<<<(unsigned)((T * kTcCols + 255) / 256), 256, 0, st>>>(n, T, eps_abs, n16, rerr, HG);
+    // centroids and radii (the loaders' pruning bound)
+    k_tile_bounds<<<(unsigned)T, 128, 0, st>>>(n, ld, Dp, X, cent, rad);
+    s.r = KnnRows{n, T, X, img, n16, rerr, HG, cent, rad};
+    return cudaGetLastError();
+}
+
+static void free_side(KnnSide &s, cudaStream_t st) {
+    if (s.block) cudaFreeAsync(s.block, st);
+    s.block = nullptr;
+}
+
 static cudaError_t knn_mark(pxsne_ctx *c, int which, cudaStream_t st) {
     cudaError_t e;
     if (!c->knn_ev[which] && (e = cudaEventCreate(&c->knn_ev[which]))) return e;
@@ -1552,7 +1589,8 @@ cudaError_t launch_knn(pxsne_ctx *c, const float *Xdev, int64_t n, int32_t D, in
                 cur = nxt;
             }
         }
-        float *piv = nullptr, *Xs = nullptr, *ns = nullptr;
+        float *piv = nullptr, *Xs = nullptr;
+        const int ld = (D + 3) & ~3;  // floats per ordered row
         uint32_t *cell = nullptr, *order = nullptr, *ccnt = nullptr;
         if ((e = cudaMallocAsync(&piv, (size_t)m * (D + 1) * sizeof(float), st))) return e;
         if ((e = cudaMallocAsync(&cell, (size_t)n * sizeof(uint32_t), st))) return e;
@@ -1562,8 +1600,7 @@ cudaError_t launch_knn(pxsne_ctx *c, const float *Xdev, int64_t n, int32_t D, in
         double *dsum = nullptr;
         if ((e = cudaMallocAsync(&dpiv, (size_t)n * sizeof(float), st))) return e;
         if ((e = cudaMallocAsync(&dsum, sizeof(double), st))) return e;
-        if ((e = cudaMallocAsync(&Xs, (size_t)n * D * sizeof(float), st))) return e;
-        if ((e = cudaMallocAsync(&ns, (size_t)n * sizeof(float), st))) return e;
+        if ((e = cudaMallocAsync(&Xs, (size_t)n * ld * sizeof(float), st))) return e;
         float *pn = piv + (size_t)m * D;
         if ((e = cudaMemcpyAsync(piv, hq.data(), (size_t)m * D * sizeof(float),
                                  cudaMemcpyHostToDevice, st)))
@@ -1670,33 +1707,12 @@ cudaError_t launch_knn(pxsne_ctx *c, const float *Xdev, int64_t n, int32_t D, in
             cudaFreeAsync(seg2, st);
             cudaFreeAsync(pref, st);
         }
-        k_gather_rows<<<(unsigned)((n * D + 255) / 256), 256, 0, st>>>(n, D, order, Xdev, nrm, Xs,
-                                                                       ns);
+        k_gather_rows<<<(unsigned)((n * ld + 255) / 256), 256, 0, st>>>(n, D, ld, order, Xdev, Xs);
         if ((e = cudaGetLastError())) return e;
         // the search runs on the ordered rows
-        const float *Xo = Xs;
-        const int64_t T = (n + kTcCols - 1) / kTcCols;
-        const size_t img_bytes = (size_t)T * kTcRows * Dp * 2;
-        uint8_t *img = nullptr;
-        float *HG = nullptr;
-        if ((e = cudaMallocAsync(&img, img_bytes, st))) return e;
-        if ((e = cudaMallocAsync(&HG, (size_t)T * kHG * sizeof(float), st))) return e;
-        const int64_t nchunks = T * kTcRows * (Dp / 8);
-        k_to_half_img<<<(unsigned)((nchunks + 255) / 256), 256, 0, st>>>(n, D, Dp, T, scale, Xo,
-                                                                          img);
-        float *n16 = nullptr, *rerr = nullptr;
-        if ((e = cudaMallocAsync(&n16, (size_t)n * sizeof(float), st))) return e;
-        if ((e = cudaMallocAsync(&rerr, (size_t)n * sizeof(float), st))) return e;
-        k_round_err<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, D, scale, Xo, n16, rerr);
-        k_tile_norms<<<(unsigned)((T * kTcCols + 255) / 256), 256, 0, st>>>(n, T, eps_abs, n16,
-                                                                           rerr, HG);
-        if ((e = cudaGetLastError())) return e;
-        // tile centroids and radii (the loader's pruning bound)
-        float *cent = nullptr, *rad = nullptr;
-        if ((e = cudaMallocAsync(&cent, (size_t)T * Dp * sizeof(float), st))) return e;
-        if ((e = cudaMallocAsync(&rad, (size_t)T * sizeof(float), st))) return e;
-        k_tile_bounds<<<(unsigned)T, 128, 0, st>>>(n, D, Dp, Xo, cent, rad);
-        if ((e = cudaGetLastError())) return e;
+        KnnSide main_side, samp_side;
+        if ((e = make_side(n, ld, Dp, scale, eps_abs, Xs, main_side, st))) return e;
+        const int64_t T = main_side.r.T;
         c->knn_tiles = T;
         if ((e = cudaFuncSetAttribute(k_knn_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)smem_tc)))
@@ -1704,39 +1720,61 @@ cudaError_t launch_knn(pxsne_ctx *c, const float *Xdev, int64_t n, int32_t D, in
         KnnTcArgs ka;
         ka.n = n;
         ka.T = T;
-        ka.D = D;
+        ka.D = ld;
         ka.Dp = Dp;
         ka.k = k;
         ka.inv_s2 = inv_s2;
         ka.kappa = kappa;
         ka.eps_abs = eps_abs;
-        ka.X = Xo;
-        ka.img = img;
-        ka.nrm = n16;
-        ka.rerr = rerr;
-        ka.HG = HG;
+        ka.X = Xs;
+        ka.img = main_side.r.img;
+        ka.nrm = main_side.r.nrm;
+        ka.rerr = main_side.r.rerr;
+        ka.HG = main_side.r.HG;
         ka.order = order;
         ka.out_idx = idx;
         ka.out_d2 = d2;
         ka.err = err;
         ka.stats = &c->sc->knn_exact;
-        ka.cent = cent;
-        ka.rad = rad;
+        ka.cent = main_side.r.cent;
+        ka.rad = main_side.r.rad;
         ka.cand = nullptr;
         ka.W = 0;
+        ka.qlist = nullptr;
         // (the search's time includes its candidate lists)
         if ((e = knn_mark(c, 0, st))) return e;
         int32_t *cand = nullptr;
         if (probe > 0) {
             const int W = (int)std::min<int64_t>(probe, T);
             if ((e = cudaMallocAsync(&cand, (size_t)T * W * sizeof(int32_t), st))) return e;
-            k_tile_cands<<<(unsigned)T, kCandThreads, 0, st>>>(T, Dp, cent, W, cand);
+            k_tile_cands<<<(unsigned)T, kCandThreads, 0, st>>>(T, Dp, ka.cent, W, cand);
             if ((e = cudaGetLastError())) return e;
             ka.cand = cand;
             ka.W = W;
         }
-        k_knn_tc<<<(unsigned)T, kTcThreads, smem_tc, st>>>(ka);
-        if ((e = cudaGetLastError())) return e;
+        uint32_t *failed = nullptr;
+        float *Xsamp = nullptr;
+        uint32_t one_pass = (uint32_t)T;  // query tiles of the one-pass search
+        if (probe == 0 && knn_scan_takes(n, k, Dp, smem_max)) {
+            const int64_t ms = scan_sample_rows(n);
+            if ((e = cudaMallocAsync(&Xsamp, (size_t)ms * ld * sizeof(float), st))) return e;
+            k_sample_rows<<<(unsigned)((ms * ld + 255) / 256), 256, 0, st>>>(ms, ld, Xs, Xsamp);
+            if ((e = cudaGetLastError())) return e;
+            if ((e = make_side(ms, ld, Dp, scale, 0.f, Xsamp, samp_side, st))) return e;
+            if ((e = cudaMallocAsync(&failed, (size_t)(T + 1) * sizeof(uint32_t), st))) return e;
+            const KnnScan sa{main_side.r, samp_side.r, ld,  Dp, k,   inv_s2, kappa,
+                             eps_abs,     order,       idx, d2, err, ka.stats};
+            if ((e = launch_knn_scan(sa, c->sms, failed, failed + T, st))) return e;
+            if ((e = cudaMemcpyAsync(&one_pass, failed + T, sizeof(uint32_t), cudaMemcpyDeviceToHost,
+                                     st)))
+                return e;
+            if ((e = cudaStreamSynchronize(st))) return e;
+            ka.qlist = failed;
+        }
+        if (one_pass > 0) {
+            k_knn_tc<<<one_pass, kTcThreads, smem_tc, st>>>(ka);
+            if ((e = cudaGetLastError())) return e;
+        }
         if (probe > 0 && c->p.knn_explore > 0) {
             // rounds of neighbour exploring, ping-ponging with a second pair
             // of lists; the last round writes into idx / d2
@@ -1749,7 +1787,7 @@ cudaError_t launch_knn(pxsne_ctx *c, const float *Xdev, int64_t n, int32_t D, in
             k_rank_of<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, order, rank);
             const int R = c->p.knn_explore;
             const int ke = std::min(k, kExploreNbrs);
-            const int v4 = ((D & 3) == 0) && ((reinterpret_cast<uintptr_t>(Xo) & 15) == 0);
+            const int v4 = 1;  // rows are padded to 16 bytes
             const unsigned eb = (unsigned)((n + kExploreWarps - 1) / kExploreWarps);
             // with R odd the first round reads a copy of the search's lists
             if ((R & 1) &&
@@ -1766,7 +1804,7 @@ cudaError_t launch_knn(pxsne_ctx *c, const float *Xdev, int64_t n, int32_t D, in
                 const float *di = into_main ? d22 : d2;
                 int32_t *io = into_main ? idx : idx2;
                 float *dout = into_main ? d2 : d22;
-                k_knn_explore<<<eb, kExploreWarps * 32, 0, st>>>(n, k, ke, D, v4, Xo, order, rank,
+                k_knn_explore<<<eb, kExploreWarps * 32, 0, st>>>(n, k, ke, ld, v4, Xs, order, rank,
                                                                 ii, di, io, dout);
                 if ((e = cudaGetLastError())) return e;
             }
@@ -1776,12 +1814,10 @@ cudaError_t launch_knn(pxsne_ctx *c, const float *Xdev, int64_t n, int32_t D, in
         }
         if ((e = knn_mark(c, 1, st))) return e;
         if (cand) cudaFreeAsync(cand, st);
-        cudaFreeAsync(img, st);
-        cudaFreeAsync(HG, st);
-        cudaFreeAsync(n16, st);
-        cudaFreeAsync(rerr, st);
-        cudaFreeAsync(cent, st);
-        cudaFreeAsync(rad, st);
+        free_side(main_side, st);
+        free_side(samp_side, st);
+        if (failed) cudaFreeAsync(failed, st);
+        if (Xsamp) cudaFreeAsync(Xsamp, st);
         cudaFreeAsync(amax, st);
         cudaFreeAsync(piv, st);
         cudaFreeAsync(cell, st);
@@ -1790,7 +1826,6 @@ cudaError_t launch_knn(pxsne_ctx *c, const float *Xdev, int64_t n, int32_t D, in
         cudaFreeAsync(dpiv, st);
         cudaFreeAsync(dsum, st);
         cudaFreeAsync(Xs, st);
-        cudaFreeAsync(ns, st);
         return cudaFreeAsync(nrm, st);
     }
     c->knn_path = 0;

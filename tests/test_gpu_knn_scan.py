@@ -1,0 +1,74 @@
+"""The two-pass neighbour search at its edges: the smallest sizes that it takes,
+ragged last tiles, row lengths that are no multiple of four, short and long
+lists, and rows whose candidates overflow or fall short (those tiles are
+scanned again or go to the one-pass search).  The lists are those of a full
+FP64 sort outside a 2e-5 band around the k-th distance, d2 within 1e-5 (the bars
+of every exact search)."""
+import numpy as np
+import pytest
+
+import datagen
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+def check(X, k, idx, d2):
+    n = X.shape[0]
+    io, do = oracle.knn(X, k)
+    assert (np.sort(idx, 1)[:, 1:] != np.sort(idx, 1)[:, :-1]).all()
+    assert not (idx == np.arange(n)[:, None]).any()
+    kth = do[:, -1:]
+    true = ((X[:, None, :].astype(np.float64) - X[idx].astype(np.float64)) ** 2).sum(2)
+    assert (true <= kth * (1 + 2e-5) + 1e-12).all()
+    np.testing.assert_allclose(d2, true, rtol=1e-5, atol=1e-9)
+    assert (np.diff(d2, axis=1) >= 0).all()
+    for i in range(n):
+        must = io[i][do[i] < kth[i] * (1 - 2e-5)]
+        assert np.isin(must, idx[i]).all(), i
+
+
+def lists(X, k):
+    import paper_1611_02568_gb300 as px
+    from paper_1611_02568_gb300 import build
+    build.build()
+    with px.Context(px.Params(log2_r=9, k=k, perplexity=max(1.0, k / 3.0))) as ctx:
+        try:
+            ctx.affinities(X)
+        except px.PxsneError as e:   # identical rows have no bandwidth
+            assert "bisection" in str(e)
+        out = ctx.get_knn()[:2]
+        exact, kept, path = ctx.knn_counters()
+        # (lists of over 128 entries outgrow the one-pass search's shared memory
+        # and go to the FP32 tiles)
+        assert (path == 1 and exact >= kept > 0) or k > 128
+    return out
+
+
+@pytest.mark.parametrize("n,D,k", [
+    (223, 3, 5), (227, 50, 5), (800, 8, 90), (1100, 50, 90), (2049, 127, 45), (2500, 17, 150),
+    (3001, 64, 33), (5003, 1, 12), (4000, 128, 1)])
+def test_lists_at_the_edges(n, D, k):
+    X, _ = datagen.gauss10(n % 7, n=n, D=D)
+    check(X, k, *lists(X, k))
+
+
+def test_crowded_and_sparse_rows():
+    """1,500 rows on one position (every candidate buffer of theirs overflows),
+    300 on two positions, a tight and a wide cluster."""
+    rng = np.random.default_rng(3)
+    X = rng.standard_normal((4003, 20)).astype(np.float32)
+    X[:1500] = X[0]
+    X[1500:1650], X[1650:1800] = 9.0, 9.25
+    X[1800:2400] = 30.0 + 1e-3 * rng.standard_normal((600, 20))
+    X[2400:2500] *= 40.0
+    X = X[rng.permutation(X.shape[0])]
+    check(X, 30, *lists(X, 30))
+
+
+def test_one_dimension_far_apart():
+    """Neighbourhoods that the stratified sample meets unevenly: points at
+    geometric distances, whose thresholds fall short or overshoot."""
+    x = np.concatenate([1.02 ** np.arange(1200), -(1.02 ** np.arange(1200))])
+    X = np.stack([x, 0.5 * x], 1).astype(np.float32)
+    check(X, 20, *lists(X, 20))
