@@ -19,7 +19,6 @@ constexpr int kMaxL = 14;           // screen up to 2^14 x 2^14 (Morton keys < 2
 constexpr int64_t kMaxN = 1 << 24;  // cell counts are exact floats below 2^24
 constexpr int kTravWarps = 8;       // warps per CTA in the traversal
 constexpr int kTravStack = 48;      // entries per warp; depth <= 3L - 2 <= 40
-constexpr int kExactLevel = 8;      // cells of 2^24 ulps and fewer
 // The traversal's kernel by the number of points (late states of 10- and
 // 100-component mixtures, us per iteration).  Below kTravPointTo one warp per
 // point: 46 against 102 at n = 2000 and 108 against 150 at 20,000, but 187
@@ -146,7 +145,8 @@ __device__ __forceinline__ uint32_t rescale_exact(u64 a, u64 gamma, double q, u6
 // whose lower corner is `base` (S_off = S - N base, the sum of the points'
 // offsets in the cell, exact), split at bit 16 as the layout in common.cuh
 // asks.  The offset is one FP32 quotient (relative error about 2^-23 of the
-// cell width, a fraction of an ulp at the leaves).
+// cell width, a fraction of an ulp at the leaves); a cell of one point has that
+// point's coordinates exactly.
 __device__ __forceinline__ void record_axis(uint32_t N, u64 S, uint32_t base, int sh,
                                             float &hi, float &lo) {
     const u64 soff = S - (u64)N * base;
@@ -154,6 +154,10 @@ __device__ __forceinline__ void record_axis(uint32_t N, u64 S, uint32_t base, in
     c = fminf(c, 4294967040.0f);
     uint32_t q = (uint32_t)c;
     float fr = c - (float)q;
+    if (N == 1u) {  // a single point: exact
+        q = (uint32_t)soff;
+        fr = 0.f;
+    }
     const uint32_t wmax = sh >= 32 ? 0xffffffffu : ((1u << sh) - 1u);
     if (q > wmax) {  // rounding at the cell's far edge
         q = wmax;
@@ -295,15 +299,16 @@ struct pxsne_ctx {
     // the 3-D embedding (dim = 3): positions, velocities, gains and forces
     // per point as 4-wide vectors (the fourth lane unused), zhat as three
     // int64 per point, and the octree's per-level counts and exact sums, its
-    // records {c_hi x, y, z, N} and {c_lo x, y, z, 0} per cell
+    // records by sibling groups (dim3.cu), and the cells' starts among their
+    // siblings' points (the counting sort)
     int dim = 2;
     uint4 *z3 = nullptr;
     long long *zhat3 = nullptr;
     float4 *u3 = nullptr, *gains3 = nullptr, *Frep3 = nullptr, *Fattr3 = nullptr;
     uint32_t *cnt3 = nullptr;
     unsigned long long *sum3 = nullptr;  // [3][cells]
-    float4 *rec3a = nullptr, *rec3b = nullptr;
-    int64_t *vstart3 = nullptr;          // exclusive scan of the voxel counts
+    float4 *rec3 = nullptr;
+    uint32_t *pref3 = nullptr;
 
     pxsne::DevScalars *sc = nullptr;
     bool state_ready = false;

@@ -9,10 +9,12 @@
 //   k3_update           Eq. grad and the gains/momentum step per coordinate
 //   k3_snap             the exact-integer rescale of Sec. 4.2 per axis, the
 //                       voxel snap and the leaf histogram (counts, exact sums)
-//   k3_perm, k3_reduce  the counting sort of the points by voxel; the
-//                       octree's upper levels with their cells' records
+//   k3_level, k3_top, k3_perm  the octree's upper levels with their cells'
+//                       records; the counting sort of the points by voxel
 //   k3_traverse         Barnes-Hut (Eq. bh_criteria) on the octree, one point
-//                       per lane, 32 points of consecutive voxels per warp
+//                       per lane, 32 points of consecutive voxels per warp, the
+//                       siblings as packed FP32 pairs; k3_traverse_pt the same
+//                       for small sets, one warp per point
 //   k3_attract          Eq. grad's first term over P, one warp per row
 //   k3_kl, k3_centre_y  Eq. cost_func; the embedding's output
 //
@@ -28,28 +30,34 @@ namespace pxsne {
 namespace {
 
 constexpr double kR3 = 4294967296.0;  // 2^32 ulps per axis
-constexpr int kT3Warps = 8;           // warps per traversal CTA
+constexpr int kT3Warps = 4;           // warps per traversal CTA
 constexpr int kT3Stack = 72;          // entries per warp; depth <= 7 L + 1 <= 64
 
 __host__ __device__ inline int64_t off3(int l) { return ((int64_t(1) << (3 * l)) - 1) / 7; }
 
+// Every third bit from bit 0 (10 of them), and back.
+__device__ __forceinline__ uint32_t spread3(uint32_t x) {
+    x &= 0x3ffu;
+    x = (x | (x << 16)) & 0x030000ffu;
+    x = (x | (x << 8)) & 0x0300f00fu;
+    x = (x | (x << 4)) & 0x030c30c3u;
+    return (x | (x << 2)) & 0x09249249u;
+}
+__device__ __forceinline__ uint32_t gather3(uint32_t x) {
+    x &= 0x09249249u;
+    x = (x | (x >> 2)) & 0x030c30c3u;
+    x = (x | (x >> 4)) & 0x0300f00fu;
+    x = (x | (x >> 8)) & 0x030000ffu;
+    return (x | (x >> 16)) & 0x3ffu;
+}
+
 // Morton key of voxel (px, py, pz): bit b of x at 3b, of y at 3b + 1, of z at 3b + 2.
 __device__ __forceinline__ uint32_t morton3(uint32_t px, uint32_t py, uint32_t pz) {
-    uint32_t m = 0u;
-#pragma unroll
-    for (int b = 0; b < 10; b++)
-        m |= (((px >> b) & 1u) << (3 * b)) | (((py >> b) & 1u) << (3 * b + 1)) |
-             (((pz >> b) & 1u) << (3 * b + 2));
-    return m;
+    return spread3(px) | (spread3(py) << 1) | (spread3(pz) << 2);
 }
 
 // Coordinate `axis` (0, 1, 2) of a cell from its Morton index.
-__device__ __forceinline__ uint32_t demorton3(uint32_t m, int axis) {
-    uint32_t v = 0u;
-#pragma unroll
-    for (int b = 0; b < 10; b++) v |= ((m >> (3 * b + axis)) & 1u) << b;
-    return v;
-}
+__device__ __forceinline__ uint32_t demorton3(uint32_t m, int axis) { return gather3(m >> axis); }
 
 __device__ __forceinline__ float rcp3(float x) {
     float r;
@@ -276,76 +284,182 @@ __global__ void k3_snap(int n, int L, int rescale, float theta, const long long 
     atomicAdd(&sz[m], (u64)zv[2]);
 }
 
-// Record of cell at (level l, Morton c): {c_hi x, y, z, N} and {c_lo x, y,
-// z, 0}, the centre of mass split at bit 16 as in 2-D (record_axis); zeros
-// for an empty cell.
-__device__ __forceinline__ void put_record3(int l, int64_t c, int64_t at, uint32_t N, u64 X, u64 Y,
-                                            u64 Zs, float4 *__restrict__ ra,
-                                            float4 *__restrict__ rb) {
-    if (N == 0u) {
-        ra[at] = make_float4(0.f, 0.f, 0.f, 0.f);
-        rb[at] = make_float4(0.f, 0.f, 0.f, 0.f);
-        return;
+// The records.  The eight siblings of a node share a group of 56 floats, as
+// in 2-D a structure of arrays: the negated halves -c_hi_x [8], -c_lo_x [8], and
+// the same for y and z, of their centres of mass (record_axis), then their
+// counts [8].  The group of the children (level l + 1) of cell m of level l is
+// group off3(l) + m, so that child c of group G has its own children in group
+// 8 G + 1 + c.  Only groups with a point are written; an empty sibling's centre
+// weighs nothing.
+constexpr int kGroup3 = 56;  // floats per sibling group, 14 float4s
+
+__device__ __forceinline__ void put_record3(float *rec, int l, int64_t c, uint32_t N, u64 X, u64 Y,
+                                            u64 Zs) {
+    float *g = rec + (off3(l - 1) + (c >> 3)) * kGroup3 + (c & 7);
+    float h[3] = {0.f, 0.f, 0.f}, e[3] = {0.f, 0.f, 0.f};
+    if (N != 0u) {
+        const int sh = 32 - l;
+        record_axis(N, X, demorton3((uint32_t)c, 0) << sh, sh, h[0], e[0]);
+        record_axis(N, Y, demorton3((uint32_t)c, 1) << sh, sh, h[1], e[1]);
+        record_axis(N, Zs, demorton3((uint32_t)c, 2) << sh, sh, h[2], e[2]);
     }
-    const int sh = 32 - l;
-    float hx, lx, hy, ly, hz, lz;
-    const uint32_t bx = l > 0 ? demorton3((uint32_t)c, 0) << sh : 0u;
-    const uint32_t by = l > 0 ? demorton3((uint32_t)c, 1) << sh : 0u;
-    const uint32_t bz = l > 0 ? demorton3((uint32_t)c, 2) << sh : 0u;
-    record_axis(N, X, bx, sh, hx, lx);
-    record_axis(N, Y, by, sh, hy, ly);
-    record_axis(N, Zs, bz, sh, hz, lz);
-    ra[at] = make_float4(hx, hy, hz, (float)N);
-    rb[at] = make_float4(lx, ly, lz, 0.f);
+#pragma unroll
+    for (int d = 0; d < 3; d++) {
+        g[16 * d] = -h[d];
+        g[16 * d + 8] = -e[d];
+    }
+    g[48] = (float)N;
 }
 
-// Cells of level l from their eight children at level l + 1: one thread per
-// child (coalesced), which writes the child's record (and, clear = the
-// children are the leaves, sets an occupied leaf back to zero once read, so
-// the next histogram starts from zeros without a memset of every leaf); the
-// eight threads of a parent add up by shuffles.  At l = 0 the root's own
-// record is written too.
-__global__ void k3_reduce(int l, int clear, uint32_t *cnt, u64 *sx, u64 *sy, u64 *sz,
-                          float4 *__restrict__ ra, float4 *__restrict__ rb) {
-    const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;  // child at level l + 1
-    const bool in = k < (int64_t(1) << (3 * (l + 1)));
-    const int64_t at = off3(l + 1) + k;
-    uint32_t N = 0u;
+// The sum over the eight threads of a sibling group, for all of them.
+__device__ __forceinline__ void sum8(unsigned mask, uint32_t &N, u64 &X, u64 &Y, u64 &Zs) {
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) {
+        N += __shfl_xor_sync(mask, N, o);
+        X += __shfl_xor_sync(mask, X, o);
+        Y += __shfl_xor_sync(mask, Y, o);
+        Zs += __shfl_xor_sync(mask, Zs, o);
+    }
+}
+
+// One level of the octree from the one below: a thread per sibling group of
+// level h.  Writes the group's records, the count and sums of its parent, and
+// the children's starts among the group's points: a point's place in the
+// counting sort is the sum of its cells' starts over the levels, so no scan of
+// the voxels is needed.  clear: the cells are the leaves, and an occupied one
+// goes back to zero once read (the next histogram starts from zeros without a
+// memset of every leaf).  A group without a point costs its 32 bytes of counts
+// and a zero for its parent: what bounds the kernel on a sparse grid is how many
+// bytes of counts are in flight, hence the whole group per thread.  n = 200,000
+// on 256^3, all levels: 0.10 ms; a thread per cell 0.39, three levels per CTA of
+// 512 cells 0.33, and with every cell's sums read and records written and a scan
+// of the voxel counts 0.44.
+__global__ void __launch_bounds__(256)
+    k3_level(int h, int clear, uint32_t *cnt, u64 *sx, u64 *sy, u64 *sz, float4 *__restrict__ rec,
+             uint32_t *__restrict__ pref) {
+    const int64_t grp = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (grp >= (int64_t(1) << (3 * (h - 1)))) return;
+    const int64_t up = off3(h - 1) + grp, at = off3(h) + 8 * grp;
+    uint32_t N[8];
+    uint32_t gN = 0u;
+    // (off3(h) is odd: the counts of a group are not 16-byte aligned, the
+    // threads of a warp still read one run of bytes)
+#pragma unroll
+    for (int c = 0; c < 8; c++) {
+        N[c] = cnt[at + c];
+        gN += N[c];
+    }
+    cnt[up] = gN;
+    if (gN == 0u) return;
+    uint32_t run = 0u;
+#pragma unroll
+    for (int c = 0; c < 8; c++) {
+        if (N[c] != 0u) {
+            pref[at + c] = run;
+            if (clear) cnt[at + c] = 0u;
+        }
+        run += N[c];
+    }
+    float4 *g = rec + (off3(h - 1) + grp) * (kGroup3 / 4);
+    g[12] = make_float4((float)N[0], (float)N[1], (float)N[2], (float)N[3]);
+    g[13] = make_float4((float)N[4], (float)N[5], (float)N[6], (float)N[7]);
+    const int sh = 32 - h;
+#pragma unroll
+    for (int d = 0; d < 3; d++) {
+        u64 *s = d == 0 ? sx : d == 1 ? sy : sz;
+        u64 S[8], sum = 0ull;
+#pragma unroll
+        for (int c = 0; c < 8; c++) S[c] = N[c] != 0u ? s[at + c] : 0ull;
+        // the group's corner, and whether child c lies on its far side
+        const uint32_t base = gather3((uint32_t)(grp >> d)) << (sh + 1);
+        float hi[8], lo[8];
+#pragma unroll
+        for (int c = 0; c < 8; c++) {
+            hi[c] = lo[c] = 0.f;
+            if (N[c] != 0u) {
+                record_axis(N[c], S[c], base + (((uint32_t)c >> d) & 1u) * (1u << sh), sh, hi[c], lo[c]);
+                if (clear) s[at + c] = 0ull;
+            }
+            sum += S[c];
+        }
+        s[up] = sum;
+        g[4 * d] = make_float4(-hi[0], -hi[1], -hi[2], -hi[3]);
+        g[4 * d + 1] = make_float4(-hi[4], -hi[5], -hi[6], -hi[7]);
+        g[4 * d + 2] = make_float4(-lo[0], -lo[1], -lo[2], -lo[3]);
+        g[4 * d + 3] = make_float4(-lo[4], -lo[5], -lo[6], -lo[7]);
+    }
+}
+
+// The top K levels in one CTA: a thread per cell of level K, whose starts among
+// all points it writes.
+template <int K>
+__global__ void __launch_bounds__(1 << (3 * K))
+    k3_top(int clear, uint32_t *cnt, u64 *sx, u64 *sy, u64 *sz, float *__restrict__ rec,
+           uint32_t *__restrict__ pref) {
+    constexpr int NT = 1 << (3 * K);
+    constexpr unsigned MASK = NT >= 32 ? 0xffffffffu : (1u << (NT & 31)) - 1u;
+    __shared__ uint32_t s_w[NT >= 32 ? NT / 32 : 1];
+    __shared__ uint32_t s_n[NT / 8];
+    __shared__ u64 s_s[3][NT / 8];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t at = off3(K) + tid;
+    uint32_t N = cnt[at];
     u64 X = 0ull, Y = 0ull, Zs = 0ull;
-    if (in) {
-        N = cnt[at];
+    if (N != 0u) {
         X = sx[at];
         Y = sy[at];
         Zs = sz[at];
-        put_record3(l + 1, k, at, N, X, Y, Zs, ra, rb);
-        if (clear && N != 0u) {
+        if (clear) {
             cnt[at] = 0u;
             sx[at] = 0ull;
             sy[at] = 0ull;
             sz[at] = 0ull;
         }
     }
+    uint32_t inc = N;
 #pragma unroll
-    for (int o = 1; o < 8; o <<= 1) {
-        N += __shfl_xor_sync(0xffffffffu, N, o);
-        X += __shfl_xor_sync(0xffffffffu, X, o);
-        Y += __shfl_xor_sync(0xffffffffu, Y, o);
-        Zs += __shfl_xor_sync(0xffffffffu, Zs, o);
+    for (int o = 1; o < (NT >= 32 ? 32 : NT); o <<= 1) {
+        const uint32_t t = __shfl_up_sync(MASK, inc, o);
+        if (lane >= o) inc += t;
     }
-    if (in && (k & 7) == 0) {
-        const int64_t c = k >> 3, me = off3(l) + c;
-        cnt[me] = N;
-        sx[me] = X;
-        sy[me] = Y;
-        sz[me] = Zs;
-        if (l == 0) put_record3(0, 0, me, N, X, Y, Zs, ra, rb);
+    if (lane == 31 || tid == NT - 1) s_w[warp] = inc;
+    __syncthreads();
+    uint32_t before = 0u;
+    for (int w = 0; w < warp; w++) before += s_w[w];
+    pref[at] = before + inc - N;
+#pragma unroll
+    for (int k = 0; k < K; k++) {
+        // level K - k: 8^(K - k) threads hold its cells
+        const int cells = NT >> (3 * k);
+        const bool in = tid < cells;
+        uint32_t gN = N;
+        u64 gX = X, gY = Y, gZ = Zs;
+        // (whole warps, or the CTA's only one: the shuffles need them all)
+        if (tid < ((cells + 31) & ~31)) {
+            sum8(MASK, gN, gX, gY, gZ);
+            if (in && gN != 0u) put_record3(rec, K - k, tid, N, X, Y, Zs);
+        }
+        if (in && (tid & 7) == 0) {
+            s_n[tid >> 3] = gN;
+            s_s[0][tid >> 3] = gX;
+            s_s[1][tid >> 3] = gY;
+            s_s[2][tid >> 3] = gZ;
+        }
+        __syncthreads();
+        const bool up = tid < (cells >> 3);
+        N = up ? s_n[tid] : 0u;
+        X = up ? s_s[0][tid] : 0ull;
+        Y = up ? s_s[1][tid] : 0ull;
+        Zs = up ? s_s[2][tid] : 0ull;
+        if (up) cnt[off3(K - k - 1) + tid] = N;
+        __syncthreads();
     }
 }
 
 // the counting sort by voxel: perm[start of the voxel + rank] = i; the
 // iteration counter advances here for an iteration
 __global__ void k3_perm(int n, int L, const uint4 *__restrict__ z, const uint32_t *__restrict__ rank,
-                        const int64_t *__restrict__ vstart, uint32_t *__restrict__ perm,
+                        const uint32_t *__restrict__ pref, uint32_t *__restrict__ perm,
                         DevScalars *sc, int bump_t) {
     const int F = 32 - L;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -353,8 +467,11 @@ __global__ void k3_perm(int n, int L, const uint4 *__restrict__ z, const uint32_
     if (i >= n) return;
     const uint4 v = z[i];
     const uint32_t m = morton3(v.x >> F, v.y >> F, v.z >> F);
-    const int64_t pos = vstart[m] + rank[i];
-    if (pos >= 0 && pos < n) perm[pos] = (uint32_t)i;
+    uint32_t pos = rank[i], a = m;
+    int l = L;
+    for (; l > 3; l--, a >>= 3) pos += pref[off3(l) + a];
+    pos += pref[off3(l) + a];  // the top level's starts are among all points
+    if (pos < (uint32_t)n) perm[pos] = (uint32_t)i;
     else atomicOr(&sc->err, (unsigned)PXSNE_DEVERR_STACK);
 }
 
@@ -362,24 +479,89 @@ __global__ void k3_perm(int n, int L, const uint4 *__restrict__ z, const uint32_
 // order, one per lane, and walks the octree depth-first; each stack entry is a
 // node with the mask of the lanes whose point opens it, so every point sees
 // exactly the cells its own depth-first search would, in the tree's order.
-// Children at the voxel level are always accepted (bounded depth) except a
-// point's own voxel, used without the point itself; above it Eq. bh_criteria
-// decides and the cell holding a point is opened.
-struct __align__(8) T3Entry {
-    uint32_t node, mask;  // (level << 27) | Morton index; lanes that opened it
+// As in 2-D the siblings enter the arithmetic as packed pairs straight from their
+// group's arrays, children at the voxel level are always accepted (bounded
+// depth) except a point's own voxel, used without the point itself, and above
+// it Eq. bh_criteria decides, the cell holding a point is opened, and a cell
+// of one point, whose centre is that point exactly, is accepted by all others.
+// 200,000 points on 256^3 (late state): 2.2 ms, 3.5 with one scalar child after
+// the other and single points opened down to their voxels.
+struct Point3 {
+    float2 h[3], l[3];
+};
+__device__ __forceinline__ float2 b3(float v) { return make_float2(v, v); }
+__device__ __forceinline__ Point3 point3(uint4 z) {
+    const uint32_t v[3] = {z.x, z.y, z.z};
+    Point3 p;
+#pragma unroll
+    for (int d = 0; d < 3; d++) {
+        p.h[d] = b3((float)(v[d] & 0xffff0000u));
+        p.l[d] = b3((float)(v[d] & 0xffffu));
+    }
+    return p;
+}
+__device__ __forceinline__ float2 half2of(float4 v, int p) {
+    return p ? make_float2(v.z, v.w) : make_float2(v.x, v.y);
+}
+
+// The force sums of a point, even and odd siblings apart.
+struct Sum3 {
+    float2 f[3], z;
 };
 
-__global__ void __launch_bounds__(kT3Warps * 32)
+// Pair p (0, 1) of one half (four siblings, r = its six arrays' float4s): the
+// offsets in ulps from the pair's centres.
+__device__ __forceinline__ void offset3(const float4 (&r)[6], int p, const Point3 &pt,
+                                        float2 (&dx)[3]) {
+#pragma unroll
+    for (int d = 0; d < 3; d++)
+        dx[d] = __fadd2_rn(__fadd2_rn(pt.h[d], half2of(r[2 * d], p)),
+                           __fadd2_rn(pt.l[d], half2of(r[2 * d + 1], p)));
+}
+
+// y-units and the squared distances.
+__device__ __forceinline__ float2 dist3(float2 (&dx)[3], const float2 (&s)[3]) {
+#pragma unroll
+    for (int d = 0; d < 3; d++) dx[d] = __fmul2_rn(dx[d], s[d]);
+    return __ffma2_rn(dx[0], dx[0], __ffma2_rn(dx[1], dx[1], __fmul2_rn(dx[2], dx[2])));
+}
+
+__device__ __forceinline__ void add3(Sum3 &a, float2 N, float2 d2, const float2 (&dx)[3]) {
+    const float2 w = __fadd2_rn(b3(1.0f), d2);
+    const float2 q = make_float2(rcp3(w.x), rcp3(w.y));
+    const float2 Nq = __fmul2_rn(N, q);
+    a.z = __fadd2_rn(a.z, Nq);
+    const float2 Nq2 = __fmul2_rn(Nq, q);
+#pragma unroll
+    for (int d = 0; d < 3; d++) a.f[d] = __ffma2_rn(Nq2, dx[d], a.f[d]);
+}
+
+// Takes the point itself out of its own voxel (slot of the pair's two): one
+// fewer, the centre of mass of the others.
+__device__ __forceinline__ void take_out3(int slot, float2 &N, float2 (&dx)[3]) {
+    const float Nc = slot ? N.y : N.x, r = Nc - 1.0f;
+    const float k = r > 0.0f ? Nc / r : 1.0f;
+    if (slot) {
+        N.y = r;
+        for (int d = 0; d < 3; d++) dx[d].y *= k;
+    } else {
+        N.x = r;
+        for (int d = 0; d < 3; d++) dx[d].x *= k;
+    }
+}
+
+struct __align__(8) T3Entry {
+    uint32_t node, mask;  // (children's level << 28) | their group; lanes that open it
+};
+
+template <bool OWN>
+__global__ void __launch_bounds__(kT3Warps * 32, 4)
     k3_traverse(int n, int L, const uint4 *__restrict__ z, const uint32_t *__restrict__ perm,
-                const float4 *__restrict__ ra, const float4 *__restrict__ rb, DevScalars *sc,
-                float4 *__restrict__ Frep, float *__restrict__ Zi) {
+                const float4 *__restrict__ rec, DevScalars *sc, float4 *__restrict__ Frep,
+                float *__restrict__ Zi) {
     __shared__ T3Entry s_stk[kT3Warps][kT3Stack];
     __shared__ float s_T[kMaxL + 2];
-    __shared__ int64_t s_off[kMaxL + 2];
-    if (threadIdx.x < kMaxL + 2) {
-        s_T[threadIdx.x] = sc->T3[threadIdx.x];
-        s_off[threadIdx.x] = threadIdx.x <= L ? off3(threadIdx.x) : 0;
-    }
+    if (threadIdx.x < kMaxL + 2) s_T[threadIdx.x] = sc->T3[threadIdx.x];
     __syncthreads();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int idx = (blockIdx.x * kT3Warps + w) * 32 + lane;
@@ -390,13 +572,12 @@ __global__ void __launch_bounds__(kT3Warps * 32)
     const uint32_t i = valid ? perm[idx] : 0u;
     const uint4 zi = z[i];
     const uint32_t mi = morton3(zi.x >> F, zi.y >> F, zi.z >> F);
-    const float hx = (float)(zi.x & 0xffff0000u), lx = (float)(zi.x & 0xffffu);
-    const float hy = (float)(zi.y & 0xffff0000u), ly = (float)(zi.y & 0xffffu);
-    const float hz = (float)(zi.z & 0xffff0000u), lz = (float)(zi.z & 0xffffu);
-    const float s0 = sc->sf3[0], s1 = sc->sf3[1], s2 = sc->sf3[2];
-    float fx = 0.f, fy = 0.f, fz = 0.f, zs = 0.f;
+    const uint32_t own_grp = (uint32_t)off3(L - 1) + (mi >> 3);
+    const Point3 pt = point3(zi);
+    const float2 s[3] = {b3(sc->sf3[0]), b3(sc->sf3[1]), b3(sc->sf3[2])};
+    Sum3 a{{b3(0.f), b3(0.f), b3(0.f)}, b3(0.f)};
     T3Entry *stk = s_stk[w];
-    if (lane == 0) stk[0] = T3Entry{0u, act};
+    if (lane == 0) stk[0] = T3Entry{1u << 28, act};  // the root's children: level 1, group 0
     int sp = 1;
     __syncwarp();
     bool overflow = false;
@@ -406,90 +587,189 @@ __global__ void __launch_bounds__(kT3Warps * 32)
         __syncwarp();
         top.node = __shfl_sync(0xffffffffu, top.node, 0);
         top.mask = __shfl_sync(0xffffffffu, top.mask, 0);
-        const int lc = (int)(top.node >> 27) + 1;
-        const uint32_t m0 = (top.node & 0x07ffffffu) << 3;
-        const int64_t at = s_off[lc] + m0;
+        const uint32_t grp = top.node & 0x0fffffffu;
+        const int lc = (int)(top.node >> 28);
         const bool me = (top.mask >> lane) & 1u;
-        // the eight children's first record halves (with the counts) are
-        // requested together, one latency per node; the second halves are
-        // read per child (an empty cell's is read and not used)
-        float4 rpre[8];
+        const float4 *g = rec + (size_t)grp * (kGroup3 / 4);
+        // the counts and the first half's records are requested together (both
+        // halves' took registers: 6.7 against 6.2 ms for four iterations)
+        const float4 nv[2] = {__ldg(g + 12), __ldg(g + 13)};
+        float4 rr[2][6];
 #pragma unroll
-        for (int ch = 0; ch < 8; ch++) rpre[ch] = __ldg(ra + at + ch);
+        for (int q = 0; q < 6; q++) rr[0][q] = __ldg(g + 2 * q);
         if (lc == L) {
+            const bool own = me && own_grp == grp;
+            const bool any_own = __any_sync(0xffffffffu, own);
 #pragma unroll
-            for (int ch = 0; ch < 8; ch++) {
-                const float4 r = rpre[ch];
-                const float4 q4 = __ldg(rb + at + ch);
-                const float N = r.w;
-                if (N == 0.f) continue;
-                float dx = (hx - r.x) + (lx - q4.x);
-                float dy = (hy - r.y) + (ly - q4.y);
-                float dz = (hz - r.z) + (lz - q4.z);
-                const bool own = me && (mi == m0 + (uint32_t)ch);
-                float Nf = N;
-                if (own) {  // own voxel: take the point out
-                    Nf = N - 1.0f;
-                    if (N > 1.0f) {
-                        const float k = N / Nf;
-                        dx *= k;
-                        dy *= k;
-                        dz *= k;
-                    }
+            for (int hf = 0; hf < 2; hf++) {
+                if (nv[hf].x + nv[hf].y + nv[hf].z + nv[hf].w == 0.f) continue;
+                if (hf == 1)
+                    for (int q = 0; q < 6; q++) rr[1][q] = __ldg(g + 2 * q + 1);
+                const float4(&r)[6] = rr[hf];
+#pragma unroll
+                for (int p = 0; p < 2; p++) {
+                    float2 N = half2of(nv[hf], p);
+                    if (N.x + N.y == 0.f) continue;
+                    float2 dx[3];
+                    offset3(r, p, pt, dx);
+                    if (any_own && own && (int)((mi & 7u) >> 1) == 2 * hf + p)
+                        take_out3((int)(mi & 1u), N, dx);
+                    const float2 d2 = dist3(dx, s);
+                    add3(a, make_float2(me ? N.x : 0.f, me ? N.y : 0.f), d2, dx);
                 }
-                dx *= s0;
-                dy *= s1;
-                dz *= s2;
-                const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                const bool acc = me && (Nf > 0.f);
-                const float q = rcp3(1.0f + d2);
-                const float Nq = (acc ? Nf : 0.0f) * q;
-                zs += Nq;
-                const float Nq2 = Nq * q;
-                fx = fmaf(Nq2, dx, fx);
-                fy = fmaf(Nq2, dy, fy);
-                fz = fmaf(Nq2, dz, fz);
             }
         } else {
             const float Tl = s_T[lc];
-            const uint32_t mine = mi >> (3 * (L - lc));  // the point's own cell at this level
+            const uint32_t mine = OWN ? mi >> (3 * (L - lc)) : 0u;
+            const uint32_t first = OWN ? 8u * (grp - (uint32_t)off3(lc - 1)) : 0u;
             if (sp + 8 > kT3Stack) {
                 overflow = true;
                 break;
             }
+            // lanes 0 .. 7 keep the acceptances of their child
+            unsigned taken = 0u;
 #pragma unroll
-            for (int ch = 0; ch < 8; ch++) {
-                const float4 r = rpre[ch];
-                const float4 q4 = __ldg(rb + at + ch);
-                const float N = r.w;
-                if (N == 0.f) continue;
-                const uint32_t mc = m0 + (uint32_t)ch;
-                const float dx = ((hx - r.x) + (lx - q4.x)) * s0;
-                const float dy = ((hy - r.y) + (ly - q4.y)) * s1;
-                const float dz = ((hz - r.z) + (lz - q4.z)) * s2;
-                const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                const bool far = (d2 > Tl) && (mine != mc);
-                const bool acc = me && far;
-                const float q = rcp3(1.0f + d2);
-                const float Nq = (acc ? N : 0.0f) * q;
-                zs += Nq;
-                const float Nq2 = Nq * q;
-                fx = fmaf(Nq2, dx, fx);
-                fy = fmaf(Nq2, dy, fy);
-                fz = fmaf(Nq2, dz, fz);
-                const unsigned ob = __ballot_sync(0xffffffffu, me && !far);
-                if (lane == 0) stk[sp] = T3Entry{((uint32_t)lc << 27) | mc, ob};
-                sp += ob != 0u;
+            for (int hf = 0; hf < 2; hf++) {
+                if (nv[hf].x + nv[hf].y + nv[hf].z + nv[hf].w == 0.f) continue;
+                if (hf == 1)
+                    for (int q = 0; q < 6; q++) rr[1][q] = __ldg(g + 2 * q + 1);
+                const float4(&r)[6] = rr[hf];
+#pragma unroll
+                for (int p = 0; p < 2; p++) {
+                    const int c = 4 * hf + 2 * p;
+                    const float2 N = half2of(nv[hf], p);
+                    if (N.x + N.y == 0.f) continue;
+                    float2 dx[3];
+                    offset3(r, p, pt, dx);
+                    const float2 d2 = dist3(dx, s);
+                    // the threshold of a cell of one point is 0
+                    const float2 tb = __ffma2_rn(N, b3(1e30f), b3(-1e30f));
+                    const bool a0 = me && d2.x > fminf(tb.x, Tl) && (!OWN || mine != first + c);
+                    const bool a1 = me && d2.y > fminf(tb.y, Tl) && (!OWN || mine != first + c + 1);
+                    add3(a, make_float2(a0 ? N.x : 0.f, a1 ? N.y : 0.f), d2, dx);
+                    const unsigned b0 = __ballot_sync(0xffffffffu, a0);
+                    const unsigned b1 = __ballot_sync(0xffffffffu, a1);
+                    if (lane == c) taken = b0;
+                    if (lane == c + 1) taken = b1;
+                }
+            }
+            // they push their child if it holds several points and some lane opens it
+            const float nn = lane < 8 ? __ldg(reinterpret_cast<const float *>(g + 12) + lane) : 0.f;
+            const unsigned o = top.mask & ~taken;
+            const bool push = nn > 1.f && o != 0u;
+            const unsigned pm = __ballot_sync(0xffffffffu, push);
+            if (push)
+                stk[sp + __popc(pm & ((1u << lane) - 1u))] =
+                    T3Entry{((uint32_t)(lc + 1) << 28) | (8u * grp + 1u + (uint32_t)lane), o};
+            sp += __popc(pm);
+        }
+        __syncwarp();
+    }
+    if (valid) {
+        Frep[i] = make_float4(a.f[0].x + a.f[0].y, a.f[1].x + a.f[1].y, a.f[2].x + a.f[2].y, 0.f);
+        Zi[i] = a.z.x + a.z.y;
+    }
+    if (overflow && lane == 0) atomicOr(&sc->err, (unsigned)PXSNE_DEVERR_STACK);
+}
+
+// One warp per point, up to 32 of its open nodes at a time (the 2-D kernel's
+// scheme, forces.cu): for sets too small to fill the chip with warps of 32
+// points.  A step adds at most 256 nodes of the next level, so a node of level
+// l waits at most 256 l places above kPt3Deep + 224.
+constexpr int kPt3Warps = 4;
+constexpr int kPt3Ring = 4096;
+constexpr int kPt3Deep = kPt3Ring - 256 * kMaxL3 - 256;
+static_assert(kPt3Deep >= 256, "ring of the point traversal");
+constexpr size_t kPt3Smem = (size_t)kPt3Warps * kPt3Ring * 4;
+template <bool OWN>
+__global__ void __launch_bounds__(kPt3Warps * 32)
+    k3_traverse_pt(int n, int L, const uint4 *__restrict__ z, const uint32_t *__restrict__ perm,
+                   const float4 *__restrict__ rec, const DevScalars *__restrict__ sc,
+                   float4 *__restrict__ Frep, float *__restrict__ Zi) {
+    extern __shared__ uint32_t s_ring[];
+    __shared__ float s_T[kMaxL + 2];
+    if (threadIdx.x < kMaxL + 2) s_T[threadIdx.x] = sc->T3[threadIdx.x];
+    __syncthreads();
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int idx = blockIdx.x * kPt3Warps + w;
+    if (idx >= n) return;  // whole warps; no block barrier follows
+    uint32_t *ring = s_ring + w * kPt3Ring;
+    const int F = 32 - L;
+    const uint32_t i = perm[idx];
+    const uint4 zi = z[i];
+    const uint32_t mi = morton3(zi.x >> F, zi.y >> F, zi.z >> F);
+    const uint32_t own_grp = (uint32_t)off3(L - 1) + (mi >> 3);
+    const Point3 pt = point3(zi);
+    const float2 s[3] = {b3(sc->sf3[0]), b3(sc->sf3[1]), b3(sc->sf3[2])};
+    Sum3 a{{b3(0.f), b3(0.f), b3(0.f)}, b3(0.f)};
+    const unsigned before = (1u << lane) - 1u;
+    if (lane == 0) ring[0] = 1u << 28;
+    uint32_t head = 0u, size = 1u;
+    __syncwarp();
+    while (size > 0u) {
+        const uint32_t k = min(size, 32u);
+        const uint32_t at = size <= (uint32_t)kPt3Deep ? head : head + size - k;
+        if (size <= (uint32_t)kPt3Deep) head += k;
+        size -= k;
+        const bool act = (uint32_t)lane < k;
+        const uint32_t node = act ? ring[(at + lane) & (kPt3Ring - 1)] : 1u << 28;
+        __syncwarp();
+        const uint32_t grp = node & 0x0fffffffu;
+        const int lc = (int)(node >> 28);
+        const bool leaf = lc == L;
+        const float4 *g = rec + (size_t)grp * (kGroup3 / 4);
+        const float Tl = s_T[lc];
+        const bool own = act && leaf && own_grp == grp;
+        const uint32_t mine = OWN ? mi >> (3 * (L - lc)) : 0u;
+        const uint32_t first = OWN ? 8u * (grp - (uint32_t)off3(lc - 1)) : 0u;
+        unsigned open = 0u;  // this lane's children to open
+#pragma unroll
+        for (int hf = 0; hf < 2; hf++) {
+            const float4 nv = act ? __ldg(g + 12 + hf) : make_float4(0.f, 0.f, 0.f, 0.f);
+            if (nv.x + nv.y + nv.z + nv.w == 0.f) continue;
+            float4 r[6];
+#pragma unroll
+            for (int q = 0; q < 6; q++) r[q] = __ldg(g + 2 * q + hf);
+#pragma unroll
+            for (int p = 0; p < 2; p++) {
+                const int c = 4 * hf + 2 * p;
+                const float2 N0 = half2of(nv, p);
+                float2 N = N0, dx[3];
+                offset3(r, p, pt, dx);
+                if (own && (int)((mi & 7u) >> 1) == 2 * hf + p) take_out3((int)(mi & 1u), N, dx);
+                const float2 d2 = dist3(dx, s);
+                const float2 tb = __ffma2_rn(N0, b3(1e30f), b3(-1e30f));
+                const float T0 = leaf ? -1.0f : fminf(tb.x, Tl), T1 = leaf ? -1.0f : fminf(tb.y, Tl);
+                const bool a0 = d2.x > T0 && (!OWN || leaf || mine != first + c);
+                const bool a1 = d2.y > T1 && (!OWN || leaf || mine != first + c + 1);
+                add3(a, make_float2(a0 ? N.x : 0.f, a1 ? N.y : 0.f), d2, dx);
+                // (a voxel is never opened, whatever a non-finite distance says)
+                open |= (!a0 && !leaf && N0.x > 1.f ? 1u : 0u) << c;
+                open |= (!a1 && !leaf && N0.y > 1.f ? 2u : 0u) << c;
             }
         }
         __syncwarp();
-        if (overflow) break;
+        const uint32_t child = ((uint32_t)(lc + 1) << 28) | (8u * grp + 1u);
+        uint32_t end = head + size;
+#pragma unroll
+        for (int c = 0; c < 8; c++) {
+            const bool o = (open >> c) & 1u;
+            const unsigned b = __ballot_sync(0xffffffffu, o);
+            if (o) ring[(end + __popc(b & before)) & (kPt3Ring - 1)] = child + (uint32_t)c;
+            end += __popc(b);
+        }
+        size = end - head;
+        __syncwarp();
     }
-    if (valid) {
-        Frep[i] = make_float4(fx, fy, fz, 0.f);
-        Zi[i] = zs;
+    float v[4] = {a.f[0].x + a.f[0].y, a.f[1].x + a.f[1].y, a.f[2].x + a.f[2].y, a.z.x + a.z.y};
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int d = 0; d < 4; d++) v[d] += __shfl_xor_sync(0xffffffffu, v[d], o);
+    if (lane == 0) {
+        Frep[i] = make_float4(v[0], v[1], v[2], 0.f);
+        Zi[i] = v[3];
     }
-    if (overflow && lane == 0) atomicOr(&sc->err, (unsigned)PXSNE_DEVERR_STACK);
 }
 
 // ---- Eq. grad's first term, one warp per row of P (rows padded with zero
@@ -706,14 +986,15 @@ cudaError_t alloc3(pxsne_ctx *c) {
     if ((e = alloc_n(&c->Fattr3, n))) return e;
     if ((e = alloc_n(&c->cnt3, (size_t)cells))) return e;
     if ((e = alloc_n(&c->sum3, 3 * (size_t)cells))) return e;
-    if ((e = alloc_n(&c->rec3a, (size_t)cells))) return e;
-    if ((e = alloc_n(&c->rec3b, (size_t)cells))) return e;
-    if ((e = alloc_n(&c->vstart3, (size_t)(int64_t(1) << (3 * c->L)) + 1))) return e;
+    // groups of siblings: one per cell above the leaves
+    const size_t groups = (size_t)off3(c->L);
+    if ((e = alloc_n(&c->rec3, groups * (kGroup3 / 4)))) return e;
+    if ((e = alloc_n(&c->pref3, (size_t)cells))) return e;
     // the leaf histogram starts from zeros; the first reduction clears what it read
     if ((e = cudaMemsetAsync(c->cnt3, 0, (size_t)cells * sizeof(uint32_t), c->stream))) return e;
     if ((e = cudaMemsetAsync(c->sum3, 0, 3 * (size_t)cells * sizeof(u64), c->stream))) return e;
-    c->dev_bytes += (int64_t)n * (16 + 24 + 16 * 4) + cells * (4 + 24 + 32) +
-                    ((int64_t(1) << (3 * c->L)) + 1) * 8;
+    c->dev_bytes += (int64_t)n * (16 + 24 + 16 * 4) + cells * (4 + 24) +
+                    (int64_t)groups * kGroup3 * 4 + cells * 4;
     return cudaSuccess;
 }
 
@@ -726,9 +1007,8 @@ void free3(pxsne_ctx *c) {
     free_p(c->Fattr3);
     free_p(c->cnt3);
     free_p(c->sum3);
-    free_p(c->rec3a);
-    free_p(c->rec3b);
-    free_p(c->vstart3);
+    free_p(c->rec3);
+    free_p(c->pref3);
 }
 
 cudaError_t launch_set_scalars3(pxsne_ctx *c, const double *s, int t) {
@@ -754,7 +1034,7 @@ cudaError_t launch_init3(pxsne_ctx *c, const float *Y0dev, double *scratch) {
 static cudaError_t tree3(pxsne_ctx *c, bool rescale) {
     cudaStream_t st = c->stream;
     const int L = c->L, n = (int)c->n;
-    const int64_t cells = cells3(L), leaves = int64_t(1) << (3 * L);
+    const int64_t cells = cells3(L);
     const int64_t lo = off3(L);
     uint32_t *cnt = c->cnt3;
     u64 *sx = c->sum3, *sy = c->sum3 + cells, *sz = c->sum3 + 2 * cells;
@@ -764,39 +1044,70 @@ static cudaError_t tree3(pxsne_ctx *c, bool rescale) {
     k3_snap<<<(n + 255) / 256, 256, 0, st>>>(n, L, rescale ? 1 : 0, c->p.theta, c->zhat3, c->z3,
                                               c->rank, cnt + lo, sx + lo, sy + lo, sz + lo, c->sc);
     if ((e = cudaGetLastError())) return e;
-    // the voxel order (before the leaves are cleared)
-    if ((e = scan_u32_to_i64(cnt + lo, leaves, c->vstart3, st))) return e;
-    k3_perm<<<(n + 255) / 256, 256, 0, st>>>(n, L, c->z3, c->rank, c->vstart3, c->perm, c->sc,
-                                              rescale ? 1 : 0);
+    // the octree from the bottom, and the voxel order
+    float *rec = reinterpret_cast<float *>(c->rec3);
+    for (int h = L; h > 3; h--) {
+        const int64_t m = int64_t(1) << (3 * (h - 1));
+        k3_level<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(h, h == L ? 1 : 0, cnt, sx, sy, sz,
+                                                              c->rec3, c->pref3);
+        if ((e = cudaGetLastError())) return e;
+    }
+    const int clear = L <= 3 ? 1 : 0;
+    if (L >= 3) k3_top<3><<<1, 512, 0, st>>>(clear, cnt, sx, sy, sz, rec, c->pref3);
+    else if (L == 2) k3_top<2><<<1, 64, 0, st>>>(clear, cnt, sx, sy, sz, rec, c->pref3);
+    else k3_top<1><<<1, 8, 0, st>>>(clear, cnt, sx, sy, sz, rec, c->pref3);
     if ((e = cudaGetLastError())) return e;
-    for (int l = L - 1; l >= 0; l--) {
-        const int64_t m = int64_t(1) << (3 * (l + 1));  // the children
-        k3_reduce<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(l, l == L - 1 ? 1 : 0, cnt, sx, sy,
-                                                               sz, c->rec3a, c->rec3b);
+    k3_perm<<<(n + 255) / 256, 256, 0, st>>>(n, L, c->z3, c->rank, c->pref3, c->perm, c->sc,
+                                              rescale ? 1 : 0);
+    return cudaGetLastError();
+}
+
+// Sets below kTrav3PointTo points take a warp per point: an iteration at n =
+// 2,000 on 64^3 takes 56 against 134 us, at 20,000 on 128^3 307 against 447, at
+// 40,000 on 256^3 812 against 678.
+constexpr int64_t kTrav3PointTo = 24576;
+
+static cudaError_t traverse3(pxsne_ctx *c) {
+    cudaStream_t st = c->stream;
+    const int n = (int)c->n;
+    // the own-cell test is redundant below theta = 1 (with a margin for the
+    // rounding of d^2)
+    const bool own = c->p.theta >= 0.999f;
+    if (c->n < kTrav3PointTo) {
+        cudaError_t e = cudaFuncSetAttribute(own ? k3_traverse_pt<true> : k3_traverse_pt<false>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)kPt3Smem);
+        if (e) return e;
+        const unsigned blocks = (unsigned)((n + kPt3Warps - 1) / kPt3Warps);
+        auto k = own ? k3_traverse_pt<true> : k3_traverse_pt<false>;
+        k<<<blocks, kPt3Warps * 32, kPt3Smem, st>>>(n, c->L, c->z3, c->perm, c->rec3, c->sc,
+                                                    c->Frep3, c->Zi);
+    } else {
+        const int per_block = kT3Warps * 32;
+        auto k = own ? k3_traverse<true> : k3_traverse<false>;
+        k<<<(n + per_block - 1) / per_block, per_block, 0, st>>>(n, c->L, c->z3, c->perm, c->rec3,
+                                                                 c->sc, c->Frep3, c->Zi);
     }
     return cudaGetLastError();
 }
 
-static cudaError_t forces3(pxsne_ctx *c) {
-    cudaStream_t st = c->stream;
+static cudaError_t attract3(pxsne_ctx *c, cudaStream_t st) {
     const int n = (int)c->n;
-    const int per_block = kT3Warps * 32;
-    k3_traverse<<<(n + per_block - 1) / per_block, per_block, 0, st>>>(
-        n, c->L, c->z3, c->perm, c->rec3a, c->rec3b, c->sc, c->Frep3, c->Zi);
-    cudaError_t e = cudaGetLastError();
-    if (e) return e;
     k3_attract<<<(unsigned)(((int64_t)n * 32 + 255) / 256), 256, 0, st>>>(
         n, c->rp, c->col, c->val, c->z3, c->sc, c->Fattr3);
-    if ((e = cudaGetLastError())) return e;
-    return launch_zsum(c);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_prime3(pxsne_ctx *c, bool rescale) {
     cudaError_t e = tree3(c, rescale);
     if (e) return e;
-    return forces3(c);
+    if ((e = traverse3(c))) return e;
+    if ((e = attract3(c, c->stream))) return e;
+    return launch_zsum(c);
 }
 
+// One iteration; the attraction, which needs only the rescaled positions and
+// P, runs on the side stream beside the traversal, as in 2-D.
 cudaError_t launch_iteration3(pxsne_ctx *c) {
     UpdateParams p;
     p.eta = c->p.eta;
@@ -807,15 +1118,20 @@ cudaError_t launch_iteration3(pxsne_ctx *c) {
     p.exag_iters = c->p.exag_iters;
     p.mom_switch = c->p.momentum_switch;
     const int n = (int)c->n;
-    int sms = 0, dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int blocks = std::max(1, std::min((n + 255) / 256, 4 * (sms > 0 ? sms : 1)));
+    const int blocks = std::max(1, std::min((n + 255) / 256, 4 * std::max(c->sms, 1)));
     k3_update<<<blocks, 256, 0, c->stream>>>(n, p, c->z3, c->Frep3, c->Fattr3, c->u3, c->gains3,
                                               c->zhat3, c->sc);
     cudaError_t e = cudaGetLastError();
     if (e) return e;
-    return launch_prime3(c, true);
+    if (!c->side) return launch_prime3(c, true);
+    if ((e = tree3(c, true))) return e;
+    if ((e = cudaEventRecord(c->ev_fork, c->stream))) return e;
+    if ((e = traverse3(c))) return e;
+    if ((e = launch_zsum(c))) return e;
+    if ((e = cudaStreamWaitEvent(c->side, c->ev_fork, 0))) return e;
+    if ((e = attract3(c, c->side))) return e;
+    if ((e = cudaEventRecord(c->ev_join, c->side))) return e;
+    return cudaStreamWaitEvent(c->stream, c->ev_join, 0);
 }
 
 cudaError_t launch_kl3(pxsne_ctx *c, double *out_dev) {

@@ -373,14 +373,13 @@ __global__ void __launch_bounds__(kTravWarps * 32, PPL == 1 ? 4 : 3)
                     }
                 }
             } else {
-                // Eq. bh_criteria's threshold on d^2.  A cell that holds one
-                // point stands for it exactly from level kExactLevel on (its
-                // offset in the cell is below 2^24 and so exact), so opening it
-                // down to its pixel would end in the same term: it is accepted
-                // at once by every point but the one in it, whose d^2 is 0
-                // (threshold 0).  Empty cells add nothing.
+                // Eq. bh_criteria's threshold on d^2.  The centre of a cell that
+                // holds one point is that point exactly, so opening it down to
+                // its pixel would end in the same term: it is accepted at once
+                // by every point but the one in it, whose d^2 is 0 (threshold
+                // 0).  Empty cells add nothing.
                 const float Tl = s_T[lc];
-                const float few = (CENTRE == 0 && lc >= kExactLevel) ? 1.0f : 0.0f;
+                constexpr float few = CENTRE == 0 ? 1.0f : 0.0f;
                 // room for the (at most four) entries this node may push
                 if (sp + 4 > stk_lim) {
                     overflow = true;
@@ -545,7 +544,7 @@ __global__ void __launch_bounds__(kPtWarps * 32)
         const uint32_t m = (CENTRE == 1 || OWN || COUNT) ? grp - (uint32_t)(rec_offset(lc) >> 2) : 0u;
         sib.load(rec, (int)(4u * grp), lc, m);
         const float Tl = s_T[lc];
-        const float few = (CENTRE == 0 && lc >= kExactLevel) ? 1.0f : 0.0f;
+        constexpr float few = CENTRE == 0 ? 1.0f : 0.0f;
         const bool own = leaf && act && (mi >> 2) + g0 == grp;
         const uint32_t mine = OWN ? mi >> (2 * (L - lc)) : 0u;
         bool open[4];

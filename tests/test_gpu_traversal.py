@@ -80,3 +80,39 @@ def test_every_cell_opened():
     oF, oZi, _ = oracle.bh_repulsion(z, s, L, 0.0)
     for Frep, Zi in ((a[0], a[1]), (b[0], b[1])):
         assert rel(Frep, oF) <= FORCE_TOL and rel(Zi, oZi) <= FORCE_TOL
+
+
+@pytest.mark.parametrize("n,level,theta", [
+    (40, 1, 0.5), (700, 2, 0.5), (900, 3, 1.2), (1500, 4, 0.3), (24575, 6, 0.5), (24576, 6, 0.5),
+    (24609, 5, 1.2), (24700, 7, 0.5)])
+def test_octree_across_the_kernels(n, level, theta):
+    """3-D: counts at every level, the order of the points and the forces on
+    both sides of the point traversal's limit and for the smallest octrees."""
+    import paper_1611_02568_gb300 as px
+    from paper_1611_02568_gb300 import build
+    build.build()
+    rng = np.random.default_rng([n, level])
+    z = rng.integers(0, 1 << 32, (n, 3), dtype=np.uint64)
+    m = n // 2
+    z[:m] = (1 << 30) + rng.integers(0, 1 << 27, (m, 3), dtype=np.uint64)
+    z[m:m + 4] = z[0]
+    z[-2], z[-1] = 0, (1 << 32) - 1
+    z, s = z.astype(np.uint32), np.array([40.0, 37.0, 51.0]) / 2.0 ** 32
+    rows = np.unique(np.concatenate([np.arange(min(n, 40)), np.arange(max(0, n - 40), n),
+                                     rng.integers(0, n, 800)]))
+    with px.Context(px.Params(log2_r=level, theta=theta, dim=3)) as ctx:
+        ctx.set_P(*ring_P(n))
+        for _ in range(2):   # from fresh leaves, and from the cleared ones
+            ctx.set_state(z, s)
+            Frep, Zi, _, Z = ctx.get_forces()
+            cnt_o = oracle.pyramid3(z, level)[0]
+            at = 0
+            for lv in range(level + 1):
+                assert np.array_equal(ctx.get_tree3(lv)[0], cnt_o[at:at + 8 ** lv]), lv
+                at += 8 ** lv
+            oF, oZi, _ = oracle.bh_repulsion3(z, s, level, theta, rows=rows)
+            assert rel(Frep[rows], oF) <= FORCE_TOL
+            assert rel(Zi[rows], oZi) <= FORCE_TOL
+            assert abs(Z - Zi.astype(np.float64).sum()) <= 1e-6 * Z
+            ctx.step(2)
+            ctx.sync()
