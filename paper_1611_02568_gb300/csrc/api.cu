@@ -2,6 +2,7 @@
 // per-iteration schedule (captured once as a CUDA graph) and the inspection
 // hooks.  All compute is in the kernels of tree.cu, forces.cu, update.cu and
 // affinity.cu.
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -186,7 +187,7 @@ int ensure_state(pxsne_ctx *c) {
     if (c->zblocks > 1024) c->zblocks = 1024;
     if (c->zblocks < 1) c->zblocks = 1;
     CK(c, dalloc(c, &c->zpart, c->zblocks));
-    c->klblocks = 304;
+    c->klblocks = 6 * std::max(c->sms, 1);
     CK(c, dalloc(c, &c->klpart, 2 * c->klblocks));
     return PXSNE_OK;
 }

@@ -116,3 +116,28 @@ def test_octree_across_the_kernels(n, level, theta):
             assert abs(Z - Zi.astype(np.float64).sum()) <= 1e-6 * Z
             ctx.step(2)
             ctx.sync()
+
+
+@pytest.mark.parametrize("n,level,k", [(40, 1, 32), (300, 4, 3), (5000, 11, 10), (5000, 3, 32), (20000, 9, 17)])
+def test_nbr_precision_on_uneven_states(n, level, k):
+    """The 2-D neighbour search over crowded cells, empty stretches and tied
+    positions: hit counts equal to the oracle's."""
+    import paper_1611_02568_gb300 as px
+    from paper_1611_02568_gb300 import build
+    build.build()
+    z, s = state(n, 11)
+    rng = np.random.default_rng([n, k])
+    # half of each row's list true neighbours of the index ring, half random
+    hd = np.stack([rng.permutation(n)[:k] for _ in range(50)])[rng.integers(0, 50, n)].astype(np.int32)
+    near = np.argsort(z[:, 0].astype(np.float64) * 3 + z[:, 1], kind="stable")
+    place = np.empty(n, np.int64)
+    place[near] = np.arange(n)
+    for a in range(k // 2):
+        hd[:, a] = near[(place + a + 1) % n]
+    with px.Context(px.Params(log2_r=level)) as ctx:
+        ctx.set_P(*ring_P(n))
+        ctx.set_state(z, s)
+        prec, hits = ctx.nbr_precision(k=k, knn_hd=hd, per_point=True)
+    prec_o, hits_o = oracle.nbr_precision(hd, k, z, s, per_row=True)
+    assert np.array_equal(hits, hits_o)
+    assert prec == pytest.approx(prec_o, abs=1e-15)
