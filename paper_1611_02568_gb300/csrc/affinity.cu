@@ -25,6 +25,7 @@
 
 #include "common.cuh"
 #include "knn.cuh"
+#include "sort.cuh"
 #include "tc.cuh"
 
 namespace pxsne {
@@ -1930,9 +1931,12 @@ cudaError_t launch_perplexity(pxsne_ctx *c, const float *d2, int64_t n, int32_t 
 }
 
 // ---------------------------------------------------------------- symmetrize
-__global__ void k_indeg(int64_t nk, const int32_t *__restrict__ idx, uint32_t *deg) {
+// In-degrees, and every entry's place among its target's incoming ones (one
+// atomic per entry serves both).
+__global__ void k_indeg(int64_t nk, const int32_t *__restrict__ idx, uint32_t *deg,
+                        uint32_t *__restrict__ slot) {
     const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e < nk) atomicAdd(&deg[idx[e]], 1u);
+    if (e < nk) slot[e] = atomicAdd(&deg[idx[e]], 1u);
 }
 
 // Exclusive scan of 32-bit counts into int64 offsets: per-block scan, then a
@@ -2002,164 +2006,138 @@ cudaError_t scan_u32_to_i64(const uint32_t *in, int64_t m, int64_t *out, cudaStr
 }
 
 // Row i of the union pattern: its own k entries (j, p_{j|i}) first, then the
-// incoming ones (j, p_{i|j}) for every j that lists i.
+// incoming ones (j, p_{i|j}) for every j that lists i, as keys column << 32 |
+// value bits.
+__device__ __forceinline__ u64 sym_key(int32_t col, float v) {
+    return ((u64)(uint32_t)col << 32) | __float_as_uint(v);
+}
 __global__ void k_fill(int64_t n, int k, const int32_t *__restrict__ idx,
                        const float *__restrict__ pcond, const int64_t *__restrict__ tptr,
-                       uint32_t *__restrict__ cursor, int32_t *__restrict__ tcol,
-                       float *__restrict__ tval) {
+                       const uint32_t *__restrict__ slot, u64 *__restrict__ T) {
     const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (e >= n * k) return;
     const int64_t i = e / k;
     const int a = (int)(e % k);
     const int32_t j = idx[e];
     const float p = pcond[e];
-    tcol[tptr[i] + a] = j;
-    tval[tptr[i] + a] = p;
-    const uint32_t slot = (uint32_t)k + atomicAdd(&cursor[j], 1u);
-    tcol[tptr[j] + slot] = (int32_t)i;
-    tval[tptr[j] + slot] = p;
+    T[tptr[i] + a] = sym_key(j, p);
+    T[tptr[j] + k + slot[e]] = sym_key((int32_t)i, p);
 }
 
-// Sort each temporary row by (col, position) (rank sort, one warp per row,
-// the row's columns staged in shared memory when it has at most kSmRow
-// entries), then merge equal columns (a column appears at most twice: once
-// from the row's own list, once from the other row's); count = number of
-// distinct columns.  With write == 1 the merged row goes to (col, val / 2n) at
-// rp[i], padded with (i, 0) to rp[i + 1].
-constexpr int kSmRow = 1024;
+// Each row's keys in column order, equal columns merged in place (a column
+// appears at most twice, once from the row's own list and once from the other
+// row's: their values add), cnt = the number of distinct columns.  A warp sorts
+// a row of at most 32 V keys in its registers; rows is the list of the rows to
+// take (NULL: all rows, those beyond 256 keys skipped).  n = 1M, k = 90 (180
+// keys a row on average): 3.7 ms with the longer rows' launches and the copy into
+// the CSR arrays; ranking every key against all others from shared memory, and a
+// second pass that merged, took 17.
+constexpr int kSymWarps = 4;
+template <int V>
+__global__ void __launch_bounds__(kSymWarps * 32)
+    k_sym_rows(int64_t n, const uint32_t *__restrict__ rows, const int64_t *__restrict__ tptr,
+               u64 *__restrict__ T, uint32_t *__restrict__ cnt) {
+    // element e at e + e / V: the lanes' runs of V keys do not meet in a bank
+    __shared__ u64 s_k[kSymWarps][33 * V + 32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t q = blockIdx.x * (int64_t)kSymWarps + w;
+    if (q >= n) return;
+    const int64_t row = rows ? rows[q] : q;
+    const int64_t a = tptr[row];
+    const int len = (int)(tptr[row + 1] - a);
+    if (len > 32 * V) return;  // another launch's
+    u64 key[V];
+#pragma unroll
+    for (int v = 0; v < V; v++) key[v] = v * 32 + lane < len ? T[a + v * 32 + lane] : ~0ull;
+    sort_keys<V>(key, lane);
+    u64 *sk = s_k[w];
+#pragma unroll
+    for (int v = 0; v < V; v++) sk[lane * (V + 1) + v] = key[v];
+    __syncwarp();
+    uint32_t done = 0u;
+    for (int e0 = 0; e0 < len; e0 += 32) {
+        const int e = e0 + lane;
+        const u64 x = e < len ? sk[e + e / V] : ~0ull;
+        const u64 nx = e + 1 < len ? sk[e + 1 + (e + 1) / V] : ~0ull;
+        const uint32_t c = (uint32_t)(x >> 32);
+        const bool head = e < len && (e == 0 || (uint32_t)(sk[e - 1 + (e - 1) / V] >> 32) != c);
+        const unsigned hm = __ballot_sync(0xffffffffu, head);
+        if (head) {
+            float v = __uint_as_float((uint32_t)x);
+            if (e + 1 < len && (uint32_t)(nx >> 32) == c) v += __uint_as_float((uint32_t)nx);
+            T[a + done + __popc(hm & ((1u << lane) - 1u))] = sym_key((int32_t)c, v);
+        }
+        done += (uint32_t)__popc(hm);
+    }
+    if (lane == 0) cnt[row] = done;
+}
+
+// The merged rows into the CSR, halved and divided by n, padded with (row, 0) to
+// the row's end; one warp per row.
 __global__ void __launch_bounds__(256)
-    k_sort_merge(int64_t n, int write, const int64_t *__restrict__ tptr,
-                 const int32_t *__restrict__ tcol, const float *__restrict__ tval,
-                 int32_t *__restrict__ scol, float *__restrict__ sval,
-                 uint32_t *__restrict__ cnt, const int64_t *__restrict__ rp,
-                 int32_t *__restrict__ col, float *__restrict__ val) {
-    __shared__ int32_t s_c[8][kSmRow];
+    k_sym_write(int64_t n, const int64_t *__restrict__ tptr, const u64 *__restrict__ T,
+                const uint32_t *__restrict__ cnt, const int64_t *__restrict__ rp,
+                int32_t *__restrict__ col, float *__restrict__ val) {
     const int64_t row = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31, w = (threadIdx.x >> 5) & 7;
+    const int lane = threadIdx.x & 31;
     if (row >= n) return;
-    const int64_t a = tptr[row], b = tptr[row + 1];
-    const int len = (int)(b - a);
-    if (!write) {
-        if (len <= kSmRow) {
-            // columns in shared memory, padded to a multiple of 4 with a value
-            // above every column; each pass ranks up to 8 elements per lane
-            // against all columns, read 16 bytes at a time
-            int32_t *sc = s_c[w];
-            const int len4 = (len + 3) & ~3;
-            for (int e = lane; e < len4; e += 32) sc[e] = e < len ? tcol[a + e] : 0x7fffffff;
-            __syncwarp();
-            const int4 *sc4 = reinterpret_cast<const int4 *>(sc);
-            for (int e0 = 0; e0 < len; e0 += 256) {
-                int32_t ce[8];
-                int r[8];
-#pragma unroll
-                for (int m = 0; m < 8; m++) {
-                    const int e = e0 + 32 * m + lane;
-                    ce[m] = e < len ? sc[e] : 0x7fffffff;
-                    r[m] = 0;
-                }
-                for (int f4 = 0; f4 < (len4 >> 2); f4++) {
-                    const int4 c4 = sc4[f4];
-                    const int f = 4 * f4;
-#pragma unroll
-                    for (int m = 0; m < 8; m++) {
-                        const int e = e0 + 32 * m + lane;
-                        r[m] += (c4.x < ce[m]) || (c4.x == ce[m] && f < e);
-                        r[m] += (c4.y < ce[m]) || (c4.y == ce[m] && f + 1 < e);
-                        r[m] += (c4.z < ce[m]) || (c4.z == ce[m] && f + 2 < e);
-                        r[m] += (c4.w < ce[m]) || (c4.w == ce[m] && f + 3 < e);
-                    }
-                }
-#pragma unroll
-                for (int m = 0; m < 8; m++) {
-                    const int e = e0 + 32 * m + lane;
-                    if (e < len) {
-                        scol[a + r[m]] = ce[m];
-                        sval[a + r[m]] = tval[a + e];
-                    }
-                }
-            }
-        } else {
-            return;  // a long row: k_sort_long
-        }
-        __syncwarp();
-        uint32_t u = 0;
-        for (int e0 = 0; e0 < len; e0 += 32) {
-            const int e = e0 + lane;
-            const bool head = e < len && (e == 0 || scol[a + e] != scol[a + e - 1]);
-            u += (uint32_t)__popc(__ballot_sync(0xffffffffu, head));
-        }
-        if (lane == 0) cnt[row] = u;
-    } else {
-        const float inv2n = (float)(0.5 / (double)n);
-        const int64_t o0 = rp[row];
-        uint32_t done = 0;  // distinct columns written so far
-        for (int e0 = 0; e0 < len; e0 += 32) {
-            const int e = e0 + lane;
-            int32_t ce = 0;
-            bool head = false;
-            if (e < len) {
-                ce = scol[a + e];
-                head = (e == 0 || ce != scol[a + e - 1]);
-            }
-            const unsigned hm = __ballot_sync(0xffffffffu, head);
-            if (head) {
-                float v = sval[a + e];
-                if (e + 1 < len && scol[a + e + 1] == ce) v += sval[a + e + 1];
-                const int64_t o = o0 + done + __popc(hm & ((1u << lane) - 1u));
-                col[o] = ce;
-                val[o] = v * inv2n;
-            }
-            done += (uint32_t)__popc(hm);
-        }
-        for (int64_t q = o0 + done + lane; q < rp[row + 1]; q += 32) {  // padding
-            col[q] = (int32_t)row;
-            val[q] = 0.f;
-        }
+    const float inv2n = (float)(0.5 / (double)n);
+    const int64_t a = tptr[row], o = rp[row];
+    const int len = (int)cnt[row], pad = (int)(rp[row + 1] - o);
+    for (int e = lane; e < pad; e += 32) {
+        const u64 x = e < len ? T[a + e] : sym_key((int32_t)row, 0.f);
+        col[o + e] = (int32_t)(x >> 32);
+        val[o + e] = __uint_as_float((uint32_t)x) * inv2n;
     }
 }
 
-// Rows longer than kSmRow (the hubs of the kNN graph, with thousands of
-// incoming entries): one CTA per row sorts the keys (col << 32 | position) by a
-// bitonic network in global scratch padded to a power of two, then writes the
-// sorted row and its count of distinct columns.
-__global__ void k_long_rows(int64_t n, const int64_t *__restrict__ tptr, uint32_t *list,
-                            uint32_t *nlong, uint32_t *plen) {
+// Rows of more than 256 keys by class: up to 512 and up to 1,024 (a warp's
+// registers again), and the hubs of the kNN graph beyond (a CTA each; plen =
+// their length rounded up to a power of two).
+constexpr int kSymRow = 1024;
+__global__ void k_long_rows(int64_t n, const int64_t *__restrict__ tptr, uint32_t *l0,
+                            uint32_t *l1, uint32_t *l2, uint32_t *num, uint32_t *plen) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
     const int64_t len = tptr[i + 1] - tptr[i];
-    if (len > kSmRow) {
-        const uint32_t q = atomicAdd(nlong, 1u);
+    if (len <= 256) return;
+    if (len <= 512) {
+        l0[atomicAdd(&num[0], 1u)] = (uint32_t)i;
+    } else if (len <= kSymRow) {
+        l1[atomicAdd(&num[1], 1u)] = (uint32_t)i;
+    } else {
+        const uint32_t q = atomicAdd(&num[2], 1u);
         uint32_t p2 = 1u;
         while (p2 < (uint64_t)len) p2 <<= 1;
-        list[q] = (uint32_t)i;
+        l2[q] = (uint32_t)i;
         plen[q] = p2;
     }
 }
 
+// A hub's row: one CTA sorts its keys by a bitonic network, in shared memory if
+// they fit (P <= cap), else in global scratch, and merges equal columns as above.
 __global__ void __launch_bounds__(1024)
     k_sort_long(const uint32_t *__restrict__ list, const uint32_t *__restrict__ plen,
-                const int64_t *__restrict__ soff, const int64_t *__restrict__ tptr,
-                const int32_t *__restrict__ tcol, const float *__restrict__ tval,
-                unsigned long long *scratch, int32_t *__restrict__ scol,
-                float *__restrict__ sval, uint32_t *__restrict__ cnt) {
+                const int64_t *__restrict__ soff, const int64_t *__restrict__ tptr, u64 *T,
+                u64 *scratch, int cap, uint32_t *__restrict__ cnt) {
+    extern __shared__ u64 s_keys[];
     __shared__ uint32_t s_w[32];
+    __shared__ uint32_t s_done;
     const uint32_t row = list[blockIdx.x];
     const int64_t a = tptr[row];
     const int len = (int)(tptr[row + 1] - a);
     const int P = (int)plen[blockIdx.x];
-    unsigned long long *key = scratch + soff[blockIdx.x];
-    const int tid = threadIdx.x;
-    for (int i = tid; i < P; i += blockDim.x)
-        key[i] = i < len ? (((unsigned long long)(uint32_t)tcol[a + i]) << 32) | (uint32_t)i
-                         : ~0ull;
+    u64 *key = P <= cap ? s_keys : scratch + soff[blockIdx.x];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int i = tid; i < P; i += blockDim.x) key[i] = i < len ? T[a + i] : ~0ull;
+    if (tid == 0) s_done = 0u;
     __syncthreads();
     for (int k2 = 2; k2 <= P; k2 <<= 1) {
         for (int j = k2 >> 1; j > 0; j >>= 1) {
             for (int i = tid; i < P; i += blockDim.x) {
                 const int l = i ^ j;
                 if (l > i) {
-                    const unsigned long long x = key[i], y = key[l];
+                    const u64 x = key[i], y = key[l];
                     const bool asc = (i & k2) == 0;
                     if ((x > y) == asc) {
                         key[i] = y;
@@ -2170,24 +2148,31 @@ __global__ void __launch_bounds__(1024)
             __syncthreads();
         }
     }
-    for (int i = tid; i < len; i += blockDim.x) {
-        const unsigned long long u = key[i];
-        scol[a + i] = (int32_t)(u >> 32);
-        sval[a + i] = tval[a + (uint32_t)(u & 0xffffffffull)];
+    for (int i0 = 0; i0 < len; i0 += (int)blockDim.x) {
+        const int i = i0 + tid;
+        const u64 x = i < len ? key[i] : ~0ull;
+        const uint32_t c = (uint32_t)(x >> 32);
+        const bool head = i < len && (i == 0 || (uint32_t)(key[i - 1] >> 32) != c);
+        const unsigned hm = __ballot_sync(0xffffffffu, head);
+        if (lane == 0) s_w[warp] = (uint32_t)__popc(hm);
+        __syncthreads();
+        uint32_t at = s_done;
+        for (int w = 0; w < warp; w++) at += s_w[w];
+        if (head) {
+            float v = __uint_as_float((uint32_t)x);
+            if (i + 1 < len && (uint32_t)(key[i + 1] >> 32) == c)
+                v += __uint_as_float((uint32_t)key[i + 1]);
+            T[a + at + __popc(hm & ((1u << lane) - 1u))] = sym_key((int32_t)c, v);
+        }
+        __syncthreads();
+        if (tid == 0) {
+            uint32_t t = s_done;
+            for (int w = 0; w < (int)(blockDim.x >> 5); w++) t += s_w[w];
+            s_done = t;
+        }
+        __syncthreads();
     }
-    __syncthreads();
-    uint32_t u = 0u;
-    for (int i = tid; i < len; i += blockDim.x)
-        u += (i == 0 || scol[a + i] != scol[a + i - 1]) ? 1u : 0u;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) u += __shfl_xor_sync(0xffffffffu, u, o);
-    if ((tid & 31) == 0) s_w[tid >> 5] = u;
-    __syncthreads();
-    if (tid == 0) {
-        uint32_t t = 0u;
-        for (int w = 0; w < (int)(blockDim.x >> 5); w++) t += s_w[w];
-        cnt[row] = t;
-    }
+    if (tid == 0) cnt[row] = s_done;
 }
 
 __global__ void k_round4(int64_t n, const uint32_t *in, uint32_t *out) {
@@ -2205,10 +2190,9 @@ cudaError_t build_symmetric_csr(pxsne_ctx *c, const int32_t *idx, const float *p
     cudaStream_t st = c->stream;
     cudaError_t e;
     const int64_t nk = n * k;
-    uint32_t *deg = nullptr, *cursor = nullptr;
+    uint32_t *deg = nullptr, *cursor = nullptr, *slot = nullptr;
     int64_t *tptr = nullptr;
-    int32_t *tcol = nullptr, *scol = nullptr;
-    float *tval = nullptr, *sval = nullptr;
+    u64 *T = nullptr;
 #define TRY(x)                 \
     do {                       \
         if ((e = (x))) {       \
@@ -2220,63 +2204,69 @@ cudaError_t build_symmetric_csr(pxsne_ctx *c, const int32_t *idx, const float *p
     TRY(cudaMallocAsync(&cursor, n * sizeof(uint32_t), st));
     TRY(cudaMallocAsync(&tptr, (n + 1) * sizeof(int64_t), st));
     TRY(cudaMemsetAsync(deg, 0, n * sizeof(uint32_t), st));
-    TRY(cudaMemsetAsync(cursor, 0, n * sizeof(uint32_t), st));
-    k_indeg<<<(unsigned)((nk + 255) / 256), 256, 0, st>>>(nk, idx, deg);
+    TRY(cudaMallocAsync(&slot, nk * sizeof(uint32_t), st));
+    k_indeg<<<(unsigned)((nk + 255) / 256), 256, 0, st>>>(nk, idx, deg, slot);
     TRY(cudaGetLastError());
     // temporary rows of length k + indeg(i); 2 n k entries in total
     uint32_t *len = cursor;
     k_add_const<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, deg, len, (uint32_t)k);
     TRY(cudaGetLastError());
     TRY(scan_u32_to_i64(len, n, tptr, st));
-    TRY(cudaMemsetAsync(cursor, 0, n * sizeof(uint32_t), st));
-    TRY(cudaMallocAsync(&tcol, 2 * nk * sizeof(int32_t), st));
-    TRY(cudaMallocAsync(&tval, 2 * nk * sizeof(float), st));
-    TRY(cudaMallocAsync(&scol, 2 * nk * sizeof(int32_t), st));
-    TRY(cudaMallocAsync(&sval, 2 * nk * sizeof(float), st));
-    k_fill<<<(unsigned)((nk + 255) / 256), 256, 0, st>>>(n, k, idx, pcond, tptr, cursor, tcol,
-                                                        tval);
+    TRY(cudaMallocAsync(&T, 2 * nk * sizeof(u64), st));
+    k_fill<<<(unsigned)((nk + 255) / 256), 256, 0, st>>>(n, k, idx, pcond, tptr, slot, T);
     TRY(cudaGetLastError());
     uint32_t *ucnt = deg;  // reuse
-    k_sort_merge<<<(unsigned)((n * 32 + 255) / 256), 256, 0, st>>>(
-        n, 0, tptr, tcol, tval, scol, sval, ucnt, nullptr, nullptr, nullptr);
+    k_sym_rows<8><<<(unsigned)((n + kSymWarps - 1) / kSymWarps), kSymWarps * 32, 0, st>>>(
+        n, nullptr, tptr, T, ucnt);
     TRY(cudaGetLastError());
     {
-        // long rows
-        uint32_t *list = nullptr, *nlong = nullptr, *plen = nullptr;
-        TRY(cudaMallocAsync(&list, (size_t)n * sizeof(uint32_t), st));
-        TRY(cudaMallocAsync(&plen, (size_t)n * sizeof(uint32_t), st));
-        TRY(cudaMallocAsync(&nlong, sizeof(uint32_t), st));
-        TRY(cudaMemsetAsync(nlong, 0, sizeof(uint32_t), st));
-        k_long_rows<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, tptr, list, nlong, plen);
+        // the longer rows
+        uint32_t *lists = nullptr;  // three lists and the hubs' padded lengths, then their counts
+        TRY(cudaMallocAsync(&lists, ((size_t)n * 4 + 4) * sizeof(uint32_t), st));
+        uint32_t *num = lists + (size_t)n * 4, *hubs = lists + 2 * (size_t)n, *plen = lists + 3 * (size_t)n;
+        TRY(cudaMemsetAsync(num, 0, 4 * sizeof(uint32_t), st));
+        k_long_rows<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, tptr, lists, lists + n, hubs, num,
+                                                                 plen);
         TRY(cudaGetLastError());
-        uint32_t hl = 0;
-        TRY(cudaMemcpyAsync(&hl, nlong, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
+        uint32_t hn[4] = {0u, 0u, 0u, 0u};
+        TRY(cudaMemcpyAsync(hn, num, sizeof(hn), cudaMemcpyDeviceToHost, st));
         TRY(cudaStreamSynchronize(st));
+        if (hn[0] > 0)
+            k_sym_rows<16><<<(hn[0] + kSymWarps - 1) / kSymWarps, kSymWarps * 32, 0, st>>>(
+                hn[0], lists, tptr, T, ucnt);
+        if (hn[1] > 0)
+            k_sym_rows<32><<<(hn[1] + kSymWarps - 1) / kSymWarps, kSymWarps * 32, 0, st>>>(
+                hn[1], lists + n, tptr, T, ucnt);
+        TRY(cudaGetLastError());
+        const uint32_t hl = hn[2];
         if (hl > 0) {
+            constexpr int kSmemKeys = 16384;  // 128 KB
             std::vector<uint32_t> hp(hl);
             TRY(cudaMemcpyAsync(hp.data(), plen, hl * sizeof(uint32_t), cudaMemcpyDeviceToHost,
                                 st));
             TRY(cudaStreamSynchronize(st));
             std::vector<int64_t> ho(hl);
             int64_t tot = 0;
+            uint32_t most = 0u;
             for (uint32_t q = 0; q < hl; q++) {
                 ho[q] = tot;
-                tot += hp[q];
+                if (hp[q] > kSmemKeys) tot += hp[q];
+                else most = std::max(most, hp[q]);
             }
             int64_t *soff = nullptr;
-            unsigned long long *scr = nullptr;
+            u64 *scr = nullptr;
             TRY(cudaMallocAsync(&soff, hl * sizeof(int64_t), st));
-            TRY(cudaMallocAsync(&scr, (size_t)tot * sizeof(unsigned long long), st));
+            TRY(cudaMallocAsync(&scr, (size_t)std::max<int64_t>(tot, 1) * sizeof(u64), st));
             TRY(cudaMemcpyAsync(soff, ho.data(), hl * sizeof(int64_t), cudaMemcpyHostToDevice, st));
-            k_sort_long<<<hl, 1024, 0, st>>>(list, plen, soff, tptr, tcol, tval, scr, scol, sval,
-                                             ucnt);
+            TRY(cudaFuncSetAttribute(k_sort_long, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     kSmemKeys * (int)sizeof(u64)));
+            k_sort_long<<<hl, 1024, (size_t)most * sizeof(u64), st>>>(hubs, plen, soff, tptr, T, scr,
+                                                                      (int)most, ucnt);
             TRY(cudaGetLastError());
             cudaFreeAsync(soff, st);
             cudaFreeAsync(scr, st);
         }
-        cudaFreeAsync(list, st);
-        cudaFreeAsync(plen, st);
-        cudaFreeAsync(nlong, st);
+        cudaFreeAsync(lists, st);
     }
     if (c->rp) { cudaFreeAsync(c->rp, st); c->rp = nullptr; }
     if (c->col) { cudaFreeAsync(c->col, st); c->col = nullptr; }
@@ -2299,8 +2289,8 @@ cudaError_t build_symmetric_csr(pxsne_ctx *c, const int32_t *idx, const float *p
     TRY(cudaStreamSynchronize(st));
     TRY(cudaMallocAsync(&c->col, (nnz_pad > 0 ? nnz_pad : 4) * sizeof(int32_t), st));
     TRY(cudaMallocAsync(&c->val, (nnz_pad > 0 ? nnz_pad : 4) * sizeof(float), st));
-    k_sort_merge<<<(unsigned)((n * 32 + 255) / 256), 256, 0, st>>>(
-        n, 1, tptr, tcol, tval, scol, sval, ucnt, c->rp, c->col, c->val);
+    k_sym_write<<<(unsigned)((n * 32 + 255) / 256), 256, 0, st>>>(n, tptr, T, ucnt, c->rp, c->col,
+                                                                 c->val);
     TRY(cudaGetLastError());
     c->nnz_pad = nnz_pad;
     c->nnz = nnz;
@@ -2308,10 +2298,8 @@ cudaError_t build_symmetric_csr(pxsne_ctx *c, const int32_t *idx, const float *p
     cudaFreeAsync(cursor, st);
     cudaFreeAsync(tptr, st);
     cudaFreeAsync(uscan, st);
-    cudaFreeAsync(tcol, st);
-    cudaFreeAsync(tval, st);
-    cudaFreeAsync(scol, st);
-    cudaFreeAsync(sval, st);
+    cudaFreeAsync(slot, st);
+    cudaFreeAsync(T, st);
 #undef TRY
     return cudaGetLastError();
 }

@@ -29,6 +29,7 @@
 
 #include "common.cuh"
 #include "knn.cuh"
+#include "sort.cuh"
 #include "tc.cuh"
 
 namespace pxsne {
@@ -455,41 +456,6 @@ __global__ void __launch_bounds__(kThreads, 2) k_knn_scan(const ScanArgs a) {
 // index); it is sorted by a bitonic network in registers, 8 or 16 keys per lane.
 constexpr int kPickWarps = 2;
 constexpr int kPickKeys = 512;  // most candidates within tau
-
-template <int V>
-__device__ __forceinline__ void sort_keys(u64 (&key)[V], int lane) {
-    // element lane * V + v; ascending
-#pragma unroll
-    for (int k2 = 2; k2 <= 32 * V; k2 <<= 1) {
-#pragma unroll
-        for (int j = k2 >> 1; j > 0; j >>= 1) {
-            if (j >= V) {
-                const int lj = j / V;
-                const bool upper = lane & lj;
-#pragma unroll
-                for (int v = 0; v < V; v++) {
-                    const bool up = ((lane * V + v) & k2) == 0;
-                    const u64 o = __shfl_xor_sync(0xffffffffu, key[v], lj);
-                    const bool less = o < key[v];
-                    // the lower element of an ascending pair keeps the smaller key
-                    key[v] = (less == (up != upper)) ? o : key[v];
-                }
-            } else {
-#pragma unroll
-                for (int v = 0; v < V; v++) {
-                    const int w = v ^ j;
-                    if (w > v) {
-                        const bool up = ((lane * V + v) & k2) == 0;
-                        const u64 x = key[v], y = key[w];
-                        const bool sw = (x > y) == up;
-                        key[v] = sw ? y : x;
-                        key[w] = sw ? x : y;
-                    }
-                }
-            }
-        }
-    }
-}
 
 template <int V>
 __device__ __forceinline__ void sort_buffer(u64 *keys, int cnt, int lane) {

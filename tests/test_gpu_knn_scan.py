@@ -72,3 +72,31 @@ def test_one_dimension_far_apart():
     x = np.concatenate([1.02 ** np.arange(1200), -(1.02 ** np.arange(1200))])
     X = np.stack([x, 0.5 * x], 1).astype(np.float32)
     check(X, 20, *lists(X, 20))
+
+
+def test_symmetric_rows_of_every_class():
+    """P with rows of every length class of the symmetrisation (a warp's 256,
+    512 and 1,024 keys, a CTA's shared memory and beyond): shells of points
+    around centres that are every shell point's nearest neighbour.  Pattern
+    equal to the oracle's, values within the bisection tolerance."""
+    import paper_1611_02568_gb300 as px
+    from paper_1611_02568_gb300 import build
+    build.build()
+    rng = np.random.default_rng(8)
+    parts = []
+    for g, m in enumerate((240, 280, 500, 530, 1015, 1100, 16500)):
+        x = rng.standard_normal((m, 120))
+        x *= rng.uniform(9.0, 11.0, (m, 1)) / np.linalg.norm(x, axis=1, keepdims=True)
+        x[0] = 0.0
+        x[:, g] += 200.0 * (g + 1)
+        parts.append(x)
+    X = rng.permutation(np.concatenate(parts)).astype(np.float32)
+    P, _, _, bad = oracle.affinities(X, 3.0, 5)
+    lengths = np.diff(P.row_ptr)
+    for lo, hi in ((1, 256), (256, 512), (512, 1024), (1024, 16384), (16384, 1 << 30)):
+        assert ((lengths > lo) & (lengths <= hi)).any()
+    with px.Context(px.Params(log2_r=9, k=5, perplexity=3.0)) as ctx:
+        ctx.affinities(X)
+        rp, col, val = ctx.get_P()
+    assert np.array_equal(rp, P.row_ptr) and np.array_equal(col, P.col)
+    np.testing.assert_allclose(val, P.val, rtol=2e-3, atol=1e-9)
