@@ -469,14 +469,18 @@ constexpr int kCells = 512;     // pivots (cells) of the locality order
 constexpr int kPivChunk = 128;  // pivots staged in shared memory at a time
 
 // cell[i] = the pivot nearest to row i (squared Euclidean, |p|^2 - 2 x.p in
-// FP32), pivots staged in shared memory; DP = D rounded up to 64.
+// FP32), pivots staged in shared memory; DP = D rounded up to 64.  A thread
+// holds its row in registers and takes four pivots at a time: one dot product
+// is a chain of dependent FMAs, and the registers leave two warps per scheduler
+// (n = 1M, D = 128: 6.2 ms with one at a time).
 template <int DP>
 __global__ void __launch_bounds__(256)
     k_assign_cells(int64_t n, int D, int m, const float *__restrict__ X,
                    const float *__restrict__ piv, const float *__restrict__ pn,
                    const float *__restrict__ nrm, uint32_t *__restrict__ cell,
                    float *__restrict__ dpiv) {
-    extern __shared__ float s_piv[];  // kPivChunk x DP
+    extern __shared__ float s_piv[];  // kPivChunk x DP, then the pivots' norms
+    float *s_pn = s_piv + kPivChunk * DP;
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     float xr[DP];
 #pragma unroll
@@ -484,28 +488,35 @@ __global__ void __launch_bounds__(256)
     float best = INFINITY;
     uint32_t bi = 0u;
     for (int p0 = 0; p0 < m; p0 += kPivChunk) {
-        const int pc = min(kPivChunk, m - p0);
+        const int pc = min(kPivChunk, m - p0), p4 = (pc + 3) & ~3;
         __syncthreads();
-        for (int q = threadIdx.x; q < pc * DP; q += blockDim.x) {
+        for (int q = threadIdx.x; q < p4 * DP; q += blockDim.x) {
             const int pi = q / DP, d = q % DP;
-            s_piv[q] = d < D ? piv[(int64_t)(p0 + pi) * D + d] : 0.f;
+            s_piv[q] = pi < pc && d < D ? piv[(int64_t)(p0 + pi) * D + d] : 0.f;
         }
+        for (int q = threadIdx.x; q < p4; q += blockDim.x) s_pn[q] = q < pc ? pn[p0 + q] : INFINITY;
         __syncthreads();
-        for (int pi = 0; pi < pc; pi++) {
+        for (int pi = 0; pi < p4; pi += 4) {
             const float4 *pr = reinterpret_cast<const float4 *>(s_piv + pi * DP);
-            float dot = 0.f;
+            float dot[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
             for (int d4 = 0; d4 < DP / 4; d4++) {
-                const float4 pv = pr[d4];
-                dot = fmaf(xr[4 * d4], pv.x, dot);
-                dot = fmaf(xr[4 * d4 + 1], pv.y, dot);
-                dot = fmaf(xr[4 * d4 + 2], pv.z, dot);
-                dot = fmaf(xr[4 * d4 + 3], pv.w, dot);
+#pragma unroll
+                for (int u = 0; u < 4; u++) {
+                    const float4 pv = pr[u * (DP / 4) + d4];
+                    dot[u] = fmaf(xr[4 * d4], pv.x, dot[u]);
+                    dot[u] = fmaf(xr[4 * d4 + 1], pv.y, dot[u]);
+                    dot[u] = fmaf(xr[4 * d4 + 2], pv.z, dot[u]);
+                    dot[u] = fmaf(xr[4 * d4 + 3], pv.w, dot[u]);
+                }
             }
-            const float v = fmaf(-2.0f, dot, pn[p0 + pi]);
-            if (v < best) {
-                best = v;
-                bi = (uint32_t)(p0 + pi);
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                const float v = fmaf(-2.0f, dot[u], s_pn[pi + u]);
+                if (v < best) {
+                    best = v;
+                    bi = (uint32_t)(p0 + pi + u);
+                }
             }
         }
     }
@@ -650,9 +661,20 @@ __global__ void k_rp_side(int64_t n, int D, const float *__restrict__ X,
     const float *xb = X + (int64_t)order[sg.x + ob] * D;
     const float *xi = X + (int64_t)order[r] * D;
     float p = 0.f;
-    for (int d = 0; d < D; d++) {
-        const float u = __ldg(xa + d), v = __ldg(xb + d);
-        p = fmaf(__ldg(xi + d) - 0.5f * (u + v), u - v, p);
+    auto side = [&p](float x, float u, float v) { p = fmaf(x - 0.5f * (u + v), u - v, p); };
+    if ((D & 3) == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0) {
+        // 16 bytes of the row at a time: every thread walks a row of its own
+        for (int d = 0; d < D; d += 4) {
+            const float4 x = __ldg(reinterpret_cast<const float4 *>(xi + d));
+            const float4 u = __ldg(reinterpret_cast<const float4 *>(xa + d));
+            const float4 v = __ldg(reinterpret_cast<const float4 *>(xb + d));
+            side(x.x, u.x, v.x);
+            side(x.y, u.y, v.y);
+            side(x.z, u.z, v.z);
+            side(x.w, u.w, v.w);
+        }
+    } else {
+        for (int d = 0; d < D; d++) side(__ldg(xi + d), __ldg(xa + d), __ldg(xb + d));
     }
     flag[r] = p >= 0.f ? 1u : 0u;
 }
@@ -1609,7 +1631,7 @@ cudaError_t launch_knn(pxsne_ctx *c, const float *Xdev, int64_t n, int32_t D, in
         if ((e = cudaMemcpyAsync(pn, hn.data(), (size_t)m * sizeof(float), cudaMemcpyHostToDevice,
                                  st)))
             return e;
-        const size_t smem_a = (size_t)std::min(m, kPivChunk) * Dp * sizeof(float);
+        const size_t smem_a = (size_t)kPivChunk * (Dp + 1) * sizeof(float);
         const unsigned ablocks = (unsigned)((n + 255) / 256);
         if (Dp == 64) {
             if ((e = cudaFuncSetAttribute(k_assign_cells<64>,
@@ -1846,11 +1868,12 @@ cudaError_t launch_knn(pxsne_ctx *c, const float *Xdev, int64_t n, int32_t D, in
 // ---------------------------------------------------------------- perplexity
 // Sec. 3.2: bisection on beta_i (start 1; double or halve until bracketed,
 // then halve the bracket) until |H_i - ln u| < 1e-5 or 200 steps, with the
-// exponents shifted by the row's smallest distance.
+// exponents shifted by the row's smallest distance.  VPL values per lane (k <=
+// 32 VPL; a fixed eight cost 2.8 ms at n = 1M, k = 90).
+template <int VPL>
 __global__ void __launch_bounds__(256)
     k_perplexity(int64_t n, int k, float target, const float *__restrict__ d2,
                  float *__restrict__ pcond, float *__restrict__ beta_out, DevScalars *sc) {
-    constexpr int VPL = 8;  // values per lane, k <= 256
     const int64_t row = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (row >= n) return;
@@ -1925,8 +1948,14 @@ __global__ void __launch_bounds__(256)
 
 cudaError_t launch_perplexity(pxsne_ctx *c, const float *d2, int64_t n, int32_t k,
                               float perplexity, float *pcond, float *beta) {
-    k_perplexity<<<(unsigned)((n * 32 + 255) / 256), 256, 0, c->stream>>>(
-        n, k, logf(perplexity), d2, pcond, beta, c->sc);
+    const unsigned blocks = (unsigned)((n * 32 + 255) / 256);
+    const float target = logf(perplexity);
+    auto kernel = k <= 32   ? k_perplexity<1>
+                  : k <= 64 ? k_perplexity<2>
+                  : k <= 96 ? k_perplexity<3>
+                  : k <= 128 ? k_perplexity<4>
+                             : k_perplexity<8>;
+    kernel<<<blocks, 256, 0, c->stream>>>(n, k, target, d2, pcond, beta, c->sc);
     return cudaGetLastError();
 }
 
