@@ -1481,14 +1481,14 @@ struct KnnSide {
     uint8_t *block = nullptr;
 };
 
-static cudaError_t make_side(int64_t n, int ld, int Dp, float scale, float eps_abs,
+static cudaError_t make_side(const pxsne_ctx *c, int64_t n, int ld, int Dp, float scale, float eps_abs,
                              const float *X, KnnSide &s, cudaStream_t st) {
     const int64_t T = (n + kTcCols - 1) / kTcCols;
     auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
     const size_t b_img = up((size_t)T * kTcRows * Dp * 2), b_hg = up((size_t)T * kHG * 4),
                  b_n = up((size_t)n * 4), b_c = up((size_t)T * Dp * 4), b_r = up((size_t)T * 4);
     cudaError_t e;
-    if ((e = cudaMallocAsync(&s.block, b_img + b_hg + 2 * b_n + b_c + b_r, st))) return e;
+    if ((e = palloc(c, &s.block, b_img + b_hg + 2 * b_n + b_c + b_r, st))) return e;
     uint8_t *img = s.block;
     float *HG = reinterpret_cast<float *>(img + b_img);
     float *n16 = reinterpret_cast<float *>(img + b_img + b_hg);
@@ -1522,7 +1522,7 @@ cudaError_t launch_knn(pxsne_ctx *c, const float *Xdev, int64_t n, int32_t D, in
     cudaStream_t st = c->stream;
     cudaError_t e;
     float *nrm = nullptr;
-    if ((e = cudaMallocAsync(&nrm, n * sizeof(float), st))) return e;
+    if ((e = palloc(c, &nrm, n * sizeof(float), st))) return e;
     k_row_norms<<<(unsigned)((n * 32 + 255) / 256), 256, 0, st>>>(n, D, Xdev, nrm);
     if ((e = cudaGetLastError())) return e;
     const int Dp = (D + 63) / 64 * 64;
@@ -1537,7 +1537,7 @@ cudaError_t launch_knn(pxsne_ctx *c, const float *Xdev, int64_t n, int32_t D, in
         unsigned *amax = nullptr;
         unsigned *err = &c->sc->err;
         if ((e = cudaMemsetAsync(&c->sc->knn_exact, 0, 3 * sizeof(u64), st))) return e;
-        if ((e = cudaMallocAsync(&amax, sizeof(unsigned), st))) return e;
+        if ((e = palloc(c, &amax, sizeof(unsigned), st))) return e;
         if ((e = cudaMemsetAsync(amax, 0, sizeof(unsigned), st))) return e;
         k_absmax<<<1184, 256, 0, st>>>(n * D, Xdev, amax);
         unsigned hmax = 0;
@@ -1569,8 +1569,8 @@ cudaError_t launch_knn(pxsne_ctx *c, const float *Xdev, int64_t n, int32_t D, in
             // (a host loop over the m^2 D / 2 terms of the chain took 28 ms)
             float *dp = nullptr;
             double *dd = nullptr;
-            if ((e = cudaMallocAsync(&dp, (size_t)m * D * sizeof(float), st))) return e;
-            if ((e = cudaMallocAsync(&dd, (size_t)m * m * sizeof(double), st))) return e;
+            if ((e = palloc(c, &dp, (size_t)m * D * sizeof(float), st))) return e;
+            if ((e = palloc(c, &dd, (size_t)m * m * sizeof(double), st))) return e;
             k_pivot_rows<<<(unsigned)(((int64_t)m * D + 255) / 256), 256, 0, st>>>(n, m, D, Xdev,
                                                                                   dp);
             k_pivot_d2<<<(unsigned)(((int64_t)m * m + 255) / 256), 256, 0, st>>>(m, D, dp, dd);
@@ -1615,15 +1615,15 @@ cudaError_t launch_knn(pxsne_ctx *c, const float *Xdev, int64_t n, int32_t D, in
         float *piv = nullptr, *Xs = nullptr;
         const int ld = (D + 3) & ~3;  // floats per ordered row
         uint32_t *cell = nullptr, *order = nullptr, *ccnt = nullptr;
-        if ((e = cudaMallocAsync(&piv, (size_t)m * (D + 1) * sizeof(float), st))) return e;
-        if ((e = cudaMallocAsync(&cell, (size_t)n * sizeof(uint32_t), st))) return e;
-        if ((e = cudaMallocAsync(&order, (size_t)n * sizeof(uint32_t), st))) return e;
-        if ((e = cudaMallocAsync(&ccnt, (size_t)(m + 1) * sizeof(uint32_t), st))) return e;
+        if ((e = palloc(c, &piv, (size_t)m * (D + 1) * sizeof(float), st))) return e;
+        if ((e = palloc(c, &cell, (size_t)n * sizeof(uint32_t), st))) return e;
+        if ((e = palloc(c, &order, (size_t)n * sizeof(uint32_t), st))) return e;
+        if ((e = palloc(c, &ccnt, (size_t)(m + 1) * sizeof(uint32_t), st))) return e;
         float *dpiv = nullptr;
         double *dsum = nullptr;
-        if ((e = cudaMallocAsync(&dpiv, (size_t)n * sizeof(float), st))) return e;
-        if ((e = cudaMallocAsync(&dsum, sizeof(double), st))) return e;
-        if ((e = cudaMallocAsync(&Xs, (size_t)n * ld * sizeof(float), st))) return e;
+        if ((e = palloc(c, &dpiv, (size_t)n * sizeof(float), st))) return e;
+        if ((e = palloc(c, &dsum, sizeof(double), st))) return e;
+        if ((e = palloc(c, &Xs, (size_t)n * ld * sizeof(float), st))) return e;
         float *pn = piv + (size_t)m * D;
         if ((e = cudaMemcpyAsync(piv, hq.data(), (size_t)m * D * sizeof(float),
                                  cudaMemcpyHostToDevice, st)))
@@ -1676,11 +1676,11 @@ cudaError_t launch_knn(pxsne_ctx *c, const float *Xdev, int64_t n, int32_t D, in
             const int64_t nb = (n + kCsRows - 1) / kCsRows;
             uint32_t *hist = nullptr;
             int64_t *off = nullptr;
-            if ((e = cudaMallocAsync(&hist, (size_t)(nc * nb) * sizeof(uint32_t), st))) return e;
-            if ((e = cudaMallocAsync(&off, (size_t)(nc * nb + 1) * sizeof(int64_t), st))) return e;
+            if ((e = palloc(c, &hist, (size_t)(nc * nb) * sizeof(uint32_t), st))) return e;
+            if ((e = palloc(c, &off, (size_t)(nc * nb + 1) * sizeof(int64_t), st))) return e;
             k_cell_rank<<<(unsigned)nb, kCsRows, 0, st>>>(n, nc, cell, hist, nb, nullptr, nullptr);
             if ((e = cudaGetLastError())) return e;
-            if ((e = scan_u32_to_i64(hist, (int64_t)nc * nb, off, st))) return e;
+            if ((e = scan_u32_to_i64(c, hist, (int64_t)nc * nb, off, st))) return e;
             k_cell_rank<<<(unsigned)nb, kCsRows, 0, st>>>(n, nc, cell, hist, nb, off, order);
             if ((e = cudaGetLastError())) return e;
             cudaFreeAsync(hist, st);
@@ -1701,12 +1701,12 @@ cudaError_t launch_knn(pxsne_ctx *c, const float *Xdev, int64_t n, int32_t D, in
             uint32_t *cst = nullptr, *order2 = nullptr, *flag = nullptr;
             int2 *seg = nullptr, *seg2 = nullptr;
             int64_t *pref = nullptr;
-            if ((e = cudaMallocAsync(&cst, (size_t)(m + 2) * sizeof(uint32_t), st))) return e;
-            if ((e = cudaMallocAsync(&order2, (size_t)n * sizeof(uint32_t), st))) return e;
-            if ((e = cudaMallocAsync(&flag, (size_t)n * sizeof(uint32_t), st))) return e;
-            if ((e = cudaMallocAsync(&seg, (size_t)n * sizeof(int2), st))) return e;
-            if ((e = cudaMallocAsync(&seg2, (size_t)n * sizeof(int2), st))) return e;
-            if ((e = cudaMallocAsync(&pref, (size_t)(n + 1) * sizeof(int64_t), st))) return e;
+            if ((e = palloc(c, &cst, (size_t)(m + 2) * sizeof(uint32_t), st))) return e;
+            if ((e = palloc(c, &order2, (size_t)n * sizeof(uint32_t), st))) return e;
+            if ((e = palloc(c, &flag, (size_t)n * sizeof(uint32_t), st))) return e;
+            if ((e = palloc(c, &seg, (size_t)n * sizeof(int2), st))) return e;
+            if ((e = palloc(c, &seg2, (size_t)n * sizeof(int2), st))) return e;
+            if ((e = palloc(c, &pref, (size_t)(n + 1) * sizeof(int64_t), st))) return e;
             std::vector<uint32_t> hs((size_t)m + 2);
             for (int q = 0; q <= m; q++) hs[(size_t)q] = hc[(size_t)q];
             hs[(size_t)m + 1] = (uint32_t)n;
@@ -1717,7 +1717,7 @@ cudaError_t launch_knn(pxsne_ctx *c, const float *Xdev, int64_t n, int32_t D, in
             for (int lv = 0; lv < levels; lv++) {
                 k_rp_side<<<ablocks, 256, 0, st>>>(n, D, Xdev, order, seg, lv, flag);
                 if ((e = cudaGetLastError())) return e;
-                if ((e = scan_u32_to_i64(flag, n, pref, st))) return e;
+                if ((e = scan_u32_to_i64(c, flag, n, pref, st))) return e;
                 k_rp_scatter<<<ablocks, 256, 0, st>>>(n, order, seg, flag, pref, order2, seg2);
                 if ((e = cudaGetLastError())) return e;
                 std::swap(order, order2);
@@ -1734,7 +1734,7 @@ cudaError_t launch_knn(pxsne_ctx *c, const float *Xdev, int64_t n, int32_t D, in
         if ((e = cudaGetLastError())) return e;
         // the search runs on the ordered rows
         KnnSide main_side, samp_side;
-        if ((e = make_side(n, ld, Dp, scale, eps_abs, Xs, main_side, st))) return e;
+        if ((e = make_side(c, n, ld, Dp, scale, eps_abs, Xs, main_side, st))) return e;
         const int64_t T = main_side.r.T;
         c->knn_tiles = T;
         if ((e = cudaFuncSetAttribute(k_knn_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1769,7 +1769,7 @@ cudaError_t launch_knn(pxsne_ctx *c, const float *Xdev, int64_t n, int32_t D, in
         int32_t *cand = nullptr;
         if (probe > 0) {
             const int W = (int)std::min<int64_t>(probe, T);
-            if ((e = cudaMallocAsync(&cand, (size_t)T * W * sizeof(int32_t), st))) return e;
+            if ((e = palloc(c, &cand, (size_t)T * W * sizeof(int32_t), st))) return e;
             k_tile_cands<<<(unsigned)T, kCandThreads, 0, st>>>(T, Dp, ka.cent, W, cand);
             if ((e = cudaGetLastError())) return e;
             ka.cand = cand;
@@ -1780,14 +1780,14 @@ cudaError_t launch_knn(pxsne_ctx *c, const float *Xdev, int64_t n, int32_t D, in
         uint32_t one_pass = (uint32_t)T;  // query tiles of the one-pass search
         if (probe == 0 && knn_scan_takes(n, k, Dp, smem_max)) {
             const int64_t ms = scan_sample_rows(n);
-            if ((e = cudaMallocAsync(&Xsamp, (size_t)ms * ld * sizeof(float), st))) return e;
+            if ((e = palloc(c, &Xsamp, (size_t)ms * ld * sizeof(float), st))) return e;
             k_sample_rows<<<(unsigned)((ms * ld + 255) / 256), 256, 0, st>>>(ms, ld, Xs, Xsamp);
             if ((e = cudaGetLastError())) return e;
-            if ((e = make_side(ms, ld, Dp, scale, 0.f, Xsamp, samp_side, st))) return e;
-            if ((e = cudaMallocAsync(&failed, (size_t)(T + 1) * sizeof(uint32_t), st))) return e;
+            if ((e = make_side(c, ms, ld, Dp, scale, 0.f, Xsamp, samp_side, st))) return e;
+            if ((e = palloc(c, &failed, (size_t)(T + 1) * sizeof(uint32_t), st))) return e;
             const KnnScan sa{main_side.r, samp_side.r, ld,  Dp, k,   inv_s2, kappa,
                              eps_abs,     order,       idx, d2, err, ka.stats};
-            if ((e = launch_knn_scan(sa, c->sms, failed, failed + T, st))) return e;
+            if ((e = launch_knn_scan(c, sa, c->sms, failed, failed + T, st))) return e;
             if ((e = cudaMemcpyAsync(&one_pass, failed + T, sizeof(uint32_t), cudaMemcpyDeviceToHost,
                                      st)))
                 return e;
@@ -1804,9 +1804,9 @@ cudaError_t launch_knn(pxsne_ctx *c, const float *Xdev, int64_t n, int32_t D, in
             uint32_t *rank = nullptr;
             int32_t *idx2 = nullptr;
             float *d22 = nullptr;
-            if ((e = cudaMallocAsync(&rank, (size_t)n * sizeof(uint32_t), st))) return e;
-            if ((e = cudaMallocAsync(&idx2, (size_t)n * k * sizeof(int32_t), st))) return e;
-            if ((e = cudaMallocAsync(&d22, (size_t)n * k * sizeof(float), st))) return e;
+            if ((e = palloc(c, &rank, (size_t)n * sizeof(uint32_t), st))) return e;
+            if ((e = palloc(c, &idx2, (size_t)n * k * sizeof(int32_t), st))) return e;
+            if ((e = palloc(c, &d22, (size_t)n * k * sizeof(float), st))) return e;
             k_rank_of<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, order, rank);
             const int R = c->p.knn_explore;
             const int ke = std::min(k, kExploreNbrs);
@@ -2022,11 +2022,12 @@ __global__ void k_scan_add(int64_t m, int64_t *out, const int64_t *__restrict__ 
 }
 
 // out[0..m] = exclusive scan of in[0..m) with out[m] = total (int64).
-cudaError_t scan_u32_to_i64(const uint32_t *in, int64_t m, int64_t *out, cudaStream_t st) {
+cudaError_t scan_u32_to_i64(const pxsne_ctx *c, const uint32_t *in, int64_t m, int64_t *out,
+                            cudaStream_t st) {
     const int64_t nb = (m + kScanB - 1) / kScanB;
     int64_t *bsum = nullptr;
     cudaError_t e;
-    if ((e = cudaMallocAsync(&bsum, (nb + 1) * sizeof(int64_t), st))) return e;
+    if ((e = palloc(c, &bsum, (nb + 1) * sizeof(int64_t), st))) return e;
     k_scan_blocks<<<(unsigned)(nb > 0 ? nb : 1), kScanB, 0, st>>>(m, in, out, bsum);
     k_scan_bsum<<<1, kScanB, 0, st>>>(nb, bsum, bsum + nb);
     k_scan_add<<<(unsigned)((m + 1 + 255) / 256), 256, 0, st>>>(m, out, bsum, bsum + nb);
@@ -2229,19 +2230,19 @@ cudaError_t build_symmetric_csr(pxsne_ctx *c, const int32_t *idx, const float *p
             return e;          \
         }                      \
     } while (0)
-    TRY(cudaMallocAsync(&deg, n * sizeof(uint32_t), st));
-    TRY(cudaMallocAsync(&cursor, n * sizeof(uint32_t), st));
-    TRY(cudaMallocAsync(&tptr, (n + 1) * sizeof(int64_t), st));
+    TRY(palloc(c, &deg, n * sizeof(uint32_t), st));
+    TRY(palloc(c, &cursor, n * sizeof(uint32_t), st));
+    TRY(palloc(c, &tptr, (n + 1) * sizeof(int64_t), st));
     TRY(cudaMemsetAsync(deg, 0, n * sizeof(uint32_t), st));
-    TRY(cudaMallocAsync(&slot, nk * sizeof(uint32_t), st));
+    TRY(palloc(c, &slot, nk * sizeof(uint32_t), st));
     k_indeg<<<(unsigned)((nk + 255) / 256), 256, 0, st>>>(nk, idx, deg, slot);
     TRY(cudaGetLastError());
     // temporary rows of length k + indeg(i); 2 n k entries in total
     uint32_t *len = cursor;
     k_add_const<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, deg, len, (uint32_t)k);
     TRY(cudaGetLastError());
-    TRY(scan_u32_to_i64(len, n, tptr, st));
-    TRY(cudaMallocAsync(&T, 2 * nk * sizeof(u64), st));
+    TRY(scan_u32_to_i64(c, len, n, tptr, st));
+    TRY(palloc(c, &T, 2 * nk * sizeof(u64), st));
     k_fill<<<(unsigned)((nk + 255) / 256), 256, 0, st>>>(n, k, idx, pcond, tptr, slot, T);
     TRY(cudaGetLastError());
     uint32_t *ucnt = deg;  // reuse
@@ -2251,7 +2252,7 @@ cudaError_t build_symmetric_csr(pxsne_ctx *c, const int32_t *idx, const float *p
     {
         // the longer rows
         uint32_t *lists = nullptr;  // three lists and the hubs' padded lengths, then their counts
-        TRY(cudaMallocAsync(&lists, ((size_t)n * 4 + 4) * sizeof(uint32_t), st));
+        TRY(palloc(c, &lists, ((size_t)n * 4 + 4) * sizeof(uint32_t), st));
         uint32_t *num = lists + (size_t)n * 4, *hubs = lists + 2 * (size_t)n, *plen = lists + 3 * (size_t)n;
         TRY(cudaMemsetAsync(num, 0, 4 * sizeof(uint32_t), st));
         k_long_rows<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, tptr, lists, lists + n, hubs, num,
@@ -2284,8 +2285,8 @@ cudaError_t build_symmetric_csr(pxsne_ctx *c, const int32_t *idx, const float *p
             }
             int64_t *soff = nullptr;
             u64 *scr = nullptr;
-            TRY(cudaMallocAsync(&soff, hl * sizeof(int64_t), st));
-            TRY(cudaMallocAsync(&scr, (size_t)std::max<int64_t>(tot, 1) * sizeof(u64), st));
+            TRY(palloc(c, &soff, hl * sizeof(int64_t), st));
+            TRY(palloc(c, &scr, (size_t)std::max<int64_t>(tot, 1) * sizeof(u64), st));
             TRY(cudaMemcpyAsync(soff, ho.data(), hl * sizeof(int64_t), cudaMemcpyHostToDevice, st));
             TRY(cudaFuncSetAttribute(k_sort_long, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      kSmemKeys * (int)sizeof(u64)));
@@ -2302,22 +2303,22 @@ cudaError_t build_symmetric_csr(pxsne_ctx *c, const int32_t *idx, const float *p
     if (c->val) { cudaFreeAsync(c->val, st); c->val = nullptr; }
     if (c->rowlen) { cudaFreeAsync(c->rowlen, st); c->rowlen = nullptr; }
     // true row lengths and nnz
-    TRY(cudaMallocAsync(&c->rowlen, n * sizeof(int32_t), st));
+    TRY(palloc(c, &c->rowlen, n * sizeof(int32_t), st));
     TRY(cudaMemcpyAsync(c->rowlen, ucnt, n * sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
     int64_t *uscan = nullptr;
-    TRY(cudaMallocAsync(&uscan, (n + 1) * sizeof(int64_t), st));
-    TRY(scan_u32_to_i64(ucnt, n, uscan, st));
+    TRY(palloc(c, &uscan, (n + 1) * sizeof(int64_t), st));
+    TRY(scan_u32_to_i64(c, ucnt, n, uscan, st));
     int64_t nnz = 0, nnz_pad = 0;
     TRY(cudaMemcpyAsync(&nnz, uscan + n, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     // padded offsets
     k_round4<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, ucnt, cursor);
     TRY(cudaGetLastError());
-    TRY(cudaMallocAsync(&c->rp, (n + 1) * sizeof(int64_t), st));
-    TRY(scan_u32_to_i64(cursor, n, c->rp, st));
+    TRY(palloc(c, &c->rp, (n + 1) * sizeof(int64_t), st));
+    TRY(scan_u32_to_i64(c, cursor, n, c->rp, st));
     TRY(cudaMemcpyAsync(&nnz_pad, c->rp + n, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     TRY(cudaStreamSynchronize(st));
-    TRY(cudaMallocAsync(&c->col, (nnz_pad > 0 ? nnz_pad : 4) * sizeof(int32_t), st));
-    TRY(cudaMallocAsync(&c->val, (nnz_pad > 0 ? nnz_pad : 4) * sizeof(float), st));
+    TRY(palloc(c, &c->col, (nnz_pad > 0 ? nnz_pad : 4) * sizeof(int32_t), st));
+    TRY(palloc(c, &c->val, (nnz_pad > 0 ? nnz_pad : 4) * sizeof(float), st));
     k_sym_write<<<(unsigned)((n * 32 + 255) / 256), 256, 0, st>>>(n, tptr, T, ucnt, c->rp, c->col,
                                                                  c->val);
     TRY(cudaGetLastError());

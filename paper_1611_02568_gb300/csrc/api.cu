@@ -80,6 +80,36 @@ void free_state(pxsne_ctx *c) {
     c->state_ready = false;
 }
 
+// P and the neighbour lists (pool memory, in stream order).
+void free_P(pxsne_ctx *c) {
+    auto drop = [&](auto *&p) {
+        if (p) cudaFreeAsync(p, c->stream);
+        p = nullptr;
+    };
+    drop(c->rp); drop(c->col); drop(c->val); drop(c->rowlen);
+    drop(c->knn_idx); drop(c->knn_d2); drop(c->beta);
+}
+
+// Gives back what the pool holds unused beyond kPoolKeep.
+void trim_pool(pxsne_ctx *c) {
+    if (c->pool) cudaMemPoolTrimTo(c->pool, kPoolKeep);
+}
+
+// The context's own pool; without one (not supported) the default pool serves.
+void make_pool(pxsne_ctx *c) {
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = c->device;
+    if (cudaMemPoolCreate(&c->pool, &props) != cudaSuccess) {
+        cudaGetLastError();
+        c->pool = nullptr;
+        return;
+    }
+    uint64_t keep = ~0ull;
+    cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold, &keep);
+}
+
 int check_params(const pxsne_params *p) {
     if (!p) return fail(nullptr, PXSNE_E_ARG, "params is NULL");
     if (p->log2_r < 1 || p->log2_r > kMaxL)
@@ -276,6 +306,7 @@ const char *kGroupNames[KG_COUNT] = {"k_relabel", "k_update", "k_snap_hist", "k_
 
 int check_device(pxsne_ctx *c, uint32_t *flags_out) {
     CK(c, cudaStreamSynchronize(c->stream));
+    trim_pool(c);
     unsigned err = 0;
     CK(c, cudaMemcpy(&err, &c->sc->err, sizeof(unsigned), cudaMemcpyDeviceToHost));
     if (flags_out) *flags_out = err;
@@ -352,6 +383,7 @@ int pxsne_create(pxsne_ctx **out, const pxsne_params *p, void *stream) {
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming);
     }
+    if (e == cudaSuccess) make_pool(c);
     if (e == cudaSuccess) e = dalloc(c, &c->sc, 1);
     if (e == cudaSuccess) e = cudaMemset(c->sc, 0, sizeof(DevScalars));
     if (e != cudaSuccess) {
@@ -359,6 +391,7 @@ int pxsne_create(pxsne_ctx **out, const pxsne_params *p, void *stream) {
         fail(nullptr, e == cudaErrorMemoryAllocation ? PXSNE_E_OOM : PXSNE_E_CUDA,
              "pxsne_create: %s", cudaGetErrorString(e));
         if (c->sc) cudaFree(c->sc);
+        if (c->pool) cudaMemPoolDestroy(c->pool);
         if (c->ev_join) cudaEventDestroy(c->ev_join);
         if (c->ev_fork) cudaEventDestroy(c->ev_fork);
         if (c->side) cudaStreamDestroy(c->side);
@@ -374,9 +407,10 @@ void pxsne_destroy(pxsne_ctx *c) {
     if (!c) return;
     cudaStreamSynchronize(c->stream);
     free_state(c);
-    dfree(c->rp); dfree(c->col); dfree(c->val); dfree(c->rowlen);
-    dfree(c->knn_idx); dfree(c->knn_d2); dfree(c->beta);
+    free_P(c);
     dfree(c->sc);
+    cudaStreamSynchronize(c->stream);
+    if (c->pool) cudaMemPoolDestroy(c->pool);
     for (auto &ev : c->knn_ev)
         if (ev) cudaEventDestroy(ev);
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
@@ -404,7 +438,7 @@ int pxsne_affinities(pxsne_ctx *c, const float *X, int64_t n, int32_t D, float p
     float *Xd = nullptr;
     const float *Xuse = X;
     if (!x_on_device) {
-        CK(c, cudaMallocAsync(&Xd, (size_t)n * D * sizeof(float), st));
+        CK(c, palloc(c, &Xd, (size_t)n * D * sizeof(float), st));
         CK(c, cudaMemcpyAsync(Xd, X, (size_t)n * D * sizeof(float), cudaMemcpyHostToDevice, st));
         Xuse = Xd;
     }
@@ -413,7 +447,7 @@ int pxsne_affinities(pxsne_ctx *c, const float *X, int64_t n, int32_t D, float p
         // state is replaced (a host loop over the n D values cost more than
         // the copy)
         unsigned *flag = nullptr, bad = 0u;
-        CK(c, cudaMallocAsync(&flag, sizeof(unsigned), st));
+        CK(c, palloc(c, &flag, sizeof(unsigned), st));
         CK(c, cudaMemsetAsync(flag, 0, sizeof(unsigned), st));
         CK(c, launch_nonfinite(c, Xuse, n * D, flag, st));
         CK(c, cudaMemcpyAsync(&bad, flag, sizeof(unsigned), cudaMemcpyDeviceToHost, st));
@@ -425,19 +459,18 @@ int pxsne_affinities(pxsne_ctx *c, const float *X, int64_t n, int32_t D, float p
         }
     }
     free_state(c);
-    dfree(c->rp); dfree(c->col); dfree(c->val); dfree(c->rowlen);
-    dfree(c->knn_idx); dfree(c->knn_d2); dfree(c->beta);
+    free_P(c);
     c->n = n;
     c->D = D;
     c->nnz = 0;
-    CK(c, dalloc(c, &c->knn_idx, (size_t)n * k));
-    CK(c, dalloc(c, &c->knn_d2, (size_t)n * k));
-    CK(c, dalloc(c, &c->beta, (size_t)n));
+    CK(c, palloc(c, &c->knn_idx, (size_t)n * k * sizeof(int32_t), st));
+    CK(c, palloc(c, &c->knn_d2, (size_t)n * k * sizeof(float), st));
+    CK(c, palloc(c, &c->beta, (size_t)n * sizeof(float), st));
     c->knn_k = k;
     CK(c, launch_knn(c, Xuse, n, D, k, c->knn_idx, c->knn_d2));
     if (Xd) CK(c, cudaFreeAsync(Xd, st));
     float *pcond = nullptr;
-    CK(c, cudaMallocAsync(&pcond, (size_t)n * k * sizeof(float), st));
+    CK(c, palloc(c, &pcond, (size_t)n * k * sizeof(float), st));
     CK(c, launch_perplexity(c, c->knn_d2, n, k, perplexity, pcond, c->beta));
     std::string where;
     cudaError_t e = build_symmetric_csr(c, c->knn_idx, pcond, n, k, where);
@@ -485,16 +518,15 @@ int pxsne_set_P(pxsne_ctx *c, int64_t n, const int64_t *row_ptr, const int32_t *
         }
     }
     free_state(c);
-    dfree(c->rp); dfree(c->col); dfree(c->val); dfree(c->rowlen);
-    dfree(c->knn_idx); dfree(c->knn_d2); dfree(c->beta);
+    free_P(c);
     c->knn_k = 0;
     c->n = n;
     c->nnz = nnz;
     c->nnz_pad = nnz_pad;
-    CK(c, dalloc(c, &c->rp, n + 1));
-    CK(c, dalloc(c, &c->rowlen, n));
-    CK(c, dalloc(c, &c->col, pc.size()));
-    CK(c, dalloc(c, &c->val, pv.size()));
+    CK(c, palloc(c, &c->rp, (n + 1) * 8, c->stream));
+    CK(c, palloc(c, &c->rowlen, n * 4, c->stream));
+    CK(c, palloc(c, &c->col, pc.size() * 4, c->stream));
+    CK(c, palloc(c, &c->val, pv.size() * 4, c->stream));
     CK(c, cudaMemcpyAsync(c->rp, rp.data(), (n + 1) * 8, cudaMemcpyHostToDevice, c->stream));
     CK(c, cudaMemcpyAsync(c->rowlen, len.data(), n * 4, cudaMemcpyHostToDevice, c->stream));
     CK(c, cudaMemcpyAsync(c->col, pc.data(), pc.size() * 4, cudaMemcpyHostToDevice, c->stream));
@@ -514,10 +546,10 @@ int pxsne_init(pxsne_ctx *c, const float *Y0, int y_on_device, uint64_t seed) {
         if (!Y0) return fail(c, PXSNE_E_UNSUPPORTED, "dim 3: the start Y0 must be given");
         float *Yd3 = nullptr;
         double *scr = nullptr;
-        CK(c, cudaMallocAsync(&scr, 8 * sizeof(double), st));
+        CK(c, palloc(c, &scr, 8 * sizeof(double), st));
         const float *Y3 = Y0;
         if (!y_on_device) {
-            CK(c, cudaMallocAsync(&Yd3, (size_t)n * 12, st));
+            CK(c, palloc(c, &Yd3, (size_t)n * 12, st));
             CK(c, cudaMemcpyAsync(Yd3, Y0, (size_t)n * 12, cudaMemcpyHostToDevice, st));
             Y3 = Yd3;
         }
@@ -534,10 +566,10 @@ int pxsne_init(pxsne_ctx *c, const float *Y0, int y_on_device, uint64_t seed) {
     }
     float *Yd = nullptr;
     uint32_t *mm = nullptr;
-    CK(c, cudaMallocAsync(&mm, 4 * sizeof(uint32_t), st));
+    CK(c, palloc(c, &mm, 4 * sizeof(uint32_t), st));
     const float *Yuse = Y0;
     if (!Y0 || !y_on_device) {
-        CK(c, cudaMallocAsync(&Yd, (size_t)n * 2 * sizeof(float), st));
+        CK(c, palloc(c, &Yd, (size_t)n * 2 * sizeof(float), st));
         if (Y0) {
             CK(c, cudaMemcpyAsync(Yd, Y0, (size_t)n * 8, cudaMemcpyHostToDevice, st));
         } else {
@@ -714,7 +746,7 @@ int pxsne_kl(pxsne_ctx *c, double *out) {
     if (rc) return rc;
     if (!out) return fail(c, PXSNE_E_ARG, "out is NULL");
     double *d = nullptr;
-    CK(c, cudaMallocAsync(&d, sizeof(double), c->stream));
+    CK(c, palloc(c, &d, sizeof(double), c->stream));
     if (is3(c)) CK(c, launch_kl3(c, d));
     else CK(c, launch_kl(c, d));
     CK(c, cudaMemcpyAsync(out, d, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
@@ -731,14 +763,14 @@ int pxsne_get_Y(pxsne_ctx *c, float *Y, int32_t *pix, int on_device) {
     const int64_t n = c->n;
     const size_t row = is3(c) ? 12 : 8;  // bytes of one point's values
     float *scratch = nullptr;
-    CK(c, cudaMallocAsync(&scratch, 32, st));
+    CK(c, palloc(c, &scratch, 32, st));
     float *Yd = Y;
     int32_t *Pd = pix;
     if (!on_device) {
         Yd = nullptr;
         Pd = nullptr;
-        if (Y) CK(c, cudaMallocAsync(&Yd, (size_t)n * row, st));
-        if (pix) CK(c, cudaMallocAsync(&Pd, (size_t)n * row, st));
+        if (Y) CK(c, palloc(c, &Yd, (size_t)n * row, st));
+        if (pix) CK(c, palloc(c, &Pd, (size_t)n * row, st));
     }
     if (is3(c)) CK(c, launch_centre_y3(c, Yd, Pd, reinterpret_cast<double *>(scratch)));
     else CK(c, launch_centre_y(c, Yd, Pd, scratch));
@@ -777,12 +809,12 @@ int pxsne_nbr_precision(pxsne_ctx *c, int32_t k, const int32_t *knn_hd, int32_t 
     const int64_t n = c->n;
     int32_t *dh = nullptr, *dk = nullptr;
     unsigned long long *dt = nullptr;
-    CK(c, cudaMallocAsync(&dh, (size_t)n * 4, st));
-    CK(c, cudaMallocAsync(&dt, 8, st));
+    CK(c, palloc(c, &dh, (size_t)n * 4, st));
+    CK(c, palloc(c, &dt, 8, st));
     CK(c, cudaMemsetAsync(dt, 0, 8, st));
     const int32_t *kd = knn_hd;
     if (!on_device) {
-        CK(c, cudaMallocAsync(&dk, (size_t)n * kh * 4, st));
+        CK(c, palloc(c, &dk, (size_t)n * kh * 4, st));
         CK(c, cudaMemcpyAsync(dk, knn_hd, (size_t)n * kh * 4, cudaMemcpyHostToDevice, st));
         kd = dk;
     }
@@ -896,14 +928,14 @@ int pxsne_get_tree(pxsne_ctx *c, int32_t level, uint32_t *cnt, uint64_t *sx, uin
     const size_t cells = size_t(1) << (2 * level);
     if (cnt) {
         uint32_t *d = nullptr;
-        CK(c, cudaMallocAsync(&d, cells * 4, st));
+        CK(c, palloc(c, &d, cells * 4, st));
         CK(c, launch_level_counts(c, level, d));
         CK(c, cudaMemcpyAsync(cnt, d, cells * 4, cudaMemcpyDeviceToHost, st));
         CK(c, cudaFreeAsync(d, st));
     }
     if (level == c->L && (sx || sy)) {
         u64 *d = nullptr;
-        CK(c, cudaMallocAsync(&d, cells * 16, st));
+        CK(c, palloc(c, &d, cells * 16, st));
         CK(c, launch_leaf_hist(c, nullptr, d, d + cells));
         if (sx) CK(c, cudaMemcpyAsync(sx, d, cells * 8, cudaMemcpyDeviceToHost, st));
         if (sy) CK(c, cudaMemcpyAsync(sy, d + cells, cells * 8, cudaMemcpyDeviceToHost, st));
@@ -911,7 +943,7 @@ int pxsne_get_tree(pxsne_ctx *c, int32_t level, uint32_t *cnt, uint64_t *sx, uin
     }
     if (morton) {
         uint32_t *d = nullptr;
-        CK(c, cudaMallocAsync(&d, (size_t)c->n * 4, st));
+        CK(c, palloc(c, &d, (size_t)c->n * 4, st));
         CK(c, launch_morton_keys(c, d));
         CK(c, cudaMemcpyAsync(morton, d, (size_t)c->n * 4, cudaMemcpyDeviceToHost, st));
         CK(c, cudaFreeAsync(d, st));
@@ -1241,8 +1273,8 @@ int pxsne_get_tree3(pxsne_ctx *c, int32_t level, uint32_t *cnt, uint64_t *sx, ui
         // the leaves: rebuilt from z (the iteration clears its own once read)
         uint32_t *dc = nullptr;
         u64 *ds = nullptr;
-        CK(c, cudaMallocAsync(&dc, cells * 4, st));
-        CK(c, cudaMallocAsync(&ds, cells * 24, st));
+        CK(c, palloc(c, &dc, cells * 4, st));
+        CK(c, palloc(c, &ds, cells * 24, st));
         CK(c, launch_leaf_hist3(c, dc, ds));
         if (cnt) CK(c, cudaMemcpyAsync(cnt, dc, cells * 4, cudaMemcpyDeviceToHost, st));
         uint64_t *out[3] = {sx, sy, sz};
@@ -1255,7 +1287,7 @@ int pxsne_get_tree3(pxsne_ctx *c, int32_t level, uint32_t *cnt, uint64_t *sx, ui
     }
     if (morton) {
         uint32_t *d = nullptr;
-        CK(c, cudaMallocAsync(&d, (size_t)c->n * 4, st));
+        CK(c, palloc(c, &d, (size_t)c->n * 4, st));
         CK(c, launch_morton3(c, d));
         CK(c, cudaMemcpyAsync(morton, d, (size_t)c->n * 4, cudaMemcpyDeviceToHost, st));
         CK(c, cudaFreeAsync(d, st));

@@ -228,6 +228,7 @@ struct pxsne_ctx {
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     cudaStream_t side = nullptr;          // stream of the attraction (overlaps the traversal)
+    cudaMemPool_t pool = nullptr;         // P, its lists and every call's scratch (palloc)
     int stack_limit = 0;                  // host copy of DevScalars::stack_limit
     int sms = 0;                          // streaming multiprocessors of the device
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
@@ -318,6 +319,21 @@ struct pxsne_ctx {
 
 // Launchers implemented in the .cu files (all enqueue on ctx->stream).
 namespace pxsne {
+// Stream-ordered allocation from the context's own pool (freed by
+// cudaFreeAsync).  The device's default pool gives its memory back at every
+// synchronisation, and P construction synchronises a dozen times: mapping it
+// anew each time took 5 of the 9 ms of P at n = 70,000 that were not kernels.
+// The context's pool keeps what a call frees until the call ends, then at most
+// kPoolKeep bytes (trim_pool), and goes with the context.
+constexpr size_t kPoolKeep = size_t(1) << 30;
+template <class T>
+inline cudaError_t palloc(const pxsne_ctx *c, T **p, size_t bytes, cudaStream_t st) {
+    void *v = nullptr;
+    const cudaError_t e = c->pool ? cudaMallocFromPoolAsync(&v, bytes, c->pool, st)
+                                  : cudaMallocAsync(&v, bytes, st);
+    *p = static_cast<T *>(v);
+    return e;
+}
 cudaError_t launch_init_map(pxsne_ctx *c, const float *Y0dev, uint32_t *mm_scratch);
 // Kernel groups of one iteration, in launch order (timing marks).
 enum KernelGroup {
@@ -349,7 +365,8 @@ cudaError_t launch_accumulate_counters(pxsne_ctx *c);
 constexpr int kRelabelEvery = 100;
 cudaError_t launch_relabel(pxsne_ctx *c, cudaStream_t st);
 // out[0..m] = exclusive scan of in[0..m) with out[m] = the total
-cudaError_t scan_u32_to_i64(const uint32_t *in, int64_t m, int64_t *out, cudaStream_t st);
+cudaError_t scan_u32_to_i64(const pxsne_ctx *c, const uint32_t *in, int64_t m, int64_t *out,
+                            cudaStream_t st);
 cudaError_t launch_traverse_zsum(pxsne_ctx *c);
 cudaError_t launch_update(pxsne_ctx *c, cudaEvent_t *marks = nullptr);
 cudaError_t launch_kl(pxsne_ctx *c, double *out_dev);

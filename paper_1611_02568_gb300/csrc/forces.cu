@@ -811,7 +811,7 @@ cudaError_t launch_relabel(pxsne_ctx *c, cudaStream_t st) {
                                                      c->rl2, c->zp);
     cudaError_t e = cudaGetLastError();
     if (e) return e;
-    if ((e = scan_u32_to_i64(c->rl2, n, c->rp2, st))) return e;
+    if ((e = scan_u32_to_i64(c, c->rl2, n, c->rp2, st))) return e;
     const unsigned blocks = (unsigned)(((int64_t)n * 32 + 255) / 256);
     k_relabel_rows<<<blocks, 256, 0, st>>>(n, c->aperm, c->ainv, c->rp,
                                            reinterpret_cast<const int4 *>(c->col),

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+struct pxsne_ctx;
+
 namespace pxsne {
 
 constexpr int kTcRows = 128;     // query rows per CTA (MMA M)
@@ -51,7 +53,7 @@ bool knn_scan_takes(int64_t n, int k, int Dp, int smem_max);
 // Lists of every row into out_idx / out_d2 (by row of X), except for the query
 // tiles written to failed (room for q.T) and counted in *nfailed (device),
 // whose lists are left to the one-pass search.
-cudaError_t launch_knn_scan(const KnnScan &a, int sms, uint32_t *failed, uint32_t *nfailed,
-                            cudaStream_t st);
+cudaError_t launch_knn_scan(const pxsne_ctx *c, const KnnScan &a, int sms, uint32_t *failed,
+                            uint32_t *nfailed, cudaStream_t st);
 
 }  // namespace pxsne

@@ -628,18 +628,18 @@ bool knn_scan_takes(int64_t n, int k, int Dp, int smem_max) {
            scan_smem(0, Dp, r) <= (size_t)smem_max && pick_smem(Dp) <= (size_t)smem_max;
 }
 
-cudaError_t launch_knn_scan(const KnnScan &a, int sms, uint32_t *failed, uint32_t *nfailed,
+cudaError_t launch_knn_scan(const pxsne_ctx *c, const KnnScan &a, int sms, uint32_t *failed, uint32_t *nfailed,
                             cudaStream_t st) {
     const int64_t n = a.q.n, T = a.q.T;
     const int r = sample_rank(a.k), cap = half_cap(r);
     cudaError_t e;
     float *tau = nullptr;
     uint32_t *buf = nullptr, *cnt = nullptr, *flag = nullptr;
-    if ((e = cudaMallocAsync(&tau, (size_t)n * 4, st))) return e;
-    if ((e = cudaMallocAsync(&buf, (size_t)n * 2 * cap * 4, st))) return e;
-    if ((e = cudaMallocAsync(&cnt, (size_t)n * 2 * 4, st))) return e;
+    if ((e = palloc(c, &tau, (size_t)n * 4, st))) return e;
+    if ((e = palloc(c, &buf, (size_t)n * 2 * cap * 4, st))) return e;
+    if ((e = palloc(c, &cnt, (size_t)n * 2 * 4, st))) return e;
     // flags and the retry list of the tiles, and its length
-    if ((e = cudaMallocAsync(&flag, (size_t)(2 * T + 1) * 4, st))) return e;
+    if ((e = palloc(c, &flag, (size_t)(2 * T + 1) * 4, st))) return e;
     uint32_t *retry = flag + T, *nretry = flag + 2 * T;
     if ((e = cudaMemsetAsync(flag, 0, (size_t)(2 * T + 1) * 4, st))) return e;
     if ((e = cudaMemsetAsync(nfailed, 0, 4, st))) return e;
