@@ -321,10 +321,10 @@ struct pxsne_ctx {
 namespace pxsne {
 // Stream-ordered allocation from the context's own pool (freed by
 // cudaFreeAsync).  The device's default pool gives its memory back at every
-// synchronisation, and P construction synchronises a dozen times: mapping it
-// anew each time took 5 of the 9 ms of P at n = 70,000 that were not kernels.
-// The context's pool keeps what a call frees until the call ends, then at most
-// kPoolKeep bytes (trim_pool), and goes with the context.
+// synchronisation, and P construction synchronises a dozen times, mapping it
+// anew after each.  The context's pool keeps what a call frees until the call
+// ends, then at most kPoolKeep bytes (trim_pool), and goes with the context: P
+// at n = 70,000 went from 6.4 to 5.7 ms, at 1M (8 GB of scratch) from 158 to 148.
 constexpr size_t kPoolKeep = size_t(1) << 30;
 template <class T>
 inline cudaError_t palloc(const pxsne_ctx *c, T **p, size_t bytes, cudaStream_t st) {

@@ -37,9 +37,11 @@ namespace {
 
 constexpr int kStages = 2;        // candidate-tile stages in shared memory
 constexpr int kAcc = 2;           // TMEM accumulators of 128 columns
-constexpr int kFilterWarps = 8;   // two per TMEM lane quarter, 64 columns each
-constexpr int kThreads = 32 * (kFilterWarps + 2);
-constexpr int kLoadWarp = kFilterWarps, kMmaWarp = kFilterWarps + 1;
+// Filter warps: one per TMEM lane quarter in the sample pass (MODE 0), so that a
+// row has one list, and two, of 64 columns each, in the other; then the loader's
+// and the MMA issuer's warp.
+constexpr int filter_warps(int mode) { return mode == 0 ? 4 : 8; }
+constexpr int scan_threads(int mode) { return 32 * (filter_warps(mode) + 2); }
 
 struct ScanArgs {
     KnnRows q, c;           // query rows; candidate rows (the sample or the rows themselves)
@@ -61,13 +63,26 @@ __device__ __forceinline__ int64_t tile_at(int64_t own, int64_t i, int64_t T) {
 }
 
 // Shared memory: A tile, kStages candidate tiles, kAcc x kHG floats, then for
-// the sample pass the lists (128 rows x 2 halves x rs floats, rs odd) and per
-// filter warp 32 x 32 staged values.
+// the sample pass the lists (128 rows x rs floats, rs odd).  At k = 90 two CTAs
+// fit on an SM in both passes.
 __host__ __device__ inline size_t scan_smem(int mode, int Dp, int r) {
     size_t b = (size_t)(1 + kStages) * kTcRows * Dp * 2 + (size_t)kAcc * kHG * 4 + 1024;
-    if (mode == 0)
-        b += (size_t)2 * kTcRows * (r | 1) * 4 + (size_t)kFilterWarps * 32 * 32 * 4;
+    if (mode == 0) b += (size_t)kTcRows * (r | 1) * 4;
     return b;
+}
+
+// v[j] of 32 registers by a tree of selections.
+__device__ __forceinline__ float pick32(const uint32_t (&v)[32], int j) {
+    uint32_t t[16];
+#pragma unroll
+    for (int q = 0; q < 16; q++) t[q] = (j & 1) ? v[2 * q + 1] : v[2 * q];
+#pragma unroll
+    for (int q = 0; q < 8; q++) t[q] = (j & 2) ? t[2 * q + 1] : t[2 * q];
+#pragma unroll
+    for (int q = 0; q < 4; q++) t[q] = (j & 4) ? t[2 * q + 1] : t[2 * q];
+#pragma unroll
+    for (int q = 0; q < 2; q++) t[q] = (j & 8) ? t[2 * q + 1] : t[2 * q];
+    return __uint_as_float((j & 16) ? t[1] : t[0]);
 }
 
 // MODE 0: the sample pass; MODE 1: the candidates.  One CTA per 128 query rows,
@@ -78,7 +93,10 @@ __host__ __device__ inline size_t scan_smem(int mode, int Dp, int r) {
 // and add and one funnel shift that collects the sign bits of e_j - t, e_j =
 // (1-eps)|c~_j|^2 - 2 q~.c~_j, with the chunk's largest kappa |q~||c~| in t.
 template <int MODE>
-__global__ void __launch_bounds__(kThreads, 2) k_knn_scan(const ScanArgs a) {
+__global__ void __launch_bounds__(scan_threads(MODE), 2) k_knn_scan(const ScanArgs a) {
+    constexpr int kFilterWarps = filter_warps(MODE), kThreads = scan_threads(MODE);
+    constexpr int kLoadWarp = kFilterWarps, kMmaWarp = kFilterWarps + 1;
+    constexpr int kChunks = 16 / kFilterWarps;  // 32-column chunks of a tile per warp
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t bar_a, bar_sf[kStages], bar_se[kStages], bar_tf[kAcc], bar_te[kAcc],
         bar_hf[kAcc], bar_he[kAcc];
@@ -95,14 +113,13 @@ __global__ void __launch_bounds__(kThreads, 2) k_knn_scan(const ScanArgs a) {
     float *hbuf = reinterpret_cast<float *>(sB + (size_t)kStages * tile_bytes);
     const int rs = a.r | 1;
     float *lists = hbuf + kAcc * kHG;
-    float *stage = lists + 2 * kTcRows * rs;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (MODE == 1 && a.qlist && blockIdx.x >= *a.qcount) return;
     const int64_t qt = MODE == 1 && a.qlist ? a.qlist[blockIdx.x] : blockIdx.x, q0 = qt * kTcRows;
     const int64_t own = MODE == 0 ? min(T - 1, qt / kScanStride) : qt;
 
     if (MODE == 0)
-        for (int e = tid; e < 2 * kTcRows * rs; e += kThreads) lists[e] = INFINITY;
+        for (int e = tid; e < kTcRows * rs; e += kThreads) lists[e] = INFINITY;
     if (warp == kMmaWarp) tc::tmem_alloc(&tslot, kAcc * kTcCols);
     if (tid == 0) {
         tc::mbar_init(&bar_a, 1);
@@ -162,10 +179,9 @@ __global__ void __launch_bounds__(kThreads, 2) k_knn_scan(const ScanArgs a) {
                 }
             }
             if (MODE == 0) {
-                // a row's threshold is at most either half-list's root
                 taum = 0.f;
 #pragma unroll
-                for (int w = 0; w < 4; w++) taum = fmaxf(taum, fminf(s_taumax[w], s_taumax[w + 4]));
+                for (int w = 0; w < kFilterWarps; w++) taum = fmaxf(taum, s_taumax[w]);
             }
             const float lbd = sqrtf(dd) * 0.9999f - rq - (in ? a.c.rad[tl] : 0.f);
             const bool skip = in && il > 0 && lbd > 0.f && lbd * lbd > taum * 1.0001f;
@@ -280,8 +296,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_knn_scan(const ScanArgs a) {
                 tc::mbar_wait(&bar_tf[j % kAcc], (uint32_t)((j / kAcc) & 1), kTcPolls);
         }
     } else {
-        // ---- filter: warps quarter and quarter + 4 own query rows q0 + 32
-        // quarter + lane; warp `half` takes columns 64 half .. +63
+        // ---- filter: warp `quarter` (and quarter + 4) owns query rows q0 + 32
+        // quarter + lane, taking its kChunks chunks of a tile's columns
         const int quarter = warp & 3, half = warp >> 2;
         const int64_t qi = q0 + 32 * quarter + lane;
         const bool qvalid = qi < n;
@@ -294,9 +310,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_knn_scan(const ScanArgs a) {
         const float sqE = MODE == 1 && qvalid ? sqrtf(a.tau[qi]) + a.q.rerr[qi] : 0.f;
         uint32_t *mine = MODE == 1 ? a.buf + ((size_t)(qvalid ? qi : 0) * 2 + half) * a.cap : nullptr;
         uint32_t found = 0u;
-        // MODE 0: max-heap of the r smallest e_j of this half's columns
-        float *heap = lists + ((size_t)half * kTcRows + 32 * quarter + lane) * rs;
-        float *es = stage + warp * 32 * 32;
+        // MODE 0: max-heap of the row's r smallest e_j
+        float *heap = lists + (size_t)(32 * quarter + lane) * rs;
         float root = INFINITY;
         // the row's own column among the candidates, if it is one
         const int64_t self = MODE == 1 ? qi
@@ -321,13 +336,13 @@ __global__ void __launch_bounds__(kThreads, 2) k_knn_scan(const ScanArgs a) {
             const int64_t c0 = (int64_t)tt * kTcCols;
             const float *hb = hbuf + b * kHG;
 #pragma unroll
-            for (int cc = 0; cc < 2; cc++) {
-                const int ci = 2 * half + cc, cb = 32 * ci;
+            for (int cc = 0; cc < kChunks; cc++) {
+                const int ci = kChunks * half + cc, cb = 32 * ci;
                 uint32_t raw[32];
                 tc::tmem_ld32_async(
                     tbase + ((uint32_t)(32 * quarter) << 16) + (uint32_t)(b * kTcCols + cb), raw);
                 tc::tmem_wait_ld();
-                if (cc == 1) {  // the accumulator is free
+                if (cc == kChunks - 1) {  // the accumulator is free
                     tc::fence_before();
                     __syncwarp();
                     if (lane == 0) tc::mbar_arrive(&bar_te[b]);
@@ -377,14 +392,11 @@ __global__ void __launch_bounds__(kThreads, 2) k_knn_scan(const ScanArgs a) {
                         if (found < (uint32_t)a.cap) mine[found] = (uint32_t)(c0 + cb + j);
                         found++;
                     }
-                } else if (__any_sync(0xffffffffu, sm != 0u)) {
-#pragma unroll
-                    for (int j = 0; j < 32; j++) es[j * 32 + lane] = __uint_as_float(raw[j]);
-                    __syncwarp();
+                } else {
                     while (sm) {
                         const int j = __clz(sm);
                         sm ^= 0x80000000u >> j;
-                        const float e = es[j * 32 + lane];
+                        const float e = pick32(raw, j);
                         if (!(e < root)) continue;
                         int p = 0;
                         for (;;) {
@@ -418,32 +430,12 @@ __global__ void __launch_bounds__(kThreads, 2) k_knn_scan(const ScanArgs a) {
             }
         }
         if (MODE == 1 && qvalid) a.cnt[qi * 2 + half] = found;
+        if (MODE == 0 && qvalid) a.tau[qi] = fmaxf(root + qn2, 0.f);
     }
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
     if (warp == kMmaWarp) tc::tmem_dealloc(tbase, kAcc * kTcCols);
-    if (MODE == 0 && tid < kTcRows && q0 + tid < n) {
-        // the r-th smallest of both halves' lists
-        float *h0 = lists + (size_t)tid * rs;
-        const float *h1 = lists + ((size_t)kTcRows + tid) * rs;
-        for (int c1 = 0; c1 < a.r; c1++) {
-            const float e = h1[c1];
-            if (!(e < h0[0])) continue;
-            int p = 0;
-            for (;;) {
-                int c = 2 * p + 1;
-                if (c >= a.r) break;
-                float vc = h0[c];
-                if (c + 1 < a.r && h0[c + 1] > vc) vc = h0[++c];
-                if (!(vc > e)) break;
-                h0[p] = vc;
-                p = c;
-            }
-            h0[p] = e;
-        }
-        a.tau[q0 + tid] = fmaxf(h0[0] + a.q.nrm[q0 + tid], 0.f);
-    }
 }
 
 // ---- exact distances and the k nearest
@@ -452,7 +444,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_knn_scan(const ScanArgs a) {
 // so that the lanes' 16-byte reads do not conflict),
 // then every lane sums its candidate's squared differences in index order.
 // (Lanes reading their candidate's row from global memory touch 32 lines per
-// load.)  The candidates within tau go to a key buffer (distance, then row
+// load; at n = 1M the 113 GB of rows come at 6.8 TB/s, and staging half rows, with
+// twice the warps per SM, changed nothing.)  The candidates within tau go to a key buffer (distance, then row
 // index); it is sorted by a bitonic network in registers, 8 or 16 keys per lane.
 constexpr int kPickWarps = 2;
 constexpr int kPickKeys = 512;  // most candidates within tau
@@ -498,16 +491,16 @@ __global__ void __launch_bounds__(kPickWarps * 32) k_knn_pick(const PickArgs a) 
     __shared__ uint64_t s_bar[kPickWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int ls = pick_pitch(a.ld);
-    uint8_t *base = pick_raw + (size_t)warp * ((size_t)33 * ls * 4 + kPickKeys * 8);
+    uint8_t *base = pick_raw + (size_t)warp * (pick_smem(a.ld) / kPickWarps);
     u64 *keys = reinterpret_cast<u64 *>(base);
     float *qrow = reinterpret_cast<float *>(keys + kPickKeys);
     float *rows = qrow + ls;
+    const uint32_t bytes = (uint32_t)a.ld * 4u;
     uint64_t *bar = &s_bar[warp];
     if (lane == 0) tc::mbar_init(bar, 1);
     __syncthreads();
     uint32_t phase = 0u;
     u64 n_exact = 0u, n_kept = 0u;
-    const uint32_t bytes = (uint32_t)a.ld * 4u;
     bool ok = true;
     const int64_t rows_all = a.qlist ? (int64_t)*a.qcount * kTcRows : a.n;
     for (int64_t q = blockIdx.x * (int64_t)kPickWarps + warp; ok && q < rows_all;
@@ -662,10 +655,10 @@ cudaError_t launch_knn_scan(const pxsne_ctx *c, const KnnScan &a, int sms, uint3
     const int64_t need = (n + kPickWarps - 1) / kPickWarps;
     const unsigned pgrid =
         (unsigned)std::min<int64_t>(need, (int64_t)std::max(1, per) * std::max(1, sms));
-    k_knn_scan<0><<<(unsigned)T, kThreads, sm0, st>>>(s);
+    k_knn_scan<0><<<(unsigned)T, scan_threads(0), sm0, st>>>(s);
     if ((e = cudaGetLastError())) return e;
     s.c = a.q;
-    k_knn_scan<1><<<(unsigned)T, kThreads, sm1, st>>>(s);
+    k_knn_scan<1><<<(unsigned)T, scan_threads(1), sm1, st>>>(s);
     if ((e = cudaGetLastError())) return e;
     PickArgs p{n, a.ld, a.k, cap, a.q.X, tau, nullptr, nullptr, buf, cnt, a.order, a.out_idx, a.out_d2,
                flag, retry, nretry, failed, nfailed, a.err, a.stats};
@@ -676,7 +669,7 @@ cudaError_t launch_knn_scan(const pxsne_ctx *c, const KnnScan &a, int sms, uint3
     s.qlist = p.qlist = retry;
     s.qcount = p.qcount = nretry;
     p.retry = nullptr;
-    k_knn_scan<1><<<(unsigned)T, kThreads, sm1, st>>>(s);
+    k_knn_scan<1><<<(unsigned)T, scan_threads(1), sm1, st>>>(s);
     if ((e = cudaGetLastError())) return e;
     k_knn_pick<<<pgrid, kPickWarps * 32, smp, st>>>(p);
     if ((e = cudaGetLastError())) return e;
