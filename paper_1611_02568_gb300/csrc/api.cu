@@ -213,9 +213,8 @@ int ensure_state(pxsne_ctx *c) {
         CK(c, dalloc(c, &c->lvl_sx[k], lvl + 4));
         CK(c, dalloc(c, &c->lvl_sy[k], lvl + 4));
     }
-    c->zblocks = (int)((n + 4095) / 4096);
-    if (c->zblocks > 1024) c->zblocks = 1024;
-    if (c->zblocks < 1) c->zblocks = 1;
+    // (about four values per thread: the sum is latency)
+    c->zblocks = (int)std::min<int64_t>(512, std::max<int64_t>(1, (n + 2047) / 2048));
     CK(c, dalloc(c, &c->zpart, c->zblocks));
     c->klblocks = 6 * std::max(c->sms, 1);
     CK(c, dalloc(c, &c->klpart, 2 * c->klblocks));

@@ -201,6 +201,17 @@ __host__ __device__ inline u64 screen_extent(int32_t r, int L) {
     return r > 0 ? (u64)r << (32 - L) : (u64(1) << 32);
 }
 
+// BH acceptance threshold of level l from the axes' y-units per ulp: a cell's
+// diagonal in y-units squared is W^2 (s0^2 + s1^2), W = 2^(32-l) ulps, and Eq.
+// bh_criteria accepts when r_c^2 < theta^2 d^2.
+__device__ inline float bh_threshold(int l, int L, double s0, double s1, float theta) {
+    const double th2 = (double)theta * (double)theta;
+    if (l > L) return INFINITY;
+    const double W2 = ldexp(1.0, 64 - 2 * l);
+    const double rc2 = W2 * (s0 * s0 + s1 * s1);
+    return th2 > 0.0 ? (float)(rc2 / th2) : INFINITY;
+}
+
 // Derived per-iteration scalars from s (called by one thread).
 __device__ inline void derive_scalars(DevScalars *sc, float theta, int L) {
     const double s0 = sc->s[0], s1 = sc->s[1];
@@ -208,15 +219,7 @@ __device__ inline void derive_scalars(DevScalars *sc, float theta, int L) {
     sc->inv_s[1] = 1.0 / s1;
     sc->sf[0] = (float)s0;
     sc->sf[1] = (float)s1;
-    const double th2 = (double)theta * (double)theta;
-    for (int l = 0; l <= kMaxL + 1; l++) {
-        if (l > L) { sc->T[l] = INFINITY; continue; }
-        // diagonal of a level-l cell in y-units, squared: W^2 (s0^2 + s1^2),
-        // W = 2^(32-l) ulps; Eq. bh_criteria accepts when r_c^2 < theta^2 d^2
-        double W2 = ldexp(1.0, 64 - 2 * l);
-        double rc2 = W2 * (s0 * s0 + s1 * s1);
-        sc->T[l] = th2 > 0.0 ? (float)(rc2 / th2) : INFINITY;
-    }
+    for (int l = 0; l <= kMaxL + 1; l++) sc->T[l] = bh_threshold(l, L, s0, s1, theta);
 }
 
 

@@ -33,27 +33,35 @@ __global__ void k_snap_hist(int n, int L, int rescale, float theta, u64 Rx, u64 
         gx = (u64)(sc->mm[par][2] - mnx) + 1ull;
         gy = (u64)(sc->mm[par][3] - mny) + 1ull;
         // R_d / gamma_d is the same for every point: one FP64 division per
-        // CTA (FP64 issues at a small fraction of the FP32 rate)
-        if (threadIdx.x == 0) {
-            s_q[0] = (double)Rx / (double)gx;
-            s_q[1] = (double)Ry / (double)gy;
-        }
+        // CTA and axis (FP64 issues at a small fraction of the FP32 rate)
+        if (threadIdx.x < 2)
+            s_q[threadIdx.x] = threadIdx.x == 0 ? (double)Rx / (double)gx : (double)Ry / (double)gy;
         __syncthreads();
         qx = s_q[0];
         qy = s_q[1];
-        if (tid == 0) {
-            sc->n_accept = 0ull;
-            sc->n_test = 0ull;
-            sc->n_steps = 0ull;
-            sc->n_nodes = 0ull;
-            // Eq. beta_scaling carried as s_d <- (s_d * gamma_d) / R_d
-            sc->s[0] = (sc->s[0] * (double)gx) / (double)Rx;
-            sc->s[1] = (sc->s[1] * (double)gy) / (double)Ry;
-            derive_scalars(sc, theta, L);
-            sc->mm[par ^ 1][0] = 0x7fffffffffffffffll;
-            sc->mm[par ^ 1][1] = 0x7fffffffffffffffll;
-            sc->mm[par ^ 1][2] = (i64)0x8000000000000000ull;
-            sc->mm[par ^ 1][3] = (i64)0x8000000000000000ull;
+        if (tid < 32) {
+            // Eq. beta_scaling carried as s_d <- (s_d * gamma_d) / R_d, and what
+            // derives from it, a lane per FP64 division (one thread forming all
+            // of them took 5 of the kernel's 10 us at n = 2000)
+            const double s0 = (sc->s[0] * (double)gx) / (double)Rx;
+            const double s1 = (sc->s[1] * (double)gy) / (double)Ry;
+            __syncwarp();
+            if (tid == 0) {
+                sc->s[0] = s0;
+                sc->s[1] = s1;
+                sc->sf[0] = (float)s0;
+                sc->sf[1] = (float)s1;
+                sc->n_accept = 0ull;
+                sc->n_test = 0ull;
+                sc->n_steps = 0ull;
+                sc->n_nodes = 0ull;
+                sc->mm[par ^ 1][0] = 0x7fffffffffffffffll;
+                sc->mm[par ^ 1][1] = 0x7fffffffffffffffll;
+                sc->mm[par ^ 1][2] = (i64)0x8000000000000000ull;
+                sc->mm[par ^ 1][3] = (i64)0x8000000000000000ull;
+            }
+            if (tid <= kMaxL + 1) sc->T[tid] = bh_threshold(tid, L, s0, s1, theta);
+            else if (tid < kMaxL + 4) sc->inv_s[tid - kMaxL - 2] = 1.0 / (tid == kMaxL + 2 ? s0 : s1);
         }
     }
     if (!rescale && tid == 0) {
@@ -301,30 +309,72 @@ __device__ __forceinline__ void put_record(float4 *rec, float *recn, int l, uint
     recn[rec_offset(l) + m] = (float)N;
 }
 
-// Levels h0-1 .. 0 from the sums of level h0 (4^h0 cells in c0/x0/y0, whose
-// records are written), by one CTA of 256 threads, ping-ponging through
-// c1/x1/y1; also blk_off = the exclusive scan of the level-h0 counts (each the
-// pixel total of one first-pass CTA).
-__device__ void pyr_top(int h0, uint32_t *c0, u64 *x0, u64 *y0, uint32_t *c1, u64 *x1, u64 *y1,
-                        float4 *rec, float *recn, uint32_t *blk_off, uint32_t *s_warp) {
-    const int tid = threadIdx.x;
-    const int nb = 1 << (2 * h0);
-    // blk_off: each thread scans a contiguous segment (16-byte loads when the
-    // segments are multiples of four)
-    const int seg = (nb + 255) / 256;
-    const int a = tid * seg, e = min(nb, a + seg);
-    uint32_t v = 0u;
-    if ((seg & 3) == 0) {
-        for (int i = a; i < e; i += 4) {
-            const uint4 q = __ldcg(reinterpret_cast<const uint4 *>(c0 + i));
-            v += q.x + q.y + q.z + q.w;
+// The four cells 4 g .. 4 g + 3 of a level (counts c, sums x, y) added up.
+__device__ __forceinline__ void sum_group(const uint32_t *c, const u64 *x, const u64 *y, int g,
+                                          bool sums, uint32_t &N, u64 &X, u64 &Y) {
+    const uint4 q4 = __ldcg(reinterpret_cast<const uint4 *>(c) + g);
+    N = q4.x + q4.y + q4.z + q4.w;
+    X = Y = 0ull;
+    if (!sums) return;
+    const ulonglong2 xa = __ldcg(reinterpret_cast<const ulonglong2 *>(x) + 2 * g);
+    const ulonglong2 xb = __ldcg(reinterpret_cast<const ulonglong2 *>(x) + 2 * g + 1);
+    const ulonglong2 ya = __ldcg(reinterpret_cast<const ulonglong2 *>(y) + 2 * g);
+    const ulonglong2 yb = __ldcg(reinterpret_cast<const ulonglong2 *>(y) + 2 * g + 1);
+    X = xa.x + xa.y + xb.x + xb.y;
+    Y = ya.x + ya.y + yb.x + yb.y;
+}
+
+// The last CTA's share for 256 cells of level h0 and more (h0 >= 4): a thread
+// adds up its run of cells level by level down to one cell of level 4, and the
+// levels above follow by shuffles, so that the cells are read once instead of
+// every level through global memory.  Bound by the chain of dependent loads and
+// barriers (one CTA): the pyramid's launch takes 14 us instead of 19 for a
+// 2048^2 screen and 54 instead of 61 for 4096^2 (n = 70,000 and 1M).
+__device__ void pyr_top_wide(int h0, const uint32_t *c0, const u64 *x0, const u64 *y0, float4 *rec,
+                             float *recn, uint32_t *blk_off, uint32_t *s_warp, uint32_t *s_n,
+                             u64 *s_x, u64 *s_y) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const bool sums = rec != nullptr;
+    const int seg = (1 << (2 * h0)) >> 8;  // 1, 4, 16 or 64 cells per thread
+    uint32_t N = 0u;
+    u64 X = 0ull, Y = 0ull;
+    if (seg == 1) {
+        N = __ldcg(c0 + tid);
+        if (sums) {
+            X = __ldcg(x0 + tid);
+            Y = __ldcg(y0 + tid);
         }
+    } else if (seg == 4) {
+        sum_group(c0, x0, y0, tid, sums, N, X, Y);
+        put_record(rec, recn, h0 - 1, (uint32_t)tid, N, X, Y);
     } else {
-        for (int i = a; i < e; i++) v += __ldcg(c0 + i);
+        for (int q = 0; q < seg / 16; q++) {
+            uint32_t n2 = 0u;
+            u64 x2 = 0ull, y2 = 0ull;
+            const int at = tid * (seg / 16) + q;  // cell of level h0 - 2
+#pragma unroll
+            for (int g = 0; g < 4; g++) {
+                uint32_t n1;
+                u64 x1, y1;
+                sum_group(c0, x0, y0, 4 * at + g, sums, n1, x1, y1);
+                put_record(rec, recn, h0 - 1, (uint32_t)(4 * at + g), n1, x1, y1);
+                n2 += n1;
+                x2 += x1;
+                y2 += y1;
+            }
+            put_record(rec, recn, h0 - 2, (uint32_t)at, n2, x2, y2);
+            N += n2;
+            X += x2;
+            Y += y2;
+        }
+        if (seg == 64) put_record(rec, recn, h0 - 3, (uint32_t)tid, N, X, Y);
     }
-    uint32_t run = block_excl_scan(v, 256, s_warp);
-    if ((seg & 3) == 0) {
-        for (int i = a; i < e; i += 4) {
+    // the pixel starts of the first pass's CTAs
+    uint32_t run = block_excl_scan(N, 256, s_warp);
+    if (seg == 1) {
+        blk_off[tid] = run;
+    } else {
+        for (int i = tid * seg; i < (tid + 1) * seg; i += 4) {
             const uint4 q = __ldcg(reinterpret_cast<const uint4 *>(c0 + i));
             uint4 o;
             o.x = run;
@@ -334,13 +384,49 @@ __device__ void pyr_top(int h0, uint32_t *c0, u64 *x0, u64 *y0, uint32_t *c1, u6
             run = o.w + q.w;
             *reinterpret_cast<uint4 *>(blk_off + i) = o;
         }
-    } else {
-        for (int i = a; i < e; i++) {
-            const uint32_t ci = __ldcg(c0 + i);
-            blk_off[i] = run;
-            run += ci;
-        }
     }
+    // levels 3 (4 threads) and 2 (16), then 1 and 0 across the warps
+#pragma unroll
+    for (int o = 1; o <= 16; o <<= 1) {
+        N += __shfl_xor_sync(0xffffffffu, N, o);
+        X += __shfl_xor_sync(0xffffffffu, X, o);
+        Y += __shfl_xor_sync(0xffffffffu, Y, o);
+        if (o == 2 && (lane & 3) == 0) put_record(rec, recn, 3, (uint32_t)(tid >> 2), N, X, Y);
+        if (o == 8 && (lane & 15) == 0) put_record(rec, recn, 2, (uint32_t)(tid >> 4), N, X, Y);
+    }
+    __syncthreads();
+    if (lane == 0) {
+        s_n[warp] = N;
+        s_x[warp] = X;
+        s_y[warp] = Y;
+    }
+    __syncthreads();
+    if (tid < 4)
+        put_record(rec, recn, 1, (uint32_t)tid, s_n[2 * tid] + s_n[2 * tid + 1],
+                   s_x[2 * tid] + s_x[2 * tid + 1], s_y[2 * tid] + s_y[2 * tid + 1]);
+    if (tid == 4) {
+        uint32_t n = 0u;
+        u64 x = 0ull, y = 0ull;
+        for (int w = 0; w < 8; w++) {
+            n += s_n[w];
+            x += s_x[w];
+            y += s_y[w];
+        }
+        put_record(rec, recn, 0, 0u, n, x, y);
+    }
+}
+
+// Levels h0-1 .. 0 from the sums of level h0 (4^h0 cells in c0/x0/y0, whose
+// records are written), by one CTA of 256 threads, ping-ponging through
+// c1/x1/y1; also blk_off = the exclusive scan of the level-h0 counts (each the
+// pixel total of one first-pass CTA).  For fewer than 256 cells (h0 < 4).
+__device__ void pyr_top(int h0, uint32_t *c0, u64 *x0, u64 *y0, uint32_t *c1, u64 *x1, u64 *y1,
+                        float4 *rec, float *recn, uint32_t *blk_off, uint32_t *s_warp) {
+    const int tid = threadIdx.x;
+    const int nb = 1 << (2 * h0);
+    const uint32_t v = tid < nb ? __ldcg(c0 + tid) : 0u;
+    const uint32_t run = block_excl_scan(v, 256, s_warp);
+    if (tid < nb) blk_off[tid] = run;
     uint32_t *cc = c0, *cn = c1;
     u64 *xc = x0, *xn = x1, *yc = y0, *yn = y1;
     const bool sums = rec != nullptr;
@@ -486,7 +572,10 @@ __global__ void __launch_bounds__(256)
     __syncthreads();
     if (!s_last) return;
     __threadfence();
-    pyr_top(h - 5, out_cnt, out_sx, out_sy, scr_cnt, scr_sx, scr_sy, rec, recn, blk_off, s_warp);
+    if (h >= 9)
+        pyr_top_wide(h - 5, out_cnt, out_sx, out_sy, rec, recn, blk_off, s_warp, s_n, s_x, s_y);
+    else
+        pyr_top(h - 5, out_cnt, out_sx, out_sy, scr_cnt, scr_sx, scr_sy, rec, recn, blk_off, s_warp);
     if (tid == 0) {
         sc->pyr_ticket = 0u;
         if (bump_t) sc->t += 1;

@@ -141,3 +141,36 @@ def test_nbr_precision_on_uneven_states(n, level, k):
     prec_o, hits_o = oracle.nbr_precision(hd, k, z, s, per_row=True)
     assert np.array_equal(hits, hits_o)
     assert prec == pytest.approx(prec_o, abs=1e-15)
+
+
+@pytest.mark.parametrize("n,level,centre", [
+    (2047, 8, 0), (2048, 10, 0), (2049, 7, 1), (2049, 10, 1), (65535, 9, 0), (65536, 8, 0)])
+def test_upper_levels_sums_and_rows(n, level, centre):
+    """Counts of every level and the forces that read the upper levels'
+    records (a wide criterion) on screens whose top is built by each of the
+    two ways, Z on both sides of one CTA's share (FP64: 1e-12), and the
+    attraction on both sides of a warp's one row and four."""
+    import paper_1611_02568_gb300 as px
+    from paper_1611_02568_gb300 import build
+    build.build()
+    z, s = state(n, 11)
+    row, col, val = ring_P(n)
+    rows = np.unique(np.concatenate([np.arange(40), np.arange(n - 40, n),
+                                     np.random.default_rng(2).integers(0, n, 800)]))
+    with px.Context(px.Params(log2_r=level, theta=1.5, centre_mode=centre)) as ctx:
+        ctx.set_P(row, col, val)
+        for _ in range(2):   # from fresh leaves, and from the cleared ones
+            ctx.set_state(z, s)
+            Frep, Zi, Fattr, Z = ctx.get_forces()
+            cnt_o = oracle.pyramid(z, level)[0]
+            for lv in range(level + 1):
+                at = oracle.level_offset(lv)
+                assert np.array_equal(ctx.get_tree(lv)[0], cnt_o[at:at + 4 ** lv]), lv
+            mo = oracle.leaf_keys(z, level)[2]
+            assert np.array_equal(ctx.get_tree(0, morton=True)[3], mo)
+    oF, oZi, _ = oracle.bh_repulsion(z, s, level, 1.5, rows=rows, centre_mode=centre)
+    oA = oracle.attraction(oracle.CSR(row, col.astype(np.int32), val), z, s)
+    assert rel(Frep[rows], oF) <= FORCE_TOL
+    assert rel(Zi[rows], oZi) <= FORCE_TOL
+    assert rel(Fattr, oA) <= FORCE_TOL
+    assert abs(Z - Zi.astype(np.float64).sum()) <= 1e-12 * Z
