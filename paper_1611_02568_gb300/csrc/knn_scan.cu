@@ -35,7 +35,10 @@
 namespace pxsne {
 namespace {
 
-constexpr int kStages = 2;        // candidate-tile stages in shared memory
+// Candidate-tile stages in shared memory, and slots of the tiles' norms: four
+// where two CTAs still fit on an SM with them, else two.  (D = 128, n = 1M, one
+// CTA of four stages: 60 ms for the second pass, two of two: 45.)
+__host__ __device__ constexpr int stages(int mode, int Dp) { return mode == 1 && Dp <= 64 ? 4 : 2; }
 constexpr int kAcc = 2;           // TMEM accumulators of 128 columns
 // Filter warps: one per TMEM lane quarter in the sample pass (MODE 0), so that a
 // row has one list, and two, of 64 columns each, in the other; then the loader's
@@ -56,17 +59,24 @@ struct ScanArgs {
     u64 *stats;
 };
 
+// MODE 1: the visits decided before the first tile, 32 a word (2 KB; all visits
+// up to n = 2.1M).  The loader alone took 1.4 us for each 32 visits, of which it
+// keeps about four, while its two stages ran dry: with all warps deciding first,
+// the second pass takes 45 ms instead of 56 at n = 1M, D = 128.
+constexpr int kKeepWords = 512;
+
 // The i-th candidate tile a CTA visits: outward from its own neighbourhood.
 __device__ __forceinline__ int64_t tile_at(int64_t own, int64_t i, int64_t T) {
     const int64_t off = (i & 1) ? (i + 1) / 2 : -(i / 2);
     return ((own + off) % T + T) % T;
 }
 
-// Shared memory: A tile, kStages candidate tiles, kAcc x kHG floats, then for
+// Shared memory: A tile, the stages of candidate tiles and of kHG floats, then for
 // the sample pass the lists (128 rows x rs floats, rs odd).  At k = 90 two CTAs
 // fit on an SM in both passes.
 __host__ __device__ inline size_t scan_smem(int mode, int Dp, int r) {
-    size_t b = (size_t)(1 + kStages) * kTcRows * Dp * 2 + (size_t)kAcc * kHG * 4 + 1024;
+    size_t b = (size_t)(1 + stages(mode, Dp)) * kTcRows * Dp * 2 +
+               (size_t)stages(mode, Dp) * kHG * 4 + 1024;
     if (mode == 0) b += (size_t)kTcRows * (r | 1) * 4;
     return b;
 }
@@ -92,19 +102,20 @@ __device__ __forceinline__ float pick32(const uint32_t (&v)[32], int j) {
 // filter warps, two per quarter of the rows.  A value costs a packed half FMA
 // and add and one funnel shift that collects the sign bits of e_j - t, e_j =
 // (1-eps)|c~_j|^2 - 2 q~.c~_j, with the chunk's largest kappa |q~||c~| in t.
-template <int MODE>
+template <int MODE, int kStages>
 __global__ void __launch_bounds__(scan_threads(MODE), 2) k_knn_scan(const ScanArgs a) {
     constexpr int kFilterWarps = filter_warps(MODE), kThreads = scan_threads(MODE);
     constexpr int kLoadWarp = kFilterWarps, kMmaWarp = kFilterWarps + 1;
     constexpr int kChunks = 16 / kFilterWarps;  // 32-column chunks of a tile per warp
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t bar_a, bar_sf[kStages], bar_se[kStages], bar_tf[kAcc], bar_te[kAcc],
-        bar_hf[kAcc], bar_he[kAcc];
+        bar_hf[kStages], bar_he[kStages];
     __shared__ uint32_t tslot;
     __shared__ volatile int s_abort;
     __shared__ volatile float s_taumax[kFilterWarps];
     __shared__ volatile int s_tile[8];
     __shared__ float s_cq[128];
+    __shared__ uint32_t s_keep[MODE == 1 ? kKeepWords : 1];
     uint8_t *smem = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
     const int64_t n = a.q.n, T = a.c.T;
     const uint32_t tile_bytes = (uint32_t)kTcRows * a.Dp * 2;
@@ -112,7 +123,7 @@ __global__ void __launch_bounds__(scan_threads(MODE), 2) k_knn_scan(const ScanAr
     uint8_t *sB = smem + tile_bytes;
     float *hbuf = reinterpret_cast<float *>(sB + (size_t)kStages * tile_bytes);
     const int rs = a.r | 1;
-    float *lists = hbuf + kAcc * kHG;
+    float *lists = hbuf + kStages * kHG;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (MODE == 1 && a.qlist && blockIdx.x >= *a.qcount) return;
     const int64_t qt = MODE == 1 && a.qlist ? a.qlist[blockIdx.x] : blockIdx.x, q0 = qt * kTcRows;
@@ -126,67 +137,87 @@ __global__ void __launch_bounds__(scan_threads(MODE), 2) k_knn_scan(const ScanAr
         for (int s = 0; s < kStages; s++) {
             tc::mbar_init(&bar_sf[s], 1);
             tc::mbar_init(&bar_se[s], 1);
+            tc::mbar_init(&bar_hf[s], 1);
+            tc::mbar_init(&bar_he[s], kFilterWarps);
         }
         for (int b = 0; b < kAcc; b++) {
             tc::mbar_init(&bar_tf[b], 1);
             tc::mbar_init(&bar_te[b], kFilterWarps);
-            tc::mbar_init(&bar_hf[b], 1);
-            tc::mbar_init(&bar_he[b], kFilterWarps);
         }
         s_abort = 0;
         for (int w = 0; w < kFilterWarps; w++) s_taumax[w] = INFINITY;
     }
+    for (int d = tid; d < a.Dp; d += kThreads) s_cq[d] = a.q.cent[qt * a.Dp + d];
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
     const uint32_t tbase = tslot;
+    const float rq = a.q.rad[qt];
+    // The lane's tile of the visits i0 .. i0 + 31, and which of the 32 a row's
+    // neighbours can be in: its centroid is no farther than the radii and the
+    // largest threshold.
+    const auto keep32 = [&](int64_t i0, float taum, int64_t &tl) {
+        const int64_t il = i0 + lane;
+        const bool in = il < T;
+        tl = in ? tile_at(own, il, T) : 0;
+        float dd = 0.f;
+        if (in) {
+            const float4 *ct = reinterpret_cast<const float4 *>(a.c.cent + tl * a.Dp);
+            for (int d4 = 0; d4 < a.Dp / 4; d4++) {
+                const float4 c = __ldg(ct + d4);
+                const float e0 = s_cq[4 * d4] - c.x, e1 = s_cq[4 * d4 + 1] - c.y;
+                const float e2 = s_cq[4 * d4 + 2] - c.z, e3 = s_cq[4 * d4 + 3] - c.w;
+                dd = fmaf(e0, e0, fmaf(e1, e1, fmaf(e2, e2, fmaf(e3, e3, dd))));
+            }
+        }
+        const float lbd = sqrtf(dd) * 0.9999f - rq - (in ? a.c.rad[tl] : 0.f);
+        const bool skip = in && il > 0 && lbd > 0.f && lbd * lbd > taum * 1.0001f;
+        return __ballot_sync(0xffffffffu, in && !skip);
+    };
+    float taum = INFINITY;
+    if (MODE == 1) {
+        taum = 0.f;
+        for (int r = lane; r < kTcRows; r += 32)
+            if (q0 + r < n) taum = fmaxf(taum, a.tau[q0 + r]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) taum = fmaxf(taum, __shfl_xor_sync(0xffffffffu, taum, o));
+        // the thresholds being known, all warps decide about the first
+        // 32 kKeepWords visits
+        for (int w = warp; w < kKeepWords && (int64_t)w * 32 < T; w += kThreads / 32) {
+            int64_t tl;
+            const unsigned keep = keep32((int64_t)w * 32, taum, tl);
+            if (lane == 0) s_keep[w] = keep;
+        }
+        __syncthreads();
+    }
 
     if (warp == kLoadWarp) {
         // ---- loader.  The kept tiles form a sequence j = 0, 1, ... that the
         // other warps follow through s_tile; the entry after the last is -1
         // (its barriers completed without data).
-        for (int d = lane; d < a.Dp; d += 32) s_cq[d] = a.q.cent[qt * a.Dp + d];
-        float taum = INFINITY;
-        if (MODE == 1) {
-            taum = 0.f;
-            for (int r = lane; r < kTcRows; r += 32)
-                if (q0 + r < n) taum = fmaxf(taum, a.tau[q0 + r]);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) taum = fmaxf(taum, __shfl_xor_sync(0xffffffffu, taum, o));
-        }
-        __syncwarp();
-        const float rq = a.q.rad[qt];
         if (lane == 0) {
             tc::mbar_expect_tx(&bar_a, tile_bytes);
             tc::bulk_g2s(sA, a.q.img + qt * tile_bytes, tile_bytes, &bar_a);
         }
         int64_t j = 0, n_sf = 0, n_hf = 0;
         u64 n_skip = 0u;
-        bool fail = false;
+        bool fail = false, ended = false;
         for (int64_t i0 = 0; i0 <= T && !fail; i0 += 32) {
             if (__shfl_sync(0xffffffffu, s_abort, 0)) break;
-            const int64_t il = i0 + lane;
-            const bool in = il < T;
-            const int64_t tl = in ? tile_at(own, il, T) : 0;
-            float dd = 0.f;
-            if (in) {
-                const float4 *ct = reinterpret_cast<const float4 *>(a.c.cent + tl * a.Dp);
-                for (int d4 = 0; d4 < a.Dp / 4; d4++) {
-                    const float4 c = __ldg(ct + d4);
-                    const float e0 = s_cq[4 * d4] - c.x, e1 = s_cq[4 * d4 + 1] - c.y;
-                    const float e2 = s_cq[4 * d4 + 2] - c.z, e3 = s_cq[4 * d4 + 3] - c.w;
-                    dd = fmaf(e0, e0, fmaf(e1, e1, fmaf(e2, e2, fmaf(e3, e3, dd))));
-                }
-            }
             if (MODE == 0) {
                 taum = 0.f;
 #pragma unroll
                 for (int w = 0; w < kFilterWarps; w++) taum = fmaxf(taum, s_taumax[w]);
             }
-            const float lbd = sqrtf(dd) * 0.9999f - rq - (in ? a.c.rad[tl] : 0.f);
-            const bool skip = in && il > 0 && lbd > 0.f && lbd * lbd > taum * 1.0001f;
-            n_skip += (u64)__popc(__ballot_sync(0xffffffffu, skip));
-            unsigned keep = __ballot_sync(0xffffffffu, in && !skip);
+            int64_t tl;
+            unsigned keep;
+            if (MODE == 1 && i0 < 32 * kKeepWords) {
+                tl = i0 + lane < T ? tile_at(own, i0 + lane, T) : 0;
+                keep = i0 < T ? s_keep[i0 >> 5] : 0u;
+            } else {
+                keep = keep32(i0, taum, tl);
+            }
+            n_skip += (u64)(min((int64_t)32, T - i0) - __popc(keep));
             const bool last_block = i0 + 32 > T;
             while (keep || last_block) {
                 const bool end = keep == 0u;  // (only in the last block)
@@ -196,7 +227,7 @@ __global__ void __launch_bounds__(scan_threads(MODE), 2) k_knn_scan(const ScanAr
                     keep &= keep - 1u;
                     t = __shfl_sync(0xffffffffu, tl, src);
                 }
-                const int s = (int)(j % kStages), b = (int)(j % kAcc);
+                const int s = (int)(j % kStages);
                 bool ok = j < kStages ||
                           tc::mbar_wait_sleep(&bar_se[s], (uint32_t)((j / kStages - 1) & 1), kTcPolls,
                                               kTcSleepNs);
@@ -214,17 +245,17 @@ __global__ void __launch_bounds__(scan_threads(MODE), 2) k_knn_scan(const ScanAr
                     }
                     if (!end) n_sf++;
                     __syncwarp();
-                    ok = j < kAcc ||
-                         tc::mbar_wait_sleep(&bar_he[b], (uint32_t)((j / kAcc - 1) & 1), kTcPolls,
+                    ok = j < kStages ||
+                         tc::mbar_wait_sleep(&bar_he[s], (uint32_t)((j / kStages - 1) & 1), kTcPolls,
                                              kTcSleepNs);
                     ok = __all_sync(0xffffffffu, ok);
                     if (ok) {
                         if (lane == 0) {
                             if (end) {
-                                tc::mbar_arrive(&bar_hf[b]);
+                                tc::mbar_arrive(&bar_hf[s]);
                             } else {
-                                tc::mbar_expect_tx(&bar_hf[b], kHG * 4);
-                                tc::bulk_g2s(hbuf + b * kHG, a.c.HG + t * kHG, kHG * 4, &bar_hf[b]);
+                                tc::mbar_expect_tx(&bar_hf[s], kHG * 4);
+                                tc::bulk_g2s(hbuf + s * kHG, a.c.HG + t * kHG, kHG * 4, &bar_hf[s]);
                             }
                         }
                         if (!end) n_hf++;
@@ -238,6 +269,7 @@ __global__ void __launch_bounds__(scan_threads(MODE), 2) k_knn_scan(const ScanAr
                     }
                 }
                 __syncwarp();
+                ended = end && !fail;
                 if (fail || end) break;
                 j++;
             }
@@ -247,12 +279,12 @@ __global__ void __launch_bounds__(scan_threads(MODE), 2) k_knn_scan(const ScanAr
             // copies still in flight complete before the CTA exits (those of the
             // last kept tiles; after the end mark the copies into the slots it
             // reused are known complete)
-            const int64_t ws = fail ? kStages : kStages - 1, wh = fail ? kAcc : kAcc - 1;
+            const int64_t ws = ended ? kStages - 1 : kStages;
             tc::mbar_wait(&bar_a, 0u, kTcPolls);
             for (int64_t q = (n_sf > ws ? n_sf - ws : 0); q < n_sf; q++)
                 tc::mbar_wait(&bar_sf[q % kStages], (uint32_t)((q / kStages) & 1), kTcPolls);
-            for (int64_t q = (n_hf > wh ? n_hf - wh : 0); q < n_hf; q++)
-                tc::mbar_wait(&bar_hf[q % kAcc], (uint32_t)((q / kAcc) & 1), kTcPolls);
+            for (int64_t q = (n_hf > ws ? n_hf - ws : 0); q < n_hf; q++)
+                tc::mbar_wait(&bar_hf[q % kStages], (uint32_t)((q / kStages) & 1), kTcPolls);
         }
     } else if (warp == kMmaWarp) {
         // ---- MMA issuer
@@ -319,11 +351,11 @@ __global__ void __launch_bounds__(scan_threads(MODE), 2) k_knn_scan(const ScanAr
                                  ? (qi - kScanPhase) / kScanStride
                                  : -1;
         for (int64_t i = 0; i <= T; i++) {
-            const int b = (int)(i % kAcc);
-            const uint32_t par = (uint32_t)((i / kAcc) & 1);
+            const int b = (int)(i % kAcc), hs = (int)(i % kStages);
+            const uint32_t par = (uint32_t)((i / kAcc) & 1), hpar = (uint32_t)((i / kStages) & 1);
             const bool got =
                 __all_sync(0xffffffffu, tc::mbar_wait_sleep(&bar_tf[b], par, kTcPolls, kTcSleepNs) &&
-                                            tc::mbar_wait_sleep(&bar_hf[b], par, kTcPolls, kTcSleepNs) &&
+                                            tc::mbar_wait_sleep(&bar_hf[hs], hpar, kTcPolls, kTcSleepNs) &&
                                             !s_abort);
             if (!got) {
                 if (lane == 0 && !s_abort) atomicOr(a.err, (unsigned)PXSNE_DEVERR_TIMEOUT);
@@ -334,7 +366,7 @@ __global__ void __launch_bounds__(scan_threads(MODE), 2) k_knn_scan(const ScanAr
             const int tt = s_tile[i & 7];
             if (tt < 0) break;
             const int64_t c0 = (int64_t)tt * kTcCols;
-            const float *hb = hbuf + b * kHG;
+            const float *hb = hbuf + hs * kHG;
 #pragma unroll
             for (int cc = 0; cc < kChunks; cc++) {
                 const int ci = kChunks * half + cc, cb = 32 * ci;
@@ -421,7 +453,7 @@ __global__ void __launch_bounds__(scan_threads(MODE), 2) k_knn_scan(const ScanAr
                 }
             }
             __syncwarp();
-            if (lane == 0) tc::mbar_arrive(&bar_he[b]);
+            if (lane == 0) tc::mbar_arrive(&bar_he[hs]);
             if (MODE == 0) {
                 float tm = qvalid ? root + qn2 : -INFINITY;
 #pragma unroll
@@ -642,9 +674,11 @@ cudaError_t launch_knn_scan(const pxsne_ctx *c, const KnnScan &a, int sms, uint3
     ScanArgs s{a.q, a.s, a.Dp, r, a.inv_s2, a.kappa, a.eps_abs, tau, nullptr, nullptr, buf, cnt, cap,
                a.err, a.stats};
     const int sm0 = (int)scan_smem(0, a.Dp, r), sm1 = (int)scan_smem(1, a.Dp, r);
-    if ((e = cudaFuncSetAttribute(k_knn_scan<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm0)))
+    const auto scan1 = stages(1, a.Dp) == 4 ? k_knn_scan<1, 4> : k_knn_scan<1, 2>;
+    if ((e = cudaFuncSetAttribute(k_knn_scan<0, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  sm0)))
         return e;
-    if ((e = cudaFuncSetAttribute(k_knn_scan<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm1)))
+    if ((e = cudaFuncSetAttribute(scan1, cudaFuncAttributeMaxDynamicSharedMemorySize, sm1)))
         return e;
     const int smp = (int)pick_smem(a.ld);
     if ((e = cudaFuncSetAttribute(k_knn_pick, cudaFuncAttributeMaxDynamicSharedMemorySize, smp)))
@@ -655,10 +689,10 @@ cudaError_t launch_knn_scan(const pxsne_ctx *c, const KnnScan &a, int sms, uint3
     const int64_t need = (n + kPickWarps - 1) / kPickWarps;
     const unsigned pgrid =
         (unsigned)std::min<int64_t>(need, (int64_t)std::max(1, per) * std::max(1, sms));
-    k_knn_scan<0><<<(unsigned)T, scan_threads(0), sm0, st>>>(s);
+    k_knn_scan<0, 2><<<(unsigned)T, scan_threads(0), sm0, st>>>(s);
     if ((e = cudaGetLastError())) return e;
     s.c = a.q;
-    k_knn_scan<1><<<(unsigned)T, scan_threads(1), sm1, st>>>(s);
+    scan1<<<(unsigned)T, scan_threads(1), sm1, st>>>(s);
     if ((e = cudaGetLastError())) return e;
     PickArgs p{n, a.ld, a.k, cap, a.q.X, tau, nullptr, nullptr, buf, cnt, a.order, a.out_idx, a.out_d2,
                flag, retry, nretry, failed, nfailed, a.err, a.stats};
@@ -669,7 +703,7 @@ cudaError_t launch_knn_scan(const pxsne_ctx *c, const KnnScan &a, int sms, uint3
     s.qlist = p.qlist = retry;
     s.qcount = p.qcount = nretry;
     p.retry = nullptr;
-    k_knn_scan<1><<<(unsigned)T, scan_threads(1), sm1, st>>>(s);
+    scan1<<<(unsigned)T, scan_threads(1), sm1, st>>>(s);
     if ((e = cudaGetLastError())) return e;
     k_knn_pick<<<pgrid, kPickWarps * 32, smp, st>>>(p);
     if ((e = cudaGetLastError())) return e;

@@ -74,6 +74,24 @@ def test_one_dimension_far_apart():
     check(X, 20, *lists(X, 20))
 
 
+def test_more_tiles_than_are_decided_first():
+    """Visits beyond the first 16,384 tiles, which the loader decides itself:
+    sampled rows against a brute force in FP64."""
+    import torch
+    rng = np.random.default_rng(12)
+    n, k = 16384 * 128 + 3 * 4096 + 77, 3
+    X = rng.standard_normal((n, 3)).astype(np.float32)
+    idx, d2 = lists(X, k)
+    dX = torch.from_numpy(X).cuda().double()
+    for i in (0, 77, n // 2, n - 1, *rng.integers(0, n, 40)):
+        t = ((dX - dX[i]) ** 2).sum(1)
+        t[i] = torch.inf
+        want = torch.topk(t, k, largest=False).values.cpu().numpy()
+        got = t[torch.from_numpy(idx[i].astype(np.int64)).cuda()].cpu().numpy()
+        np.testing.assert_allclose(got, want, rtol=2e-5)
+        np.testing.assert_allclose(d2[i], got, rtol=1e-5)
+
+
 def test_symmetric_rows_of_every_class():
     """P with rows of every length class of the symmetrisation (a warp's 256,
     512 and 1,024 keys, a CTA's shared memory and beyond): shells of points
