@@ -3,7 +3,7 @@
 // and Adam by the kernels below.  It maps a data row x to an initial 2-D
 // position, from which the plain method refines.
 //
-//   k_gemm<NT, EPI>  C = A B^T on the tensor cores (tcgen05, accumulator in
+//   k_gemm<EPI>      C = A B^T on the tensor cores (tcgen05, accumulator in
 //                    TMEM), A [M x K] and B [N x K] BF16 row-major; fused
 //                    epilogues: bias + GELU (forward), GELU' (backward), FP32
 //                    atomic accumulation (weight gradients, split over K)
@@ -43,6 +43,13 @@ __device__ __forceinline__ float gelu_df(float z) {
            z * expf(-0.5f * z * z) * 0.39894228040143268f;
 }
 
+// Columns of a block.  The GEMMs of a batch are bound by their epilogues, which
+// 64 columns left to 128 CTAs of four warps on 152 SMs; 32 columns and rows
+// stored 16 bytes a lane: forward 15.6 to 8.3 us a GEMM of 4,096 rows, the
+// gradient through GELU' 21.6 to 10.1, the weight gradients (16-byte additions)
+// 8.2 to 6.9.
+constexpr int NT = 32;
+
 enum { EPI_Z_GELU = 0, EPI_DGELU = 1, EPI_ATOMIC = 2 };
 
 struct Epi {
@@ -59,7 +66,7 @@ struct Epi {
 };
 
 // C[m0:m0+128, n0:n0+NT] = sum over this CTA's K range of A B^T.
-template <int NT, int EPI>
+template <int EPI>
 __global__ void __launch_bounds__(kGemmThreads)
     k_gemm(int M, int N, int K, int k_split, const bf16 *__restrict__ A, int lda,
            const bf16 *__restrict__ B, int ldb, Epi ep) {
@@ -76,7 +83,7 @@ __global__ void __launch_bounds__(kGemmThreads)
     const int kb0 = blockIdx.z * k_split;
     const int kb1 = min(K, kb0 + k_split);
     const int chunks = (kb1 - kb0) / 64;
-    if (warp == 0) tc::tmem_alloc(&tslot, NT < 32 ? 32 : NT);
+    if (warp == 0) tc::tmem_alloc(&tslot, NT);
     if (tid == 0) {
         tc::mbar_init(&mbar[0], 1);
         tc::mbar_init(&mbar[1], 1);
@@ -89,8 +96,8 @@ __global__ void __launch_bounds__(kGemmThreads)
     const uint32_t idesc = tc::idesc_f16(128, NT, 1);
     // the next 64-column chunk of both operands is requested into registers
     // while the current one is multiplied (the weight gradients of a batch of
-    // 4,096 rows: 26 us a GEMM without, 8 with it and slices of 256 rows; the
-    // forward ones 19 and 15)
+    // 4,096 rows in blocks of 64 columns: 26 us a GEMM without, 8 with it and
+    // slices of 256 rows; the forward ones 19 and 15)
     constexpr int QA = 128 * 8 / kGemmThreads, QB = NT * 8 / kGemmThreads;
     uint4 ra[QA], rb[QB];
     auto fetch = [&](int i) {
@@ -109,6 +116,18 @@ __global__ void __launch_bounds__(kGemmThreads)
         }
     };
     if (chunks > 0) fetch(0);
+    // EPI_DGELU: the pre-activations of this block, requested ahead as well
+    constexpr int kRowQuads = 128 * NT / 4 / kGemmThreads;
+    float4 zq[kRowQuads];
+    if (EPI == EPI_DGELU) {
+#pragma unroll
+        for (int u = 0; u < kRowQuads; u++) {
+            const int q = tid + u * kGemmThreads, gr = m0 + (q >> 3);
+            zq[u] = gr < ep.rows ? *reinterpret_cast<const float4 *>(ep.Z + (size_t)gr * ep.ld + n0 +
+                                                                     4 * (q & 7))
+                                 : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    }
     for (int i = 0; i < chunks; i++) {
         const int s = i & 1;
         if (i >= 2 && !tc::mbar_wait(&mbar[s], (uint32_t)(((i - 2) >> 1) & 1), kGemmPolls))
@@ -147,97 +166,121 @@ __global__ void __launch_bounds__(kGemmThreads)
     if (!ok && lane == 0 && chunks > 0) atomicOr(ep.err, (unsigned)PXSNE_DEVERR_TIMEOUT);
     if (!ok && lane == 0) s_abort = 1;
     tc::fence_after();
-    // Epilogue, 32 columns at a time: each thread holds one row of the block
-    // (TMEM lane = row); values pass through shared memory (the operand
-    // stages are free now) so that row-major stores, loads and atomics are
-    // made by a warp along a row, coalesced.  Transposed stores go straight
-    // from the row's thread (consecutive rows, coalesced as well).
+    // Epilogue: each thread holds one row of the block (TMEM lane = row); values
+    // pass through shared memory (the operand stages are free now) so that
+    // row-major stores, loads and atomics run along the rows, 16 bytes a lane
+    // where N is the hidden width.  Transposed stores go straight from the row's
+    // thread (consecutive rows, coalesced as well).
     __syncthreads();
     ok = !s_abort;  // the same in every warp (the barriers below need it)
     if (ok) {
-        constexpr int SP = 33;  // padded row pitch: conflict-free both ways
+        constexpr int SP = 36;  // padded row pitch: conflict-free 16 bytes a lane both ways
         float *sZ = reinterpret_cast<float *>(smem);
         float *sH = sZ + 128 * SP;
         const int rl = 32 * warp + lane, row = m0 + rl;
         const bool rv = row < ep.rows;
-#pragma unroll 1
-        for (int cb = 0; cb < NT; cb += 32) {
-            const int colb = n0 + cb;
-            if (EPI == EPI_DGELU) {
-                // the pre-activations of this block, loaded along rows
-                for (int r = warp; r < 128; r += kGemmThreads / 32) {
-                    const int gr = m0 + r, gc = colb + lane;
-                    sZ[r * SP + lane] = (gr < ep.rows && gc < N) ? ep.Z[(size_t)gr * ep.ld + gc] : 0.f;
-                }
-                __syncthreads();
-            }
-            float v[32];
-            tc::tmem_ld32(tbase + ((uint32_t)(32 * warp) << 16) + (uint32_t)cb, v);
+        if (EPI == EPI_DGELU) {
 #pragma unroll
-            for (int j = 0; j < 32; j++) {
-                const int col = colb + j;
-                if (EPI == EPI_Z_GELU) {
-                    const float z = v[j] + (col < N ? ep.bias[col] : 0.f);
-                    const float h = gelu_f(z);
-                    sZ[rl * SP + j] = z;
-                    sH[rl * SP + j] = h;
-                    if (ep.HT && rv && col < N) ep.HT[(size_t)col * ep.ldT + row] = __float2bfloat16_rn(h);
-                } else if (EPI == EPI_DGELU) {
-                    const float g = v[j] * gelu_df(sZ[rl * SP + j]);
-                    sH[rl * SP + j] = g;
-                    if (ep.HT && rv && col < N) ep.HT[(size_t)col * ep.ldT + row] = __float2bfloat16_rn(g);
-                } else {
-                    sZ[rl * SP + j] = v[j];
-                }
+            for (int u = 0; u < kRowQuads; u++) {
+                const int q = tid + u * kGemmThreads;
+                *reinterpret_cast<float4 *>(sZ + (q >> 3) * SP + 4 * (q & 7)) = zq[u];
             }
             __syncthreads();
-            if (EPI == EPI_DGELU) {
-                // the bias gradient: a warp sums its rows of one column per lane
-                float t = 0.f;
-                for (int r = warp; r < 128 && m0 + r < ep.rows; r += kGemmThreads / 32)
-                    t += __bfloat162float(__float2bfloat16_rn(sH[r * SP + lane]));
-                if (colb + lane < N) atomicAdd(ep.colsum + colb + lane, t);
-            }
-            for (int r = warp; r < 128; r += kGemmThreads / 32) {
-                const int gr = m0 + r, gc = colb + lane;
-                if (gr >= ep.rows || gc >= N) continue;
-                const size_t o = (size_t)gr * ep.ld + gc;
+        }
+        float v[32];
+        tc::tmem_ld32(tbase + ((uint32_t)(32 * warp) << 16), v);
+        if (EPI == EPI_ATOMIC) {
+#pragma unroll
+            for (int j = 0; j < 32; j += 4)
+                *reinterpret_cast<float4 *>(sZ + rl * SP + j) =
+                    make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+        } else {
+#pragma unroll
+            for (int j = 0; j < 32; j += 4) {
+                float4 *pz = reinterpret_cast<float4 *>(sZ + rl * SP + j);
+                float4 h;
                 if (EPI == EPI_Z_GELU) {
-                    ep.Z[o] = sZ[r * SP + lane];
-                    if (ep.H) ep.H[o] = __float2bfloat16_rn(sH[r * SP + lane]);
-                } else if (EPI == EPI_DGELU) {
-                    if (ep.H) ep.H[o] = __float2bfloat16_rn(sH[r * SP + lane]);
+                    const float4 bq = __ldg(reinterpret_cast<const float4 *>(ep.bias + n0 + j));
+                    const float4 z = make_float4(v[j] + bq.x, v[j + 1] + bq.y, v[j + 2] + bq.z,
+                                                 v[j + 3] + bq.w);
+                    *pz = z;
+                    h = make_float4(gelu_f(z.x), gelu_f(z.y), gelu_f(z.z), gelu_f(z.w));
                 } else {
-                    atomicAdd(ep.acc + o, sZ[r * SP + lane]);
+                    const float4 z = *pz;
+                    h = make_float4(v[j] * gelu_df(z.x), v[j + 1] * gelu_df(z.y),
+                                    v[j + 2] * gelu_df(z.z), v[j + 3] * gelu_df(z.w));
+                }
+                *reinterpret_cast<float4 *>(sH + rl * SP + j) = h;
+                if (ep.HT && rv) {
+                    bf16 *t = ep.HT + (size_t)(n0 + j) * ep.ldT + row;
+                    t[0] = __float2bfloat16_rn(h.x);
+                    t[ep.ldT] = __float2bfloat16_rn(h.y);
+                    t[2 * ep.ldT] = __float2bfloat16_rn(h.z);
+                    t[3 * ep.ldT] = __float2bfloat16_rn(h.w);
                 }
             }
-            __syncthreads();
+        }
+        __syncthreads();
+        if (EPI == EPI_DGELU) {
+            // the bias gradient: a warp sums its rows of one column per lane
+            float t = 0.f;
+            for (int r = warp; r < 128 && m0 + r < ep.rows; r += kGemmThreads / 32)
+                t += __bfloat162float(__float2bfloat16_rn(sH[r * SP + lane]));
+            atomicAdd(ep.colsum + n0 + lane, t);
+        }
+        if (EPI == EPI_ATOMIC && (N & 3) == 0 && (ep.ld & 3) == 0) {
+#pragma unroll
+            for (int u = 0; u < kRowQuads; u++) {
+                const int q = tid + u * kGemmThreads, r = q >> 3, c = 4 * (q & 7);
+                if (m0 + r < ep.rows && n0 + c < N)
+                    atomicAdd(reinterpret_cast<float4 *>(ep.acc + (size_t)(m0 + r) * ep.ld + n0 + c),
+                              *reinterpret_cast<const float4 *>(sZ + r * SP + c));
+            }
+        } else if (EPI == EPI_ATOMIC) {
+            const int gc = n0 + lane;
+            for (int r = warp; r < 128 && m0 + r < ep.rows; r += kGemmThreads / 32)
+                if (gc < N) atomicAdd(ep.acc + (size_t)(m0 + r) * ep.ld + gc, sZ[r * SP + lane]);
+        } else {
+#pragma unroll
+            for (int u = 0; u < kRowQuads; u++) {
+                const int q = tid + u * kGemmThreads, r = q >> 3, c = 4 * (q & 7);
+                if (m0 + r >= ep.rows) continue;
+                const size_t o = (size_t)(m0 + r) * ep.ld + n0 + c;
+                if (EPI == EPI_Z_GELU)
+                    *reinterpret_cast<float4 *>(ep.Z + o) =
+                        *reinterpret_cast<const float4 *>(sZ + r * SP + c);
+                const float4 h = *reinterpret_cast<const float4 *>(sH + r * SP + c);
+                __align__(8) bf16 hb[4] = {__float2bfloat16_rn(h.x), __float2bfloat16_rn(h.y),
+                                           __float2bfloat16_rn(h.z), __float2bfloat16_rn(h.w)};
+                *reinterpret_cast<uint2 *>(ep.H + o) = *reinterpret_cast<const uint2 *>(hb);
+            }
         }
     }
     tc::fence_before();
     __syncthreads();
-    if (warp == 0) tc::tmem_dealloc(tbase, NT < 32 ? 32 : NT);
+    if (warp == 0) tc::tmem_dealloc(tbase, NT);
 }
 
-template <int NT, int EPI>
+template <int EPI>
 cudaError_t gemm(cudaStream_t st, int M, int N, int K, int k_split, const bf16 *A, int lda,
                  const bf16 *B, int ldb, const Epi &ep) {
     const size_t smem = 2 * (128 * 128 + NT * 128) + 1024;
-    cudaError_t e = cudaFuncSetAttribute(k_gemm<NT, EPI>,
+    cudaError_t e = cudaFuncSetAttribute(k_gemm<EPI>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e) return e;
     const dim3 g((M + 127) / 128, (N + NT - 1) / NT, (K + k_split - 1) / k_split);
-    k_gemm<NT, EPI><<<g, kGemmThreads, smem, st>>>(M, N, K, k_split, A, lda, B, ldb, ep);
+    k_gemm<EPI><<<g, kGemmThreads, smem, st>>>(M, N, K, k_split, A, lda, B, ldb, ep);
     return cudaGetLastError();
 }
 
-// Output layer: a CTA takes 32 consecutive rows of the batch, a warp 4 of
+// Output layer: a CTA takes 16 consecutive rows of the batch, a warp 2 of
 // them, a lane 8 of the 256 hidden units of a row (16-byte loads and stores).
 // With targets: loss (sum of squared errors / m), dy = 2 (y - t) / m,
 // dz2 = (W3^T dy) * GELU'(z2), row-major and transposed (the transposed copy
 // is staged in shared memory and written 8 rows per 16-byte store), and
 // dL/dW3, dL/db3 and dL/db2 accumulated per CTA and added atomically.
-constexpr int kOutRows = 32;
+// (32 rows a CTA, 128 of them for 4,096 rows: 10.6 us; 16: 8.4.)
+constexpr int kOutRows = 16;
 __global__ void __launch_bounds__(256)
     k_out_layer(int m, int rows_pad, const bf16 *__restrict__ H2, const float *__restrict__ Z2,
                 const bf16 *__restrict__ W3, const float *__restrict__ b3,
@@ -315,7 +358,7 @@ __global__ void __launch_bounds__(256)
     }
     if (!T) return;
     __syncthreads();
-    // transposed copy: thread c writes unit c of the CTA's 32 rows, 8 rows per
+    // transposed copy: thread c writes unit c of the CTA's rows, 8 rows per
     // 16-byte store
     {
         const int c = threadIdx.x;
@@ -334,7 +377,7 @@ __global__ void __launch_bounds__(256)
         atomicAdd(&gb2[c], t);
     }
     // the warps' sums meet in shared memory first: 512 atomics per CTA on the
-    // same addresses instead of 4,096 (82 us a batch of 4,096 rows, 11 now)
+    // same addresses instead of 4,096 (82 us a batch of 4,096 rows, then 11)
 #pragma unroll
     for (int o = 0; o < 2; o++)
 #pragma unroll
@@ -767,13 +810,13 @@ int forward_backward(pxsne_mlp *M, int m, bool train) {
     e.Z = M->Z1;
     e.H = M->H1;
     e.HT = train ? M->H1T : nullptr;
-    MCK(M, (gemm<64, EPI_Z_GELU>(st, rp, kH, M->dp, M->dp, M->Xb, M->dp, M->W1b, M->dp, e)));
+    MCK(M, (gemm<EPI_Z_GELU>(st, rp, kH, M->dp, M->dp, M->Xb, M->dp, M->W1b, M->dp, e)));
     // layer 2
     e.bias = M->w + L.b2;
     e.Z = M->Z2;
     e.H = M->H2;
     e.HT = nullptr;
-    MCK(M, (gemm<64, EPI_Z_GELU>(st, rp, kH, kH, kH, M->H1, kH, M->W2b, kH, e)));
+    MCK(M, (gemm<EPI_Z_GELU>(st, rp, kH, kH, kH, M->H1, kH, M->W2b, kH, e)));
     // output layer (+ loss, dW3, db3, dZ2)
     const int ob = (rp + kOutRows - 1) / kOutRows;
     k_out_layer<<<ob, 256, 0, st>>>(m, rp, M->H2, M->Z2, M->W3b, M->w + L.b3,
@@ -781,13 +824,13 @@ int forward_backward(pxsne_mlp *M, int m, bool train) {
                                     M->g + L.W3, M->g + L.b3, M->g + L.b2, M->loss);
     MCK(M, cudaGetLastError());
     if (!train) return PXSNE_OK;
-    // dW2 = dZ2^T H1 (K = batch rows, split in 1024-row slices)
+    // dW2 = dZ2^T H1 (K = batch rows, split in slices of kSplitK)
     Epi a{};
     a.err = M->derr;
     a.ld = kH;
     a.rows = kH;
     a.acc = M->g + L.W2;
-    MCK(M, (gemm<64, EPI_ATOMIC>(st, kH, kH, rp, kSplitK, M->dZ2T, rp, M->H1T, rp, a)));
+    MCK(M, (gemm<EPI_ATOMIC>(st, kH, kH, rp, kSplitK, M->dZ2T, rp, M->H1T, rp, a)));
     // dZ1 = (dZ2 W2) * GELU'(Z1)
     Epi b{};
     b.err = M->derr;
@@ -798,11 +841,11 @@ int forward_backward(pxsne_mlp *M, int m, bool train) {
     b.H = M->dZ1;
     b.HT = M->dZ1T;
     b.colsum = M->g + L.b1;
-    MCK(M, (gemm<64, EPI_DGELU>(st, rp, kH, kH, kH, M->dZ2, kH, M->W2Tb, kH, b)));
+    MCK(M, (gemm<EPI_DGELU>(st, rp, kH, kH, kH, M->dZ2, kH, M->W2Tb, kH, b)));
     // dW1 = dZ1^T X
     a.ld = M->d;
     a.acc = M->g + L.W1;
-    MCK(M, (gemm<64, EPI_ATOMIC>(st, kH, M->d, rp, kSplitK, M->dZ1T, rp, M->XT, rp, a)));
+    MCK(M, (gemm<EPI_ATOMIC>(st, kH, M->d, rp, kSplitK, M->dZ1T, rp, M->XT, rp, a)));
     return PXSNE_OK;
 }
 

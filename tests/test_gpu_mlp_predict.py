@@ -50,3 +50,29 @@ def test_predict(n, d):
     net64 = oracle.MLP.from_flat(weights64(w, sizes), d, 256)
     _, ref, _ = oracle.mlp(net64, bf16(X[rows]))
     assert np.linalg.norm(host[rows] - ref) <= 1e-2 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("n,d", [(1, 3), (127, 64), (129, 65), (1000, 100), (4096, 50), (8192, 128)])
+def test_gradient_sizes(n, d):
+    """Loss and gradient where the last block of rows is ragged and where the
+    weight gradients' rows are and are not multiples of 16 bytes.  Four stored
+    tensors (h1, h2, dz2, dz1) lie between the input and W1's gradient, each
+    rounded by at most 2^-9 of an element: 0.8 %, the bar is 1 %."""
+    import paper_1611_02568_gb300 as px
+    from paper_1611_02568_gb300 import build
+    build.build()
+    rng = np.random.default_rng([n, d, 1])
+    X = bf16(0.5 * rng.standard_normal((n, d)))
+    T = rng.standard_normal((n, 2)).astype(np.float32)
+    with px.MLP(d, seed=2) as net:
+        w = bf16(net.get_params())
+        net.set_params(w)
+        loss, g = net.loss_grad(X, T)
+    ref = oracle.MLP.from_flat(w.astype(np.float64), d, 256)
+    loss_o, _, g_o = oracle.mlp(ref, X, T, grad=True)
+    assert abs(loss - loss_o) <= 1e-2 * loss_o
+    go = oracle.MLP.from_flat(g_o, d, 256)
+    gg = oracle.MLP.from_flat(g.astype(np.float64), d, 256)
+    for name in ("W1", "b1", "W2", "b2", "W3", "b3"):
+        a, b = getattr(gg, name), getattr(go, name)
+        assert np.linalg.norm(a - b) <= 1e-2 * np.linalg.norm(b), name
