@@ -256,7 +256,7 @@ int prime(pxsne_ctx *c) {
     k_iota<<<(n + 255) / 256, 256, 0, c->stream>>>(n, c->perm);
     CK(c, cudaGetLastError());
     CK(c, launch_tree(c, false));
-    // a state set from outside: P relabelled for its Morton order before the
+    // a state set from outside: P relabelled for its tree order before the
     // first attraction
     CK(c, launch_relabel(c, c->stream));
     c->since_relabel = 0;
@@ -265,7 +265,7 @@ int prime(pxsne_ctx *c) {
     return PXSNE_OK;
 }
 
-// The attraction's relabelled copy of P follows the Morton order of the last
+// The attraction's relabelled copy of P follows the tree order of the last
 // tree; it is refreshed every kRelabelEvery iterations (before the update).
 cudaError_t relabel_if_due(pxsne_ctx *c) {
     if (is3(c) || c->since_relabel < kRelabelEvery) return cudaSuccess;

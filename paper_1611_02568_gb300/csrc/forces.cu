@@ -1,7 +1,7 @@
 // Forces of the PixelSNE gradient (Eq. grad) on the pixel-aligned tree.
 //
 //   k_bh_traverse  repulsion by Barnes-Hut (Sec. 3.3, Eq. bh_criteria) on the
-//                  dense pyramid, one warp per 32 points of the Morton order
+//                  dense pyramid, one warp per 32 points in tree order
 //                  (64 with geometric centres), the siblings as packed FP32
 //                  pairs; each point keeps its own accept/open decisions (lane
 //                  masks per stack entry), so it sees exactly the cells its
@@ -17,7 +17,7 @@
 
 namespace pxsne {
 
-// One warp = 32 PPL points consecutive in Morton order, PPL (1 or 2) per lane.
+// One warp = 32 PPL points consecutive in tree order, PPL (1 or 2) per lane.
 // Each stack
 // entry is a node whose four children are to be tested, with the mask of the
 // lanes whose point opened it, so every point sees exactly the cells its own
@@ -89,7 +89,7 @@ __device__ __forceinline__ float lo_bits(uint32_t v) {
 // Eq. grad, first term: Fattr_i = sum_j p_ij w_ij (y_i - y_j), one warp per
 // row (row lengths vary with the in-degree of the kNN graph; a warp per row
 // keeps long rows from stalling short ones).  It runs over the relabelled copy
-// of P (rows and columns in the Morton order of a recent state), so a row's
+// of P (rows and columns in the tree order of a recent state), so a row's
 // gathered positions zp[j] lie close together in memory, and writes each row's
 // force back under the point's own index.  Each lane keeps four entries in
 // flight; P is streamed with evict-first loads so that the positions stay in
@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(kTravWarps * 32, PPL == 1 ? 4 : 3)
     const unsigned before = (1u << lane) - 1u;
     uint32_t n_acc = 0u, n_tst = 0u, n_stp = 0u, n_nod = 0u;
     TravEntry<PPL> *stk = s_stk[w];
-    // Each warp takes the next 32 PPL points of the Morton order until none are
+    // Each warp takes the next 32 PPL points of the tree order until none are
     // left: a warp whose points are cheap moves on instead of idling until
     // the slowest warp of its CTA is done.
     for (;;) {
@@ -669,7 +669,7 @@ __global__ void __launch_bounds__(256)
     }
 }
 
-// Relabelling: new label r is the point perm[r] (Morton order of the last
+// Relabelling: new label r is the point perm[r] (tree order of the last
 // tree).  Maps, padded row lengths under the new labels, and the positions.
 __global__ void k_relabel_maps(int n, const uint32_t *__restrict__ perm,
                                const int64_t *__restrict__ rp, const uint2 *__restrict__ z,

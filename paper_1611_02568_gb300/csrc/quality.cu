@@ -2,7 +2,7 @@
 // with N_D^k(i) the first k high-dimensional neighbours of point i and
 // N_d^k(i) its k nearest neighbours in the 2-D embedding.
 //
-// k_nbr_precision  one warp per point (in Morton order): exact 2-D k nearest
+// k_nbr_precision  one warp per point (in tree order): exact 2-D k nearest
 //                  neighbours by a ring search over the cells of one level of the
 //                  current tree (the points of a cell are contiguous in the
 //                  counting-sort permutation); squared distances in FP64 with
@@ -20,6 +20,17 @@ __device__ __forceinline__ double d2_fp64(uint2 a, uint2 b, double s0, double s1
     const double dx = __dmul_rn(s0, (double)((int64_t)a.x - (int64_t)b.x));
     const double dy = __dmul_rn(s1, (double)((int64_t)a.y - (int64_t)b.y));
     return __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy));
+}
+
+// The state of the Hilbert curve two levels below a cell of state s, for each of
+// the 16 pairs of Morton digits, two bits each.
+constexpr uint32_t hil_next2(uint32_t s) {
+    uint32_t w = 0u;
+    for (uint32_t q = 0u; q < 16u; q++) {
+        const uint32_t t = hil_child(s, hil_pos(s, q >> 2));
+        w |= hil_child(t, hil_pos(t, q & 3u)) << (2u * q);
+    }
+    return w;
 }
 
 // The search runs on level l0 of the tree (2^l0 cells per axis, about one point
@@ -40,6 +51,16 @@ __global__ void __launch_bounds__(kPrecWarps * 32)
                     int kh, const DevScalars *__restrict__ sc, int32_t *__restrict__ hits,
                     unsigned long long *total) {
     __shared__ unsigned s_hits[kPrecWarps];
+    __shared__ uint32_t s_next[4];
+    if (threadIdx.x == 0) {
+        constexpr uint32_t k0 = hil_next2(0u), k1 = hil_next2(1u), k2 = hil_next2(2u),
+                           k3 = hil_next2(3u);
+        s_next[0] = k0;
+        s_next[1] = k1;
+        s_next[2] = k2;
+        s_next[3] = k3;
+    }
+    __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int t = blockIdx.x * kPrecWarps + warp;
     unsigned h = 0u;
@@ -52,6 +73,7 @@ __global__ void __launch_bounds__(kPrecWarps * 32)
         const float *cell_n = recn + rec_offset(l);
         const int F = 32 - l, R = 1 << l, up = 2 * (L - l);
         const int px = (int)(zi.x >> F), py = (int)(zi.y >> F);
+        const bool hil = hil_order(L);
         const double s0 = sc->s[0], s1 = sc->s[1];
         // smallest cell side in y-units
         const double w = ldexp(s0 < s1 ? s0 : s1, F);
@@ -79,7 +101,22 @@ __global__ void __launch_bounds__(kPrecWarps * 32)
                         const uint32_t m = morton2((uint32_t)x, (uint32_t)y);
                         cnt = (uint32_t)cell_n[m];  // (exact float)
                         if (cnt != 0u) {
-                            const uint32_t first = m << up;
+                            uint32_t first = m << up;
+                            // along the curve the first leaf of a cell is its first
+                            // or, where the state's bit 1 is set, its last one
+                            if (hil) {
+                                uint32_t s = 0u;
+                                int b = 2 * l;
+                                if (l & 1) {
+                                    b -= 2;
+                                    s = hil_child(0u, hil_pos(0u, m >> b));
+                                }
+                                while (b > 0) {
+                                    b -= 4;
+                                    s = (s_next[s] >> (2u * ((m >> b) & 15u))) & 3u;
+                                }
+                                if (s & 2u) first += (1u << up) - 1u;
+                            }
                             start = blk_off[first >> (2 * K1)] + leaf_start[first];
                         }
                     }

@@ -70,7 +70,7 @@ __global__ void k_snap_hist(int n, int L, int rescale, float theta, u64 Rx, u64 
         sc->n_steps = 0ull;
         sc->n_nodes = 0ull;
     }
-    // Points arrive in the Morton order of a recent state, so lanes with equal
+    // Points arrive in the tree order of a recent state, so lanes with equal
     // leaf keys mostly form runs: each run adds its count and sums with one
     // set of atomics (segmented shuffle scan), and each lane's rank inside its
     // pixel is the run's base plus its position in the run.
@@ -296,7 +296,7 @@ __global__ void __launch_bounds__(1 << (2 * (K - 1)))
 // cell, 16 lanes a level-(h-3) cell, two warps a level-(h-4) cell and the CTA
 // one level-(h-5) cell.  It writes the records of levels h .. h-4, the sums of
 // level h-5 and, per CTA, the exclusive scan of the leaf counts (local start of
-// each pixel in Morton order).  With fuse_top the last CTA to finish also does
+// each pixel in tree order).  With fuse_top the last CTA to finish also does
 // the rest of the pyramid (pyr_top).
 __device__ __forceinline__ u64 shfl_xor_u64(u64 v, int o) {
     return __shfl_xor_sync(0xffffffffu, v, o);
@@ -325,39 +325,42 @@ __device__ __forceinline__ void sum_group(const uint32_t *c, const u64 *x, const
 }
 
 // The last CTA's share for 256 cells of level h0 and more (h0 >= 4): a thread
-// adds up its run of cells level by level down to one cell of level 4, and the
+// adds up its cells level by level down to one cell of level 4, taken in the
+// order of the Hilbert curve (hil_order holds wherever this runs), and the
 // levels above follow by shuffles, so that the cells are read once instead of
 // every level through global memory.  Bound by the chain of dependent loads and
 // barriers (one CTA): the pyramid's launch takes 14 us instead of 19 for a
-// 2048^2 screen and 54 instead of 61 for 4096^2 (n = 70,000 and 1M).
+// 1024^2 screen (n = 70,000).
 __device__ void pyr_top_wide(int h0, const uint32_t *c0, const u64 *x0, const u64 *y0, float4 *rec,
                              float *recn, uint32_t *blk_off, uint32_t *s_warp, uint32_t *s_n,
                              u64 *s_x, u64 *s_y) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const bool sums = rec != nullptr;
     const int seg = (1 << (2 * h0)) >> 8;  // 1, 4, 16 or 64 cells per thread
+    uint32_t state = 0u;
+    const int g = (int)hil_morton((uint32_t)tid, 4, state);  // the thread's cell of level 4
     uint32_t N = 0u;
     u64 X = 0ull, Y = 0ull;
     if (seg == 1) {
-        N = __ldcg(c0 + tid);
+        N = __ldcg(c0 + g);
         if (sums) {
-            X = __ldcg(x0 + tid);
-            Y = __ldcg(y0 + tid);
+            X = __ldcg(x0 + g);
+            Y = __ldcg(y0 + g);
         }
     } else if (seg == 4) {
-        sum_group(c0, x0, y0, tid, sums, N, X, Y);
-        put_record(rec, recn, h0 - 1, (uint32_t)tid, N, X, Y);
+        sum_group(c0, x0, y0, g, sums, N, X, Y);
+        put_record(rec, recn, h0 - 1, (uint32_t)g, N, X, Y);
     } else {
         for (int q = 0; q < seg / 16; q++) {
             uint32_t n2 = 0u;
             u64 x2 = 0ull, y2 = 0ull;
-            const int at = tid * (seg / 16) + q;  // cell of level h0 - 2
+            const int at = g * (seg / 16) + q;  // cell of level h0 - 2
 #pragma unroll
-            for (int g = 0; g < 4; g++) {
+            for (int k = 0; k < 4; k++) {
                 uint32_t n1;
                 u64 x1, y1;
-                sum_group(c0, x0, y0, 4 * at + g, sums, n1, x1, y1);
-                put_record(rec, recn, h0 - 1, (uint32_t)(4 * at + g), n1, x1, y1);
+                sum_group(c0, x0, y0, 4 * at + k, sums, n1, x1, y1);
+                put_record(rec, recn, h0 - 1, (uint32_t)(4 * at + k), n1, x1, y1);
                 n2 += n1;
                 x2 += x1;
                 y2 += y1;
@@ -367,22 +370,20 @@ __device__ void pyr_top_wide(int h0, const uint32_t *c0, const u64 *x0, const u6
             X += x2;
             Y += y2;
         }
-        if (seg == 64) put_record(rec, recn, h0 - 3, (uint32_t)tid, N, X, Y);
+        if (seg == 64) put_record(rec, recn, h0 - 3, (uint32_t)g, N, X, Y);
     }
-    // the pixel starts of the first pass's CTAs
+    // the pixel starts of the first pass's CTAs, along the curve
     uint32_t run = block_excl_scan(N, 256, s_warp);
     if (seg == 1) {
-        blk_off[tid] = run;
+        blk_off[g] = run;
     } else {
-        for (int i = tid * seg; i < (tid + 1) * seg; i += 4) {
-            const uint4 q = __ldcg(reinterpret_cast<const uint4 *>(c0 + i));
-            uint4 o;
-            o.x = run;
-            o.y = o.x + q.x;
-            o.z = o.y + q.y;
-            o.w = o.z + q.z;
-            run = o.w + q.w;
-            *reinterpret_cast<uint4 *>(blk_off + i) = o;
+        for (int i = 0; i < seg / 4; i++) {
+            uint32_t st = state;
+            const uint32_t at =
+                (uint32_t)(g * (seg / 4)) + hil_morton((uint32_t)i, seg == 4 ? 0 : seg == 16 ? 1 : 2, st);
+            const uint4 q = __ldcg(reinterpret_cast<const uint4 *>(c0) + at);
+            reinterpret_cast<uint4 *>(blk_off)[at] = hil_starts(st, q, run);
+            run += q.x + q.y + q.z + q.w;
         }
     }
     // levels 3 (4 threads) and 2 (16), then 1 and 0 across the warps
@@ -391,8 +392,8 @@ __device__ void pyr_top_wide(int h0, const uint32_t *c0, const u64 *x0, const u6
         N += __shfl_xor_sync(0xffffffffu, N, o);
         X += __shfl_xor_sync(0xffffffffu, X, o);
         Y += __shfl_xor_sync(0xffffffffu, Y, o);
-        if (o == 2 && (lane & 3) == 0) put_record(rec, recn, 3, (uint32_t)(tid >> 2), N, X, Y);
-        if (o == 8 && (lane & 15) == 0) put_record(rec, recn, 2, (uint32_t)(tid >> 4), N, X, Y);
+        if (o == 2 && (lane & 3) == 0) put_record(rec, recn, 3, (uint32_t)(g >> 2), N, X, Y);
+        if (o == 8 && (lane & 15) == 0) put_record(rec, recn, 2, (uint32_t)(g >> 4), N, X, Y);
     }
     __syncthreads();
     if (lane == 0) {
@@ -402,7 +403,7 @@ __device__ void pyr_top_wide(int h0, const uint32_t *c0, const u64 *x0, const u6
     }
     __syncthreads();
     if (tid < 4)
-        put_record(rec, recn, 1, (uint32_t)tid, s_n[2 * tid] + s_n[2 * tid + 1],
+        put_record(rec, recn, 1, hil_quad(0u, (uint32_t)tid), s_n[2 * tid] + s_n[2 * tid + 1],
                    s_x[2 * tid] + s_x[2 * tid + 1], s_y[2 * tid] + s_y[2 * tid + 1]);
     if (tid == 4) {
         uint32_t n = 0u;
@@ -475,7 +476,12 @@ __global__ void __launch_bounds__(256)
     __shared__ bool s_last;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t b = blockIdx.x;
-    const uint32_t cell0 = b * 1024u + 4u * (uint32_t)tid;
+    // the thread's cell of level h - 1: along the Hilbert curve, or in Morton order
+    const bool hil = hil_order(h);
+    const uint32_t bstate = hil ? hil_state(b, h - 5) : 0u;
+    uint32_t state = bstate;
+    const uint32_t g = hil ? hil_morton((uint32_t)tid, 4, state) : (uint32_t)tid;
+    const uint32_t cell0 = b * 1024u + 4u * g;
     // rec == NULL: a count-only tree (geometric centres), no sums read or kept
     const bool sums = rec != nullptr;
     const uint4 c4 = reinterpret_cast<const uint4 *>(in_cnt)[cell0 >> 2];
@@ -505,7 +511,7 @@ __global__ void __launch_bounds__(256)
         const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o);
         if (lane >= o) inc += t;
     }
-    put_record(rec, recn, h - 1, b * 256u + (uint32_t)tid, N, X, Y);
+    put_record(rec, recn, h - 1, b * 256u + g, N, X, Y);
     // levels h-2 (4 lanes) and h-3 (16 lanes)
 #pragma unroll
     for (int o = 1; o <= 2; o <<= 1) {
@@ -515,7 +521,7 @@ __global__ void __launch_bounds__(256)
             Y += shfl_xor_u64(Y, o);
         }
     }
-    if ((lane & 3) == 0) put_record(rec, recn, h - 2, b * 64u + (uint32_t)(tid >> 2), N, X, Y);
+    if ((lane & 3) == 0) put_record(rec, recn, h - 2, b * 64u + (g >> 2), N, X, Y);
 #pragma unroll
     for (int o = 4; o <= 8; o <<= 1) {
         N += __shfl_xor_sync(0xffffffffu, N, o);
@@ -524,7 +530,7 @@ __global__ void __launch_bounds__(256)
             Y += shfl_xor_u64(Y, o);
         }
     }
-    if ((lane & 15) == 0) put_record(rec, recn, h - 3, b * 16u + (uint32_t)(tid >> 4), N, X, Y);
+    if ((lane & 15) == 0) put_record(rec, recn, h - 3, b * 16u + (g >> 4), N, X, Y);
     N += __shfl_xor_sync(0xffffffffu, N, 16);
     if (sums) {
         X += shfl_xor_u64(X, 16);
@@ -541,15 +547,21 @@ __global__ void __launch_bounds__(256)
     for (int w = 0; w < warp; w++) before += s_n[w];
     const uint32_t e0 = before + inc - (c4.x + c4.y + c4.z + c4.w);
     uint4 st;
-    st.x = e0;
-    st.y = e0 + c4.x;
-    st.z = st.y + c4.y;
-    st.w = st.z + c4.z;
+    if (hil) {
+        st = hil_starts(state, c4, e0);
+    } else {
+        st.x = e0;
+        st.y = e0 + c4.x;
+        st.z = st.y + c4.y;
+        st.w = st.z + c4.z;
+    }
     reinterpret_cast<uint4 *>(leaf_start)[cell0 >> 2] = st;
     // level h-4: pairs of warps; level h-5: the CTA
-    if (tid < 4)
-        put_record(rec, recn, h - 4, b * 4u + (uint32_t)tid, s_n[2 * tid] + s_n[2 * tid + 1],
+    if (tid < 4) {
+        const uint32_t q = hil ? hil_quad(bstate, (uint32_t)tid) : (uint32_t)tid;
+        put_record(rec, recn, h - 4, b * 4u + q, s_n[2 * tid] + s_n[2 * tid + 1],
                    s_x[2 * tid] + s_x[2 * tid + 1], s_y[2 * tid] + s_y[2 * tid + 1]);
+    }
     if (tid == 0) {
         uint32_t n5 = 0u;
         u64 x5 = 0ull, y5 = 0ull;
@@ -572,7 +584,7 @@ __global__ void __launch_bounds__(256)
     __syncthreads();
     if (!s_last) return;
     __threadfence();
-    if (h >= 9)
+    if (hil)
         pyr_top_wide(h - 5, out_cnt, out_sx, out_sy, rec, recn, blk_off, s_warp, s_n, s_x, s_y);
     else
         pyr_top(h - 5, out_cnt, out_sx, out_sy, scr_cnt, scr_sx, scr_sy, rec, recn, blk_off, s_warp);

@@ -174,3 +174,10 @@ def test_upper_levels_sums_and_rows(n, level, centre):
     assert rel(Zi[rows], oZi) <= FORCE_TOL
     assert rel(Fattr, oA) <= FORCE_TOL
     assert abs(Z - Zi.astype(np.float64).sum()) <= 1e-12 * Z
+
+
+@pytest.mark.parametrize("n,level,k", [(3000, 10, 5), (3000, 12, 5), (9000, 10, 10)])
+def test_cells_along_the_curve(n, level, k):
+    """The first point of a cell on the screens whose points follow the Hilbert
+    curve, for cells of even and odd levels."""
+    test_nbr_precision_on_uneven_states(n, level, k)
