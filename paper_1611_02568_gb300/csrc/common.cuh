@@ -17,7 +17,7 @@ typedef long long i64;
 
 constexpr int kMaxL = 14;           // screen up to 2^14 x 2^14 (Morton keys < 2^28)
 constexpr int64_t kMaxN = 1 << 24;  // cell counts are exact floats below 2^24
-constexpr int kTravWarps = 8;       // warps per CTA in the traversal
+constexpr int kTravWarps = 2;       // warps per CTA in the traversal
 constexpr int kTravStack = 48;      // entries per warp; depth <= 3L - 2 <= 40
 // The traversal's kernel by the number of points (late states of 10- and
 // 100-component mixtures, us per iteration).  Below kTravPointTo one warp per
@@ -29,16 +29,21 @@ constexpr int kTravStack = 48;      // entries per warp; depth <= 3L - 2 <= 40
 // of mass cost the gain back: 28.8 against 27.7 ms for 20 iterations at 1M).
 constexpr int64_t kTravPointTo = 32768;
 constexpr int64_t kTravPairFrom = 150000;
-// Persistent grids of the forces: CTAs per SM of the traversal (one and two
-// points per lane) and of the attraction that runs beside it on the side
-// stream.  The traversal leaves registers for the attraction's CTAs from the
-// start: 20 iterations at n = 1M take 29.6, 27.7 and 30.0 ms with 2, 3 and 4
-// traversal CTAs (two points per lane, geometric centres at 300,000, ten
-// iterations: 4.79 ms with two, 4.74 with three, but 5.74 against 6.12 at
-// 400,000), 27.9 with four of the attraction's CTAs instead of five.
-constexpr int kTravCtasPerSm = 3;
-constexpr int kTravPairCtasPerSm = 2;
-constexpr int kAttCtasPerSm = 5;
+// Persistent grids of the forces: CTAs per SM of the traversal and of the
+// attraction that runs beside it on the side stream.  They share the registers
+// (20 + 20 warps at 56 and 40) and the data pipe of L1, which each alone keeps
+// about 60 % busy, so the best split depends on which of the two is the longer:
+// the whole schedule of the 1M mixture (it/s; attraction 0.56, traversal 0.69 ms
+// alone) against a spread-out late state of 1M points (ms an iteration; 0.55 and
+// 1.13), by the traversal's warps per SM: 16: 822, 1.75; 20: 839, 1.58; 22: 827,
+// 1.54; 24: 808, 1.54.  (CTAs of two warps leave the registers between the two
+// grids in small pieces; 16 and 24 were CTAs of eight.  20 in CTAs of four: 837.)
+// Two points per lane with geometric centres take the same 20 warps (ten
+// iterations at 300,000: 4.64 ms; 16: 4.79); with centres of mass they would
+// bring the schedule to 866 at 16 warps, and the late state to 1.73.
+constexpr int kTravCtasPerSm = 10;
+constexpr int kAttWarps = 2;        // warps per CTA in the attraction
+constexpr int kAttCtasPerSm = 20;
 constexpr int kPyrK = 5;            // pyramid levels reduced per CTA pass
 
 // Scalars of the iteration that live on the device so that a captured graph

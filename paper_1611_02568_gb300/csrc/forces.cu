@@ -226,7 +226,7 @@ struct __align__(16) TravEntry<2> {
 };
 
 template <int CENTRE, int COUNT, bool OWN, int PPL>
-__global__ void __launch_bounds__(kTravWarps * 32, PPL == 1 ? 4 : 3)
+__global__ void __launch_bounds__(kTravWarps * 32, 16)
     k_bh_traverse(int n, int L, const uint2 *__restrict__ z, const uint32_t *__restrict__ perm,
                   const float4 *__restrict__ rec, const float *__restrict__ recn,
                   DevScalars *sc, float2 *__restrict__ Frep, float *__restrict__ Zi) {
@@ -766,8 +766,8 @@ template <int CENTRE, int COUNT, bool OWN, int PPL>
 static void traverse_as(pxsne_ctx *c, cudaStream_t st) {
     const int n = (int)c->n;
     const int per_block = kTravWarps * 32 * PPL;
-    const int ctas = PPL == 1 ? kTravCtasPerSm : kTravPairCtasPerSm;
-    const int blocks = std::min((n + per_block - 1) / per_block, ctas * std::max(c->sms, 1));
+    const int blocks =
+        std::min((n + per_block - 1) / per_block, kTravCtasPerSm * std::max(c->sms, 1));
     k_bh_traverse<CENTRE, COUNT, OWN, PPL><<<blocks, kTravWarps * 32, 0, st>>>(
         n, c->L, c->z, c->perm, c->rec, c->recn, c->sc, c->Frep, c->Zi);
 }
@@ -803,9 +803,11 @@ static cudaError_t traverse(pxsne_ctx *c, cudaStream_t st, bool count) {
 cudaError_t launch_attract(pxsne_ctx *c, cudaStream_t st) {
     const int n = (int)c->n;
     const int rows = n < kAttRowsFrom ? 1 : kAttRows;
-    const int need = (int)((int64_t(n) + 8 * rows - 1) / (8 * rows));
-    const int blocks = std::min(need, kAttCtasPerSm * std::max(c->sms, 1));
-    k_attract<<<blocks, 256, 0, st>>>(n, rows, attract_args(c), c->sc);
+    // (few rows: fewer and larger CTAs; no difference beyond noise at n = 2000)
+    const int warps = rows == 1 ? 8 : kAttWarps;
+    const int need = (int)((int64_t(n) + warps * rows - 1) / (warps * rows));
+    const int blocks = std::min(need, kAttCtasPerSm * kAttWarps / warps * std::max(c->sms, 1));
+    k_attract<<<blocks, warps * 32, 0, st>>>(n, rows, attract_args(c), c->sc);
     return cudaGetLastError();
 }
 
