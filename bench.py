@@ -188,7 +188,7 @@ def group_bytes(n, nnz, L, nonempty=None, occupied=None):
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) from an
 # ncu capture of the current kernels, by (workload, n); emptied whenever a
 # kernel changes, until the capture is taken again
-TRAFFIC_BYTES = {("gmm128", 1_000_000): {"k_bh_traverse": 45.49e6 + 2.10e6}}
+TRAFFIC_BYTES = {("gmm128", 1_000_000): {"k_bh_traverse": 36.42e6 + 1.82e6}}
 TRAFFIC_SOURCE = ("profiles/traversal_gmm128_n1M_dram.md (one-pass ncu capture of the "
                   "9th launch, t about 2)")
 
@@ -660,12 +660,15 @@ def run_gpu(args):
     kskip, kpairs = ctx.knn_pruning()
     # the products the tensor cores actually formed: the (query tile,
     # candidate tile) pairs of 128 x 128 rows not skipped by the tile bound,
-    # 2 * 128 * 128 * Dp FLOP each (rows padded to the tiles, D to Dp)
+    # 2 * 128 * 128 * Dp FLOP each (rows padded to the tiles, D to Dp); the time
+    # also holds the pass over the sample and the exact distances, and the rows
+    # kept are those within the search's threshold (heap insertions where the
+    # one-pass search k_knn_tc did a tile)
     Dp = (X.shape[1] + 63) // 64 * 64
     knn_dense = 2.0 * n * n * X.shape[1]
     knn_flop = (kpairs - kskip) * 2.0 * 128 * 128 * Dp if kpairs else knn_dense
     pk, pk_kind = measured_peaks()
-    knn = {"kernel": "k_knn_tc" if kpath == 1 else "k_knn_tile", "ms": knn_ms,
+    knn = {"kernel": "k_knn_scan" if kpath == 1 else "k_knn_tile", "ms": knn_ms,
            "bound": "tensor", "achieved": knn_flop / (knn_ms / 1e3) / 1e12,
            "peak": pk["bf16_tflops"], "unit": "TFLOP/s",
            "frac": knn_flop / (knn_ms / 1e3) / 1e12 / pk["bf16_tflops"],
