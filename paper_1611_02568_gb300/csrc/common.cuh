@@ -29,6 +29,17 @@ constexpr int kTravStack = 48;      // entries per warp; depth <= 3L - 2 <= 40
 // of mass cost the gain back: 28.8 against 27.7 ms for 20 iterations at 1M).
 constexpr int64_t kTravPointTo = 32768;
 constexpr int64_t kTravPairFrom = 150000;
+// Crowded screens (half a point per pixel and more, centres of mass): consecutive
+// points lie close together and the attraction takes as long as the traversal,
+// which then keeps to 16 warps per SM instead of 20, and from kTravCrowdedPair on
+// takes two points per lane (600 iterations of a 100-component mixture from its
+// start, it/s, 20 warps, 16 warps, 16 with two points per lane: 200,000 points
+// on 512^2 3,979, 4,150, 3,863; 400,000 2,271, 2,379, 2,353; 700,000 on 1024^2
+// 1,291, 1,316, 1,335; 1M on 512^2 964, 1,008, 1,025, on 1024^2 921, 941, 974).
+// Spread-out states of a sparse screen pay for it (1M on 2048^2: 1.58, 1.75 and
+// 1.73 ms an iteration).
+constexpr int64_t kTravCrowdedPair = 600000;
+inline bool trav_crowded(int64_t n, int L) { return 2 * n >= (int64_t(1) << (2 * L)); }
 // Persistent grids of the forces: CTAs per SM of the traversal and of the
 // attraction that runs beside it on the side stream.  They share the registers
 // (20 + 20 warps at 56 and 40) and the data pipe of L1, which each alone keeps
@@ -42,6 +53,7 @@ constexpr int64_t kTravPairFrom = 150000;
 // iterations at 300,000: 4.64 ms; 16: 4.79); with centres of mass they would
 // bring the schedule to 866 at 16 warps, and the late state to 1.73.
 constexpr int kTravCtasPerSm = 10;
+constexpr int kTravCrowdedCtasPerSm = 8;
 constexpr int kAttWarps = 2;        // warps per CTA in the attraction
 constexpr int kAttCtasPerSm = 20;
 constexpr int kPyrK = 5;            // pyramid levels reduced per CTA pass

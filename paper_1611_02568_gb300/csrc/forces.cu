@@ -766,8 +766,8 @@ template <int CENTRE, int COUNT, bool OWN, int PPL>
 static void traverse_as(pxsne_ctx *c, cudaStream_t st) {
     const int n = (int)c->n;
     const int per_block = kTravWarps * 32 * PPL;
-    const int blocks =
-        std::min((n + per_block - 1) / per_block, kTravCtasPerSm * std::max(c->sms, 1));
+    const int ctas = CENTRE == 0 && trav_crowded(n, c->L) ? kTravCrowdedCtasPerSm : kTravCtasPerSm;
+    const int blocks = std::min((n + per_block - 1) / per_block, ctas * std::max(c->sms, 1));
     k_bh_traverse<CENTRE, COUNT, OWN, PPL><<<blocks, kTravWarps * 32, 0, st>>>(
         n, c->L, c->z, c->perm, c->rec, c->recn, c->sc, c->Frep, c->Zi);
 }
@@ -779,10 +779,11 @@ static void traverse_n(pxsne_ctx *c, cudaStream_t st) {
         const int n = (int)c->n;
         k_bh_traverse_pt<CENTRE, COUNT, OWN><<<(n + kPtWarps - 1) / kPtWarps, kPtWarps * 32, 0, st>>>(
             n, c->L, c->z, c->perm, c->rec, c->recn, c->sc, c->Frep, c->Zi);
-    } else if (CENTRE == 0 || c->n < kTravPairFrom) {
-        traverse_as<CENTRE, COUNT, OWN, 1>(c, st);
+    } else if (CENTRE == 0 ? trav_crowded(c->n, c->L) && c->n >= kTravCrowdedPair
+                           : c->n >= kTravPairFrom) {
+        traverse_as<CENTRE, COUNT, OWN, 2>(c, st);
     } else {
-        traverse_as<CENTRE, COUNT, OWN, CENTRE == 0 ? 1 : 2>(c, st);
+        traverse_as<CENTRE, COUNT, OWN, 1>(c, st);
     }
 }
 

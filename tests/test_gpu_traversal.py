@@ -181,3 +181,24 @@ def test_cells_along_the_curve(n, level, k):
     """The first point of a cell on the screens whose points follow the Hilbert
     curve, for cells of even and odd levels."""
     test_nbr_precision_on_uneven_states(n, level, k)
+
+
+@pytest.mark.parametrize("n,level", [(599_999, 9), (600_000, 9), (600_001, 10), (600_001, 11)])
+def test_forces_on_crowded_screens(n, level):
+    """Two points per lane and one on both sides of the rule between them
+    (600,000 points, half a point per pixel)."""
+    import paper_1611_02568_gb300 as px
+    from paper_1611_02568_gb300 import build
+    build.build()
+    z, s = state(n, 13)
+    rng = np.random.default_rng(3)
+    rows = np.unique(np.concatenate([np.arange(70), np.arange(n - 70, n), rng.integers(0, n, 600)]))
+    with px.Context(px.Params(log2_r=level)) as ctx:
+        ctx.set_P(*ring_P(n))
+        ctx.set_state(z, s)
+        Frep, Zi, _, Z = ctx.get_forces()
+        assert ctx.sync() == 0
+    oF, oZi, _ = oracle.bh_repulsion(z, s, level, 0.5, rows=rows)
+    assert rel(Frep[rows], oF) <= FORCE_TOL
+    assert rel(Zi[rows], oZi) <= FORCE_TOL
+    assert abs(Z - Zi.astype(np.float64).sum()) <= 1e-12 * Z
