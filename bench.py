@@ -658,15 +658,15 @@ def run_gpu(args):
     knn_ms = ctx.knn_time_ms()
     kx, ki, kpath = ctx.knn_counters()
     kskip, kpairs = ctx.knn_pruning()
-    # the products the tensor cores actually formed: the (query tile,
-    # candidate tile) pairs of 128 x 128 rows not skipped by the tile bound,
-    # 2 * 128 * 128 * Dp FLOP each (rows padded to the tiles, D to Dp); the time
-    # also holds the pass over the sample and the exact distances, and the rows
+    # the products the tensor cores actually formed, in all passes: those of the
+    # (query tile, candidate tile) pairs of 128 x 128 rows not skipped by the
+    # tile bound, 2 * 128 * 128 * Dp FLOP each (rows padded to the tiles, D to
+    # Dp); the time also holds the exact distances, and the rows
     # kept are those within the search's threshold (heap insertions where the
     # one-pass search k_knn_tc did a tile)
     Dp = (X.shape[1] + 63) // 64 * 64
     knn_dense = 2.0 * n * n * X.shape[1]
-    knn_flop = (kpairs - kskip) * 2.0 * 128 * 128 * Dp if kpairs else knn_dense
+    knn_flop = ctx.knn_work()[0] * 2.0 * 128 * 128 * Dp if kpairs else knn_dense
     pk, pk_kind = measured_peaks()
     knn = {"kernel": "k_knn_scan" if kpath == 1 else "k_knn_tile", "ms": knn_ms,
            "bound": "tensor", "achieved": knn_flop / (knn_ms / 1e3) / 1e12,

@@ -347,9 +347,18 @@ int pxsne_get_knn_counters(pxsne_ctx *ctx, uint64_t *exact, uint64_t *inserted, 
 /* Tile pruning of the last tensor-core neighbour search: (query tile,
  * candidate tile) pairs of 128 x 128 rows it skipped because the triangle
  * inequality on the tiles' centroids and radii put every candidate beyond the
- * query rows' current k-th distances, and the number of pairs (T^2).  Both 0
- * after the FP32 search.  Any pointer may be NULL.  Synchronises. */
+ * query rows' current k-th distances (the rows' thresholds in the two-pass
+ * search, whose first pass over all candidates is the one that counts), and the
+ * number of pairs (T^2).  Both 0 after the FP32 search.  Any pointer may be
+ * NULL.  Synchronises. */
 int pxsne_get_knn_pruning(pxsne_ctx *ctx, uint64_t *skipped_pairs, uint64_t *pairs);
+
+/* What the passes of the last tensor-core neighbour search did: products =
+ * tile products of 128 x 128 rows formed by all of them (the pass over the
+ * sample included), and of the two-pass search the query tiles that it scanned
+ * a second time and those whose lists it left to the one-pass search.  All 0
+ * after the FP32 search.  Any pointer may be NULL.  Synchronises. */
+int pxsne_get_knn_work(pxsne_ctx *ctx, uint64_t *products, uint64_t *again, uint64_t *left);
 
 /* Device time in milliseconds of the last neighbour-search kernel (the brute
  * force of Sec. 3.3's kNN pattern; CUDA events around its launch on the

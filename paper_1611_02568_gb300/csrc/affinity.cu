@@ -1008,7 +1008,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_knn_tc(const KnnTcArgs a) {
             }
         }
         if (lane == 0) {
-            atomicAdd(&a.stats[2], n_skip);
+            // (a tile left over by the two-pass search has been counted there)
+            if (!a.qlist) atomicAdd(&a.stats[2], n_skip);
+            atomicAdd(&a.stats[3], (u64)n_sf);
             // copies still in flight complete before the CTA exits: those of
             // the last kept tiles (kept tile q used stage q % 2 and h slot
             // q % 4).  After the end mark the copies into the slots it reused
@@ -1536,7 +1538,7 @@ cudaError_t launch_knn(pxsne_ctx *c, const float *Xdev, int64_t n, int32_t D, in
         c->knn_path = 1;
         unsigned *amax = nullptr;
         unsigned *err = &c->sc->err;
-        if ((e = cudaMemsetAsync(&c->sc->knn_exact, 0, 3 * sizeof(u64), st))) return e;
+        if ((e = cudaMemsetAsync(&c->sc->knn_exact, 0, 6 * sizeof(u64), st))) return e;
         if ((e = palloc(c, &amax, sizeof(unsigned), st))) return e;
         if ((e = cudaMemsetAsync(amax, 0, sizeof(unsigned), st))) return e;
         k_absmax<<<1184, 256, 0, st>>>(n * D, Xdev, amax);

@@ -1012,6 +1012,19 @@ int pxsne_get_knn_pruning(pxsne_ctx *c, uint64_t *skipped_pairs, uint64_t *pairs
     return PXSNE_OK;
 }
 
+int pxsne_get_knn_work(pxsne_ctx *c, uint64_t *products, uint64_t *again, uint64_t *left) {
+    if (!c) return PXSNE_E_ARG;
+    DevScalars h;
+    CK(c, cudaMemcpyAsync(&h, c->sc, sizeof(DevScalars), cudaMemcpyDeviceToHost, c->stream));
+    int rc = check_device(c, nullptr);
+    if (rc) return rc;
+    const bool tc_path = c->knn_path == 1;
+    if (products) *products = tc_path ? h.knn_products : 0u;
+    if (again) *again = tc_path ? h.knn_again : 0u;
+    if (left) *left = tc_path ? h.knn_left : 0u;
+    return PXSNE_OK;
+}
+
 int pxsne_get_knn_counters(pxsne_ctx *c, uint64_t *exact, uint64_t *inserted, int32_t *path) {
     if (!c) return PXSNE_E_ARG;
     DevScalars h;

@@ -88,7 +88,11 @@ struct DevScalars {
                             // over the counting traversals since the last reset
     u64 knn_exact;       // exact distances computed by the last neighbour search
     u64 knn_insert;      // list insertions of the last neighbour search
-    u64 knn_skip;        // (query tile, candidate tile) pairs it skipped by the tile bound
+    u64 knn_skip;        // (query tile, candidate tile) pairs it skipped by the tile bound,
+                         // each query tile counted by the first pass over all tiles only
+    u64 knn_products;    // tile products formed, all passes together
+    u64 knn_again;       // query tiles that the two-pass search scanned a second time
+    u64 knn_left;        // query tiles that it left to the one-pass search
     // the 3-D embedding (dim = 3): the same scalars for three axes
     double s3[3], inv_s3[3];
     float sf3[3];

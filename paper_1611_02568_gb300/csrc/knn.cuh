@@ -38,7 +38,9 @@ struct KnnScan {
     int32_t *out_idx;
     float *out_d2;
     unsigned *err;
-    unsigned long long *stats;  // exact distances, kept candidates, skipped tile pairs
+    // exact distances, kept candidates, skipped tile pairs, tile products, query
+    // tiles scanned again and left to the one-pass search (DevScalars::knn_*)
+    unsigned long long *stats;
 };
 
 // The sample takes the ordered rows kScanPhase + i kScanStride.

@@ -275,7 +275,9 @@ __global__ void __launch_bounds__(scan_threads(MODE), 2) k_knn_scan(const ScanAr
             }
         }
         if (lane == 0) {
-            if (MODE == 1) atomicAdd(&a.stats[2], n_skip);
+            // (the second scan's tiles were counted by the first)
+            if (MODE == 1 && !a.qlist) atomicAdd(&a.stats[2], n_skip);
+            atomicAdd(&a.stats[3], (u64)n_sf);
             // copies still in flight complete before the CTA exits (those of the
             // last kept tiles; after the end mark the copies into the slots it
             // reused are known complete)
@@ -605,9 +607,13 @@ __global__ void __launch_bounds__(kPickWarps * 32) k_knn_pick(const PickArgs a) 
                 }
                 if (wider > tau && wider < 3.402823466e38f) {
                     a.tau[row] = wider;
-                    if (atomicOr(&a.flag[t], 1u) == 0u) a.retry[atomicAdd(a.nretry, 1u)] = t;
+                    if (atomicOr(&a.flag[t], 1u) == 0u) {
+                        a.retry[atomicAdd(a.nretry, 1u)] = t;
+                        atomicAdd(&a.stats[4], 1ull);
+                    }
                 } else if (!(atomicOr(&a.flag[t], 2u) & 2u)) {
                     a.failed[atomicAdd(a.nfailed, 1u)] = t;
+                    atomicAdd(&a.stats[5], 1ull);
                 }
                 if (!ok) atomicOr(a.err, (unsigned)PXSNE_DEVERR_TIMEOUT);
             }
