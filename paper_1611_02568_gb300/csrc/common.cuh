@@ -284,6 +284,17 @@ __device__ inline float bh_threshold(int l, int L, double s0, double s1, float t
     return th2 > 0.0 ? (float)(rc2 / th2) : INFINITY;
 }
 
+// A cell of one point, whose centre is that point, is accepted by every point but
+// itself, so its threshold on d^2 is 0 where any other's d^2 is above 0.  That
+// fails where the square of an axis's y-units per ulp (sf; the smallest offset is
+// one ulp) underflows: there every point accepts it, itself included, and takes
+// its own term, 1, out of its sum again.  fma(N, kManyT, base) is at most 0 for N
+// <= 1 and beyond every d^2 whose kernel value is not flushed to 0 (2^126) for
+// more.
+constexpr float kManyT = 0x1p127f;
+__device__ __forceinline__ float single_base(bool always) { return always ? -1.25f * kManyT : -kManyT; }
+__device__ __forceinline__ bool underflows(float sf) { return !(sf * sf > 0.f); }
+
 // Derived per-iteration scalars from s (called by one thread).
 __device__ inline void derive_scalars(DevScalars *sc, float theta, int L) {
     const double s0 = sc->s[0], s1 = sc->s[1];

@@ -550,6 +550,20 @@ __device__ __forceinline__ void take_out3(int slot, float2 &N, float2 (&dx)[3]) 
     }
 }
 
+// Cells of one point are accepted by all others by the same rule as in 2-D
+// (single_base, common.cuh).
+__device__ __forceinline__ bool tiny3(const float2 (&s)[3]) {
+    return underflows(s[0].x) || underflows(s[1].x) || underflows(s[2].x);
+}
+// What a point (its voxel's Morton index mi) has to take out of its sum.
+template <bool OWN>
+__device__ __forceinline__ float own_single3(float base, const float4 *__restrict__ rec, int L,
+                                             uint32_t mi) {
+    if (OWN || base == -kManyT || L < 2) return 0.f;
+    const float *g = reinterpret_cast<const float *>(rec) + (off3(L - 2) + (mi >> 6)) * kGroup3;
+    return g[48 + ((mi >> 3) & 7u)] == 1.f ? 1.f : 0.f;
+}
+
 struct __align__(8) T3Entry {
     uint32_t node, mask;  // (children's level << 28) | their group; lanes that open it
 };
@@ -575,6 +589,7 @@ __global__ void __launch_bounds__(kT3Warps * 32, 4)
     const uint32_t own_grp = (uint32_t)off3(L - 1) + (mi >> 3);
     const Point3 pt = point3(zi);
     const float2 s[3] = {b3(sc->sf3[0]), b3(sc->sf3[1]), b3(sc->sf3[2])};
+    const float base = single_base(OWN || tiny3(s));
     Sum3 a{{b3(0.f), b3(0.f), b3(0.f)}, b3(0.f)};
     T3Entry *stk = s_stk[w];
     if (lane == 0) stk[0] = T3Entry{1u << 28, act};  // the root's children: level 1, group 0
@@ -642,8 +657,7 @@ __global__ void __launch_bounds__(kT3Warps * 32, 4)
                     float2 dx[3];
                     offset3(r, p, pt, dx);
                     const float2 d2 = dist3(dx, s);
-                    // the threshold of a cell of one point is 0
-                    const float2 tb = __ffma2_rn(N, b3(1e30f), b3(-1e30f));
+                    const float2 tb = __ffma2_rn(N, b3(kManyT), b3(base));
                     const bool a0 = me && d2.x > fminf(tb.x, Tl) && (!OWN || mine != first + c);
                     const bool a1 = me && d2.y > fminf(tb.y, Tl) && (!OWN || mine != first + c + 1);
                     add3(a, make_float2(a0 ? N.x : 0.f, a1 ? N.y : 0.f), d2, dx);
@@ -667,7 +681,7 @@ __global__ void __launch_bounds__(kT3Warps * 32, 4)
     }
     if (valid) {
         Frep[i] = make_float4(a.f[0].x + a.f[0].y, a.f[1].x + a.f[1].y, a.f[2].x + a.f[2].y, 0.f);
-        Zi[i] = a.z.x + a.z.y;
+        Zi[i] = a.z.x + a.z.y - own_single3<OWN>(base, rec, L, mi);
     }
     if (overflow && lane == 0) atomicOr(&sc->err, (unsigned)PXSNE_DEVERR_STACK);
 }
@@ -701,6 +715,7 @@ __global__ void __launch_bounds__(kPt3Warps * 32)
     const uint32_t own_grp = (uint32_t)off3(L - 1) + (mi >> 3);
     const Point3 pt = point3(zi);
     const float2 s[3] = {b3(sc->sf3[0]), b3(sc->sf3[1]), b3(sc->sf3[2])};
+    const float base = single_base(OWN || tiny3(s));
     Sum3 a{{b3(0.f), b3(0.f), b3(0.f)}, b3(0.f)};
     const unsigned before = (1u << lane) - 1u;
     if (lane == 0) ring[0] = 1u << 28;
@@ -738,7 +753,7 @@ __global__ void __launch_bounds__(kPt3Warps * 32)
                 offset3(r, p, pt, dx);
                 if (own && (int)((mi & 7u) >> 1) == 2 * hf + p) take_out3((int)(mi & 1u), N, dx);
                 const float2 d2 = dist3(dx, s);
-                const float2 tb = __ffma2_rn(N0, b3(1e30f), b3(-1e30f));
+                const float2 tb = __ffma2_rn(N0, b3(kManyT), b3(base));
                 const float T0 = leaf ? -1.0f : fminf(tb.x, Tl), T1 = leaf ? -1.0f : fminf(tb.y, Tl);
                 const bool a0 = d2.x > T0 && (!OWN || leaf || mine != first + c);
                 const bool a1 = d2.y > T1 && (!OWN || leaf || mine != first + c + 1);
@@ -768,7 +783,7 @@ __global__ void __launch_bounds__(kPt3Warps * 32)
         for (int d = 0; d < 4; d++) v[d] += __shfl_xor_sync(0xffffffffu, v[d], o);
     if (lane == 0) {
         Frep[i] = make_float4(v[0], v[1], v[2], 0.f);
-        Zi[i] = v[3];
+        Zi[i] = v[3] - own_single3<OWN>(base, rec, L, mi);
     }
 }
 

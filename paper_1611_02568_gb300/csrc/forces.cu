@@ -225,18 +225,41 @@ struct __align__(16) TravEntry<2> {
     uint32_t node, m[2], pad;
 };
 
+// The threshold's term for cells of one point (single_base; geometric centres: no
+// such rule).  It is read with the level's threshold where it is no constant: a
+// register for it across the walk cost 1.5 % of an iteration at n = 70,000.
+template <int CENTRE, bool OWN>
+__device__ __forceinline__ constexpr bool trav_const() {
+    return CENTRE != 0 || OWN;
+}
+template <int CENTRE, bool OWN>
+__device__ __forceinline__ float trav_base(const DevScalars *sc) {
+    if (CENTRE != 0) return 0.f;
+    return single_base(OWN || underflows(sc->sf[0]) || underflows(sc->sf[1]));
+}
+
+// What a point (its pixel's Morton index mi) has to take out of its sum: 1 where
+// every point accepts cells of one point (single_base) and it is alone in a cell
+// above the pixels.
+template <int CENTRE, bool OWN>
+__device__ __forceinline__ float own_single(float base, const float *__restrict__ recn, int L,
+                                            uint32_t mi) {
+    if (CENTRE != 0 || OWN || base == -kManyT || L < 2) return 0.f;
+    return recn[rec_offset(L - 1) + (mi >> 2)] == 1.f ? 1.f : 0.f;
+}
+
 template <int CENTRE, int COUNT, bool OWN, int PPL>
 __global__ void __launch_bounds__(kTravWarps * 32, 16)
     k_bh_traverse(int n, int L, const uint2 *__restrict__ z, const uint32_t *__restrict__ perm,
                   const float4 *__restrict__ rec, const float *__restrict__ recn,
                   DevScalars *sc, float2 *__restrict__ Frep, float *__restrict__ Zi) {
     __shared__ TravEntry<PPL> s_stk[kTravWarps][kTravStack];
-    __shared__ float s_T[kMaxL + 2];
+    __shared__ float2 s_T[kMaxL + 2];  // a level's threshold on d^2, and single_base
     const int stk_lim = sc->stack_limit > 0 ? min(max(sc->stack_limit, 4), kTravStack) : kTravStack;
     // COUNT: (tested, accepted, warp steps) by level of the child
     __shared__ u64 s_lv[COUNT ? kMaxL + 2 : 1][3];
     if (threadIdx.x < kMaxL + 2) {
-        s_T[threadIdx.x] = sc->T[threadIdx.x];
+        s_T[threadIdx.x] = make_float2(sc->T[threadIdx.x], trav_base<CENTRE, OWN>(sc));
         if (COUNT) s_lv[threadIdx.x][0] = s_lv[threadIdx.x][1] = s_lv[threadIdx.x][2] = 0ull;
     }
     __syncthreads();
@@ -376,9 +399,10 @@ __global__ void __launch_bounds__(kTravWarps * 32, 16)
                 // Eq. bh_criteria's threshold on d^2.  The centre of a cell that
                 // holds one point is that point exactly, so opening it down to
                 // its pixel would end in the same term: it is accepted at once
-                // by every point but the one in it, whose d^2 is 0 (threshold
-                // 0).  Empty cells add nothing.
-                const float Tl = s_T[lc];
+                // by every point but the one in it (single_base).  Empty cells
+                // add nothing.
+                const float2 Tb = s_T[lc];
+                const float Tl = Tb.x, base = trav_const<CENTRE, OWN>() ? trav_base<CENTRE, OWN>(sc) : Tb.y;
                 constexpr float few = CENTRE == 0 ? 1.0f : 0.0f;
                 // room for the (at most four) entries this node may push
                 if (sp + 4 > stk_lim) {
@@ -389,7 +413,7 @@ __global__ void __launch_bounds__(kTravWarps * 32, 16)
 #pragma unroll
                 for (int p = 0; p < 2; p++) {
                     const float2 N = p ? make_float2(nv.z, nv.w) : make_float2(nv.x, nv.y);
-                    const float2 tb = fma2(N, bc2(1e30f), bc2(-1e30f * few));
+                    const float2 tb = fma2(N, bc2(kManyT), bc2(base));
                     const float T0 = fminf(tb.x, Tl), T1 = fminf(tb.y, Tl);
 #pragma unroll
                     for (int a = 0; a < PPL; a++) {
@@ -397,7 +421,7 @@ __global__ void __launch_bounds__(kTravWarps * 32, 16)
                         // theta < 1 (the point and the centre of mass lie in the
                         // cell, so d <= r_c < r_c / theta); tested explicitly
                         // otherwise
-                        const uint32_t mine = OWN ? mi[a] >> (2 * (L - lc)) : 0u;
+                        const uint32_t mine = OWN || COUNT ? mi[a] >> (2 * (L - lc)) : 0u;
                         float2 dx, dy;
                         sib.offset(p, pt[a], dx, dy);
                         dx = mul2(dx, sf0);
@@ -405,16 +429,18 @@ __global__ void __launch_bounds__(kTravWarps * 32, 16)
                         const float2 d2 = fma2(dx, dx, mul2(dy, dy));
                         const bool a0 = me[a] && d2.x > T0 && (!OWN || mine != 4u * m + 2u * p);
                         const bool a1 = me[a] && d2.y > T1 && (!OWN || mine != 4u * m + 2u * p + 1u);
-                        if (COUNT) {
+                        if (COUNT) {  // (its own cell is no interaction)
+                            const bool c0 = a0 && mine != 4u * m + 2u * p;
+                            const bool c1 = a1 && mine != 4u * m + 2u * p + 1u;
                             if (N.x != 0.f) {
                                 n_tst += me[a];
-                                n_acc += a0;
-                                count_level(s_lv[lc], me[a], a0, a == 0, lane);
+                                n_acc += c0;
+                                count_level(s_lv[lc], me[a], c0, a == 0, lane);
                             }
                             if (N.y != 0.f) {
                                 n_tst += me[a];
-                                n_acc += a1;
-                                count_level(s_lv[lc], me[a], a1, a == 0, lane);
+                                n_acc += c1;
+                                count_level(s_lv[lc], me[a], c1, a == 0, lane);
                             }
                         }
                         const float2 w1 = add2(bc2(1.0f), d2);
@@ -454,7 +480,7 @@ __global__ void __launch_bounds__(kTravWarps * 32, 16)
         for (int a = 0; a < PPL; a++)
             if ((act[a] >> lane) & 1u) {
                 Frep[i[a]] = make_float2(fx[a].x + fx[a].y, fy[a].x + fy[a].y);
-                Zi[i[a]] = zs[a].x + zs[a].y;
+                Zi[i[a]] = zs[a].x + zs[a].y - own_single<CENTRE, OWN>(s_T[0].y, recn, L, mi[a]);
             }
         if (overflow && lane == 0) atomicOr(&sc->err, (unsigned)PXSNE_DEVERR_STACK);
         __syncwarp();
@@ -516,6 +542,7 @@ __global__ void __launch_bounds__(kPtWarps * 32)
     uint32_t *ring = s_ring[w];
     const int F = 32 - L;
     const float2 sf0 = bc2(sc->sf[0]), sf1 = bc2(sc->sf[1]);
+    const float base = trav_base<CENTRE, OWN>(sc);
     const unsigned before = (1u << lane) - 1u;
     const uint32_t g0 = (uint32_t)(rec_offset(L) >> 2);
     const uint32_t i = perm[idx];
@@ -546,7 +573,7 @@ __global__ void __launch_bounds__(kPtWarps * 32)
         const float Tl = s_T[lc];
         constexpr float few = CENTRE == 0 ? 1.0f : 0.0f;
         const bool own = leaf && act && (mi >> 2) + g0 == grp;
-        const uint32_t mine = OWN ? mi >> (2 * (L - lc)) : 0u;
+        const uint32_t mine = OWN || COUNT ? mi >> (2 * (L - lc)) : 0u;
         bool open[4];
         if (COUNT && act) n_nod++;
 #pragma unroll
@@ -574,14 +601,17 @@ __global__ void __launch_bounds__(kPtWarps * 32)
             dy = mul2(dy, sf1);
             const float2 d2 = fma2(dx, dx, mul2(dy, dy));
             // thresholds as above; a pixel is always accepted
-            const float2 tb = fma2(N0, bc2(1e30f), bc2(-1e30f * few));
+            const float2 tb = fma2(N0, bc2(kManyT), bc2(base));
             const float T0 = leaf ? -1.0f : fminf(tb.x, Tl), T1 = leaf ? -1.0f : fminf(tb.y, Tl);
             const bool a0 = d2.x > T0 && (!OWN || leaf || mine != 4u * m + 2u * p);
             const bool a1 = d2.y > T1 && (!OWN || leaf || mine != 4u * m + 2u * p + 1u);
             if (COUNT) {
                 const bool f0 = N0.x != 0.f, f1 = N0.y != 0.f;
                 const uint32_t ts = (f0 ? 1u : 0u) + (f1 ? 1u : 0u);
-                const uint32_t ac = (f0 && a0 && N.x > 0.f ? 1u : 0u) + (f1 && a1 && N.y > 0.f ? 1u : 0u);
+                // (its own cell above the pixels is no interaction)
+                const bool c0 = a0 && (leaf || mine != 4u * m + 2u * p);
+                const bool c1 = a1 && (leaf || mine != 4u * m + 2u * p + 1u);
+                const uint32_t ac = (f0 && c0 && N.x > 0.f ? 1u : 0u) + (f1 && c1 && N.y > 0.f ? 1u : 0u);
                 n_tst += ts;
                 n_acc += ac;
                 n_stp += ts;
@@ -622,7 +652,7 @@ __global__ void __launch_bounds__(kPtWarps * 32)
     }
     if (lane == 0) {
         Frep[i] = make_float2(vx, vy);
-        Zi[i] = vz;
+        Zi[i] = vz - own_single<CENTRE, OWN>(base, recn, L, mi);
     }
     if (COUNT) {
 #pragma unroll
