@@ -1119,10 +1119,14 @@ int pxsne_mlp_predict(pxsne_mlp *M, const float *X, int64_t n, float *Y, int on_
     if (!M || !X || !Y || n < 1) return mfail(M, PXSNE_E_ARG, "bad arguments");
     int rc = PXSNE_OK;
     cudaStream_t st = M->stream;
-    // (the fused kernels read the caller's rows in place)
+    // the fused kernels read the caller's rows in place, kInfRows at a time, unless
+    // the outputs of one round could overwrite rows of the next
     const bool fused = M->dp <= kInfMaxK;
-    if (!(fused && on_device) && (rc = stage_data(M, X, nullptr, n, on_device))) return rc;
-    const float *Xd = fused && on_device ? X : M->Xd;
+    const uintptr_t x0 = reinterpret_cast<uintptr_t>(X), y0 = reinterpret_cast<uintptr_t>(Y);
+    const bool apart = y0 >= x0 + (uintptr_t)n * M->d * 4 || x0 >= y0 + (uintptr_t)n * 8;
+    const bool in_place = fused && on_device && apart;
+    if (!in_place && (rc = stage_data(M, X, nullptr, n, on_device))) return rc;
+    const float *Xd = in_place ? X : M->Xd;
     float *Yd = Y;
     if (!on_device) MCK(M, mal(&Yd, (size_t)n * 2));
     if (fused) {
