@@ -445,6 +445,12 @@ int pxsne_mlp_train(pxsne_mlp *m, const float *X, const float *T, int64_t n, int
 /* Y = MLP(X) for n rows. */
 int pxsne_mlp_predict(pxsne_mlp *m, const float *X, int64_t n, float *Y, int on_device);
 
+/* Test hook of the prediction kernels' bounded waits: with 1 <= polls <= 65536
+ * every CTA's last operand region never arrives, and a wait gives up after
+ * polls polls of at most 2 us each; pxsne_mlp_predict then returns
+ * PXSNE_E_DEVICE and the network stays usable.  0 restores the waits. */
+int pxsne_mlp_test_stall(pxsne_mlp *m, int32_t polls);
+
 /* PCA pre-processing (Sec. 5.1.1 reduces every dataset to 50 dimensions
  * before P): Xout (n x dout) = (X - mean) V with V the dout leading
  * eigenvectors of the sample covariance (X - mean)^T (X - mean) / (n - 1).

@@ -132,6 +132,7 @@ def load(path: str | None = None):
     L.pxsne_mlp_train.argtypes = [vp, vp, vp, i64, i32, i32, C.c_float, u64,
                                   C.POINTER(C.c_double), C.c_int]
     L.pxsne_mlp_predict.argtypes = [vp, vp, i64, vp, C.c_int]
+    L.pxsne_mlp_test_stall.argtypes = [vp, i32]
     L.pxsne_embed_align.argtypes = [vp, vp, i64, vp, C.c_int]
     L.pxsne_pca.argtypes = [vp, i64, i32, i32, vp, vp, vp, C.c_int, u64]
     L.pxsne_device_bytes.argtypes = [vp]
@@ -566,6 +567,11 @@ class MLP:
         return Y
 
 
+    def test_stall(self, polls):
+        """Let the prediction's waits run out (test hook; 0 restores them)."""
+        self._ck(self.L.pxsne_mlp_test_stall(self.h, int(polls)))
+
+
 def embed_align(Y, Yref=None):
     """Centre, scale to unit RMS and (with Yref, whose row i is the same point
     as row i of Y) orthogonally align Y (numpy)."""
@@ -623,7 +629,7 @@ EXPORTED = ["pxsne_default_params", "pxsne_create", "pxsne_destroy", "pxsne_last
             "pxsne_get_knn_counters", "pxsne_set_schedule", "pxsne_mlp_create",
             "pxsne_mlp_destroy", "pxsne_mlp_last_error", "pxsne_mlp_num_params",
             "pxsne_mlp_set_params", "pxsne_mlp_get_params", "pxsne_mlp_loss_grad",
-            "pxsne_mlp_train", "pxsne_mlp_predict", "pxsne_embed_align",
+            "pxsne_mlp_train", "pxsne_mlp_predict", "pxsne_mlp_test_stall", "pxsne_embed_align",
             "pxsne_nbr_precision", "pxsne_pca", "pxsne_measure_peaks",
             "pxsne_get_level_counters", "pxsne_save", "pxsne_load", "pxsne_get_params",
             "pxsne_test_stack_limit", "pxsne_get_tree3"]

@@ -447,16 +447,19 @@ struct InfArgs {
     const float *b3;
     float *Y;
     unsigned *err;
+    int polls;                // limit of every wait
+    int stall;                // test hook: the last operand region never comes
 };
 
 template <int LAYER>
 __global__ void __launch_bounds__(kInfThreads, 1) k_infer(const InfArgs a) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t bar_full[8], bar_empty[8], bar_tf[2], bar_te[2];
+    __shared__ uint64_t bar_p[LAYER == 2 ? 4 : 1][4];  // a quarter's partial sums, tile i in i & 3
     __shared__ uint32_t tslot;
     __shared__ volatile int s_abort;
     __shared__ float s_bias[kH], s_w3[2][kH];
-    __shared__ float s_part[2][128][2];
+    __shared__ float s_part[LAYER == 2 ? 4 : 1][128][2];
     uint8_t *smem = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
     const int K = a.K, regions = K / 64, NS = inf_stages<LAYER>(K);
     uint8_t *sW = smem, *sA = smem + (size_t)kH * K * 2;
@@ -483,6 +486,8 @@ __global__ void __launch_bounds__(kInfThreads, 1) k_infer(const InfArgs a) {
             tc::mbar_init(&bar_tf[q], 1);
             tc::mbar_init(&bar_te[q], kInfEpi);
         }
+        if (LAYER == 2)
+            for (int q = 0; q < 16; q++) tc::mbar_init(&bar_p[q >> 2][q & 3], 1);
         s_abort = 0;
     }
     tc::fence_proxy_async();
@@ -500,9 +505,10 @@ __global__ void __launch_bounds__(kInfThreads, 1) k_infer(const InfArgs a) {
                 const int s = (int)(j % NS);
                 ok = __all_sync(0xffffffffu,
                                 (j < NS || tc::mbar_wait_sleep(&bar_empty[s], (uint32_t)((j / NS - 1) & 1),
-                                                               kGemmPolls, 2000u)) &&
+                                                               a.polls, 2000u)) &&
                                     !s_abort);
                 if (!ok) break;
+                if (a.stall && t + gridDim.x >= a.tiles && g == regions - 1) break;
                 uint8_t *dst = sA + (size_t)s * kReg;
                 if (LAYER == 1) {
                     const int lt = tid - 32 * kInfEpi;
@@ -554,10 +560,10 @@ __global__ void __launch_bounds__(kInfThreads, 1) k_infer(const InfArgs a) {
             for (int64_t t = blockIdx.x; t < a.tiles && ok; t += gridDim.x, i++) {
                 const int b = (int)(i & 1);
                 if (i >= 2)
-                    ok = tc::mbar_wait_sleep(&bar_te[b], (uint32_t)((i / 2 - 1) & 1), kGemmPolls, 2000u);
+                    ok = tc::mbar_wait_sleep(&bar_te[b], (uint32_t)((i / 2 - 1) & 1), a.polls, 2000u);
                 for (int g = 0; g < regions && ok; g++, j++) {
                     const int s = (int)(j % NS);
-                    ok = tc::mbar_wait_sleep(&bar_full[s], (uint32_t)((j / NS) & 1), kGemmPolls, 2000u) &&
+                    ok = tc::mbar_wait_sleep(&bar_full[s], (uint32_t)((j / NS) & 1), a.polls, 2000u) &&
                          !s_abort;
                     if (!ok) break;
                     tc::fence_after();
@@ -586,7 +592,7 @@ __global__ void __launch_bounds__(kInfThreads, 1) k_infer(const InfArgs a) {
         for (int64_t t = blockIdx.x; t < a.tiles; t += gridDim.x, i++) {
             const int b = (int)(i & 1);
             const bool got = __all_sync(
-                0xffffffffu, tc::mbar_wait_sleep(&bar_tf[b], (uint32_t)((i / 2) & 1), kGemmPolls, 2000u) &&
+                0xffffffffu, tc::mbar_wait_sleep(&bar_tf[b], (uint32_t)((i / 2) & 1), a.polls, 2000u) &&
                                  !s_abort);
             if (!got) {
                 if (lane == 0 && !s_abort) atomicOr(a.err, (unsigned)PXSNE_DEVERR_TIMEOUT);
@@ -627,16 +633,31 @@ __global__ void __launch_bounds__(kInfThreads, 1) k_infer(const InfArgs a) {
                 }
             }
             if (LAYER == 2) {
-                // the halves' sums meet in the first one's warp
-                if (half == 1) {
-                    s_part[b][r][0] = y0;
-                    s_part[b][r][1] = y1;
-                }
-                asm volatile("bar.sync %0, 64;" ::"r"(1 + quarter) : "memory");
+                // the halves' sums meet in the first one's warp, through an
+                // mbarrier: a named barrier would have no limit where one of the
+                // two warps gives up.  The second half is at most three tiles
+                // ahead (tile i + 3 comes after this warp has released tile i +
+                // 1), so four slots are never written while one is read.
+                const int p = (int)(i & 3);
                 const int64_t row = t * 128 + r;
-                if (half == 0 && row < a.rows) {
-                    a.Y[2 * row] = y0 + s_part[b][r][0] + a.b3[0];
-                    a.Y[2 * row + 1] = y1 + s_part[b][r][1] + a.b3[1];
+                if (half == 1) {
+                    s_part[p][r][0] = y0;
+                    s_part[p][r][1] = y1;
+                    __syncwarp();
+                    if (lane == 0) tc::mbar_arrive(&bar_p[quarter][p]);
+                } else {
+                    bool met = tc::mbar_wait(&bar_p[quarter][p], (uint32_t)((i >> 2) & 1), 1);
+                    for (int q = 1; !met && q < a.polls && !s_abort; q++)
+                        met = tc::mbar_wait_sleep(&bar_p[quarter][p], (uint32_t)((i >> 2) & 1), 1, 2000u);
+                    if (!__all_sync(0xffffffffu, met)) {
+                        if (lane == 0 && !s_abort) atomicOr(a.err, (unsigned)PXSNE_DEVERR_TIMEOUT);
+                        s_abort = 1;
+                        break;
+                    }
+                    if (row < a.rows) {
+                        a.Y[2 * row] = y0 + s_part[p][r][0] + a.b3[0];
+                        a.Y[2 * row + 1] = y1 + s_part[p][r][1] + a.b3[1];
+                    }
                 }
             }
         }
@@ -750,6 +771,7 @@ struct pxsne_mlp {
     // inference: operand images of H1 for inf_cap rows (at most kInfRows)
     uint8_t *H1img = nullptr;
     int64_t inf_cap = 0;
+    int stall_polls = 0;  // test hook (pxsne_mlp_test_stall)
 };
 
 namespace {
@@ -896,6 +918,8 @@ int infer(pxsne_mlp *M, const float *X, int64_t n, float *Y) {
         const unsigned grid = (unsigned)std::min<int64_t>(a.tiles, std::max(1, sms));
         a.H1 = M->H1img;
         a.err = M->derr;
+        a.stall = M->stall_polls > 0;
+        a.polls = a.stall ? M->stall_polls : kGemmPolls;
         a.d = M->d;
         a.K = M->dp;
         a.X = X + base * M->d;
@@ -1113,6 +1137,13 @@ int pxsne_mlp_train(pxsne_mlp *M, const float *X, const float *T, int64_t n, int
     }
     if (final_loss) *final_loss = last;
     return check_dev(M);
+}
+
+int pxsne_mlp_test_stall(pxsne_mlp *M, int32_t polls) {
+    if (!M) return PXSNE_E_ARG;
+    if (polls < 0 || polls > 65536) return mfail(M, PXSNE_E_ARG, "polls outside [0, 65536]");
+    M->stall_polls = polls;
+    return PXSNE_OK;
 }
 
 int pxsne_mlp_predict(pxsne_mlp *M, const float *X, int64_t n, float *Y, int on_device) {
