@@ -402,6 +402,11 @@ int pxsne_measure_peaks(void *stream, double *l2_read_gbs, double *fp32_tflops,
  * usable.  Takes effect from the next traversal.  Synchronises. */
 int pxsne_test_stack_limit(pxsne_ctx *ctx, int32_t entries);
 
+/* Test hook of a full device: a single request for more than `bytes` of device
+ * memory for P, the neighbour lists or a call's scratch fails as if there were no
+ * room for it (0: no limit). */
+int pxsne_test_alloc_limit(pxsne_ctx *ctx, int64_t bytes);
+
 /* Total bytes of device memory the context holds. */
 int64_t pxsne_device_bytes(const pxsne_ctx *ctx);
 

@@ -140,6 +140,7 @@ def load(path: str | None = None):
     L.pxsne_get_level_counters.argtypes = [vp, C.POINTER(u64), i32]
     L.pxsne_save.argtypes = [vp, C.c_char_p]
     L.pxsne_test_stack_limit.argtypes = [vp, i32]
+    L.pxsne_test_alloc_limit.argtypes = [vp, i64]
     L.pxsne_load.argtypes = [C.POINTER(vp), C.c_char_p, vp]
     L.pxsne_get_params.argtypes = [vp, C.POINTER(_CParams)]
     L.pxsne_get_tree3.argtypes = [vp, i32, vp, vp, vp, vp, vp]
@@ -463,6 +464,10 @@ class Context:
         """Lower the traversal's stack room (test hook; 0 restores it)."""
         self._ck(self.L.pxsne_test_stack_limit(self.h, int(entries)))
 
+    def test_alloc_limit(self, nbytes):
+        """Let larger device allocations fail (test hook; 0: no limit)."""
+        self._ck(self.L.pxsne_test_alloc_limit(self.h, int(nbytes)))
+
     def knn_pruning(self):
         """(skipped (query tile, candidate tile) pairs, all pairs) of the last
         tensor-core neighbour search."""
@@ -632,4 +637,4 @@ EXPORTED = ["pxsne_default_params", "pxsne_create", "pxsne_destroy", "pxsne_last
             "pxsne_mlp_train", "pxsne_mlp_predict", "pxsne_mlp_test_stall", "pxsne_embed_align",
             "pxsne_nbr_precision", "pxsne_pca", "pxsne_measure_peaks",
             "pxsne_get_level_counters", "pxsne_save", "pxsne_load", "pxsne_get_params",
-            "pxsne_test_stack_limit", "pxsne_get_tree3"]
+            "pxsne_test_stack_limit", "pxsne_test_alloc_limit", "pxsne_get_tree3"]

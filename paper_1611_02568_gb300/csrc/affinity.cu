@@ -1507,8 +1507,8 @@ static cudaError_t make_side(const pxsne_ctx *c, int64_t n, int ld, int Dp, floa
     return cudaGetLastError();
 }
 
-static void free_side(KnnSide &s, cudaStream_t st) {
-    if (s.block) cudaFreeAsync(s.block, st);
+static void free_side(const pxsne_ctx *c, KnnSide &s, cudaStream_t st) {
+    if (s.block) pfree(c, s.block, st);
     s.block = nullptr;
 }
 
@@ -1583,8 +1583,8 @@ cudaError_t launch_knn(pxsne_ctx *c, const float *Xdev, int64_t n, int32_t D, in
             if ((e = cudaMemcpyAsync(hd.data(), dd, (size_t)m * m * sizeof(double),
                                      cudaMemcpyDeviceToHost, st)))
                 return e;
-            if ((e = cudaFreeAsync(dp, st))) return e;
-            if ((e = cudaFreeAsync(dd, st))) return e;
+            if ((e = pfree(c, dp, st))) return e;
+            if ((e = pfree(c, dd, st))) return e;
             if ((e = cudaStreamSynchronize(st))) return e;
         }
         {
@@ -1685,8 +1685,8 @@ cudaError_t launch_knn(pxsne_ctx *c, const float *Xdev, int64_t n, int32_t D, in
             if ((e = scan_u32_to_i64(c, hist, (int64_t)nc * nb, off, st))) return e;
             k_cell_rank<<<(unsigned)nb, kCsRows, 0, st>>>(n, nc, cell, hist, nb, off, order);
             if ((e = cudaGetLastError())) return e;
-            cudaFreeAsync(hist, st);
-            cudaFreeAsync(off, st);
+            pfree(c, hist, st);
+            pfree(c, off, st);
         }
         const int probe = c->p.knn_probe;
         {
@@ -1725,12 +1725,12 @@ cudaError_t launch_knn(pxsne_ctx *c, const float *Xdev, int64_t n, int32_t D, in
                 std::swap(order, order2);
                 std::swap(seg, seg2);
             }
-            cudaFreeAsync(cst, st);
-            cudaFreeAsync(order2, st);
-            cudaFreeAsync(flag, st);
-            cudaFreeAsync(seg, st);
-            cudaFreeAsync(seg2, st);
-            cudaFreeAsync(pref, st);
+            pfree(c, cst, st);
+            pfree(c, order2, st);
+            pfree(c, flag, st);
+            pfree(c, seg, st);
+            pfree(c, seg2, st);
+            pfree(c, pref, st);
         }
         k_gather_rows<<<(unsigned)((n * ld + 255) / 256), 256, 0, st>>>(n, D, ld, order, Xdev, Xs);
         if ((e = cudaGetLastError())) return e;
@@ -1833,25 +1833,25 @@ cudaError_t launch_knn(pxsne_ctx *c, const float *Xdev, int64_t n, int32_t D, in
                                                                 ii, di, io, dout);
                 if ((e = cudaGetLastError())) return e;
             }
-            cudaFreeAsync(rank, st);
-            cudaFreeAsync(idx2, st);
-            cudaFreeAsync(d22, st);
+            pfree(c, rank, st);
+            pfree(c, idx2, st);
+            pfree(c, d22, st);
         }
         if ((e = knn_mark(c, 1, st))) return e;
-        if (cand) cudaFreeAsync(cand, st);
-        free_side(main_side, st);
-        free_side(samp_side, st);
-        if (failed) cudaFreeAsync(failed, st);
-        if (Xsamp) cudaFreeAsync(Xsamp, st);
-        cudaFreeAsync(amax, st);
-        cudaFreeAsync(piv, st);
-        cudaFreeAsync(cell, st);
-        cudaFreeAsync(order, st);
-        cudaFreeAsync(ccnt, st);
-        cudaFreeAsync(dpiv, st);
-        cudaFreeAsync(dsum, st);
-        cudaFreeAsync(Xs, st);
-        return cudaFreeAsync(nrm, st);
+        if (cand) pfree(c, cand, st);
+        free_side(c, main_side, st);
+        free_side(c, samp_side, st);
+        if (failed) pfree(c, failed, st);
+        if (Xsamp) pfree(c, Xsamp, st);
+        pfree(c, amax, st);
+        pfree(c, piv, st);
+        pfree(c, cell, st);
+        pfree(c, order, st);
+        pfree(c, ccnt, st);
+        pfree(c, dpiv, st);
+        pfree(c, dsum, st);
+        pfree(c, Xs, st);
+        return pfree(c, nrm, st);
     }
     c->knn_path = 0;
     const size_t smem = (size_t)D * (kQR + kCT) * 4 + (size_t)kQR * k * 8 + kQR * 4 +
@@ -1864,7 +1864,7 @@ cudaError_t launch_knn(pxsne_ctx *c, const float *Xdev, int64_t n, int32_t D, in
                                                                           idx, d2);
     if ((e = cudaGetLastError())) return e;
     if ((e = knn_mark(c, 1, st))) return e;
-    return cudaFreeAsync(nrm, st);
+    return pfree(c, nrm, st);
 }
 
 // ---------------------------------------------------------------- perplexity
@@ -2034,7 +2034,7 @@ cudaError_t scan_u32_to_i64(const pxsne_ctx *c, const uint32_t *in, int64_t m, i
     k_scan_bsum<<<1, kScanB, 0, st>>>(nb, bsum, bsum + nb);
     k_scan_add<<<(unsigned)((m + 1 + 255) / 256), 256, 0, st>>>(m, out, bsum, bsum + nb);
     if ((e = cudaGetLastError())) return e;
-    return cudaFreeAsync(bsum, st);
+    return pfree(c, bsum, st);
 }
 
 // Row i of the union pattern: its own k entries (j, p_{j|i}) first, then the
@@ -2295,17 +2295,17 @@ cudaError_t build_symmetric_csr(pxsne_ctx *c, const int32_t *idx, const float *p
             k_sort_long<<<hl, 1024, (size_t)most * sizeof(u64), st>>>(hubs, plen, soff, tptr, T, scr,
                                                                       (int)most, ucnt);
             TRY(cudaGetLastError());
-            cudaFreeAsync(soff, st);
-            cudaFreeAsync(scr, st);
+            pfree(c, soff, st);
+            pfree(c, scr, st);
         }
-        cudaFreeAsync(lists, st);
+        pfree(c, lists, st);
     }
     if (c->rp) { cudaFreeAsync(c->rp, st); c->rp = nullptr; }
     if (c->col) { cudaFreeAsync(c->col, st); c->col = nullptr; }
     if (c->val) { cudaFreeAsync(c->val, st); c->val = nullptr; }
     if (c->rowlen) { cudaFreeAsync(c->rowlen, st); c->rowlen = nullptr; }
     // true row lengths and nnz
-    TRY(palloc(c, &c->rowlen, n * sizeof(int32_t), st));
+    TRY(pkeep(c, &c->rowlen, n * sizeof(int32_t), st));
     TRY(cudaMemcpyAsync(c->rowlen, ucnt, n * sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
     int64_t *uscan = nullptr;
     TRY(palloc(c, &uscan, (n + 1) * sizeof(int64_t), st));
@@ -2315,23 +2315,23 @@ cudaError_t build_symmetric_csr(pxsne_ctx *c, const int32_t *idx, const float *p
     // padded offsets
     k_round4<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, ucnt, cursor);
     TRY(cudaGetLastError());
-    TRY(palloc(c, &c->rp, (n + 1) * sizeof(int64_t), st));
+    TRY(pkeep(c, &c->rp, (n + 1) * sizeof(int64_t), st));
     TRY(scan_u32_to_i64(c, cursor, n, c->rp, st));
     TRY(cudaMemcpyAsync(&nnz_pad, c->rp + n, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     TRY(cudaStreamSynchronize(st));
-    TRY(palloc(c, &c->col, (nnz_pad > 0 ? nnz_pad : 4) * sizeof(int32_t), st));
-    TRY(palloc(c, &c->val, (nnz_pad > 0 ? nnz_pad : 4) * sizeof(float), st));
+    TRY(pkeep(c, &c->col, (nnz_pad > 0 ? nnz_pad : 4) * sizeof(int32_t), st));
+    TRY(pkeep(c, &c->val, (nnz_pad > 0 ? nnz_pad : 4) * sizeof(float), st));
     k_sym_write<<<(unsigned)((n * 32 + 255) / 256), 256, 0, st>>>(n, tptr, T, ucnt, c->rp, c->col,
                                                                  c->val);
     TRY(cudaGetLastError());
     c->nnz_pad = nnz_pad;
     c->nnz = nnz;
-    cudaFreeAsync(deg, st);
-    cudaFreeAsync(cursor, st);
-    cudaFreeAsync(tptr, st);
-    cudaFreeAsync(uscan, st);
-    cudaFreeAsync(slot, st);
-    cudaFreeAsync(T, st);
+    pfree(c, deg, st);
+    pfree(c, cursor, st);
+    pfree(c, tptr, st);
+    pfree(c, uscan, st);
+    pfree(c, slot, st);
+    pfree(c, T, st);
 #undef TRY
     return cudaGetLastError();
 }

@@ -30,8 +30,22 @@ int fail(pxsne_ctx *c, int code, const char *fmt, ...) {
     return code;
 }
 
+// Gives back what the pool holds unused beyond kPoolKeep.
+void trim_pool(pxsne_ctx *c) {
+    if (c->pool) cudaMemPoolTrimTo(c->pool, kPoolKeep);
+}
+
+// What a call that ends early holds goes back to the device.
+void give_back(pxsne_ctx *c) {
+    pfree_from(c, 0, c->stream);
+    cudaStreamSynchronize(c->stream);
+    trim_pool(c);
+    cudaGetLastError();
+}
+
 int cuda_fail(pxsne_ctx *c, cudaError_t e, const char *what) {
     cudaGetLastError();
+    if (c) give_back(c);
     return fail(c, e == cudaErrorMemoryAllocation ? PXSNE_E_OOM : PXSNE_E_CUDA, "%s: %s (%s)",
                 what, cudaGetErrorName(e), cudaGetErrorString(e));
 }
@@ -90,9 +104,12 @@ void free_P(pxsne_ctx *c) {
     drop(c->knn_idx); drop(c->knn_d2); drop(c->beta);
 }
 
-// Gives back what the pool holds unused beyond kPoolKeep.
-void trim_pool(pxsne_ctx *c) {
-    if (c->pool) cudaMemPoolTrimTo(c->pool, kPoolKeep);
+// After a failure that left P incomplete: the context holds none.
+void drop_P(pxsne_ctx *c) {
+    free_P(c);
+    c->n = c->nnz = c->nnz_pad = 0;
+    c->knn_k = 0;
+    give_back(c);
 }
 
 // The context's own pool; without one (not supported) the default pool serves.
@@ -423,9 +440,8 @@ const char *pxsne_last_error(const pxsne_ctx *c) {
     return c ? c->err.c_str() : g_create_err.c_str();
 }
 
-int pxsne_affinities(pxsne_ctx *c, const float *X, int64_t n, int32_t D, float perplexity,
-                     int x_on_device) {
-    if (!c) return PXSNE_E_ARG;
+static int affinities(pxsne_ctx *c, const float *X, int64_t n, int32_t D, float perplexity,
+                      int x_on_device, bool &replaced) {
     if (!X) return fail(c, PXSNE_E_ARG, "X is NULL");
     const int k = c->p.k;
     if (n < 2 || n > kMaxN) return fail(c, PXSNE_E_ARG, "n = %lld outside [2, 2^24]", (long long)n);
@@ -450,32 +466,42 @@ int pxsne_affinities(pxsne_ctx *c, const float *X, int64_t n, int32_t D, float p
         CK(c, cudaMemsetAsync(flag, 0, sizeof(unsigned), st));
         CK(c, launch_nonfinite(c, Xuse, n * D, flag, st));
         CK(c, cudaMemcpyAsync(&bad, flag, sizeof(unsigned), cudaMemcpyDeviceToHost, st));
-        CK(c, cudaFreeAsync(flag, st));
+        CK(c, pfree(c, flag, st));
         CK(c, cudaStreamSynchronize(st));
         if (bad) {
-            if (Xd) CK(c, cudaFreeAsync(Xd, st));
+            give_back(c);
             return fail(c, PXSNE_E_ARG, "X has a non-finite entry");
         }
     }
     free_state(c);
     free_P(c);
+    replaced = true;
     c->n = n;
     c->D = D;
     c->nnz = 0;
-    CK(c, palloc(c, &c->knn_idx, (size_t)n * k * sizeof(int32_t), st));
-    CK(c, palloc(c, &c->knn_d2, (size_t)n * k * sizeof(float), st));
-    CK(c, palloc(c, &c->beta, (size_t)n * sizeof(float), st));
+    CK(c, pkeep(c, &c->knn_idx, (size_t)n * k * sizeof(int32_t), st));
+    CK(c, pkeep(c, &c->knn_d2, (size_t)n * k * sizeof(float), st));
+    CK(c, pkeep(c, &c->beta, (size_t)n * sizeof(float), st));
     c->knn_k = k;
     CK(c, launch_knn(c, Xuse, n, D, k, c->knn_idx, c->knn_d2));
-    if (Xd) CK(c, cudaFreeAsync(Xd, st));
+    if (Xd) CK(c, pfree(c, Xd, st));
     float *pcond = nullptr;
     CK(c, palloc(c, &pcond, (size_t)n * k * sizeof(float), st));
     CK(c, launch_perplexity(c, c->knn_d2, n, k, perplexity, pcond, c->beta));
     std::string where;
     cudaError_t e = build_symmetric_csr(c, c->knn_idx, pcond, n, k, where);
     if (e != cudaSuccess) return cuda_fail(c, e, where.c_str());
-    CK(c, cudaFreeAsync(pcond, st));
+    CK(c, pfree(c, pcond, st));
     return check_device(c, nullptr);
+}
+
+int pxsne_affinities(pxsne_ctx *c, const float *X, int64_t n, int32_t D, float perplexity,
+                     int x_on_device) {
+    if (!c) return PXSNE_E_ARG;
+    bool replaced = false;
+    const int rc = affinities(c, X, n, D, perplexity, x_on_device, replaced);
+    if (replaced && (rc == PXSNE_E_OOM || rc == PXSNE_E_CUDA)) drop_P(c);
+    return rc;
 }
 
 int pxsne_set_P(pxsne_ctx *c, int64_t n, const int64_t *row_ptr, const int32_t *col,
@@ -522,16 +548,23 @@ int pxsne_set_P(pxsne_ctx *c, int64_t n, const int64_t *row_ptr, const int32_t *
     c->n = n;
     c->nnz = nnz;
     c->nnz_pad = nnz_pad;
-    CK(c, palloc(c, &c->rp, (n + 1) * 8, c->stream));
-    CK(c, palloc(c, &c->rowlen, n * 4, c->stream));
-    CK(c, palloc(c, &c->col, pc.size() * 4, c->stream));
-    CK(c, palloc(c, &c->val, pv.size() * 4, c->stream));
-    CK(c, cudaMemcpyAsync(c->rp, rp.data(), (n + 1) * 8, cudaMemcpyHostToDevice, c->stream));
-    CK(c, cudaMemcpyAsync(c->rowlen, len.data(), n * 4, cudaMemcpyHostToDevice, c->stream));
-    CK(c, cudaMemcpyAsync(c->col, pc.data(), pc.size() * 4, cudaMemcpyHostToDevice, c->stream));
-    CK(c, cudaMemcpyAsync(c->val, pv.data(), pv.size() * 4, cudaMemcpyHostToDevice, c->stream));
-    CK(c, cudaStreamSynchronize(c->stream));
-    return PXSNE_OK;
+    const auto fill = [&]() -> int {
+        cudaStream_t st = c->stream;
+        CK(c, pkeep(c, &c->rp, (n + 1) * 8, st));
+        CK(c, pkeep(c, &c->rowlen, n * 4, st));
+        CK(c, pkeep(c, &c->col, pc.size() * 4, st));
+        CK(c, pkeep(c, &c->val, pv.size() * 4, st));
+        CK(c, cudaMemcpyAsync(c->rp, rp.data(), (n + 1) * 8, cudaMemcpyHostToDevice, st));
+        CK(c, cudaMemcpyAsync(c->rowlen, len.data(), n * 4, cudaMemcpyHostToDevice, st));
+        CK(c, cudaMemcpyAsync(c->col, pc.data(), pc.size() * 4, cudaMemcpyHostToDevice, st));
+        CK(c, cudaMemcpyAsync(c->val, pv.data(), pv.size() * 4, cudaMemcpyHostToDevice, st));
+        CK(c, cudaStreamSynchronize(st));
+        trim_pool(c);
+        return PXSNE_OK;
+    };
+    const int rc = fill();
+    if (rc) drop_P(c);
+    return rc;
 }
 
 int pxsne_init(pxsne_ctx *c, const float *Y0, int y_on_device, uint64_t seed) {
@@ -557,8 +590,8 @@ int pxsne_init(pxsne_ctx *c, const float *Y0, int y_on_device, uint64_t seed) {
         CK(c, launch_init3(c, Y3, scr));
         rc = prime(c);
         if (rc) return rc;
-        if (Yd3) CK(c, cudaFreeAsync(Yd3, st));
-        CK(c, cudaFreeAsync(scr, st));
+        if (Yd3) CK(c, pfree(c, Yd3, st));
+        CK(c, pfree(c, scr, st));
         rc = check_device(c, nullptr);
         if (rc) c->state_ready = false;
         return rc;
@@ -581,8 +614,8 @@ int pxsne_init(pxsne_ctx *c, const float *Y0, int y_on_device, uint64_t seed) {
     CK(c, launch_init_map(c, Yuse, mm));
     rc = prime(c);
     if (rc) return rc;
-    if (Yd) CK(c, cudaFreeAsync(Yd, st));
-    CK(c, cudaFreeAsync(mm, st));
+    if (Yd) CK(c, pfree(c, Yd, st));
+    CK(c, pfree(c, mm, st));
     rc = check_device(c, nullptr);
     if (rc) {
         c->state_ready = false;
@@ -749,7 +782,7 @@ int pxsne_kl(pxsne_ctx *c, double *out) {
     if (is3(c)) CK(c, launch_kl3(c, d));
     else CK(c, launch_kl(c, d));
     CK(c, cudaMemcpyAsync(out, d, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    CK(c, cudaFreeAsync(d, c->stream));
+    CK(c, pfree(c, d, c->stream));
     return check_device(c, nullptr);
 }
 
@@ -776,14 +809,14 @@ int pxsne_get_Y(pxsne_ctx *c, float *Y, int32_t *pix, int on_device) {
     if (!on_device) {
         if (Y) {
             CK(c, cudaMemcpyAsync(Y, Yd, (size_t)n * row, cudaMemcpyDeviceToHost, st));
-            CK(c, cudaFreeAsync(Yd, st));
+            CK(c, pfree(c, Yd, st));
         }
         if (pix) {
             CK(c, cudaMemcpyAsync(pix, Pd, (size_t)n * row, cudaMemcpyDeviceToHost, st));
-            CK(c, cudaFreeAsync(Pd, st));
+            CK(c, pfree(c, Pd, st));
         }
     }
-    CK(c, cudaFreeAsync(scratch, st));
+    CK(c, pfree(c, scratch, st));
     if (async) {
         CK(c, cudaGetLastError());
         return PXSNE_OK;
@@ -821,9 +854,9 @@ int pxsne_nbr_precision(pxsne_ctx *c, int32_t k, const int32_t *knn_hd, int32_t 
     unsigned long long tot = 0;
     CK(c, cudaMemcpyAsync(&tot, dt, 8, cudaMemcpyDeviceToHost, st));
     if (hits) CK(c, cudaMemcpyAsync(hits, dh, (size_t)n * 4, cudaMemcpyDeviceToHost, st));
-    CK(c, cudaFreeAsync(dh, st));
-    CK(c, cudaFreeAsync(dt, st));
-    if (dk) CK(c, cudaFreeAsync(dk, st));
+    CK(c, pfree(c, dh, st));
+    CK(c, pfree(c, dt, st));
+    if (dk) CK(c, pfree(c, dk, st));
     rc = check_device(c, nullptr);
     if (rc) return rc;
     if (precision) *precision = (double)tot / ((double)k * (double)n);
@@ -930,7 +963,7 @@ int pxsne_get_tree(pxsne_ctx *c, int32_t level, uint32_t *cnt, uint64_t *sx, uin
         CK(c, palloc(c, &d, cells * 4, st));
         CK(c, launch_level_counts(c, level, d));
         CK(c, cudaMemcpyAsync(cnt, d, cells * 4, cudaMemcpyDeviceToHost, st));
-        CK(c, cudaFreeAsync(d, st));
+        CK(c, pfree(c, d, st));
     }
     if (level == c->L && (sx || sy)) {
         u64 *d = nullptr;
@@ -938,14 +971,14 @@ int pxsne_get_tree(pxsne_ctx *c, int32_t level, uint32_t *cnt, uint64_t *sx, uin
         CK(c, launch_leaf_hist(c, nullptr, d, d + cells));
         if (sx) CK(c, cudaMemcpyAsync(sx, d, cells * 8, cudaMemcpyDeviceToHost, st));
         if (sy) CK(c, cudaMemcpyAsync(sy, d + cells, cells * 8, cudaMemcpyDeviceToHost, st));
-        CK(c, cudaFreeAsync(d, st));
+        CK(c, pfree(c, d, st));
     }
     if (morton) {
         uint32_t *d = nullptr;
         CK(c, palloc(c, &d, (size_t)c->n * 4, st));
         CK(c, launch_morton_keys(c, d));
         CK(c, cudaMemcpyAsync(morton, d, (size_t)c->n * 4, cudaMemcpyDeviceToHost, st));
-        CK(c, cudaFreeAsync(d, st));
+        CK(c, pfree(c, d, st));
     }
     return check_device(c, nullptr);
 }
@@ -1257,6 +1290,13 @@ int pxsne_get_params(const pxsne_ctx *c, pxsne_params *p) {
     return PXSNE_OK;
 }
 
+int pxsne_test_alloc_limit(pxsne_ctx *c, int64_t bytes) {
+    if (!c) return PXSNE_E_ARG;
+    if (bytes < 0) return fail(c, PXSNE_E_ARG, "bytes < 0");
+    c->alloc_limit = (size_t)bytes;
+    return PXSNE_OK;
+}
+
 int pxsne_test_stack_limit(pxsne_ctx *c, int32_t entries) {
     if (!c) return PXSNE_E_ARG;
     if (entries != 0 && (entries < 4 || entries > kTravStack))
@@ -1294,15 +1334,15 @@ int pxsne_get_tree3(pxsne_ctx *c, int32_t level, uint32_t *cnt, uint64_t *sx, ui
             if (out[d])
                 CK(c, cudaMemcpyAsync(out[d], ds + d * cells, cells * 8, cudaMemcpyDeviceToHost,
                                       st));
-        CK(c, cudaFreeAsync(dc, st));
-        CK(c, cudaFreeAsync(ds, st));
+        CK(c, pfree(c, dc, st));
+        CK(c, pfree(c, ds, st));
     }
     if (morton) {
         uint32_t *d = nullptr;
         CK(c, palloc(c, &d, (size_t)c->n * 4, st));
         CK(c, launch_morton3(c, d));
         CK(c, cudaMemcpyAsync(morton, d, (size_t)c->n * 4, cudaMemcpyDeviceToHost, st));
-        CK(c, cudaFreeAsync(d, st));
+        CK(c, pfree(c, d, st));
     }
     return check_device(c, nullptr);
 }

@@ -6,7 +6,9 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <cstddef>
 #include <string>
+#include <vector>
 
 #include "pxsne.h"
 
@@ -315,6 +317,8 @@ struct pxsne_ctx {
     bool own_stream = false;
     cudaStream_t side = nullptr;          // stream of the attraction (overlaps the traversal)
     cudaMemPool_t pool = nullptr;         // P, its lists and every call's scratch (palloc)
+    mutable std::vector<void *> scratch;  // what the running call has allocated and not freed
+    size_t alloc_limit = 0;               // test hook: a larger request fails (0: none)
     int stack_limit = 0;                  // host copy of DevScalars::stack_limit
     int sms = 0;                          // streaming multiprocessors of the device
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
@@ -413,12 +417,37 @@ namespace pxsne {
 // at n = 70,000 went from 6.4 to 5.7 ms, at 1M (8 GB of scratch) from 158 to 148.
 constexpr size_t kPoolKeep = size_t(1) << 30;
 template <class T>
-inline cudaError_t palloc(const pxsne_ctx *c, T **p, size_t bytes, cudaStream_t st) {
+inline cudaError_t pkeep(const pxsne_ctx *c, T **p, size_t bytes, cudaStream_t st) {
     void *v = nullptr;
-    const cudaError_t e = c->pool ? cudaMallocFromPoolAsync(&v, bytes, c->pool, st)
-                                  : cudaMallocAsync(&v, bytes, st);
+    cudaError_t e = cudaErrorMemoryAllocation;
+    if (c->alloc_limit == 0 || bytes <= c->alloc_limit)
+        e = c->pool ? cudaMallocFromPoolAsync(&v, bytes, c->pool, st) : cudaMallocAsync(&v, bytes, st);
     *p = static_cast<T *>(v);
     return e;
+}
+// A call's scratch: as pkeep, and recorded until pfree, so that a call that ends
+// early leaves nothing behind (give_back).
+template <class T>
+inline cudaError_t palloc(const pxsne_ctx *c, T **p, size_t bytes, cudaStream_t st) {
+    const cudaError_t e = pkeep(c, p, bytes, st);
+    if (e == cudaSuccess) c->scratch.push_back(*p);
+    return e;
+}
+inline cudaError_t pfree(const pxsne_ctx *c, void *p, cudaStream_t st) {
+    auto &s = c->scratch;
+    for (size_t q = s.size(); q-- > 0;)
+        if (s[q] == p) {
+            s.erase(s.begin() + (std::ptrdiff_t)q);
+            break;
+        }
+    return cudaFreeAsync(p, st);
+}
+// Frees the scratch allocated since it held `from` blocks.
+inline void pfree_from(const pxsne_ctx *c, size_t from, cudaStream_t st) {
+    while (c->scratch.size() > from) {
+        cudaFreeAsync(c->scratch.back(), st);
+        c->scratch.pop_back();
+    }
 }
 cudaError_t launch_init_map(pxsne_ctx *c, const float *Y0dev, uint32_t *mm_scratch);
 // Kernel groups of one iteration, in launch order (timing marks).

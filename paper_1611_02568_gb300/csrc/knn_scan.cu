@@ -713,10 +713,10 @@ cudaError_t launch_knn_scan(const pxsne_ctx *c, const KnnScan &a, int sms, uint3
     if ((e = cudaGetLastError())) return e;
     k_knn_pick<<<pgrid, kPickWarps * 32, smp, st>>>(p);
     if ((e = cudaGetLastError())) return e;
-    cudaFreeAsync(tau, st);
-    cudaFreeAsync(buf, st);
-    cudaFreeAsync(cnt, st);
-    return cudaFreeAsync(flag, st);
+    pfree(c, tau, st);
+    pfree(c, buf, st);
+    pfree(c, cnt, st);
+    return pfree(c, flag, st);
 }
 
 }  // namespace pxsne
