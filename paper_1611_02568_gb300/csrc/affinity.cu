@@ -1782,19 +1782,38 @@ cudaError_t launch_knn(pxsne_ctx *c, const float *Xdev, int64_t n, int32_t D, in
         uint32_t one_pass = (uint32_t)T;  // query tiles of the one-pass search
         if (probe == 0 && knn_scan_takes(n, k, Dp, smem_max)) {
             const int64_t ms = scan_sample_rows(n);
-            if ((e = palloc(c, &Xsamp, (size_t)ms * ld * sizeof(float), st))) return e;
-            k_sample_rows<<<(unsigned)((ms * ld + 255) / 256), 256, 0, st>>>(ms, ld, Xs, Xsamp);
-            if ((e = cudaGetLastError())) return e;
-            if ((e = make_side(c, ms, ld, Dp, scale, 0.f, Xsamp, samp_side, st))) return e;
-            if ((e = palloc(c, &failed, (size_t)(T + 1) * sizeof(uint32_t), st))) return e;
-            const KnnScan sa{main_side.r, samp_side.r, ld,  Dp, k,   inv_s2, kappa,
-                             eps_abs,     order,       idx, d2, err, ka.stats};
-            if ((e = launch_knn_scan(c, sa, c->sms, failed, failed + T, st))) return e;
-            if ((e = cudaMemcpyAsync(&one_pass, failed + T, sizeof(uint32_t), cudaMemcpyDeviceToHost,
-                                     st)))
+            const size_t held = c->scratch.size();
+            auto two_passes = [&]() -> cudaError_t {
+                cudaError_t q;
+                if ((q = palloc(c, &Xsamp, (size_t)ms * ld * sizeof(float), st))) return q;
+                k_sample_rows<<<(unsigned)((ms * ld + 255) / 256), 256, 0, st>>>(ms, ld, Xs, Xsamp);
+                if ((q = cudaGetLastError())) return q;
+                if ((q = make_side(c, ms, ld, Dp, scale, 0.f, Xsamp, samp_side, st))) return q;
+                if ((q = palloc(c, &failed, (size_t)(T + 1) * sizeof(uint32_t), st))) return q;
+                const KnnScan sa{main_side.r, samp_side.r, ld,  Dp, k,   inv_s2, kappa,
+                                 eps_abs,     order,       idx, d2, err, ka.stats};
+                if ((q = launch_knn_scan(c, sa, c->sms, failed, failed + T, st))) return q;
+                if ((q = cudaMemcpyAsync(&one_pass, failed + T, sizeof(uint32_t),
+                                         cudaMemcpyDeviceToHost, st)))
+                    return q;
+                return cudaStreamSynchronize(st);
+            };
+            e = two_passes();
+            if (e == cudaErrorMemoryAllocation) {
+                // no room for the candidates (2.5 KB a row at k = 90): every tile
+                // by the one-pass search, which needs none.  (Nothing that counts
+                // has been launched: the scan allocates first.)
+                cudaGetLastError();
+                pfree_from(c, held, st);
+                Xsamp = nullptr;
+                failed = nullptr;
+                samp_side = KnnSide{};
+                one_pass = (uint32_t)T;
+            } else if (e) {
                 return e;
-            if ((e = cudaStreamSynchronize(st))) return e;
-            ka.qlist = failed;
+            } else {
+                ka.qlist = failed;
+            }
         }
         if (one_pass > 0) {
             k_knn_tc<<<one_pass, kTcThreads, smem_tc, st>>>(ka);

@@ -54,7 +54,8 @@ inline int64_t scan_sample_rows(int64_t n) {
 bool knn_scan_takes(int64_t n, int k, int Dp, int smem_max);
 // Lists of every row into out_idx / out_d2 (by row of X), except for the query
 // tiles written to failed (room for q.T) and counted in *nfailed (device),
-// whose lists are left to the one-pass search.
+// whose lists are left to the one-pass search.  cudaErrorMemoryAllocation: nothing
+// was launched (its scratch is the caller's to free).
 cudaError_t launch_knn_scan(const pxsne_ctx *c, const KnnScan &a, int sms, uint32_t *failed,
                             uint32_t *nfailed, cudaStream_t st);
 

@@ -1,7 +1,9 @@
 """What calls do where device memory is short, and what they hold afterwards:
-calls that end early, and P after a call that could not finish it.
+the neighbour search without room for its candidate buffers, calls that end
+early, and P after a call that could not finish it.
 
-Bars: statuses exactly, and at most the 1 GB that a context may keep, with 100 MB for
+Bars: the search's lists equal (both searches are exact; the data have no ties),
+statuses exactly, and at most the 1 GB that a context may keep, with 100 MB for
 everything else that a process allocates on the side."""
 import numpy as np
 import pytest
@@ -25,6 +27,23 @@ def free_bytes():
     import torch
     torch.cuda.synchronize()
     return torch.cuda.mem_get_info()[0]
+
+
+def test_search_without_room_for_candidates(px):
+    X, _ = datagen.gauss10(5, n=20_000, D=50)
+    with px.Context(px.Params(log2_r=9)) as ctx:
+        ctx.affinities(X)
+        idx, d2, beta = ctx.get_knn()
+        P = ctx.get_P()
+        products = ctx.knn_work()[0]
+        # the buffers take 51 MB, everything else at most 29
+        ctx.test_alloc_limit(40_000_000)
+        ctx.affinities(X)
+        assert ctx.knn_counters()[2] == 1 and ctx.knn_work()[0] != products
+        for a, b in zip((idx, d2, beta, *P), (*ctx.get_knn(), *ctx.get_P())):
+            assert np.array_equal(a, b)
+        skipped, pairs = ctx.knn_pruning()
+        assert 0 < skipped < pairs
 
 
 def test_a_failed_call_leaves_no_P_and_can_be_repeated(px):
