@@ -1739,9 +1739,7 @@ cudaError_t launch_knn(pxsne_ctx *c, const float *Xdev, int64_t n, int32_t D, in
         if ((e = make_side(c, n, ld, Dp, scale, eps_abs, Xs, main_side, st))) return e;
         const int64_t T = main_side.r.T;
         c->knn_tiles = T;
-        if ((e = cudaFuncSetAttribute(k_knn_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)smem_tc)))
-            return e;
+        if ((e = allow_smem(k_knn_tc))) return e;
         KnnTcArgs ka;
         ka.n = n;
         ka.T = T;
@@ -1875,9 +1873,7 @@ cudaError_t launch_knn(pxsne_ctx *c, const float *Xdev, int64_t n, int32_t D, in
     c->knn_path = 0;
     const size_t smem = (size_t)D * (kQR + kCT) * 4 + (size_t)kQR * k * 8 + kQR * 4 +
                         (size_t)(kQR + kKnnThreads / 32) * kCT * 4;
-    if ((e = cudaFuncSetAttribute(k_knn_tile, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)smem)))
-        return e;
+    if ((e = allow_smem(k_knn_tile))) return e;
     if ((e = knn_mark(c, 0, st))) return e;
     k_knn_tile<<<(unsigned)((n + kQR - 1) / kQR), kKnnThreads, smem, st>>>(n, D, k, Xdev, nrm,
                                                                           idx, d2);

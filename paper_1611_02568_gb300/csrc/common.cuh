@@ -449,6 +449,21 @@ inline void pfree_from(const pxsne_ctx *c, size_t from, cudaStream_t st) {
         c->scratch.pop_back();
     }
 }
+// Lets a kernel whose dynamic shared memory depends on the call take all that the
+// device has.  The limit belongs to the process, not to a context: set to each
+// call's own size, a thread with a smaller one lowered it between another's
+// setting and its launch, which then failed.
+template <class F>
+inline cudaError_t allow_smem(F *kernel) {
+    int dev = 0, most = 0;
+    cudaFuncAttributes fa;
+    cudaError_t e;
+    if ((e = cudaGetDevice(&dev))) return e;
+    if ((e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev))) return e;
+    if ((e = cudaFuncGetAttributes(&fa, kernel))) return e;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                most - (int)fa.sharedSizeBytes);
+}
 cudaError_t launch_init_map(pxsne_ctx *c, const float *Y0dev, uint32_t *mm_scratch);
 // Kernel groups of one iteration, in launch order (timing marks).
 enum KernelGroup {

@@ -681,14 +681,10 @@ cudaError_t launch_knn_scan(const pxsne_ctx *c, const KnnScan &a, int sms, uint3
                a.err, a.stats};
     const int sm0 = (int)scan_smem(0, a.Dp, r), sm1 = (int)scan_smem(1, a.Dp, r);
     const auto scan1 = stages(1, a.Dp) == 4 ? k_knn_scan<1, 4> : k_knn_scan<1, 2>;
-    if ((e = cudaFuncSetAttribute(k_knn_scan<0, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  sm0)))
-        return e;
-    if ((e = cudaFuncSetAttribute(scan1, cudaFuncAttributeMaxDynamicSharedMemorySize, sm1)))
-        return e;
     const int smp = (int)pick_smem(a.ld);
-    if ((e = cudaFuncSetAttribute(k_knn_pick, cudaFuncAttributeMaxDynamicSharedMemorySize, smp)))
-        return e;
+    if ((e = allow_smem(k_knn_scan<0, 2>))) return e;
+    if ((e = allow_smem(scan1))) return e;
+    if ((e = allow_smem(k_knn_pick))) return e;
     int per = 1;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_knn_pick, kPickWarps * 32, smp)))
         return e;

@@ -908,8 +908,8 @@ int infer(pxsne_mlp *M, const float *X, int64_t n, float *Y) {
     MCK(M, cudaGetDevice(&dev));
     MCK(M, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const size_t s1 = inf_smem<1>(M->dp), s2 = inf_smem<2>(kH);
-    MCK(M, cudaFuncSetAttribute(k_infer<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s1));
-    MCK(M, cudaFuncSetAttribute(k_infer<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s2));
+    MCK(M, allow_smem(k_infer<1>));
+    MCK(M, allow_smem(k_infer<2>));
     const Layout L = layout(M->d);
     for (int64_t base = 0; base < n; base += kInfRows) {
         InfArgs a{};

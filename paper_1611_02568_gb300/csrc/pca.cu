@@ -357,8 +357,7 @@ bool subspace_device(int D, int b, int iters, const double *dC, double *dwork,
     int per = (D * cb + std::max(sms, 1) - 1) / std::max(sms, 1);
     per = std::min(32, std::max(1, per));
     const size_t mul_smem = (size_t)(per * kMulK + kMulK * 32) * 8;
-    bool ok = ck(cudaFuncSetAttribute(k_chol_inv, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)ch_smem));
+    bool ok = ck(allow_smem(k_chol_inv));
     ok = ok && ck(cudaMemsetAsync(bad, 0, sizeof(int), st));
     ok = ok && ck(cudaMemcpyAsync(dQ, Q.data(), (size_t)D * b * 8, cudaMemcpyHostToDevice, st));
     if (!ok) return false;
