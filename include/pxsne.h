@@ -322,9 +322,11 @@ const char *pxsne_kernel_group_name(int32_t g);
  * of all its iterations (each counted by one extra traversal after that
  * iteration's timed groups): n_accept =
  * accepted (point, cell) pairs (the interactions of Eq. bh_criteria), n_test =
- * tested pairs (accepted + opened + the cell of the point alone), n_warp_steps = warp-level
- * (node, non-empty child) steps, n_nodes = nodes opened by a
- * warp.  Any pointer may be NULL.  Synchronises. */
+ * tested pairs (accepted + opened + the cell of the point alone), n_warp_steps =
+ * the warps' steps, each what a warp tests at once: one non-empty child of a node
+ * for its 32 points (64 with two points per lane), or, below 32,768 points, the
+ * same child of up to 32 nodes of a level for its one point; n_nodes = nodes opened
+ * by a warp.  Any pointer may be NULL.  Synchronises. */
 int pxsne_get_counters(pxsne_ctx *ctx, uint64_t *n_accept, uint64_t *n_test,
                        uint64_t *n_warp_steps, uint64_t *n_nodes);
 

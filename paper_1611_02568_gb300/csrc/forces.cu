@@ -612,14 +612,18 @@ __global__ void __launch_bounds__(kPtWarps * 32)
                 const bool c0 = a0 && (leaf || mine != 4u * m + 2u * p);
                 const bool c1 = a1 && (leaf || mine != 4u * m + 2u * p + 1u);
                 const uint32_t ac = (f0 && c0 && N.x > 0.f ? 1u : 0u) + (f1 && c1 && N.y > 0.f ? 1u : 0u);
+                // a warp step: the lanes that test their nodes' same child at
+                // once, those of each level counted apart
+                const unsigned m0 = __match_any_sync(0xffffffffu, f0 ? lc : -1);
+                const unsigned m1 = __match_any_sync(0xffffffffu, f1 ? lc : -1);
+                const uint32_t st = (f0 && lane == __ffs(m0) - 1 ? 1u : 0u) +
+                                    (f1 && lane == __ffs(m1) - 1 ? 1u : 0u);
                 n_tst += ts;
                 n_acc += ac;
-                n_stp += ts;
-                if (ts) {
-                    atomicAdd(&sc->lvl[lc][0], (u64)ts);
-                    atomicAdd(&sc->lvl[lc][2], (u64)ts);
-                }
+                n_stp += st;
+                if (ts) atomicAdd(&sc->lvl[lc][0], (u64)ts);
                 if (ac) atomicAdd(&sc->lvl[lc][1], (u64)ac);
+                if (st) atomicAdd(&sc->lvl[lc][2], (u64)st);
             }
             const float2 w1 = add2(bc2(1.0f), d2);
             const float2 q = make_float2(rcp1(w1.x), rcp1(w1.y));
