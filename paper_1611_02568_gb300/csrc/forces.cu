@@ -910,9 +910,10 @@ cudaError_t launch_forces(pxsne_ctx *c, cudaEvent_t *marks) {
     return cudaSuccess;
 }
 
-// A sum of FP32 terms carried as an unevaluated pair of floats: the rounding
-// error of every addition is found exactly (Knuth's two-sum) and added to the
-// low word, so that the pair holds about 46 bits.
+// A sum of a few FP32 terms carried as an unevaluated pair of floats: the rounding
+// error of every addition is found exactly (Knuth's two-sum) and added to the low
+// word, whose own roundings leave an error of at most k^2 2^-50 of the terms'
+// absolute sum after k terms.
 struct FloatPair {
     float h, l;
     __device__ __forceinline__ void add(float x) {
@@ -924,10 +925,13 @@ struct FloatPair {
 
 // Eq. cost_func: C = sum_ij p_ij ln(p_ij Z / w_ij)
 //                  = sum p (ln p - ln w) + (sum p) ln Z,
-// one warp per row, FP32 terms accumulated as float pairs per lane and in FP64
-// across lanes and blocks, fixed order.  (FP64 additions and conversions issue
-// at a small fraction of the FP32 rate; 100,000 points, 13.5M entries: 0.40 ms
-// with two of each per entry and the partials added by one thread.)
+// one warp per row, fixed order: a lane adds up to kKlPairs FP32 terms as float
+// pairs, then those to its FP64 sums, so that what the pairs lose (2^-44 of the
+// terms at most) is no more than what FP64 additions of a lane's several hundred
+// terms would.  (FP64 additions and conversions issue at a small fraction of the
+// FP32 rate; 100,000 points, 13.5M entries: 0.40 ms with two of each per entry
+// and the partials added by one thread.)
+constexpr int kKlPairs = 8;
 __global__ void __launch_bounds__(256)
     k_kl(int n, const int64_t *__restrict__ rp, const int32_t *__restrict__ col,
          const float *__restrict__ val, const uint2 *__restrict__ z, DevScalars *sc,
@@ -937,25 +941,31 @@ __global__ void __launch_bounds__(256)
     const int lane = threadIdx.x & 31;
     const int warps_total = gridDim.x * (blockDim.x >> 5);
     const float sf0 = sc->sf[0], sf1 = sc->sf[1];
-    FloatPair acc{0.f, 0.f}, psum{0.f, 0.f};
+    double acc = 0.0, psum = 0.0;
     for (int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); row < n;
          row += warps_total) {
         const uint2 zi = z[row];
         const float xh = hi_bits(zi.x), xl = lo_bits(zi.x);
         const float yh = hi_bits(zi.y), yl = lo_bits(zi.y);
         const int64_t e1 = rp[row + 1];
-        for (int64_t e = rp[row] + lane; e < e1; e += 32) {
-            const float p = __ldcs(val + e);
-            const uint2 zj = z[__ldcs(col + e)];
-            if (!(p > 0.f)) continue;
-            const float dx = ((xh - hi_bits(zj.x)) + (xl - lo_bits(zj.x))) * sf0;
-            const float dy = ((yh - hi_bits(zj.y)) + (yl - lo_bits(zj.y))) * sf1;
-            acc.add(p * (logf(p) + log1pf(fmaf(dx, dx, dy * dy))));
-            psum.add(p);
+        for (int64_t e0 = rp[row] + lane; e0 < e1; e0 += 32 * kKlPairs) {
+            FloatPair a8{0.f, 0.f}, p8{0.f, 0.f};
+            const int64_t e8 = min(e1, e0 + 32 * kKlPairs);
+            for (int64_t e = e0; e < e8; e += 32) {
+                const float p = __ldcs(val + e);
+                const uint2 zj = z[__ldcs(col + e)];
+                if (!(p > 0.f)) continue;
+                const float dx = ((xh - hi_bits(zj.x)) + (xl - lo_bits(zj.x))) * sf0;
+                const float dy = ((yh - hi_bits(zj.y)) + (yl - lo_bits(zj.y))) * sf1;
+                a8.add(p * (logf(p) + log1pf(fmaf(dx, dx, dy * dy))));
+                p8.add(p);
+            }
+            acc += (double)a8.h + (double)a8.l;
+            psum += (double)p8.h + (double)p8.l;
         }
     }
-    const double a = block_sum_f64((double)acc.h + (double)acc.l, s_red);
-    const double ps = block_sum_f64((double)psum.h + (double)psum.l, s_red);
+    const double a = block_sum_f64(acc, s_red);
+    const double ps = block_sum_f64(psum, s_red);
     if (threadIdx.x == 0) {
         part[2 * blockIdx.x] = a;
         part[2 * blockIdx.x + 1] = ps;
