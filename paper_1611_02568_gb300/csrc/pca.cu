@@ -342,7 +342,12 @@ void subspace_host(int D, int b, int iters, const std::vector<double> &C, std::v
 // (positive diagonal here and there), so Cholesky of its Gram matrix gives the
 // columns that Gram-Schmidt does, up to rounding; the last one is done twice,
 // which leaves the columns orthonormal to FP64 rounding.  False: a
-// factorisation broke down (Q and T are not to be used) or an error.
+// factorisation broke down or an error (Q is then the start still).  It does
+// so first where the spectrum spans six decades and more: the first product's
+// columns are all alike there, while later ones have turned to directions of
+// their own.  So the flag is read after the first product: a spectrum falling as
+// 0.85^i costs PCA2MS ms before the host takes over, the whole iteration's 4 to 9
+// otherwise.
 template <class Check>
 bool subspace_device(int D, int b, int iters, const double *dC, double *dwork,
                      std::vector<double> &Q, std::vector<double> &T, cudaStream_t st, Check &&ck) {
@@ -373,22 +378,29 @@ bool subspace_device(int D, int b, int iters, const double *dC, double *dwork,
         mul(y, b, dW, other);
         std::swap(y, other);
     };
+    int hbad = 0;
     orthonormal(dQ, dY);
     for (int it = 0; it < iters; it++) {
         mul(dC, D, dQ, dY);
         std::swap(dQ, dY);
         orthonormal(dQ, dY);
+        if (it == 0) {
+            ok = ck(cudaGetLastError());
+            ok = ok && ck(cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, st));
+            ok = ok && ck(cudaStreamSynchronize(st));
+            if (!ok || hbad) return false;
+        }
     }
     orthonormal(dQ, dY);
     mul(dC, D, dQ, dY);
     k_gram<<<gram_blocks, 256, 0, st>>>(D, b, dQ, dY, dG);
-    int hbad = 0;
     ok = ck(cudaGetLastError());
     ok = ok && ck(cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, st));
-    ok = ok && ck(cudaMemcpyAsync(Q.data(), dQ, (size_t)D * b * 8, cudaMemcpyDeviceToHost, st));
-    ok = ok && ck(cudaMemcpyAsync(T.data(), dG, (size_t)b * b * 8, cudaMemcpyDeviceToHost, st));
     ok = ok && ck(cudaStreamSynchronize(st));
-    return ok && hbad == 0;
+    if (!ok || hbad) return false;
+    ok = ck(cudaMemcpyAsync(Q.data(), dQ, (size_t)D * b * 8, cudaMemcpyDeviceToHost, st));
+    ok = ok && ck(cudaMemcpyAsync(T.data(), dG, (size_t)b * b * 8, cudaMemcpyDeviceToHost, st));
+    return ok && ck(cudaStreamSynchronize(st));
 }
 
 }  // namespace
@@ -451,9 +463,6 @@ extern "C" int pxsne_pca(const float *X, int64_t n, int32_t D, int32_t dout, flo
             std::vector<double> C((size_t)D * D);
             ck(cudaMemcpyAsync(C.data(), dcov, (size_t)D * D * 8, cudaMemcpyDeviceToHost, st));
             ck(cudaStreamSynchronize(st));
-            rng.seed(seed);
-            nd.reset();
-            for (auto &q : Q) q = nd(rng);
             if (rc == PXSNE_OK) subspace_host(D, b, iters, C, Q, T);
         }
         if (rc == PXSNE_OK) {
