@@ -14,8 +14,9 @@
 // k_knn_pick then forms the exact FP32 distances of a row's candidates and
 // sorts them.  tau need not be right: every row at an exact distance of at most
 // tau is among the candidates, so if at least k candidates have one, the k
-// nearest of them are the row's k nearest; where fewer have, or a buffer
-// overflowed, the row's tile goes to the one-pass search.
+// nearest of them are the row's k nearest.  Where fewer have, or a buffer
+// overflowed, the row gets a wider or narrower threshold and its tile a second scan,
+// and where that does not do either, the tile goes to the one-pass search.
 //
 //   k_knn_scan<0>  the sample pass: tau
 //   k_knn_scan<1>  the candidates of every row
@@ -52,8 +53,9 @@ struct ScanArgs {
     float inv_s2, kappa, eps_abs;
     float *tau;             // [n] written by the sample pass, read by the other
     const uint32_t *qlist, *qcount;  // the query tiles to scan and how many; NULL: all
+    const uint32_t *flag;   // with qlist: the tiles' flags, those with kLeft not scanned
     uint32_t *buf;          // [n][2][cap] candidates (ordered positions)
-    uint32_t *cnt;          // [n][2] candidates found (may exceed cap: overflow)
+    uint32_t *cnt;          // [n][2] candidates found (more than cap: the first cap are in buf)
     int cap;
     unsigned *err;
     u64 *stats;
@@ -64,6 +66,16 @@ struct ScanArgs {
 // keeps about four, while its two stages ran dry: with all warps deciding first,
 // the second pass takes 45 ms instead of 56 at n = 1M, D = 128.
 constexpr int kKeepWords = 512;
+
+// A row with up to kHopeless times the candidates that it has room for gets a
+// narrower threshold; beyond, its distances tie or lie within the rounding of its
+// tile's rows, and the tile is left to the one-pass search.  (Whole numbers: 200,000
+// rows of 0 .. 3 in 8 dimensions, P in 34 ms, 57 with all tiles left over and 46
+// by the one-pass search alone; 10 one-hot attributes of 5 values 58, 95 and 85.
+// Where nothing helps the passes are lost: 128 dimensions, 300 off the origin, 428
+// against 426; ending the hopeless scans early saved 2 and cost 1 % of every scan.)
+constexpr uint32_t kHopeless = 4u;
+constexpr uint32_t kAgain = 1u, kLeft = 2u;  // tile flags
 
 // The i-th candidate tile a CTA visits: outward from its own neighbourhood.
 __device__ __forceinline__ int64_t tile_at(int64_t own, int64_t i, int64_t T) {
@@ -127,6 +139,7 @@ __global__ void __launch_bounds__(scan_threads(MODE), 2) k_knn_scan(const ScanAr
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (MODE == 1 && a.qlist && blockIdx.x >= *a.qcount) return;
     const int64_t qt = MODE == 1 && a.qlist ? a.qlist[blockIdx.x] : blockIdx.x, q0 = qt * kTcRows;
+    if (MODE == 1 && a.qlist && (a.flag[qt] & kLeft)) return;
     const int64_t own = MODE == 0 ? min(T - 1, qt / kScanStride) : qt;
 
     if (MODE == 0)
@@ -278,6 +291,7 @@ __global__ void __launch_bounds__(scan_threads(MODE), 2) k_knn_scan(const ScanAr
             // (the second scan's tiles were counted by the first)
             if (MODE == 1 && !a.qlist) atomicAdd(&a.stats[2], n_skip);
             atomicAdd(&a.stats[3], (u64)n_sf);
+            if (MODE == 1 && a.qlist) atomicAdd(&a.stats[4], 1ull);
             // copies still in flight complete before the CTA exits (those of the
             // last kept tiles; after the end mark the copies into the slots it
             // reused are known complete)
@@ -499,14 +513,16 @@ __device__ __forceinline__ void sort_buffer(u64 *keys, int cnt, int lane) {
 struct PickArgs {
     int64_t n;
     int ld, k, cap;
+    float enough;  // k and 3.75 deviations
     const float *X;
-    float *tau;                      // a row that falls short gets a wider one
+    float *tau;                      // a row that falls short gets a wider one, a row
+                                     // with too many a narrower one
     const uint32_t *qlist, *qcount;  // the query tiles to take and how many; NULL: all
     const uint32_t *buf, *cnt, *order;
     int32_t *out_idx;
     float *out_d2;
-    // per query tile, 1: in retry (a second scan with its rows' new
-    // thresholds), 2: in failed (the one-pass search)
+    // per query tile, kAgain: in retry (a second scan with its rows' new
+    // thresholds), kLeft: in failed (the one-pass search)
     uint32_t *flag, *retry, *nretry, *failed, *nfailed;
     unsigned *err;
     u64 *stats;
@@ -541,77 +557,91 @@ __global__ void __launch_bounds__(kPickWarps * 32) k_knn_pick(const PickArgs a) 
          q += (int64_t)gridDim.x * kPickWarps) {
         const int64_t row = a.qlist ? (int64_t)a.qlist[q / kTcRows] * kTcRows + q % kTcRows : q;
         if (row >= a.n) continue;
+        const uint32_t fl = __ldcg(&a.flag[row / kTcRows]);
         const uint32_t c0 = a.cnt[2 * row], c1 = a.cnt[2 * row + 1];
         const float tau = a.tau[row];
+        // a tile that another of its rows has left to the one-pass search
+        if (__any_sync(0xffffffffu, fl & kLeft)) continue;
         const uint32_t *b0 = a.buf + (size_t)row * 2 * a.cap, *b1 = b0 + a.cap;
-        bool good = c0 <= (uint32_t)a.cap && c1 <= (uint32_t)a.cap;
+        // the candidates that are in the buffers, and whether that is all of them
+        const uint32_t m0 = min(c0, (uint32_t)a.cap), tot = m0 + min(c1, (uint32_t)a.cap);
+        const bool all = c0 <= (uint32_t)a.cap && c1 <= (uint32_t)a.cap;
+        bool good = c0 <= kHopeless * (uint32_t)a.cap && c1 <= kHopeless * (uint32_t)a.cap;
         uint32_t kept = 0u;
-        if (good) {
-            const uint32_t tot = c0 + c1;
+        if (good)
             for (int d = lane; d < (a.ld >> 2); d += 32)
                 reinterpret_cast<float4 *>(qrow)[d] =
                     __ldg(reinterpret_cast<const float4 *>(a.X + row * a.ld) + d);
-            for (uint32_t e0 = 0u; e0 < tot; e0 += 32u) {
-                const uint32_t e = e0 + lane, m = min(32u, tot - e0);
-                const uint32_t cand = e < tot ? (e < c0 ? b0[e] : b1[e - c0]) : 0u;
-                __syncwarp();
-                tc::fence_proxy_async();
-                if (lane == 0) tc::mbar_expect_tx(bar, m * bytes);
-                __syncwarp();
-                if (e < tot) tc::bulk_g2s(rows + lane * ls, a.X + (int64_t)cand * a.ld, bytes, bar);
-                ok = __all_sync(0xffffffffu, tc::mbar_wait(bar, phase & 1u, kTcPolls));
-                phase++;
-                if (!ok) break;
-                float s = 0.f;
-                const float4 *pc = reinterpret_cast<const float4 *>(rows + lane * ls);
-                const float4 *pq = reinterpret_cast<const float4 *>(qrow);
+        for (uint32_t e0 = 0u; good && e0 < tot; e0 += 32u) {
+            const uint32_t e = e0 + lane, m = min(32u, tot - e0);
+            const uint32_t cand = e < tot ? (e < m0 ? b0[e] : b1[e - m0]) : 0u;
+            __syncwarp();
+            tc::fence_proxy_async();
+            if (lane == 0) tc::mbar_expect_tx(bar, m * bytes);
+            __syncwarp();
+            if (e < tot) tc::bulk_g2s(rows + lane * ls, a.X + (int64_t)cand * a.ld, bytes, bar);
+            ok = __all_sync(0xffffffffu, tc::mbar_wait(bar, phase & 1u, kTcPolls));
+            phase++;
+            if (!ok) break;
+            float s = 0.f;
+            const float4 *pc = reinterpret_cast<const float4 *>(rows + lane * ls);
+            const float4 *pq = reinterpret_cast<const float4 *>(qrow);
 #pragma unroll 8
-                for (int d = 0; d < (a.ld >> 2); d++) {
-                    const float4 u = pq[d], v = pc[d];
-                    float t = u.x - v.x;
-                    s = fmaf(t, t, s);
-                    t = u.y - v.y;
-                    s = fmaf(t, t, s);
-                    t = u.z - v.z;
-                    s = fmaf(t, t, s);
-                    t = u.w - v.w;
-                    s = fmaf(t, t, s);
-                }
-                const bool in = e < tot && s <= tau;
-                const unsigned im = __ballot_sync(0xffffffffu, in);
-                const uint32_t at = kept + __popc(im & ((1u << lane) - 1u));
-                if (in && at < (uint32_t)kPickKeys)
-                    keys[at] = ((u64)__float_as_uint(s) << 32) | __ldg(a.order + cand);
-                kept += __popc(im);
+            for (int d = 0; d < (a.ld >> 2); d++) {
+                const float4 u = pq[d], v = pc[d];
+                float t = u.x - v.x;
+                s = fmaf(t, t, s);
+                t = u.y - v.y;
+                s = fmaf(t, t, s);
+                t = u.z - v.z;
+                s = fmaf(t, t, s);
+                t = u.w - v.w;
+                s = fmaf(t, t, s);
             }
-            if (ok) {
-                n_exact += tot;
-                n_kept += kept;
-            }
-            good = ok && kept <= (uint32_t)kPickKeys;
+            const bool in = e < tot && s <= tau;
+            const unsigned im = __ballot_sync(0xffffffffu, in);
+            const uint32_t at = kept + __popc(im & ((1u << lane) - 1u));
+            if (in && at < (uint32_t)kPickKeys)
+                keys[at] = ((u64)__float_as_uint(s) << 32) | __ldg(a.order + cand);
+            kept += __popc(im);
         }
+        good = good && ok;
         __syncwarp();
+        const uint32_t have = min(kept, (uint32_t)kPickKeys);
         if (good) {
-            if (kept <= 256u) sort_buffer<8>(keys, (int)kept, lane);
-            else sort_buffer<16>(keys, (int)kept, lane);
+            n_exact += tot;
+            if (have <= 256u) sort_buffer<8>(keys, (int)have, lane);
+            else sort_buffer<16>(keys, (int)have, lane);
         }
-        if (!good || kept < (uint32_t)a.k) {
-            if (lane == 0) {
-                const uint32_t t = (uint32_t)(row / kTcRows);
-                // half as many rows lie within keys[kept / 2]: the same factor
-                // again should about double them
-                float wider = 0.f;
-                if (good && a.retry && kept >= 8u) {
-                    const float half = __uint_as_float((uint32_t)(keys[kept >> 1] >> 32));
-                    wider = half > 0.f ? tau * (tau / half) : 0.f;
+        if (!good || !all || kept != have || kept < (uint32_t)a.k) {
+            // A threshold that should do.  Too many candidates: the k-th nearest of
+            // those that were sorted bounds the k-th nearest; where they are a part,
+            // so in all likelihood does the one that as large a part of `enough`
+            // reach.  Too few: half of them lie within keys[kept / 2], so the same
+            // factor again should about double them.
+            float next = -1.f;
+            if (good && (kept != have || !all)) {
+                const float of = all ? (float)kept : (float)(c0 + c1) * (float)kept / (float)tot;
+                const int at = min(a.k - 1, (int)(a.enough * (float)have / of));
+                if ((uint32_t)at < have) {
+                    const float v = __uint_as_float((uint32_t)(keys[at] >> 32));
+                    if (v < tau) next = v;
                 }
-                if (wider > tau && wider < 3.402823466e38f) {
-                    a.tau[row] = wider;
-                    if (atomicOr(&a.flag[t], 1u) == 0u) {
-                        a.retry[atomicAdd(a.nretry, 1u)] = t;
-                        atomicAdd(&a.stats[4], 1ull);
-                    }
-                } else if (!(atomicOr(&a.flag[t], 2u) & 2u)) {
+            } else if (good && a.retry && kept >= 8u) {
+                const float half = __uint_as_float((uint32_t)(keys[kept >> 1] >> 32));
+                const float wider = half > 0.f ? tau * (tau / half) : 0.f;
+                if (wider > tau && wider < 3.402823466e38f) next = wider;
+            }
+            const uint32_t t = (uint32_t)(row / kTcRows);
+            if (next >= 0.f && all && kept != have) {
+                // all its candidates are at hand: the same row again
+                if (lane == 0) a.tau[row] = next;
+                q -= (int64_t)gridDim.x * kPickWarps;
+            } else if (lane == 0) {
+                if (next >= 0.f && a.retry) {
+                    a.tau[row] = next;
+                    if (!(atomicOr(&a.flag[t], kAgain) & kAgain)) a.retry[atomicAdd(a.nretry, 1u)] = t;
+                } else if (!(atomicOr(&a.flag[t], kLeft) & kLeft)) {
                     a.failed[atomicAdd(a.nfailed, 1u)] = t;
                     atomicAdd(&a.stats[5], 1ull);
                 }
@@ -620,6 +650,7 @@ __global__ void __launch_bounds__(kPickWarps * 32) k_knn_pick(const PickArgs a) 
             __syncwarp();
             continue;
         }
+        n_kept += kept;
         const int64_t orow = a.order[row];
         for (int e = lane; e < a.k; e += 32) {
             const u64 v = keys[e];
@@ -677,7 +708,7 @@ cudaError_t launch_knn_scan(const pxsne_ctx *c, const KnnScan &a, int sms, uint3
     // (a scan that gives up leaves its rows without candidates)
     if ((e = cudaMemsetAsync(tau, 0, (size_t)n * 4, st))) return e;
     if ((e = cudaMemsetAsync(cnt, 0, (size_t)n * 2 * 4, st))) return e;
-    ScanArgs s{a.q, a.s, a.Dp, r, a.inv_s2, a.kappa, a.eps_abs, tau, nullptr, nullptr, buf, cnt, cap,
+    ScanArgs s{a.q, a.s, a.Dp, r, a.inv_s2, a.kappa, a.eps_abs, tau, nullptr, nullptr, flag, buf, cnt, cap,
                a.err, a.stats};
     const int sm0 = (int)scan_smem(0, a.Dp, r), sm1 = (int)scan_smem(1, a.Dp, r);
     const auto scan1 = stages(1, a.Dp) == 4 ? k_knn_scan<1, 4> : k_knn_scan<1, 2>;
@@ -696,11 +727,11 @@ cudaError_t launch_knn_scan(const pxsne_ctx *c, const KnnScan &a, int sms, uint3
     s.c = a.q;
     scan1<<<(unsigned)T, scan_threads(1), sm1, st>>>(s);
     if ((e = cudaGetLastError())) return e;
-    PickArgs p{n, a.ld, a.k, cap, a.q.X, tau, nullptr, nullptr, buf, cnt, a.order, a.out_idx, a.out_d2,
+    PickArgs p{n, a.ld, a.k, cap, (float)a.k + 3.75f * std::sqrt((float)a.k) + 1.f, a.q.X, tau, nullptr, nullptr, buf, cnt, a.order, a.out_idx, a.out_d2,
                flag, retry, nretry, failed, nfailed, a.err, a.stats};
     k_knn_pick<<<pgrid, kPickWarps * 32, smp, st>>>(p);
     if ((e = cudaGetLastError())) return e;
-    // the tiles with a row that fell short, once more (their number is on the
+    // the tiles with a row that fell short or had too many, once more (their number is on the
     // device: CTAs past it return at once)
     s.qlist = p.qlist = retry;
     s.qcount = p.qcount = nretry;
