@@ -436,6 +436,10 @@ __host__ __device__ constexpr size_t inf_smem(int K) {
     return (size_t)kH * K * 2 + (size_t)inf_stages<LAYER>(K) * kReg + 1024;
 }
 
+static_assert(inf_smem<1>(64) <= inf_smem<1>(kInfMaxK) && inf_smem<1>(128) <= inf_smem<1>(kInfMaxK) &&
+                  inf_smem<1>(192) <= inf_smem<1>(kInfMaxK),
+              "shared memory limit of the prediction");
+
 struct InfArgs {
     int64_t rows, tiles;
     int d, K;                 // input width and its padding to 64 (LAYER 2: 256)
@@ -908,8 +912,11 @@ int infer(pxsne_mlp *M, const float *X, int64_t n, float *Y) {
     MCK(M, cudaGetDevice(&dev));
     MCK(M, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const size_t s1 = inf_smem<1>(M->dp), s2 = inf_smem<2>(kH);
-    MCK(M, allow_smem(k_infer<1>));
-    MCK(M, allow_smem(k_infer<2>));
+    // (the same limit from every network: that of the widest input, which the
+    // narrower ones' stages stay below)
+    MCK(M, cudaFuncSetAttribute(k_infer<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)inf_smem<1>(kInfMaxK)));
+    MCK(M, cudaFuncSetAttribute(k_infer<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s2));
     const Layout L = layout(M->d);
     for (int64_t base = 0; base < n; base += kInfRows) {
         InfArgs a{};
