@@ -39,9 +39,14 @@ constexpr int64_t kTravPairFrom = 150000;
 // on 512^2 3,979, 4,150, 3,863; 400,000 2,271, 2,379, 2,353; 700,000 on 1024^2
 // 1,291, 1,316, 1,335; 1M on 512^2 964, 1,008, 1,025, on 1024^2 921, 941, 974).
 // Spread-out states of a sparse screen pay for it (1M on 2048^2: 1.58, 1.75 and
-// 1.73 ms an iteration).
+// 1.73 ms an iteration).  The pixels are those of the r_1 x r_2 screen: iterations
+// 300 to 600 of 1.1M points on 1920 x 1080 run at 850 it/s so, 800 as if on the whole
+// 2048^2; 2M at 460 and 428.
 constexpr int64_t kTravCrowdedPair = 600000;
-inline bool trav_crowded(int64_t n, int L) { return 2 * n >= (int64_t(1) << (2 * L)); }
+inline bool trav_crowded(int64_t n, int L, int rx, int ry) {
+    const int64_t side = int64_t(1) << L;
+    return 2 * n >= (rx > 0 ? rx : side) * (ry > 0 ? ry : side);
+}
 // Persistent grids of the forces: CTAs per SM of the traversal and of the
 // attraction that runs beside it on the side stream.  They share the registers
 // (20 + 20 warps at 56 and 40) and the data pipe of L1, which each alone keeps
