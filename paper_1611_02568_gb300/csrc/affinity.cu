@@ -3,7 +3,9 @@
 //   k_knn_tc       brute-force k nearest neighbours on the tensor cores: FP16
 //                  dot-product tiles (tcgen05, FP32 accumulator in TMEM) filter
 //                  candidates with a rigorous error bound; survivors are
-//                  re-ranked with exact FP32 distances (the default path)
+//                  re-ranked with exact FP32 distances.  One pass, for what the
+//                  two passes of knn_scan.cu (the default path) do not take or
+//                  leave over, and for the approximate search
 //   k_knn_tile     the same search on FP32 CUDA cores (check path): a 64 x 128 tile of
 //                  approximate squared distances |q|^2 + |c|^2 - 2 q.c (FP32
 //                  dot products) filters candidates against each row's current

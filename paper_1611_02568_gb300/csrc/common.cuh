@@ -82,7 +82,7 @@ struct DevScalars {
     unsigned pyr_ticket; // last-block-done counter of the pyramid's first pass
     int stack_limit;     // entries of a traversal warp's stack in use (0: all
                          // kTravStack; lowered only by pxsne_test_stack_limit)
-    unsigned trav_next;  // next 64-point chunk of the traversal (0 between launches)
+    unsigned trav_next;  // next chunk of 32 or 64 points of the traversal (0 between launches)
     unsigned trav_done;  // traversal warps finished (the last one resets both)
     unsigned att_next;   // the same two counters for the attraction's row chunks
     unsigned att_done;

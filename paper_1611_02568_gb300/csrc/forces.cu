@@ -1,15 +1,16 @@
 // Forces of the PixelSNE gradient (Eq. grad) on the pixel-aligned tree.
 //
 //   k_bh_traverse  repulsion by Barnes-Hut (Sec. 3.3, Eq. bh_criteria) on the
-//                  dense pyramid, one warp per 32 points in tree order
-//                  (64 with geometric centres), the siblings as packed FP32
-//                  pairs; each point keeps its own accept/open decisions (lane
-//                  masks per stack entry), so it sees exactly the cells its
-//                  own depth-first search would
+//                  dense pyramid, one warp per 32 points in tree order (64
+//                  for large sets with geometric centres or on a crowded
+//                  screen), the siblings as packed FP32 pairs; each point
+//                  keeps its own accept/open decisions (lane masks per stack
+//                  entry), so it sees exactly the cells its own depth-first
+//                  search would
 //   k_bh_traverse_pt  the same for small sets, one warp per point
 //   k_attract      attraction over the CSR of P, one warp per row
 //   k_zsum         Z = sum_i Z_i in FP64, fixed summation order
-//   k_kl           Eq. cost_func in FP64 accumulation
+//   k_kl           Eq. cost_func, FP64 sums of a few terms' float pairs
 #include <algorithm>
 #include <cmath>
 
@@ -227,7 +228,8 @@ struct __align__(16) TravEntry<2> {
 
 // The threshold's term for cells of one point (single_base; geometric centres: no
 // such rule).  It is read with the level's threshold where it is no constant: a
-// register for it across the walk cost 1.5 % of an iteration at n = 70,000.
+// register for it across the walk, or a load of its own, cost 1.6 % of an iteration
+// at n = 70,000.
 template <int CENTRE, bool OWN>
 __device__ __forceinline__ constexpr bool trav_const() {
     return CENTRE != 0 || OWN;
@@ -516,8 +518,8 @@ __global__ void __launch_bounds__(kTravWarps * 32, 16)
 // tree one node after another, and the time is that chain's latency.  Here the
 // lanes take up to 32 of the point's open nodes at a time (all four children
 // of a node as two packed pairs), so that the chain is about one step per
-// level: 5 us instead of 55 at n = 2000 (20 iterations 0.93 ms, 2.05 with the
-// kernel above).  The open nodes wait in a ring in shared memory, taken oldest first
+// level: 5 us instead of 55 at n = 2000 (20 iterations 0.93 ms when it came, 2.05
+// with the kernel above; 0.72 with the smaller steps since).  The open nodes wait in a ring in shared memory, taken oldest first
 // (breadth first); above kPtDeep waiting nodes the newest are taken first,
 // which bounds the ring: such a step takes the 32 newest, of level l or deeper,
 // and puts at most 128 of level l + 1 or deeper in their place, so that a

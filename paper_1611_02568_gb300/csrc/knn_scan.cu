@@ -110,8 +110,8 @@ __device__ __forceinline__ float pick32(const uint32_t (&v)[32], int j) {
 // MODE 0: the sample pass; MODE 1: the candidates.  One CTA per 128 query rows,
 // warp roles as in the one-pass search: a loader that skips tiles beyond the
 // rows' thresholds (triangle inequality on centroids and radii) and streams
-// the others into shared memory by bulk copies, an MMA issuer, and eight
-// filter warps, two per quarter of the rows.  A value costs a packed half FMA
+// the others into shared memory by bulk copies, an MMA issuer, and the filter
+// warps, one (MODE 0) or two (MODE 1) per quarter of the rows.  A value costs a packed half FMA
 // and add and one funnel shift that collects the sign bits of e_j - t, e_j =
 // (1-eps)|c~_j|^2 - 2 q~.c~_j, with the chunk's largest kappa |q~||c~| in t.
 template <int MODE, int kStages>

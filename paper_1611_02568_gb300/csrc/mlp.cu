@@ -425,19 +425,17 @@ constexpr int kInfMaxK = 256;                            // widest padded input
 constexpr int64_t kInfRows = 131072;                     // rows of H1 kept (64 MB)
 constexpr uint32_t kReg = 128 * 128;                     // bytes of 128 rows x 64 columns
 
-template <int LAYER>
 __host__ __device__ constexpr int inf_stages(int K) {
     // 128 x 64 operand regions in flight: two tiles, or as many as fit beside
     // the weights
     return K <= 128 ? 2 * (K / 64) : 5;
 }
-template <int LAYER>
 __host__ __device__ constexpr size_t inf_smem(int K) {
-    return (size_t)kH * K * 2 + (size_t)inf_stages<LAYER>(K) * kReg + 1024;
+    return (size_t)kH * K * 2 + (size_t)inf_stages(K) * kReg + 1024;
 }
 
-static_assert(inf_smem<1>(64) <= inf_smem<1>(kInfMaxK) && inf_smem<1>(128) <= inf_smem<1>(kInfMaxK) &&
-                  inf_smem<1>(192) <= inf_smem<1>(kInfMaxK),
+static_assert(inf_smem(64) <= inf_smem(kInfMaxK) && inf_smem(128) <= inf_smem(kInfMaxK) &&
+                  inf_smem(192) <= inf_smem(kInfMaxK),
               "shared memory limit of the prediction");
 
 struct InfArgs {
@@ -465,7 +463,7 @@ __global__ void __launch_bounds__(kInfThreads, 1) k_infer(const InfArgs a) {
     __shared__ float s_bias[kH], s_w3[2][kH];
     __shared__ float s_part[LAYER == 2 ? 4 : 1][128][2];
     uint8_t *smem = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
-    const int K = a.K, regions = K / 64, NS = inf_stages<LAYER>(K);
+    const int K = a.K, regions = K / 64, NS = inf_stages(K);
     uint8_t *sW = smem, *sA = smem + (size_t)kH * K * 2;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     for (int q = tid; q < kH * (K / 8); q += kInfThreads) {
@@ -911,11 +909,11 @@ int infer(pxsne_mlp *M, const float *X, int64_t n, float *Y) {
     int sms = 0, dev = 0;
     MCK(M, cudaGetDevice(&dev));
     MCK(M, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const size_t s1 = inf_smem<1>(M->dp), s2 = inf_smem<2>(kH);
+    const size_t s1 = inf_smem(M->dp), s2 = inf_smem(kH);
     // (the same limit from every network: that of the widest input, which the
     // narrower ones' stages stay below)
     MCK(M, cudaFuncSetAttribute(k_infer<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)inf_smem<1>(kInfMaxK)));
+                                (int)inf_smem(kInfMaxK)));
     MCK(M, cudaFuncSetAttribute(k_infer<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s2));
     const Layout L = layout(M->d);
     for (int64_t base = 0; base < n; base += kInfRows) {
