@@ -148,7 +148,10 @@ const char *pxsne_last_error(const pxsne_ctx *ctx);
  * unsupported size returns an error).  perplexity <= 0 uses the
  * context's parameter.  Replaces any previous P and clears the embedding
  * state.  Synchronises.  A non-finite entry of X (checked on the device)
- * returns PXSNE_E_ARG and leaves the context as it was.  Row convergence
+ * returns PXSNE_E_ARG and leaves the context as it was.  Where squared distances
+ * of a row's k nearest are beyond FP32 (entries around 1e19 and more) and its list
+ * cannot be filled, the call returns PXSNE_E_ARG, too, and leaves the context
+ * without P.  Row convergence
  * failures set PXSNE_DEVERR_BISECT and return PXSNE_E_DEVICE (P is still
  * built from the last bracket). */
 int pxsne_affinities(pxsne_ctx *ctx, const float *X, int64_t n, int32_t D,

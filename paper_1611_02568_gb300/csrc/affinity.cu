@@ -779,7 +779,9 @@ __global__ void __launch_bounds__(kCandThreads)
                     const float e2 = s_cq[4 * d4 + 2] - c.z, e3 = s_cq[4 * d4 + 3] - c.w;
                     dd = fmaf(e0, e0, fmaf(e1, e1, fmaf(e2, e2, fmaf(e3, e3, dd))));
                 }
-                b = dd;
+                // (a distance that overflows is a far one: W tiles are listed
+                // whatever the rows hold)
+                b = dd < 3.402823466e38f ? dd : 3.402823466e38f;
             }
             if (b < s_thr) {
                 const int slot = atomicAdd(&s_cnt, 1);
@@ -1980,11 +1982,16 @@ cudaError_t launch_perplexity(pxsne_ctx *c, const float *d2, int64_t n, int32_t 
 
 // ---------------------------------------------------------------- symmetrize
 // In-degrees, and every entry's place among its target's incoming ones (one
-// atomic per entry serves both).
-__global__ void k_indeg(int64_t nk, const int32_t *__restrict__ idx, uint32_t *deg,
-                        uint32_t *__restrict__ slot) {
+// atomic per entry serves both).  A list that the search could not fill (its row's
+// squared distances overflow FP32, or a wait of the search timed out) ends in
+// entries that name no row: they are counted in *unfilled and not followed.
+__global__ void k_indeg(int64_t nk, int64_t n, const int32_t *__restrict__ idx, uint32_t *deg,
+                        uint32_t *__restrict__ slot, uint32_t *unfilled) {
     const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e < nk) slot[e] = atomicAdd(&deg[idx[e]], 1u);
+    if (e >= nk) return;
+    const uint32_t j = (uint32_t)idx[e];
+    if ((int64_t)j < n) slot[e] = atomicAdd(&deg[j], 1u);
+    else atomicAdd(unfilled, 1u);
 }
 
 // Exclusive scan of 32-bit counts into int64 offsets: per-block scan, then a
@@ -2070,7 +2077,7 @@ __global__ void k_fill(int64_t n, int k, const int32_t *__restrict__ idx,
     const int32_t j = idx[e];
     const float p = pcond[e];
     T[tptr[i] + a] = sym_key(j, p);
-    T[tptr[j] + k + slot[e]] = sym_key((int32_t)i, p);
+    if ((uint64_t)(uint32_t)j < (uint64_t)n) T[tptr[j] + k + slot[e]] = sym_key((int32_t)i, p);
 }
 
 // Each row's keys in column order, equal columns merged in place (a column
@@ -2235,7 +2242,7 @@ __global__ void k_add_const(int64_t n, const uint32_t *in, uint32_t *out, uint32
 }
 
 cudaError_t build_symmetric_csr(pxsne_ctx *c, const int32_t *idx, const float *pcond,
-                                int64_t n, int32_t k, std::string &err) {
+                                int64_t n, int32_t k, std::string &err, uint32_t &unfilled) {
     cudaStream_t st = c->stream;
     cudaError_t e;
     const int64_t nk = n * k;
@@ -2254,7 +2261,13 @@ cudaError_t build_symmetric_csr(pxsne_ctx *c, const int32_t *idx, const float *p
     TRY(palloc(c, &tptr, (n + 1) * sizeof(int64_t), st));
     TRY(cudaMemsetAsync(deg, 0, n * sizeof(uint32_t), st));
     TRY(palloc(c, &slot, nk * sizeof(uint32_t), st));
-    k_indeg<<<(unsigned)((nk + 255) / 256), 256, 0, st>>>(nk, idx, deg, slot);
+    // three lists of the longer rows and the hubs' padded lengths, then their
+    // counts and that of the entries that name no row
+    uint32_t *lists = nullptr;
+    TRY(palloc(c, &lists, ((size_t)n * 4 + 4) * sizeof(uint32_t), st));
+    uint32_t *num = lists + (size_t)n * 4, *hubs = lists + 2 * (size_t)n, *plen = lists + 3 * (size_t)n;
+    TRY(cudaMemsetAsync(num, 0, 4 * sizeof(uint32_t), st));
+    k_indeg<<<(unsigned)((nk + 255) / 256), 256, 0, st>>>(nk, n, idx, deg, slot, num + 3);
     TRY(cudaGetLastError());
     // temporary rows of length k + indeg(i); 2 n k entries in total
     uint32_t *len = cursor;
@@ -2270,16 +2283,14 @@ cudaError_t build_symmetric_csr(pxsne_ctx *c, const int32_t *idx, const float *p
     TRY(cudaGetLastError());
     {
         // the longer rows
-        uint32_t *lists = nullptr;  // three lists and the hubs' padded lengths, then their counts
-        TRY(palloc(c, &lists, ((size_t)n * 4 + 4) * sizeof(uint32_t), st));
-        uint32_t *num = lists + (size_t)n * 4, *hubs = lists + 2 * (size_t)n, *plen = lists + 3 * (size_t)n;
-        TRY(cudaMemsetAsync(num, 0, 4 * sizeof(uint32_t), st));
         k_long_rows<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, tptr, lists, lists + n, hubs, num,
                                                                  plen);
         TRY(cudaGetLastError());
         uint32_t hn[4] = {0u, 0u, 0u, 0u};
         TRY(cudaMemcpyAsync(hn, num, sizeof(hn), cudaMemcpyDeviceToHost, st));
         TRY(cudaStreamSynchronize(st));
+        unfilled = hn[3];
+        if (unfilled > 0) return cudaSuccess;  // (the caller gives the scratch back)
         if (hn[0] > 0)
             k_sym_rows<16><<<(hn[0] + kSymWarps - 1) / kSymWarps, kSymWarps * 32, 0, st>>>(
                 hn[0], lists, tptr, T, ucnt);

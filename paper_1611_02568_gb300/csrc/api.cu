@@ -441,7 +441,7 @@ const char *pxsne_last_error(const pxsne_ctx *c) {
 }
 
 static int affinities(pxsne_ctx *c, const float *X, int64_t n, int32_t D, float perplexity,
-                      int x_on_device, bool &replaced) {
+                      int x_on_device, bool &replaced, bool &lost) {
     if (!X) return fail(c, PXSNE_E_ARG, "X is NULL");
     const int k = c->p.k;
     if (n < 2 || n > kMaxN) return fail(c, PXSNE_E_ARG, "n = %lld outside [2, 2^24]", (long long)n);
@@ -489,8 +489,19 @@ static int affinities(pxsne_ctx *c, const float *X, int64_t n, int32_t D, float 
     CK(c, palloc(c, &pcond, (size_t)n * k * sizeof(float), st));
     CK(c, launch_perplexity(c, c->knn_d2, n, k, perplexity, pcond, c->beta));
     std::string where;
-    cudaError_t e = build_symmetric_csr(c, c->knn_idx, pcond, n, k, where);
+    uint32_t unfilled = 0u;
+    cudaError_t e = build_symmetric_csr(c, c->knn_idx, pcond, n, k, where, unfilled);
     if (e != cudaSuccess) return cuda_fail(c, e, where.c_str());
+    if (unfilled > 0) {
+        lost = true;
+        give_back(c);
+        uint32_t flags = 0u;
+        const int rc = check_device(c, &flags);
+        if (rc && (flags & PXSNE_DEVERR_TIMEOUT)) return rc;
+        return fail(c, PXSNE_E_ARG,
+                    "squared distances of X overflow: %u neighbour-list entries could not be filled",
+                    unfilled);
+    }
     CK(c, pfree(c, pcond, st));
     return check_device(c, nullptr);
 }
@@ -498,9 +509,10 @@ static int affinities(pxsne_ctx *c, const float *X, int64_t n, int32_t D, float 
 int pxsne_affinities(pxsne_ctx *c, const float *X, int64_t n, int32_t D, float perplexity,
                      int x_on_device) {
     if (!c) return PXSNE_E_ARG;
-    bool replaced = false;
-    const int rc = affinities(c, X, n, D, perplexity, x_on_device, replaced);
-    if (replaced && (rc == PXSNE_E_OOM || rc == PXSNE_E_CUDA)) drop_P(c);
+    // replaced: the P before is gone; lost: the new one cannot be had
+    bool replaced = false, lost = false;
+    const int rc = affinities(c, X, n, D, perplexity, x_on_device, replaced, lost);
+    if (lost || (replaced && (rc == PXSNE_E_OOM || rc == PXSNE_E_CUDA))) drop_P(c);
     return rc;
 }
 

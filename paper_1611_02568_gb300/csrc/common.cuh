@@ -514,7 +514,7 @@ cudaError_t launch_knn(pxsne_ctx *c, const float *Xdev, int64_t n, int32_t D, in
 cudaError_t launch_perplexity(pxsne_ctx *c, const float *d2, int64_t n, int32_t k,
                               float perplexity, float *pcond, float *beta);
 cudaError_t build_symmetric_csr(pxsne_ctx *c, const int32_t *idx, const float *pcond,
-                                int64_t n, int32_t k, std::string &err);
+                                int64_t n, int32_t k, std::string &err, uint32_t &unfilled);
 cudaError_t launch_level_counts(pxsne_ctx *c, int level, uint32_t *cnt);
 // counts and exact coordinate sums of the leaves of the current state (any may be NULL)
 cudaError_t launch_leaf_hist(pxsne_ctx *c, uint32_t *cnt, u64 *sx, u64 *sy);

@@ -574,7 +574,10 @@ __global__ void __launch_bounds__(kPickWarps * 32) k_knn_pick(const PickArgs a) 
                     __ldg(reinterpret_cast<const float4 *>(a.X + row * a.ld) + d);
         for (uint32_t e0 = 0u; good && e0 < tot; e0 += 32u) {
             const uint32_t e = e0 + lane, m = min(32u, tot - e0);
-            const uint32_t cand = e < tot ? (e < m0 ? b0[e] : b1[e - m0]) : 0u;
+            uint32_t cand = e < tot ? (e < m0 ? b0[e] : b1[e - m0]) : 0u;
+            // (a padding column passes the filter only where its terms are NaN)
+            const bool real = e < tot && cand < (uint32_t)a.n;
+            if (!real) cand = 0u;
             __syncwarp();
             tc::fence_proxy_async();
             if (lane == 0) tc::mbar_expect_tx(bar, m * bytes);
@@ -598,7 +601,7 @@ __global__ void __launch_bounds__(kPickWarps * 32) k_knn_pick(const PickArgs a) 
                 t = u.w - v.w;
                 s = fmaf(t, t, s);
             }
-            const bool in = e < tot && s <= tau;
+            const bool in = real && s <= tau;
             const unsigned im = __ballot_sync(0xffffffffu, in);
             const uint32_t at = kept + __popc(im & ((1u << lane) - 1u));
             if (in && at < (uint32_t)kPickKeys)
