@@ -188,7 +188,7 @@ def group_bytes(n, nnz, L, nonempty=None, occupied=None):
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) from an
 # ncu capture of the current kernels, by (workload, n); emptied whenever a
 # kernel changes, until the capture is taken again
-TRAFFIC_BYTES = {("gmm128", 1_000_000): {"k_bh_traverse": 36.42e6 + 1.82e6}}
+TRAFFIC_BYTES = {("gmm128", 1_000_000): {"k_bh_traverse": 36.42e6 + 1.79e6}}
 TRAFFIC_SOURCE = ("profiles/traversal_gmm128_n1M_dram.md (one-pass ncu capture of the "
                   "9th launch, t about 2)")
 

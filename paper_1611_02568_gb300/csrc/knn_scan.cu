@@ -7,7 +7,7 @@
 // kScanStride-th in the locality order, so every neighbourhood is sampled in
 // proportion) finds, per row, the r-th smallest approximate distance to the
 // sample: a threshold tau that with r = k / 8 + 3.75 sigma + 1 lies above the
-// true k-th distance for all but two rows in 10^4, and that about 8 r rows
+// true k-th distance for all but two rows in 10^4 at most, and that about 8 r rows
 // reach.  The second pass has that threshold from its first tile on: it keeps
 // no list, every candidate whose rigorous bound (below) does not exceed tau is
 // appended to the row's buffer in global memory, and two CTAs fit on an SM.
@@ -670,9 +670,10 @@ __global__ void __launch_bounds__(kPickWarps * 32) k_knn_pick(const PickArgs a) 
 }
 
 // Entries of a sample list: of the k nearest, k / kScanStride are in the sample
-// on average; 3.75 standard deviations and one more leave a chance of about
-// 2e-4 per row that the threshold comes out below the k-th distance (the tile
-// is then scanned again, about 3 % of them; four and a half deviations would
+// on average; 3.75 standard deviations and one more leave a chance of at most
+// 2e-4 per row that the threshold comes out below the k-th distance, less than
+// that where the locality order spreads the sample evenly (the tile is then scanned
+// again: 0.65 % of them at n = 1M, 0.9 % at 10M; four and a half deviations would
 // spare that but bring 12 % more candidates to every row).
 int sample_rank(int k) {
     const double m = (double)k / kScanStride;

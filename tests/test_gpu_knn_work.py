@@ -2,9 +2,9 @@
 tile pairs, the products formed, and the query tiles that the two-pass search
 scanned again or left to the one-pass search.
 
-Bars: counts, exactly.  A row's threshold comes out short with a chance of about
-2e-4, so that of 60,000 rows about 12 send their tile to the second scan (none:
-a chance of 6e-6); a row with more identical partners than its buffer or the
+Bars: counts, exactly.  A row's threshold comes out short with a chance of at most
+2e-4 (5e-5 on the bench's mixtures), so that of these 60,000 rows some send their
+tile to the second scan; a row with more identical partners than its buffer or the
 sort hold must leave its tile."""
 import numpy as np
 import pytest
