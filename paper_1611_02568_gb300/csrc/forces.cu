@@ -10,7 +10,7 @@
 //   k_bh_traverse_pt  the same for small sets, one warp per point
 //   k_attract      attraction over the CSR of P, one warp per row
 //   k_zsum         Z = sum_i Z_i in FP64, fixed summation order
-//   k_kl           Eq. cost_func, FP64 sums of a few terms' float pairs
+//   k_kl           Eq. cost_func, sums in three floats and FP64
 #include <algorithm>
 #include <cmath>
 
@@ -917,28 +917,31 @@ cudaError_t launch_forces(pxsne_ctx *c, cudaEvent_t *marks) {
     return cudaSuccess;
 }
 
-// A sum of a few FP32 terms carried as an unevaluated pair of floats: the rounding
-// error of every addition is found exactly (Knuth's two-sum) and added to the low
-// word, whose own roundings leave an error of at most k^2 2^-50 of the terms'
-// absolute sum after k terms.
-struct FloatPair {
-    float h, l;
-    __device__ __forceinline__ void add(float x) {
-        const float s = __fadd_rn(h, x), b = __fsub_rn(s, h);
-        l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(s, b)), __fsub_rn(x, b)));
-        h = s;
+// A sum of FP32 terms carried as three floats: the rounding error of every
+// addition to one word is found exactly (Knuth's two-sum) and added to the next, and
+// only the last one rounds.  After N terms the error is at most N^3 2^-74 of their
+// absolute sum, which is less than that of N FP64 additions (N 2^-53) up to 1,400
+// terms; with roundings of either sign it is about N^1.5 2^-72 against N^0.5 2^-54.
+struct FloatSum {
+    float h, m, l;
+    static __device__ __forceinline__ float two_sum(float &a, float x) {
+        const float s = __fadd_rn(a, x), b = __fsub_rn(s, a);
+        const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, b)), __fsub_rn(x, b));
+        a = s;
+        return e;
     }
+    __device__ __forceinline__ void add(float x) { l = __fadd_rn(l, two_sum(m, two_sum(h, x))); }
+    __device__ __forceinline__ double sum() const { return (double)h + ((double)m + (double)l); }
 };
 
 // Eq. cost_func: C = sum_ij p_ij ln(p_ij Z / w_ij)
 //                  = sum p (ln p - ln w) + (sum p) ln Z,
-// one warp per row, fixed order: a lane adds up to kKlPairs FP32 terms as float
-// pairs, then those to its FP64 sums, so that what the pairs lose (2^-44 of the
-// terms at most) is no more than what FP64 additions of a lane's several hundred
-// terms would.  (FP64 additions and conversions issue at a small fraction of the
-// FP32 rate; 100,000 points, 13.5M entries: 0.40 ms with two of each per entry
-// and the partials added by one thread.)
-constexpr int kKlPairs = 8;
+// one warp per row, fixed order: a lane's FP32 terms (700 of them at n = 1M) in three
+// floats, FP64 across lanes and blocks.  FP64 additions and conversions issue at a
+// small fraction of the FP32 rate: 100,000 points, 13.5M entries, the whole call
+// 278 us; 284 with two floats, whose error of 2^-37 on a row of 200,000 entries is
+// more than FP64's, 296 with two floats and FP64 after every row (288 with the
+// three); the kernel alone took 400 with two FP64 additions per entry.
 __global__ void __launch_bounds__(256)
     k_kl(int n, const int64_t *__restrict__ rp, const int32_t *__restrict__ col,
          const float *__restrict__ val, const uint2 *__restrict__ z, DevScalars *sc,
@@ -948,29 +951,24 @@ __global__ void __launch_bounds__(256)
     const int lane = threadIdx.x & 31;
     const int warps_total = gridDim.x * (blockDim.x >> 5);
     const float sf0 = sc->sf[0], sf1 = sc->sf[1];
-    double acc = 0.0, psum = 0.0;
+    FloatSum ka{0.f, 0.f, 0.f}, kp{0.f, 0.f, 0.f};
     for (int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); row < n;
          row += warps_total) {
         const uint2 zi = z[row];
         const float xh = hi_bits(zi.x), xl = lo_bits(zi.x);
         const float yh = hi_bits(zi.y), yl = lo_bits(zi.y);
         const int64_t e1 = rp[row + 1];
-        for (int64_t e0 = rp[row] + lane; e0 < e1; e0 += 32 * kKlPairs) {
-            FloatPair a8{0.f, 0.f}, p8{0.f, 0.f};
-            const int64_t e8 = min(e1, e0 + 32 * kKlPairs);
-            for (int64_t e = e0; e < e8; e += 32) {
-                const float p = __ldcs(val + e);
-                const uint2 zj = z[__ldcs(col + e)];
-                if (!(p > 0.f)) continue;
-                const float dx = ((xh - hi_bits(zj.x)) + (xl - lo_bits(zj.x))) * sf0;
-                const float dy = ((yh - hi_bits(zj.y)) + (yl - lo_bits(zj.y))) * sf1;
-                a8.add(p * (logf(p) + log1pf(fmaf(dx, dx, dy * dy))));
-                p8.add(p);
-            }
-            acc += (double)a8.h + (double)a8.l;
-            psum += (double)p8.h + (double)p8.l;
+        for (int64_t e = rp[row] + lane; e < e1; e += 32) {
+            const float p = __ldcs(val + e);
+            const uint2 zj = z[__ldcs(col + e)];
+            if (!(p > 0.f)) continue;
+            const float dx = ((xh - hi_bits(zj.x)) + (xl - lo_bits(zj.x))) * sf0;
+            const float dy = ((yh - hi_bits(zj.y)) + (yl - lo_bits(zj.y))) * sf1;
+            ka.add(p * (logf(p) + log1pf(fmaf(dx, dx, dy * dy))));
+            kp.add(p);
         }
     }
+    const double acc = ka.sum(), psum = kp.sum();
     const double a = block_sum_f64(acc, s_red);
     const double ps = block_sum_f64(psum, s_red);
     if (threadIdx.x == 0) {

@@ -1,8 +1,8 @@
 """The KL's sums over P keep 64 bits: the KL of a P whose one long row has values
 over twelve decades equals the sum of the KLs of its even and its odd entries,
 whose FP32 terms are the same.  Bar: 2^-42 of the terms' absolute sum (each of
-the three sums is off by at most 2^-44 of its terms in its pairs of floats and a
-few units of FP64; about 2^-38 with a pair of floats over a lane's whole share)."""
+the three sums is off by about 2^-53 of its terms in its three floats and a few
+units of FP64; about 2^-38 with two floats)."""
 import numpy as np
 import pytest
 
