@@ -552,8 +552,10 @@ __device__ __forceinline__ void take_out3(int slot, float2 &N, float2 (&dx)[3]) 
 
 // Cells of one point are accepted by all others by the same rule as in 2-D
 // (single_base, common.cuh).
-__device__ __forceinline__ bool tiny3(const float2 (&s)[3]) {
-    return underflows(s[0].x) || underflows(s[1].x) || underflows(s[2].x);
+template <bool OWN>
+__device__ __forceinline__ float base3(const DevScalars *sc) {
+    return single_base(OWN || underflows(sc->sf3[0]) || underflows(sc->sf3[1]) ||
+                       underflows(sc->sf3[2]));
 }
 // What a point (its voxel's Morton index mi) has to take out of its sum.
 template <bool OWN>
@@ -574,8 +576,8 @@ __global__ void __launch_bounds__(kT3Warps * 32, 4)
                 const float4 *__restrict__ rec, DevScalars *sc, float4 *__restrict__ Frep,
                 float *__restrict__ Zi) {
     __shared__ T3Entry s_stk[kT3Warps][kT3Stack];
-    __shared__ float s_T[kMaxL + 2];
-    if (threadIdx.x < kMaxL + 2) s_T[threadIdx.x] = sc->T3[threadIdx.x];
+    __shared__ float2 s_T[kMaxL + 2];  // a level's threshold on d^2, and single_base
+    if (threadIdx.x < kMaxL + 2) s_T[threadIdx.x] = make_float2(sc->T3[threadIdx.x], base3<OWN>(sc));
     __syncthreads();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int idx = (blockIdx.x * kT3Warps + w) * 32 + lane;
@@ -589,7 +591,6 @@ __global__ void __launch_bounds__(kT3Warps * 32, 4)
     const uint32_t own_grp = (uint32_t)off3(L - 1) + (mi >> 3);
     const Point3 pt = point3(zi);
     const float2 s[3] = {b3(sc->sf3[0]), b3(sc->sf3[1]), b3(sc->sf3[2])};
-    const float base = single_base(OWN || tiny3(s));
     Sum3 a{{b3(0.f), b3(0.f), b3(0.f)}, b3(0.f)};
     T3Entry *stk = s_stk[w];
     if (lane == 0) stk[0] = T3Entry{1u << 28, act};  // the root's children: level 1, group 0
@@ -634,7 +635,8 @@ __global__ void __launch_bounds__(kT3Warps * 32, 4)
                 }
             }
         } else {
-            const float Tl = s_T[lc];
+            const float2 Tb = s_T[lc];
+            const float Tl = Tb.x, base = OWN ? single_base(true) : Tb.y;
             const uint32_t mine = OWN ? mi >> (3 * (L - lc)) : 0u;
             const uint32_t first = OWN ? 8u * (grp - (uint32_t)off3(lc - 1)) : 0u;
             if (sp + 8 > kT3Stack) {
@@ -681,7 +683,7 @@ __global__ void __launch_bounds__(kT3Warps * 32, 4)
     }
     if (valid) {
         Frep[i] = make_float4(a.f[0].x + a.f[0].y, a.f[1].x + a.f[1].y, a.f[2].x + a.f[2].y, 0.f);
-        Zi[i] = a.z.x + a.z.y - own_single3<OWN>(base, rec, L, mi);
+        Zi[i] = a.z.x + a.z.y - own_single3<OWN>(s_T[0].y, rec, L, mi);
     }
     if (overflow && lane == 0) atomicOr(&sc->err, (unsigned)PXSNE_DEVERR_STACK);
 }
@@ -715,7 +717,7 @@ __global__ void __launch_bounds__(kPt3Warps * 32)
     const uint32_t own_grp = (uint32_t)off3(L - 1) + (mi >> 3);
     const Point3 pt = point3(zi);
     const float2 s[3] = {b3(sc->sf3[0]), b3(sc->sf3[1]), b3(sc->sf3[2])};
-    const float base = single_base(OWN || tiny3(s));
+    const float base = base3<OWN>(sc);
     Sum3 a{{b3(0.f), b3(0.f), b3(0.f)}, b3(0.f)};
     const unsigned before = (1u << lane) - 1u;
     if (lane == 0) ring[0] = 1u << 28;
